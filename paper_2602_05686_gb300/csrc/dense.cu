@@ -1,13 +1,23 @@
 // Coarsest level (Sec. 4: the coarsest level is solved directly).  A_L
-// (n_L <= a few thousand) is densified and factored A_L = L L^T by a blocked
-// right-looking Cholesky in FP64 (32 x 32 tiles); then the inverses of the
-// diagonal blocks of COARSE_BS rows, W_KK = L_KK^-1, are formed by blocked
-// forward substitution on the identity.  Every coarse solve is block
-// substitution: per diagonal block a row-parallel product with the blocks
-// already solved and one with W_KK (forward with L, backward with L^T and
-// W_KK^T), so it uses every SM instead of running row-by-row sweeps.  L^T and
-// W^T are stored explicitly so all products read contiguous rows.
+// (n_L <= a few thousand) is factored A_L = L L^T by a tiled Cholesky in FP64
+// (32 x 32 tiles) inside its skyline; then the inverses of the diagonal
+// blocks of COARSE_BS rows, W_KK = L_KK^-1, are formed by blocked forward
+// substitution on the identity.  Every coarse solve is block substitution:
+// per diagonal block a row-parallel product with the blocks already solved
+// and one with W_KK (forward with L, backward with L^T and W_KK^T), so it uses
+// every SM instead of running row-by-row sweeps.  L^T and W^T are stored
+// explicitly so all products read contiguous rows.
+//
+// Skyline: Cholesky without pivoting creates no entry left of a row's first
+// nonzero, so with f_i the first nonzero tile column of tile row i, L_ij = 0
+// for j < f_i, and a product of a zero tile changes nothing.  Factor, inverses
+// and solve skip those tiles.  The coarse operators are numbered along the
+// mesh (aggregates by ascending root index), so their skylines hold 0.06
+// (4225-row square) to 0.45 (3989-row 3D level) of the lower triangle and
+// 0.002 to 0.16 of the dense factor's tile products.
 #include <math.h>
+
+#include <vector>
 
 #include "common.cuh"
 #include "profile.cuh"
@@ -17,246 +27,337 @@
 namespace sa {
 
 constexpr int NB = 32;
+constexpr int CH_THREADS = 256;
+constexpr int CH_STRIP = 16;             // columns of one inverse task
+constexpr int CH_BT = (int)(COARSE_BS / NB);  // tiles per diagonal block
+constexpr uint32_t CH_INV = 0x80000000u;      // task word of an inverse strip
 
-__global__ void k_densify(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                          const double* __restrict__ v, double* __restrict__ M) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  for (int64_t p = rp[i]; p < rp[i + 1]; ++p) M[i * n + ci[p]] = v[p];
-}
-
-__global__ void k_set_identity(int64_t n, double* __restrict__ W) {
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n * n) W[t] = (t / n == t % n) ? 1.0 : 0.0;
-}
-
-// factor the diagonal tile (k,k) in place (err = 1 on a non-positive pivot)
-// and write the inverse of the factored tile, L_kk^-1 (lower triangular), to
-// Dinv + k NB^2: the panel and inverse solves then become tile products
-__global__ void k_potrf_diag(int64_t n, double* __restrict__ M, int k, int* __restrict__ err,
-                             double* __restrict__ Dinv) {
-  __shared__ double T[NB][NB + 1];
-  __shared__ double rinv[NB];
-  const int64_t o = (int64_t)k * NB;
-  const int bs = (int)((n - o) < NB ? (n - o) : NB);
-  for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
-    int r = t / NB, c = t % NB;
-    T[r][c] = (r < bs && c < bs) ? M[(o + r) * n + o + c] : 0.0;
+// f[i]: first nonzero tile column of tile row i (columns ascend, the first
+// entry of a row is its smallest column; at most the diagonal tile)
+__global__ void k_sky_first(int64_t n, int nb, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                            int32_t* __restrict__ f) {
+  const int i = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
+  if (i >= nb) return;
+  const int64_t r = (int64_t)i * NB + (threadIdx.x & 31);
+  int c = i;
+  if (r < n && rp[r + 1] > rp[r]) {
+    const int t = ci[rp[r]] / NB;
+    c = t < i ? t : i;
   }
+  c = __reduce_min_sync(FULL, c);
+  if ((threadIdx.x & 31) == 0) f[i] = c;
+}
+
+// the skyline of tile row blockIdx.x as dense rows: zeros, then the entries of
+// the lower triangle (and of the diagonal tile)
+__global__ void k_densify_sky(int64_t n, const int32_t* __restrict__ f, const int64_t* __restrict__ rp,
+                              const int32_t* __restrict__ ci, const double* __restrict__ v, double* __restrict__ M) {
+  const int64_t o = (int64_t)blockIdx.x * NB;
+  const int64_t c0 = (int64_t)f[blockIdx.x] * NB, c1 = o + NB < n ? o + NB : n;
+  const int64_t r1 = o + NB < n ? o + NB : n;
+  for (int64_t r = o; r < r1; ++r)
+    for (int64_t c = c0 + threadIdx.x; c < c1; c += blockDim.x) M[r * n + c] = 0.0;
   __syncthreads();
-  for (int j = 0; j < bs; ++j) {
-    if (threadIdx.x == 0) {
-      double d = T[j][j];
-      if (!(d > 0.0)) { atomicOr(err, 1); d = 1.0; }
-      d = sqrt(d);
-      T[j][j] = d;
-      rinv[j] = 1.0 / d;
+  const int w = (int)(threadIdx.x >> 5), nw = (int)(blockDim.x >> 5), lane = lane_id();
+  for (int64_t r = o + w; r < r1; r += nw)
+    for (int64_t p = rp[r] + lane; p < rp[r + 1]; p += 32) {
+      const int32_t c = ci[p];
+      if (c < c1) M[r * n + c] = v[p];
     }
-    __syncthreads();
-    const double ri = rinv[j];
-    for (int r = j + 1 + threadIdx.x; r < bs; r += blockDim.x) T[r][j] *= ri;
-    __syncthreads();
-    // thread (warp w, lane r) owns T[r][w + 8q], q = 0..3 (256 threads)
-    {
-      const int r = (int)(threadIdx.x & 31), w = (int)(threadIdx.x >> 5);
-      if (r > j && r < bs) {
-        const double lrj = T[r][j];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int c = w + 8 * q;
-          if (c > j && c <= r) T[r][c] -= lrj * T[c][j];
+}
+
+struct CholView {
+  int64_t n;
+  int nb;
+  const int32_t* f;      // first tile column of each tile row
+  const int32_t* off;    // flag index of tile (i, f_i); tile (i, j) at off[i] + j - f[i]
+  const uint32_t* task;
+  int ntask;
+  double *M, *LT, *W, *WT, *Dinv;
+  int* flag;             // 1: the tile of L is written (and, on the diagonal, its inverse)
+  int* ticket;
+  int* err;              // 1: pivot not positive; 2: a wait ran out
+};
+
+// bounded wait of one thread for *p: false when it ran out or another wait did
+__device__ bool ch_poll(const int* p, int* err) {
+  for (int it = 0; it < (1 << 24); ++it) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    if (v) return true;
+    if (it > 64) {
+      __nanosleep(64);
+      if ((it & 1023) == 0 && (*(volatile int*)err & 2)) return false;
+    }
+  }
+  atomicOr(err, 2);
+  return false;
+}
+
+__device__ __forceinline__ void ch_publish(int* p) {
+  // the block's writes are ordered before the flag: barrier (by the caller),
+  // then this thread's fence and release
+  __threadfence();
+  asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(1) : "memory");
+}
+
+// factor the tile in T (rows and columns < bs) in place and form its inverse
+// in Y (lower triangular, zero elsewhere).  What bounds it is the chain
+// sqrt -> 1/x -> scale -> update of the next pivot, about 1490 cycles per
+// column of FP64 latency (dependent DFMA 65 cycles, sqrt 640, divide 606,
+// measured), so warp 0 runs only that chain (a row per lane) while the other
+// warps apply the previous column to the columns right of the next one and
+// form the previous row of the inverse; one barrier per column.  Warp 4
+// shares warp 0's scheduler (and its FP64 issue) and stays idle.
+__device__ __forceinline__ void potrf_inv(int bs, double (*T)[NB + 1], double (*Y)[NB + 1], double* rinv, int* err) {
+  const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
+  double l = 0.0;  // warp 0: row `lane` of the previous column of L
+  for (int j = 0; j <= bs; ++j) {
+    if (warp == 0) {
+      if (j < bs) {
+        double t = T[lane][j];
+        if (j > 0) {
+          const double lj = __shfl_sync(FULL, l, j);
+          if (lane >= j) t = fma(-l, lj, t);
+        }
+        double d = __shfl_sync(FULL, t, j);
+        if (!(d > 0.0)) {
+          if (lane == 0) atomicOr(err, 1);
+          d = 1.0;
+        }
+        d = sqrt(d);
+        const double ri = 1.0 / d;
+        l = lane == j ? d : (lane > j ? t * ri : 0.0);
+        if (lane >= j) T[lane][j] = l;
+        if (lane == 0) rinv[j] = ri;
+      }
+    } else if (warp != 4 && j > 0) {
+      const int m = j - 1, wi = warp < 4 ? warp - 1 : warp - 2;
+      const int nd = (m >> 2) + 1;                      // groups of four columns of the inverse's row m
+      const int nu = bs - (j + 1) > 0 ? bs - (j + 1) : 0;  // columns j + 1 ... of the update
+      for (int it = wi; it < nd + nu; it += 6) {
+        if (it < nd) {
+          // row m of the inverse by forward substitution, L y = e_c: eight
+          // lanes per column split the dot product
+          const int c = it * 4 + (lane >> 3), g = lane & 7;
+          double part = 0.0;
+          if (m > c)
+            for (int q = c + g; q < m; q += 8) part = fma(T[m][q], Y[q][c], part);
+          part += __shfl_xor_sync(FULL, part, 4, 8);
+          part += __shfl_xor_sync(FULL, part, 2, 8);
+          part += __shfl_xor_sync(FULL, part, 1, 8);
+          if (g == 0 && c <= m) Y[m][c] = ((m == c ? 1.0 : 0.0) - part) * rinv[m];
+        } else {
+          const int q = j + 1 + (it - nd);
+          if (lane >= q && lane < bs) T[lane][q] = fma(-T[lane][m], T[q][m], T[lane][q]);
         }
       }
     }
     __syncthreads();
   }
-  for (int t = threadIdx.x; t < bs * bs; t += blockDim.x) {
-    int r = t / bs, c = t % bs;
-    M[(o + r) * n + o + c] = (c <= r) ? T[r][c] : 0.0;
-  }
-  // inverse by forward substitution, L y = e_c for every column c: eight
-  // threads per column (one warp holds four columns) split each row's dot
-  // product and combine it with shuffles
-  __shared__ double Y[NB][NB + 1];
-  {
-    const int c = threadIdx.x >> 3, g = threadIdx.x & 7;
-    for (int r = 0; r < NB; ++r) {
-      double part = 0.0;
-      if (r < bs && c < bs && r > c)
-        for (int q = c + g; q < r; q += 8) part += T[r][q] * Y[q][c];
-      part += __shfl_xor_sync(FULL, part, 4, 8);
-      part += __shfl_xor_sync(FULL, part, 2, 8);
-      part += __shfl_xor_sync(FULL, part, 1, 8);
-      if (g == 0) {
-        double y = 0.0;
-        if (r < bs && c < bs && r >= c) y = ((r == c ? 1.0 : 0.0) - part) * rinv[r];
-        Y[r][c] = y;
+}
+
+// One launch factors the matrix and inverts its diagonal blocks.  A task is
+// one tile of L (left-looking: all its products, then its solve or its own
+// factor) or a strip of CH_STRIP columns of one W_KK; tasks are numbered so
+// that a task reads only tiles of lower-numbered tasks, CTAs draw tickets in
+// that order and wait (bounded) on the tiles' flags.  The lowest unfinished
+// task never waits for one that no CTA has drawn, so the launch makes
+// progress with any number of resident CTAs.
+// Every tile sees the products of the blocked right-looking form in the same
+// order (per product a sum over the tile's 32 columns, subtracted from the
+// tile; tile columns ascending), so the factor is bitwise that form's.
+// Before: one launch per panel step and two more streams, a diagonal tile in
+// a single CTA's 45 us; 4225-row square 34.4 ms, 814 rows 3.9 ms, 3528 rows
+// 35.1 ms.
+__global__ void __launch_bounds__(CH_THREADS) k_chol(CholView C) {
+  __shared__ double As[2][NB][NB + 1];
+  __shared__ double Bs[2][NB][NB + 1];
+  __shared__ double rinv[NB];
+  __shared__ int s_task;
+  const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t n = C.n;
+  for (;;) {
+    __syncthreads();  // the previous task's reads of shared memory
+    if (tid == 0) s_task = atomicAdd(C.ticket, 1);
+    __syncthreads();
+    const int tk = s_task;
+    if (tk >= C.ntask) return;
+    const uint32_t tw = C.task[tk];
+    if (tw & CH_INV) {
+      // columns c0 .. c0 + CH_STRIP - 1 of W_KK: for tile rows i downwards
+      // X = (I)_i - sum_m L_im W_m,  W_i = L_ii^-1 X
+      const int q = (int)((tw >> 16) & 0x7fff), s = (int)(tw & 0xffff);
+      const int64_t c0 = (int64_t)q * COARSE_BS + (int64_t)s * CH_STRIP;
+      const int jt = (int)(c0 / NB);
+      const int e = (q + 1) * CH_BT < C.nb ? (q + 1) * CH_BT : C.nb;
+      const int cw = (int)(n - c0 < CH_STRIP ? n - c0 : CH_STRIP);
+      const int r = tid >> 4, c = tid & 15;  // outputs (r, c) and (r + 16, c)
+      int buf = 0;
+      for (int i = jt; i < e; ++i) {
+        const int64_t oi = (int64_t)i * NB;
+        const int bi = (int)(n - oi < NB ? n - oi : NB);
+        const int fi = C.f[i];
+        double x0 = c0 + c == oi + r ? 1.0 : 0.0, x1 = c0 + c == oi + r + 16 ? 1.0 : 0.0;
+        for (int m = fi > jt ? fi : jt; m < i; ++m) {
+          const bool ok = tid != 0 || ch_poll(&C.flag[C.off[i] + m - fi], C.err);
+          if (!__syncthreads_and(ok)) return;
+          const int64_t om = (int64_t)m * NB;
+          for (int t = tid; t < NB * NB; t += CH_THREADS) {
+            const int a = t / NB, b = t % NB;
+            As[buf][a][b] = a < bi ? __ldcg(&C.M[(oi + a) * n + om + b]) : 0.0;
+          }
+          for (int t = tid; t < NB * CH_STRIP; t += CH_THREADS) {
+            const int a = t / CH_STRIP, b = t % CH_STRIP;
+            Bs[buf][a][b] = b < cw ? __ldcg(&C.W[(om + a) * n + c0 + b]) : 0.0;
+          }
+          __syncthreads();
+          double s0 = 0.0, s1 = 0.0;
+#pragma unroll 8
+          for (int u = 0; u < NB; ++u) {
+            const double b = Bs[buf][u][c];
+            s0 = fma(As[buf][r][u], b, s0);
+            s1 = fma(As[buf][r + 16][u], b, s1);
+          }
+          x0 -= s0;
+          x1 -= s1;
+          buf ^= 1;
+        }
+        const bool ok = tid != 0 || ch_poll(&C.flag[C.off[i] + i - fi], C.err);
+        if (!__syncthreads_and(ok)) return;
+        const double* D = C.Dinv + (int64_t)i * NB * NB;
+        for (int t = tid; t < NB * NB; t += CH_THREADS) As[buf][t / NB][t % NB] = __ldcg(&D[t]);
+        Bs[buf][r][c] = x0;
+        Bs[buf][r + 16][c] = x1;
+        __syncthreads();
+        double w0 = 0.0, w1 = 0.0;
+        for (int u = 0; u <= r; ++u) w0 = fma(As[buf][r][u], Bs[buf][u][c], w0);
+        for (int u = 0; u <= r + 16; ++u) w1 = fma(As[buf][r + 16][u], Bs[buf][u][c], w1);
+        if (c < cw) {
+          if (r < bi) {
+            C.W[(oi + r) * n + c0 + c] = w0;
+            C.WT[(c0 + c) * n + oi + r] = w0;
+          }
+          if (r + 16 < bi) {
+            C.W[(oi + r + 16) * n + c0 + c] = w1;
+            C.WT[(c0 + c) * n + oi + r + 16] = w1;
+          }
+        }
+        buf ^= 1;
+        __syncthreads();  // this strip's rows of W before they are read back
       }
-      __syncwarp();
+      continue;
     }
-  }
-  __syncthreads();
-  double* D = Dinv + (int64_t)k * NB * NB;
-  for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) D[t] = Y[t / NB][t % NB];
-}
-
-// L_ik = A_ik L_kk^-T for block rows i > k: a tile product with the stored
-// L_kk^-1 (one CTA of 256 threads per block row, 4 outputs per thread)
-__global__ void k_trsm_panel(int64_t n, double* __restrict__ M, int k, const double* __restrict__ Dinv) {
-  __shared__ double Li[NB][NB + 1];
-  __shared__ double X[NB][NB + 1];
-  const int64_t ok = (int64_t)k * NB;
-  const int bk = (int)((n - ok) < NB ? (n - ok) : NB);
-  const int64_t oi = (int64_t)(k + 1 + blockIdx.x) * NB;
-  const int bi = (int)((n - oi) < NB ? (n - oi) : NB);
-  const double* D = Dinv + (int64_t)k * NB * NB;
-  for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
-    int r = t / NB, c = t % NB;
-    Li[r][c] = D[t];
-    X[r][c] = (r < bi && c < bk) ? M[(oi + r) * n + ok + c] : 0.0;
-  }
-  __syncthreads();
-  double out[NB * NB / 256];
+    const int i = (int)(tw >> 15), j = (int)(tw & 0x7fff);
+    const int fi = C.f[i], fj = C.f[j];
+    const int64_t oi = (int64_t)i * NB, oj = (int64_t)j * NB;
+    const int bi = (int)(n - oi < NB ? n - oi : NB), bj = (int)(n - oj < NB ? n - oj : NB);
+    const bool diag = i == j;
+    // this thread's elements of the tile: off the diagonal rows warp + 8u of
+    // column `lane`; on it the lower triangle's 528 elements in order
+    int er[4], ec[4];
+    double acc[4];
 #pragma unroll
-  for (int u = 0; u < NB * NB / 256; ++u) {
-    const int t = threadIdx.x + u * 256, r = t / NB, c = t % NB;
-    double acc = 0.0;  // (L^-T)_qc = (L^-1)_cq, nonzero for q <= c
-    for (int q = 0; q <= c; ++q) acc += X[r][q] * Li[c][q];
-    out[u] = acc;
-  }
-  __syncthreads();
+    for (int u = 0; u < 4; ++u) {
+      er[u] = warp + 8 * u;
+      ec[u] = lane;
+      if (diag) {
+        const int t = tid + CH_THREADS * u;
+        int a = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+        while ((a + 1) * (a + 2) / 2 <= t) ++a;
+        while (a * (a + 1) / 2 > t) --a;
+        er[u] = a;
+        ec[u] = t - a * (a + 1) / 2;
+      }
+      acc[u] = er[u] < bi && ec[u] < bj ? __ldcg(&C.M[(oi + er[u]) * n + oj + ec[u]]) : 0.0;
+    }
+    int buf = 0;
+    for (int k = fi > fj ? fi : fj; k < j; ++k) {
+      bool ok = true;
+      if (tid == 0) ok = ch_poll(&C.flag[C.off[i] + k - fi], C.err);
+      if (tid == 32 && !diag) ok = ch_poll(&C.flag[C.off[j] + k - fj], C.err);
+      if (!__syncthreads_and(ok)) return;
+      const int64_t ok_ = (int64_t)k * NB;
+      for (int t = tid; t < NB * NB; t += CH_THREADS) {
+        const int a = t / NB, b = t % NB;
+        As[buf][a][b] = a < bi ? __ldcg(&C.M[(oi + a) * n + ok_ + b]) : 0.0;
+        if (!diag) Bs[buf][a][b] = a < bj ? __ldcg(&C.M[(oj + a) * n + ok_ + b]) : 0.0;
+      }
+      __syncthreads();
+      if (diag) {
 #pragma unroll
-  for (int u = 0; u < NB * NB / 256; ++u) {
-    const int t = threadIdx.x + u * 256, r = t / NB, c = t % NB;
-    if (r < bi && c < bk) M[(oi + r) * n + ok + c] = out[u];
-  }
-}
-
-__device__ __forceinline__ void tri_index(int64_t idx, int* ti, int* tj) {
-  // idx -> (ti, tj) with 0 <= tj <= ti, idx = ti (ti+1) / 2 + tj
-  int t = (int)((sqrt(8.0 * (double)idx + 1.0) - 1.0) * 0.5);
-  while ((int64_t)(t + 1) * (t + 2) / 2 <= idx) ++t;
-  while ((int64_t)t * (t + 1) / 2 > idx) --t;
-  *ti = t;
-  *tj = (int)(idx - (int64_t)t * (t + 1) / 2);
-}
-
-// C -= A B^T on one NB x NB tile; 256 threads, 4 outputs each
-__device__ __forceinline__ void tile_gemm_nt_sub(int64_t n, double* __restrict__ M, int64_t oc_r, int64_t oc_c,
-                                                 int br, int bc, const double* __restrict__ Abase, int64_t oa_r,
-                                                 int64_t oa_c, const double* __restrict__ Bbase, int64_t ob_r,
-                                                 int64_t ob_c, int bkk, int64_t lda, int64_t ldb) {
-  __shared__ double As[NB][NB + 1];
-  __shared__ double Bs[NB][NB + 1];
-  for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
-    int r = t / NB, c = t % NB;
-    As[r][c] = (r < br && c < bkk) ? Abase[(oa_r + r) * lda + oa_c + c] : 0.0;
-    Bs[r][c] = (r < bc && c < bkk) ? Bbase[(ob_r + r) * ldb + ob_c + c] : 0.0;
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
-    int r = t / NB, c = t % NB;
-    if (r < br && c < bc) {
-      double s = 0.0;
+        for (int u = 0; u < 3; ++u) {
+          if (er[u] < NB) {
+            double s = 0.0;
 #pragma unroll 8
-      for (int m = 0; m < NB; ++m) s += As[r][m] * Bs[c][m];
-      M[(oc_r + r) * n + oc_c + c] -= s;
-    }
-  }
-}
-
-// trailing update after panel k: A_ij -= L_ik L_jk^T for tiles first <= j <= i
-// (col_only: the tiles of block column j = first only)
-__global__ void k_syrk_update(int64_t n, double* __restrict__ M, int k, int first, int col_only) {
-  int ti, tj;
-  if (col_only) {
-    ti = (int)blockIdx.x;
-    tj = 0;
-  } else {
-    tri_index(blockIdx.x, &ti, &tj);
-  }
-  const int i = first + ti, j = first + tj;
-  const int64_t oi = (int64_t)i * NB, oj = (int64_t)j * NB, ok = (int64_t)k * NB;
-  const int bi = (int)((n - oi) < NB ? (n - oi) : NB);
-  const int bj = (int)((n - oj) < NB ? (n - oj) : NB);
-  const int bk = (int)((n - ok) < NB ? (n - ok) : NB);
-  tile_gemm_nt_sub(n, M, oi, oj, bi, bj, M, oi, ok, M, oj, ok, bk, n, n);
-}
-
-// W_ij <- L_ii^-1 W_ij for block columns j0 <= j <= i, a tile product with
-// the stored L_ii^-1 (one CTA of 256 threads per j, 4 outputs per thread)
-__global__ void k_trsm_lower_left(int64_t n, const double* __restrict__ Dinv, double* __restrict__ W, int i,
-                                  int j0) {
-  __shared__ double Li[NB][NB + 1];
-  __shared__ double X[NB][NB + 1];
-  const int j = j0 + (int)blockIdx.x;
-  const int64_t oi = (int64_t)i * NB, oj = (int64_t)j * NB;
-  const int bi = (int)((n - oi) < NB ? (n - oi) : NB);
-  const int bj = (int)((n - oj) < NB ? (n - oj) : NB);
-  const double* D = Dinv + (int64_t)i * NB * NB;
-  for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
-    int r = t / NB, c = t % NB;
-    Li[r][c] = D[t];
-    X[r][c] = (r < bi && c < bj) ? W[(oi + r) * n + oj + c] : 0.0;
-  }
-  __syncthreads();
-  double out[NB * NB / 256];
-#pragma unroll
-  for (int u = 0; u < NB * NB / 256; ++u) {
-    const int t = threadIdx.x + u * 256, r = t / NB, c = t % NB;
-    double acc = 0.0;
-    for (int q = 0; q <= r; ++q) acc += Li[r][q] * X[q][c];
-    out[u] = acc;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int u = 0; u < NB * NB / 256; ++u) {
-    const int t = threadIdx.x + u * 256, r = t / NB, c = t % NB;
-    if (r < bi && c < bj) W[(oi + r) * n + oj + c] = out[u];
-  }
-}
-
-// W_mj -= L_mi W_ij for block rows m >= m0 (m0 > i), block columns
-// j0 <= j < j0 + ncolb (j <= i)
-__global__ void k_gemm_left(int64_t n, const double* __restrict__ L, double* __restrict__ W, int i, int ncolb,
-                            int m0, int j0) {
-  const int m = m0 + (int)blockIdx.x / ncolb;
-  const int j = j0 + (int)blockIdx.x % ncolb;
-  const int64_t om = (int64_t)m * NB, oi = (int64_t)i * NB, oj = (int64_t)j * NB;
-  const int bm = (int)((n - om) < NB ? (n - om) : NB);
-  const int bi = (int)((n - oi) < NB ? (n - oi) : NB);
-  const int bj = (int)((n - oj) < NB ? (n - oj) : NB);
-  __shared__ double As[NB][NB + 1];
-  __shared__ double Bs[NB][NB + 1];
-  for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
-    int r = t / NB, c = t % NB;
-    As[r][c] = (r < bm && c < bi) ? L[(om + r) * n + oi + c] : 0.0;   // L_mi
-    Bs[r][c] = (r < bi && c < bj) ? W[(oi + r) * n + oj + c] : 0.0;   // W_ij
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
-    int r = t / NB, c = t % NB;
-    if (r < bm && c < bj) {
-      double s = 0.0;
+            for (int m = 0; m < NB; ++m) s = fma(As[buf][er[u]][m], As[buf][ec[u]][m], s);
+            acc[u] -= s;
+          }
+        }
+      } else {
+        double s[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 8
-      for (int q = 0; q < NB; ++q) s += As[r][q] * Bs[q][c];
-      W[(om + r) * n + oj + c] -= s;
+        for (int m = 0; m < NB; ++m) {
+          const double b = Bs[buf][lane][m];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) s[u] = fma(As[buf][warp + 8 * u][m], b, s[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[u] -= s[u];
+      }
+      buf ^= 1;
     }
-  }
-}
-
-__global__ void k_transpose_dense(int64_t n, const double* __restrict__ W, double* __restrict__ WT) {
-  __shared__ double t[32][33];
-  int64_t bx = (int64_t)blockIdx.x * 32, by = (int64_t)blockIdx.y * 32;
-  int x = threadIdx.x, y = threadIdx.y;
-  for (int k = y; k < 32; k += 8) {
-    int64_t r = by + k, c = bx + x;
-    t[k][x] = (r < n && c < n) ? W[r * n + c] : 0.0;
-  }
-  __syncthreads();
-  for (int k = y; k < 32; k += 8) {
-    int64_t r = bx + k, c = by + x;
-    if (r < n && c < n) WT[r * n + c] = t[x][k];
+    double(*T)[NB + 1] = As[buf];
+    double(*Y)[NB + 1] = Bs[buf];
+    if (diag) {
+      for (int t = tid; t < NB * NB; t += CH_THREADS) {
+        T[t / NB][t % NB] = 0.0;
+        Y[t / NB][t % NB] = 0.0;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < 3; ++u)
+        if (er[u] < NB) T[er[u]][ec[u]] = acc[u];
+      __syncthreads();
+      potrf_inv(bi, T, Y, rinv, C.err);
+      double* D = C.Dinv + (int64_t)i * NB * NB;
+      for (int t = tid; t < NB * NB; t += CH_THREADS) {
+        const int a = t / NB, b = t % NB;
+        D[t] = Y[a][b];
+        if (a < bi && b < bi) {
+          C.M[(oi + a) * n + oi + b] = b <= a ? T[a][b] : 0.0;
+          C.LT[(oi + a) * n + oi + b] = a <= b ? T[b][a] : 0.0;
+        }
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) T[er[u]][ec[u]] = acc[u];
+      const bool ok = tid != 0 || ch_poll(&C.flag[C.off[j] + j - fj], C.err);
+      if (!__syncthreads_and(ok)) return;
+      const double* D = C.Dinv + (int64_t)j * NB * NB;
+      for (int t = tid; t < NB * NB; t += CH_THREADS) Y[t / NB][t % NB] = __ldcg(&D[t]);
+      __syncthreads();
+      // L_ij = X L_jj^-T: row `lane`, columns warp + 8u (uniform trip counts)
+      double o[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int c = warp + 8 * u;
+        double a = 0.0;  // (L^-T)_qc = (L^-1)_cq, nonzero for q <= c
+        for (int q = 0; q <= c; ++q) a = fma(T[lane][q], Y[c][q], a);
+        o[u] = a;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < 4; ++u) T[lane][warp + 8 * u] = o[u];
+      __syncthreads();
+      for (int t = tid; t < NB * NB; t += CH_THREADS) {
+        const int a = t / NB, b = t % NB;
+        if (a < bi && b < bj) C.M[(oi + a) * n + oj + b] = T[a][b];
+        if (b < bi && a < bj) C.LT[(oj + a) * n + oi + b] = T[b][a];
+      }
+    }
+    __syncthreads();
+    if (tid == 0) ch_publish(&C.flag[C.off[i] + j - fi]);
   }
 }
 
@@ -264,15 +365,9 @@ DenseJob::~DenseJob() {
   // left without dense_finish (an error in between): the temporaries are
   // released on the caller's stream after this returns, so the dense
   // launches must have ended first
-  if (pending) {
-    if (sd) cudaStreamSynchronize(sd);
-    if (s2) cudaStreamSynchronize(s2);
-  }
+  if (pending && sd) cudaStreamSynchronize(sd);
   if (e_fork) cudaEventDestroy(e_fork);
   if (e_done) cudaEventDestroy(e_done);
-  if (e_main) cudaEventDestroy(e_main);
-  if (e_side) cudaEventDestroy(e_side);
-  if (s2) cudaStreamDestroy(s2);   // pending work still completes
   if (sd) cudaStreamDestroy(sd);
 }
 
@@ -282,43 +377,79 @@ int dense_start(Alloc& al, int64_t n, const int64_t* rp, const int32_t* ci, cons
   job.main = s;
   job.n = n;
   if (n <= 0) return SA_OK;
+  const int nb = (int)((n + NB - 1) / NB);
   SA_TRY(F.L.alloc(&al, n * n));
   SA_TRY(F.LT.alloc(&al, n * n));
   SA_TRY(F.W.alloc(&al, n * n));
   SA_TRY(F.WT.alloc(&al, n * n));
-  SA_TRY(job.err.alloc(&al, 1));
-  SA_TRY(memset_d(F.L.p, 0, F.L.bytes(), s));
-  SA_TRY(memset_d(job.err.p, 0, sizeof(int), s));
-  k_densify<<<blocks_for(n, 128), 128, 0, s>>>(n, rp, ci, v, F.L.p);
-  SA_LAUNCHED();
-  const int nb = (int)((n + NB - 1) / NB);
+  SA_TRY(job.err.alloc(&al, 2));  // error bits, ticket counter
+  SA_TRY(memset_d(job.err.p, 0, 2 * sizeof(int), s));
+  // host tables, uploaded as one block: first tile column of each tile row,
+  // end of the tile rows that reach each tile column (both kept for the
+  // solve), flag offsets, tasks
+  std::vector<int32_t> tab(3 * (size_t)nb + 1);
+  {
+    Buf<int32_t> f_dev;
+    SA_TRY(f_dev.alloc(&al, nb));
+    k_sky_first<<<blocks_for((int64_t)nb * 32, 256), 256, 0, s>>>(n, nb, rp, ci, f_dev.p);
+    SA_LAUNCHED();
+    SA_TRY(copy_d2h(tab.data(), f_dev.p, sizeof(int32_t) * nb, s));
+  }
+  int32_t ntile = 0;
+  {
+    const int32_t* f = tab.data();
+    int32_t *env = tab.data() + nb, *off = tab.data() + 2 * nb;
+    for (int j = 0; j < nb; ++j) env[j] = j + 1;
+    off[0] = 0;
+    for (int i = 0; i < nb; ++i) {
+      off[i + 1] = off[i] + (i - f[i] + 1);
+      if (env[f[i]] < i + 1) env[f[i]] = i + 1;
+    }
+    for (int j = 1; j < nb; ++j)
+      if (env[j] < env[j - 1]) env[j] = env[j - 1];
+    ntile = off[nb];
+  }
+  // tasks: tiles by columns; a diagonal block's inverse strips once its last
+  // column is numbered
+  tab.reserve(tab.size() + (size_t)ntile + (size_t)(n / CH_STRIP) + 1);
+  for (int j = 0; j < nb; ++j) {
+    const int e = tab[nb + j];
+    for (int i = j; i < e; ++i)
+      if (tab[i] <= j) tab.push_back((i << 15) | j);
+    if ((j + 1) % CH_BT == 0 || j + 1 == nb) {
+      const int q = j / CH_BT;
+      const int64_t r0 = (int64_t)q * COARSE_BS, r1 = (int64_t)(j + 1) * NB < n ? (int64_t)(j + 1) * NB : n;
+      for (int64_t c = r0; c < r1; c += CH_STRIP)
+        tab.push_back((int32_t)(CH_INV | ((uint32_t)q << 16) | (uint32_t)((c - r0) / CH_STRIP)));
+    }
+  }
+  const int64_t nt = (int64_t)tab.size() - (3 * (int64_t)nb + 1);
+  SA_TRY(F.sky.alloc(&al, (int64_t)tab.size()));
+  SA_TRY(job.flag.alloc(&al, ntile));
   SA_TRY(job.Dinv.alloc(&al, (int64_t)nb * NB * NB));
+  // (pageable source: the copy has left it when the call returns)
+  SA_TRY(copy_h2d(F.sky.p, tab.data(), sizeof(int32_t) * tab.size(), s));
+  SA_TRY(memset_d(job.flag.p, 0, job.flag.bytes(), s));
+  // L^T rows are read up to the last tile row that reaches them; tiles of
+  // that range outside another row's skyline stay zero
+  SA_TRY(memset_d(F.LT.p, 0, F.LT.bytes(), s));
+  k_densify_sky<<<(unsigned)nb, 256, 0, s>>>(n, F.sky.p, rp, ci, v, F.L.p);
+  SA_LAUNCHED();
   // The factor runs on its own stream `sd`, forked from the caller's stream
   // after the dense copy; the caller goes on with work that does not read
   // the factor (Chebyshev bounds, SELL packing) and joins in dense_finish.
-  // Within it, look-ahead on a second stream: after panel k, `sd` updates
-  // only block column k+1 and goes on to factor panel k+1, while `s2`
-  // updates the rest of the trailing matrix (columns >= k+2); `sd` waits for
-  // that before it updates column k+2.  The same for the diagonal-block
-  // inverses: row i+1 on `sd`, rows >= i+2 of the same diagonal block on
-  // `s2`.  Without the extra streams everything runs on the caller's stream
-  // in the same order.
-  // Both streams get the highest priority: the factor is the setup's
-  // critical path (a chain of small panel launches), the work it overlaps
-  // has slack, and the block scheduler then hands free SM slots to the
-  // factor first.
+  // It gets the highest priority: the factor is the setup's critical path,
+  // the work it overlaps has slack.  Without the extra stream it runs on the
+  // caller's.
   int prio_lo = 0, prio_hi = 0;
   if (cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi) != cudaSuccess) {
     cudaGetLastError();
     prio_hi = 0;
   }
-  bool own = cudaStreamCreateWithPriority(&job.sd, cudaStreamNonBlocking, prio_hi) == cudaSuccess &&
-             cudaEventCreateWithFlags(&job.e_fork, cudaEventDisableTiming) == cudaSuccess &&
-             cudaEventCreateWithFlags(&job.e_done, cudaEventDisableTiming) == cudaSuccess;
-  bool la = own && cudaStreamCreateWithPriority(&job.s2, cudaStreamNonBlocking, prio_hi) == cudaSuccess &&
-            cudaEventCreateWithFlags(&job.e_main, cudaEventDisableTiming) == cudaSuccess &&
-            cudaEventCreateWithFlags(&job.e_side, cudaEventDisableTiming) == cudaSuccess;
-  if (!la) cudaGetLastError();
+  const bool own = cudaStreamCreateWithPriority(&job.sd, cudaStreamNonBlocking, prio_hi) == cudaSuccess &&
+                   cudaEventCreateWithFlags(&job.e_fork, cudaEventDisableTiming) == cudaSuccess &&
+                   cudaEventCreateWithFlags(&job.e_done, cudaEventDisableTiming) == cudaSuccess;
+  if (!own) cudaGetLastError();
   cudaStream_t m = s;
   if (own) {
     SA_CUDA(cudaEventRecord(job.e_fork, s));
@@ -326,84 +457,14 @@ int dense_start(Alloc& al, int64_t n, const int64_t* rp, const int32_t* ci, cons
     m = job.sd;
   }
   job.pending = own;
-  cudaStream_t s2 = job.s2;
-  double* M = F.L.p;
-  double* D = job.Dinv.p;
   const int ph = prof_begin(m, PK_S_DENSE, job.level, 0.0);
-  bool side_pending = false;
-  for (int k = 0; k < nb; ++k) {
-    k_potrf_diag<<<1, 256, 0, m>>>(n, M, k, job.err.p, D);
-    count_launch();
-    const int r = nb - k - 1;
-    if (r > 0) {
-      k_trsm_panel<<<r, 256, 0, m>>>(n, M, k, D);
-      count_launch();
-      if (la) {
-        if (side_pending) SA_CUDA(cudaStreamWaitEvent(m, job.e_side, 0));
-        k_syrk_update<<<r, 256, 0, m>>>(n, M, k, k + 1, 1);
-        count_launch();
-        if (r > 1) {
-          SA_CUDA(cudaEventRecord(job.e_main, m));
-          SA_CUDA(cudaStreamWaitEvent(s2, job.e_main, 0));
-          k_syrk_update<<<(unsigned)((int64_t)(r - 1) * r / 2), 256, 0, s2>>>(n, M, k, k + 2, 0);
-          count_launch();
-          SA_CUDA(cudaEventRecord(job.e_side, s2));
-          side_pending = true;
-        } else {
-          side_pending = false;
-        }
-      } else {
-        k_syrk_update<<<(unsigned)((int64_t)r * (r + 1) / 2), 256, 0, m>>>(n, M, k, k + 1, 0);
-        count_launch();
-      }
-    }
-    SA_LAUNCHED();
-  }
-  if (la && side_pending) SA_CUDA(cudaStreamWaitEvent(m, job.e_side, 0));
-  // W_KK = L_KK^-1 for the diagonal blocks of COARSE_BS rows, block row by
-  // block row (NB rows) inside each.  A pivot that was not positive is
-  // recorded in err and replaced by 1, so the inverse is computed on finite
-  // data either way; dense_finish reports it.  The strict upper triangle of
-  // L outside the NB x NB diagonal tiles still holds A: the solve reads
-  // only the lower triangle of L and the diagonal blocks of W.
-  k_set_identity<<<blocks_for(n * n, 256), 256, 0, m>>>(n, F.W.p);
-  count_launch();
-  side_pending = false;
-  constexpr int BB = (int)(COARSE_BS / NB);  // NB-blocks per diagonal block
-  for (int i = 0; i < nb; ++i) {
-    const int j0 = (i / BB) * BB;                   // first NB-block column of this diagonal block
-    const int e = j0 + BB < nb ? j0 + BB : nb;      // end of its NB-block rows
-    const int ncolb = i + 1 - j0;
-    k_trsm_lower_left<<<(unsigned)ncolb, 256, 0, m>>>(n, D, F.W.p, i, j0);
-    count_launch();
-    const int r = e - i - 1;
-    if (r > 0) {
-      if (la) {
-        if (side_pending) SA_CUDA(cudaStreamWaitEvent(m, job.e_side, 0));
-        k_gemm_left<<<(unsigned)ncolb, 256, 0, m>>>(n, M, F.W.p, i, ncolb, i + 1, j0);
-        count_launch();
-        if (r > 1) {
-          SA_CUDA(cudaEventRecord(job.e_main, m));
-          SA_CUDA(cudaStreamWaitEvent(s2, job.e_main, 0));
-          k_gemm_left<<<(unsigned)((r - 1) * ncolb), 256, 0, s2>>>(n, M, F.W.p, i, ncolb, i + 2, j0);
-          count_launch();
-          SA_CUDA(cudaEventRecord(job.e_side, s2));
-          side_pending = true;
-        } else {
-          side_pending = false;
-        }
-      } else {
-        k_gemm_left<<<(unsigned)(r * ncolb), 256, 0, m>>>(n, M, F.W.p, i, ncolb, i + 1, j0);
-        count_launch();
-      }
-    }
-    SA_LAUNCHED();
-  }
-  if (la && side_pending) SA_CUDA(cudaStreamWaitEvent(m, job.e_side, 0));
-  dim3 tb(32, 8), tg((unsigned)((n + 31) / 32), (unsigned)((n + 31) / 32));
-  k_transpose_dense<<<tg, tb, 0, m>>>(n, F.W.p, F.WT.p);
-  SA_LAUNCHED();
-  k_transpose_dense<<<tg, tb, 0, m>>>(n, F.L.p, F.LT.p);
+  CholView C;
+  C.n = n; C.nb = nb; C.f = F.sky.p; C.off = F.sky.p + 2 * nb;
+  C.task = reinterpret_cast<const uint32_t*>(F.sky.p + 3 * nb + 1); C.ntask = (int)nt;
+  C.M = F.L.p; C.LT = F.LT.p; C.W = F.W.p; C.WT = F.WT.p; C.Dinv = job.Dinv.p;
+  C.flag = job.flag.p; C.ticket = job.err.p + 1; C.err = job.err.p;
+  const int64_t g = 2 * (int64_t)num_sms();
+  k_chol<<<(unsigned)(nt < g ? nt : g), CH_THREADS, 0, m>>>(C);
   SA_LAUNCHED();
   prof_end(m, ph);
   if (own) SA_CUDA(cudaEventRecord(job.e_done, m));
@@ -418,6 +479,10 @@ int dense_finish(DenseJob& job) {
   }
   int h_err = 0;
   SA_TRY(copy_d2h(&h_err, job.err.p, sizeof(int), job.main));
+  if (h_err & 2) {
+    set_error_text("coarse factor: a wait for a tile ran out");
+    return SA_ERR_CUDA;
+  }
   return h_err ? SA_ERR_NOT_SPD : SA_OK;
 }
 
@@ -438,23 +503,35 @@ int dense_finish(DenseJob& job) {
 // ---------------------------------------------------------------------------
 constexpr int TRI_WARPS = 4;
 
+// The products with L and L^T (MODE 2, 3) leave out the columns outside the
+// skyline (`sky`: the first tile column of each tile row, or the end of the
+// tile rows that reach each tile column): a lane starts at the first of its
+// own columns inside it, so the sums are those over the whole range.
 // the row i of one step (a block of TRI_WARPS warps per row)
 template <int MODE, int K>
 __device__ __forceinline__ void tri_row_at(int64_t n, int64_t r0, int64_t r1, const double* __restrict__ M,
-                                           const double* __restrict__ v, const double* __restrict__ rhs,
-                                           double* __restrict__ out, int64_t i) {
+                                           const int32_t* __restrict__ sky, const double* __restrict__ v,
+                                           const double* __restrict__ rhs, double* __restrict__ out, int64_t i) {
   __shared__ double sh[TRI_WARPS][K];
   const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
   const int64_t lo = MODE == 0 ? r0 : (MODE == 1 ? i : (MODE == 2 ? 0 : r1));
   const int64_t hi = MODE == 0 ? i + 1 : (MODE == 1 ? r1 : (MODE == 2 ? r0 : n));
   const int64_t seg = (((hi - lo) + TRI_WARPS - 1) / TRI_WARPS + 31) & ~(int64_t)31;
   const int64_t b = lo + warp * seg;
-  const int64_t e = b + seg < hi ? b + seg : hi;
+  int64_t e = b + seg < hi ? b + seg : hi;
   const double* __restrict__ Mi = M + i * n;
   double sum[K];
 #pragma unroll
   for (int c = 0; c < K; ++c) sum[c] = 0.0;
   int64_t j = b + lane;
+  if (MODE == 2) {
+    const int64_t f = (int64_t)sky[i / NB] * NB;
+    if (j < f) j += (f - j + 31) & ~(int64_t)31;
+  }
+  if (MODE == 3) {
+    const int64_t g = (int64_t)sky[i / NB] * NB;
+    if (e > g) e = g;
+  }
   for (; j + 96 < e; j += 128) {
     const double w0 = __ldcs(&Mi[j]), w1 = __ldcs(&Mi[j + 32]), w2 = __ldcs(&Mi[j + 64]), w3 = __ldcs(&Mi[j + 96]);
 #pragma unroll
@@ -488,10 +565,11 @@ __device__ __forceinline__ void tri_row_at(int64_t n, int64_t r0, int64_t r1, co
 template <int MODE, int K>
 __global__ void __launch_bounds__(TRI_WARPS * 32) k_tri_row(int64_t n, int64_t r0, int64_t r1,
                                                             const double* __restrict__ M,
+                                                            const int32_t* __restrict__ sky,
                                                             const double* __restrict__ v,
                                                             const double* __restrict__ rhs,
                                                             double* __restrict__ out) {
-  tri_row_at<MODE, K>(n, r0, r1, M, v, rhs, out, r0 + blockIdx.x);
+  tri_row_at<MODE, K>(n, r0, r1, M, sky, v, rhs, out, r0 + blockIdx.x);
 }
 
 // the same step for several problems in one launch (group solve): block
@@ -511,7 +589,7 @@ __global__ void __launch_bounds__(TRI_WARPS * 32) k_g_tri(const GTri* __restrict
   }
   __syncthreads();
   const GTri& D = d[s_seg];
-  tri_row_at<MODE, 1>(D.n, D.r0, D.r1, D.M, D.v, D.rhs, D.out, D.r0 + (int64_t)(blockIdx.x - D.blk0));
+  tri_row_at<MODE, 1>(D.n, D.r0, D.r1, D.M, D.sky, D.v, D.rhs, D.out, D.r0 + (int64_t)(blockIdx.x - D.blk0));
 }
 
 int launch_g_tri(cudaStream_t st, int mode, const GTri* d, int m, unsigned blocks) {
@@ -538,20 +616,20 @@ static int coarse_solve_k(cudaStream_t st, const CoarseView& F, const double* b,
     const int64_t r0 = q * COARSE_BS, r1 = r0 + COARSE_BS < n ? r0 + COARSE_BS : n;
     const unsigned g = (unsigned)(r1 - r0);
     if (q > 0) {
-      k_tri_row<2, K><<<g, T, 0, st>>>(n, r0, r1, F.L, y, b, t);
+      k_tri_row<2, K><<<g, T, 0, st>>>(n, r0, r1, F.L, F.first, y, b, t);
       SA_LAUNCHED();
     }
-    k_tri_row<0, K><<<g, T, 0, st>>>(n, r0, r1, F.W, q > 0 ? t : b, nullptr, y);
+    k_tri_row<0, K><<<g, T, 0, st>>>(n, r0, r1, F.W, nullptr, q > 0 ? t : b, nullptr, y);
     SA_LAUNCHED();
   }
   for (int q = nbk - 1; q >= 0; --q) {
     const int64_t r0 = q * COARSE_BS, r1 = r0 + COARSE_BS < n ? r0 + COARSE_BS : n;
     const unsigned g = (unsigned)(r1 - r0);
     if (q < nbk - 1) {
-      k_tri_row<3, K><<<g, T, 0, st>>>(n, r0, r1, F.LT, x, y, t);
+      k_tri_row<3, K><<<g, T, 0, st>>>(n, r0, r1, F.LT, F.end, x, y, t);
       SA_LAUNCHED();
     }
-    k_tri_row<1, K><<<g, T, 0, st>>>(n, r0, r1, F.WT, q < nbk - 1 ? t : y, nullptr, x);
+    k_tri_row<1, K><<<g, T, 0, st>>>(n, r0, r1, F.WT, nullptr, q < nbk - 1 ? t : y, nullptr, x);
     SA_LAUNCHED();
   }
   return SA_OK;

@@ -57,6 +57,7 @@ struct GTri {
   uint32_t blk0;
   int64_t n, r0, r1;
   const double* M;
+  const int32_t* sky;  // modes 2 and 3: the factor's skyline (CoarseView first / end)
   const double* v;
   const double* rhs;
   double* out;

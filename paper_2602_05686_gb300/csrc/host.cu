@@ -838,8 +838,8 @@ static int setup_impl(const sa_problem* P, const sa_options* o, sa_handle h) {
   Level& Lc = *h->lev[nlev - 1];
   if (Lc.n > 16384) return SA_ERR_STAGNATION;
   h->nL = Lc.n;
-  // a15: the coarse Cholesky factor and its diagonal-block inverses, on
-  // streams of their own: the Chebyshev bounds and the packing of the
+  // a15: the coarse Cholesky factor and its diagonal-block inverses, on a
+  // stream of their own: the Chebyshev bounds and the packing of the
   // hierarchy below overlap it (the packing stores the addresses of the
   // factor's arrays, not their contents)
   DenseJob dj;
@@ -1420,6 +1420,7 @@ int sa_free(sa_handle h) {
   h->cf.LT.release();
   h->cf.W.release();
   h->cf.WT.release();
+  h->cf.sky.release();
   h->r.release(); h->p.release(); h->q.release(); h->rprev.release(); h->t.release();
   h->part.release(); h->dots.release(); h->xb.release(); h->bb.release(); h->cg.release();
   h->it_dev.release(); h->ctl.release();
@@ -1718,7 +1719,7 @@ struct GroupVcycle {
           const int64_t r0 = q * COARSE_BS, r1 = r0 + COARSE_BS < c.n ? r0 + COARSE_BS : c.n;
           GTri g = {};
           g.blk0 = blk; g.n = c.n; g.r0 = r0; g.r1 = r1;
-          if (mode == 2) { g.M = c.F.L; g.v = c.y; g.rhs = c.bin; g.out = c.t; }
+          if (mode == 2) { g.M = c.F.L; g.sky = c.F.first; g.v = c.y; g.rhs = c.bin; g.out = c.t; }
           else { g.M = c.F.W; g.v = q > 0 ? c.t : c.bin; g.rhs = nullptr; g.out = c.y; }
           v.push_back(g);
           blk += (uint32_t)(r1 - r0);
@@ -1737,7 +1738,7 @@ struct GroupVcycle {
           const int64_t r0 = q * COARSE_BS, r1 = r0 + COARSE_BS < c.n ? r0 + COARSE_BS : c.n;
           GTri g = {};
           g.blk0 = blk; g.n = c.n; g.r0 = r0; g.r1 = r1;
-          if (mode == 3) { g.M = c.F.LT; g.v = c.x; g.rhs = c.y; g.out = c.t; }
+          if (mode == 3) { g.M = c.F.LT; g.sky = c.F.end; g.v = c.x; g.rhs = c.y; g.out = c.t; }
           else { g.M = c.F.WT; g.v = t > 0 ? c.t : c.y; g.rhs = nullptr; g.out = c.x; }
           v.push_back(g);
           blk += (uint32_t)(r1 - r0);

@@ -55,8 +55,14 @@ int launch_interleave(cudaStream_t st, int64_t n, int k, int K, const double* sr
 // instead of n^3 / 3 for the whole inverse).
 constexpr int64_t COARSE_BS = 1024;
 
+// Only the skyline of L is stored (tiles of 32 x 32 from each tile row's
+// first nonzero tile column on), the rest of L is unset.
 struct CoarseFactor {
   Buf<double> L, LT, W, WT;
+  // per tile row of 32: the first tile column of its skyline; then per tile
+  // column the end of the tile rows that reach it; then the factorisation's
+  // own tables
+  Buf<int32_t> sky;
 };
 
 struct CoarseView {
@@ -65,23 +71,27 @@ struct CoarseView {
   const double* LT = nullptr;
   const double* W = nullptr;
   const double* WT = nullptr;
+  const int32_t* first = nullptr;  // skyline: first tile column per tile row
+  const int32_t* end = nullptr;    // ... and end of the tile rows per tile column
 };
 
 inline CoarseView coarse_view(const CoarseFactor& F, int64_t n) {
   CoarseView v;
   v.n = n; v.L = F.L.p; v.LT = F.LT.p; v.W = F.W.p; v.WT = F.WT.p;
+  v.first = F.sky.p; v.end = F.sky.p + (n + 31) / 32;
   return v;
 }
 
-// dense_start enqueues the whole factorisation on streams of its own, forked
+// dense_start enqueues the whole factorisation on a stream of its own, forked
 // from al.stream after the dense copy of A; dense_finish makes al.stream wait
 // for it and reports a pivot that was not positive (SA_ERR_NOT_SPD).  Work on
 // al.stream in between must not read the factor.
 struct DenseJob {
   Buf<double> Dinv;
-  Buf<int> err;
-  cudaStream_t main = nullptr, sd = nullptr, s2 = nullptr;
-  cudaEvent_t e_fork = nullptr, e_done = nullptr, e_main = nullptr, e_side = nullptr;
+  Buf<int> err;           // error bits, ticket counter
+  Buf<int32_t> flag;      // per tile of L: written
+  cudaStream_t main = nullptr, sd = nullptr;
+  cudaEvent_t e_fork = nullptr, e_done = nullptr;
   int64_t n = 0;
   int level = 0;         // for the setup-phase profile
   bool pending = false;  // forked and not yet joined
