@@ -8,6 +8,7 @@
 // bitwise.
 #include "common.cuh"
 #include "profile.cuh"
+#include "reduce.cuh"
 #include "solve.cuh"
 #include "vcycle.cuh"
 #include "vkern.cuh"
@@ -1018,8 +1019,7 @@ static MatView<double> sell_view(const Sell<double>& A) {
 }
 
 int launch_bsell_spmv_dot(cudaStream_t st, const Sell<double>& A, int K, const double* P, double* Q, double* part,
-                          int* nparts) {
-  *nparts = (int)g256(A.n);
+                          const Fin& fin) {
   const MatView<double> mv = sell_view(A);
   // the matrix once; P read and Q written for each of the K columns
   const double bytes = (8.0 + A.idx_bytes()) * A.nnz + 8.0 * (A.nslices + 1) + (A.idx16 ? 4.0 * A.nslices : 0.0) +
@@ -1031,7 +1031,7 @@ int launch_bsell_spmv_dot(cudaStream_t st, const Sell<double>& A, int K, const d
   else k_bsell_spmv_dot<8><<<g256(A.n), 256, 0, st>>>(mv, P, Q, part);
   prof_end(st, pi);
   SA_LAUNCHED();
-  return SA_OK;
+  return launch_fin_wide(st, part, (int)g256(A.n), fin);
 }
 
 int launch_bsell_residual64(cudaStream_t st, const Sell<double>& A, int K, const double* B, const double* X,

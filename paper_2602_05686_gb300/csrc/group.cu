@@ -5,6 +5,7 @@
 // index of the segment, so the results are the one-problem results bit for
 // bit.
 #include "group.cuh"
+#include "reduce.cuh"
 
 namespace sa {
 
@@ -157,7 +158,24 @@ __device__ __forceinline__ double g_sell_row(const GCg& D, const double* __restr
   return D.c16 ? sell_row16<double>(D.sp, D.base, D.c16, D.v, x, i) : sell_row<double>(D.sp, D.ci, D.v, x, i);
 }
 
-// rows geometry (blocks of 256): residual, operator product with p.q partials
+// the problem's last block: sums of its partials, then the scalar step
+template <int NV, int NT>
+__device__ __forceinline__ void g_tail(const GCg& D) {
+  __shared__ double res[NV];
+  if (!last_block(D.tick, D.nblk)) return;
+  fin_sums<NV, NT>(D.part, (int)D.nblk, RED_BLOCKS, res);
+  if (threadIdx.x != 0) return;
+  switch (D.tail) {
+    case GT_ALPHA: cg_alpha_step(D.cg, res[0]); break;
+    case GT_BETA: cg_beta_step(D.cg, res[0], NV > 1 ? res[NV - 1] : 0.0, D.flexible); break;
+    default:
+      D.gather[0] = res[0];
+      D.gather[1] = (double)D.cg->breakdown;
+      break;
+  }
+}
+
+// rows geometry (blocks of 256): residual, operator product with p.q
 __global__ void __launch_bounds__(256) k_g_cg_rows(int op, const GCg* __restrict__ d, int m) {
   const int k = seg_of(d, m);
   const GCg& D = d[k];
@@ -183,22 +201,27 @@ __global__ void __launch_bounds__(256) k_g_cg_rows(int op, const GCg* __restrict
     t = warp_sum(t);
     if (lane == 0) D.part[blk] = t;
   }
+  g_tail<1, 256>(D);
 }
 
-// reduction geometry (RED_BLOCKS blocks of RED_THREADS per problem)
-__global__ void __launch_bounds__(RED_THREADS) k_g_cg_red(int op, const GCg* __restrict__ d) {
-  const int k = (int)(blockIdx.x / RED_BLOCKS);
-  const unsigned blk = blockIdx.x % RED_BLOCKS;
+// reduction geometry: each problem the blocks of its one-vector kernels
+// (red_blocks(n) of RED_THREADS: the fixed grid less the blocks without
+// elements; sixteen small problems in full grids spent 25 us a launch on
+// block sums of zeros)
+__global__ void __launch_bounds__(RED_THREADS) k_g_cg_red(int op, const GCg* __restrict__ d, int m) {
+  const int k = seg_of(d, m);
   const GCg& D = d[k];
+  const unsigned blk = blockIdx.x - D.blk0;
   const int64_t n = D.n;
-  const int64_t stride = (int64_t)RED_BLOCKS * blockDim.x;
+  const int64_t stride = (int64_t)D.nblk * blockDim.x;
   if (op == GC_DOTS) {
-    double acc[3] = {0.0, 0.0, 0.0};
+    double acc[2] = {0.0, 0.0};
     for (int64_t i = (int64_t)blk * blockDim.x + threadIdx.x; i < n; i += stride) {
       acc[0] = fma(D.a0[i], D.b0[i], acc[0]);
       if (D.a1) acc[1] = fma(D.a1[i], D.b1[i], acc[1]);
     }
-    g_block_sum_to<3>(acc, D.part, RED_BLOCKS, blk);
+    g_block_sum_to<2>(acc, D.part, RED_BLOCKS, blk);
+    g_tail<2, RED_THREADS>(D);
   } else if (op == GC_UPDATE) {
     const double alpha = D.cg->alpha;
     double acc[1] = {0.0};
@@ -211,6 +234,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_g_cg_red(int op, const GCg* __r
       acc[0] = fma(ri, ri, acc[0]);
     }
     g_block_sum_to<1>(acc, D.part, 0, blk);
+    g_tail<1, RED_THREADS>(D);
   } else {  // GC_PUPDATE
     const double beta = D.cg->beta;
     for (int64_t i = (int64_t)blk * blockDim.x + threadIdx.x; i < n; i += stride)
@@ -218,78 +242,10 @@ __global__ void __launch_bounds__(RED_THREADS) k_g_cg_red(int op, const GCg* __r
   }
 }
 
-// one block of 1024 per problem: the partial sums in index order
-__global__ void __launch_bounds__(1024) k_g_cg_finish(const GCg* __restrict__ d) {
-  const GCg& D = d[blockIdx.x];
-  double acc[3] = {0.0, 0.0, 0.0};
-  for (int t = threadIdx.x; t < D.np; t += blockDim.x)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) acc[k] += D.part[(int64_t)k * D.stride + t];
-  __shared__ double sh[3][32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    double t = warp_sum(acc[k]);
-    if (lane == 0) sh[k][w] = t;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < 3; ++k) {
-      double s = 0.0;
-      for (int q = 0; q < nw; ++q) s += sh[k][q];
-      D.dots[k] = s;
-    }
-  }
-}
-
-// one thread per problem: alpha, beta, the host gather
-__global__ void k_g_cg_scalar(int op, const GCg* __restrict__ d, int m) {
-  const int k = (int)(blockIdx.x * blockDim.x + threadIdx.x);
-  if (k >= m) return;
-  const GCg& D = d[k];
-  CgScalars* s = D.cg;
-  if (op == GC_ALPHA) {
-    double pq = D.dots[0];
-    s->pq = pq;
-    if (!(pq > 0.0)) { s->breakdown = 1; s->alpha = 0.0; return; }
-    s->alpha = s->rz / pq;
-  } else if (op == GC_BETA) {
-    double rz_new = D.dots[0];
-    if (D.flexible < 0) {
-      s->rz = rz_new;
-      s->beta = 0.0;
-      s->breakdown = 0;
-      return;
-    }
-    double num = D.flexible ? rz_new - D.dots[1] : rz_new;
-    s->beta = num / s->rz;
-    s->rz = rz_new;
-  } else {  // GC_GATHER
-    D.gather[2 * k] = D.dots[0];
-    D.gather[2 * k + 1] = (double)s->breakdown;
-  }
-}
-
 int launch_g_cg(cudaStream_t st, int op, const GCg* d, int m, unsigned blocks) {
-  if (m <= 0) return SA_OK;
-  switch (op) {
-    case GC_RESID:
-    case GC_SPMV_DOT:
-      if (blocks == 0) return SA_OK;
-      k_g_cg_rows<<<blocks, 256, 0, st>>>(op, d, m);
-      break;
-    case GC_DOTS:
-    case GC_UPDATE:
-    case GC_PUPDATE:
-      k_g_cg_red<<<(unsigned)m * RED_BLOCKS, RED_THREADS, 0, st>>>(op, d);
-      break;
-    case GC_FINISH:
-      k_g_cg_finish<<<(unsigned)m, 1024, 0, st>>>(d);
-      break;
-    default:
-      k_g_cg_scalar<<<1, GROUP_MAX, 0, st>>>(op, d, m);
-      break;
-  }
+  if (m <= 0 || blocks == 0) return SA_OK;
+  if (op == GC_RESID || op == GC_SPMV_DOT) k_g_cg_rows<<<blocks, 256, 0, st>>>(op, d, m);
+  else k_g_cg_red<<<blocks, RED_THREADS, 0, st>>>(op, d, m);
   SA_LAUNCHED();
   return SA_OK;
 }

@@ -66,18 +66,22 @@ struct GTri {
 // outer FP64 CG of one problem
 enum GCgOp {
   GC_RESID = 0,     // t = b - A x                 (rows)
-  GC_SPMV_DOT = 1,  // q = A p, p.q partials       (rows)
-  GC_DOTS = 2,      // dots of (a0,b0), (a1,b1)   (RED_BLOCKS per problem)
-  GC_FINISH = 3,    // partials -> dots            (one block per problem)
-  GC_ALPHA = 4,     //                             (one thread per problem)
-  GC_UPDATE = 5,    // x, r, r_prev, r.r partials  (RED_BLOCKS per problem)
-  GC_BETA = 6,      //                             (one thread per problem)
-  GC_PUPDATE = 7,   // p = z + beta p              (RED_BLOCKS per problem)
-  GC_GATHER = 8     // rr, breakdown -> host block (one thread per problem)
+  GC_SPMV_DOT = 1,  // q = A p, p.q                (rows)
+  GC_DOTS = 2,      // dots of (a0,b0), (a1,b1)    (red_blocks per problem)
+  GC_UPDATE = 3,    // x, r, r_prev, r.r           (red_blocks per problem)
+  GC_PUPDATE = 4    // p = z + beta p              (red_blocks per problem)
+};
+
+// what a problem's last block does with the sums of its partials (reduce.cuh)
+enum GCgTail {
+  GT_ALPHA = 0,
+  GT_BETA = 1,
+  GT_GATHER = 2     // (first sum, breakdown) -> host block
 };
 
 struct GCg {
-  uint32_t blk0;    // rows geometry: first block of this problem
+  uint32_t blk0;    // first block of this problem in the launch
+  uint32_t nblk;    // its blocks
   int64_t n;
   // FP64 SELL fine operator
   const int64_t* sp;
@@ -100,11 +104,11 @@ struct GCg {
   const double* q;
   CgScalars* cg;
   double* part;
-  double* dots;       // finish target / alpha, beta source
-  int np, stride;     // finish: partial count and stride
+  unsigned* tick;     // ticket of the problem's finishing block
+  int tail;           // GCgTail
   int flexible;       // beta: -1 initialise, 0 plain, 1 flexible
   int first;          // pupdate
-  double* gather;     // GC_GATHER: 2 doubles per problem (r.r, breakdown)
+  double* gather;     // GT_GATHER: this problem's 2 doubles (sum, breakdown)
 };
 
 template <typename T>

@@ -16,6 +16,7 @@
 #include "group.cuh"
 #include "kernels.cuh"
 #include "profile.cuh"
+#include "reduce.cuh"
 #include "solve.cuh"
 #include "vcycle.cuh"
 
@@ -56,6 +57,8 @@ struct sa_handle_s {
   sa::Sell<double> A0s;  // fine operator (unscaled) for the outer CG
   // Krylov workspace (FP64, fine level)
   sa::Buf<double> r, p, q, rprev, t, part, dots, xb, bb;
+  sa::Buf<double> wsum;      // group sums of the wide finish
+  sa::Buf<unsigned> tick;    // ticket of the finishing block (zero between launches)
   sa::Buf<sa::CgScalars> cg;
   double* host_pin = nullptr;  // pinned readback buffer
   int zero_guess = 0;          // set for one sa_solve_batch_zero call: x is output only
@@ -262,6 +265,9 @@ static int alloc_workspace(sa_handle h) {
   int64_t np = blocks_for(n * 32, 256) + RED_BLOCKS;
   SA_TRY(h->part.alloc(&al, 3 * np));
   SA_TRY(h->dots.alloc(&al, 8));
+  SA_TRY(h->wsum.alloc(&al, 32 * KMAX_BLOCK));
+  SA_TRY(h->tick.alloc(&al, 1));
+  SA_TRY(memset_d(h->tick.p, 0, sizeof(unsigned), al.stream));
   SA_TRY(h->cg.alloc(&al, 1));
   SA_TRY(h->it_dev.alloc(&al, 1));
   SA_TRY(h->ctl.alloc(&al, 1));
@@ -281,9 +287,34 @@ static int precondition(sa_handle h, const double* r, double** z) {
   return vh_vcycle<double>(h->v64, h->al.stream, r, z);
 }
 
+// what a reduction's last block does with its sums: stored at `out`, then
+// the scalar step `op` on the handle's CG scalars
+static Fin fin_one(sa_handle h, int op, double* out, int flexible = 0) {
+  Fin f;
+  f.op = op;
+  f.out = out;
+  f.tick = h->tick.p;
+  f.wsum = h->wsum.p;
+  f.cg = h->cg.p;
+  f.flexible = flexible;
+  return f;
+}
+static Fin fin_block(sa_handle h, int K, int op, double* out, int flexible = 0) {
+  Fin f = fin_one(h, op, out, flexible);
+  f.cg = h->kS.p;
+  f.k = K;
+  f.active = h->kact.p;
+  return f;
+}
+// ||v||^2 at out
+static int norm2(sa_handle h, const double* v, double* out) {
+  return launch_dots(h->al.stream, h->n, v, v, nullptr, nullptr, h->part.p, fin_one(h, FIN_STORE, out));
+}
+
 // outer-CG operator products on the FP64 SELL copy of the fine operator
-static int op_spmv_dot(sa_handle h, const double* p, double* q, double* part, int* np) {
-  return launch_sell_spmv_dot(h->al.stream, h->A0s, p, q, part, np);
+// (q = A p, then alpha from p.q)
+static int op_spmv_alpha(sa_handle h, const double* p, double* q) {
+  return launch_sell_spmv_dot(h->al.stream, h->A0s, p, q, h->part.p, fin_one(h, FIN_ALPHA, h->dots.p));
 }
 static int op_residual(sa_handle h, const double* b, const double* x, double* r) {
   return launch_sell_residual64(h->al.stream, h->A0s, b, x, r);
@@ -324,7 +355,7 @@ static int cg_eager_dev(sa_handle h, const double* b, double* x, double tol, sa_
   int status = SA_ERR_NO_CONVERGENCE, it = 0;
   double r0 = 0.0;
   SA_TRY(op_residual(h, b, x, h->r.p));
-  SA_TRY(launch_dots(s, n, h->r.p, h->r.p, nullptr, nullptr, nullptr, nullptr, h->part.p, h->dots.p));
+  SA_TRY(norm2(h, h->r.p, h->dots.p));
   SA_CUDA(cudaMemcpyAsync(hp, h->dots.p, sizeof(double), cudaMemcpyDeviceToHost, s));
   SA_CUDA(cudaStreamSynchronize(s));
   r0 = sqrt(hp[0]);
@@ -332,18 +363,14 @@ static int cg_eager_dev(sa_handle h, const double* b, double* x, double tol, sa_
     double* z = nullptr;
     SA_TRY(precondition(h, h->r.p, &z));
     SA_TRY(launch_cg_pupdate(s, n, h->cg.p, z, h->p.p, 1));
-    SA_TRY(launch_dots(s, n, h->r.p, z, nullptr, nullptr, nullptr, nullptr, h->part.p, h->dots.p));
-    SA_TRY(launch_cg_beta(s, h->cg.p, h->dots.p, -1));
+    SA_TRY(launch_dots(s, n, h->r.p, z, nullptr, nullptr, h->part.p, fin_one(h, FIN_BETA, h->dots.p, -1)));
     const int maxit = h->opt.maxit;
     for (it = 1; it <= maxit; ++it) {
-      int np = 0;
       PROF(PK_CG_SPMV, 0, (8.0 + h->A0s.idx_bytes()) * L0.nnz + 8.0 * (h->A0s.nslices + 1) + 16.0 * n,
-           op_spmv_dot(h, h->p.p, h->q.p, h->part.p, &np));
-      SA_TRY(launch_finish(s, h->part.p, np, h->dots.p));
-      SA_TRY(launch_cg_alpha(s, h->cg.p, h->dots.p));
+           op_spmv_alpha(h, h->p.p, h->q.p));
       PROF(PK_CG_VEC, 0, (flexible ? 56.0 : 48.0) * n,
-           launch_cg_update(s, n, h->cg.p, h->p.p, h->q.p, x, h->r.p, flexible ? h->rprev.p : nullptr, h->part.p));
-      SA_TRY(launch_finish(s, h->part.p, RED_BLOCKS, h->dots.p + 4));
+           launch_cg_update(s, n, h->cg.p, h->p.p, h->q.p, x, h->r.p, flexible ? h->rprev.p : nullptr, h->part.p,
+                            fin_one(h, FIN_STORE, h->dots.p + 4)));
       SA_CUDA(cudaMemcpyAsync(hp, h->dots.p + 4, sizeof(double), cudaMemcpyDeviceToHost, s));
       SA_CUDA(cudaMemcpyAsync(hp + 1, &h->cg.p->breakdown, sizeof(int), cudaMemcpyDeviceToHost, s));
       SA_CUDA(cudaStreamSynchronize(s));
@@ -352,7 +379,7 @@ static int cg_eager_dev(sa_handle h, const double* b, double* x, double tol, sa_
       if (brk) { status = SA_ERR_BREAKDOWN; break; }
       if (sqrt(hp[0]) <= tol * r0) {
         SA_TRY(op_residual(h, b, x, h->t.p));
-        SA_TRY(launch_dots(s, n, h->t.p, h->t.p, nullptr, nullptr, nullptr, nullptr, h->part.p, h->dots.p + 4));
+        SA_TRY(norm2(h, h->t.p, h->dots.p + 4));
         SA_CUDA(cudaMemcpyAsync(hp, h->dots.p + 4, sizeof(double), cudaMemcpyDeviceToHost, s));
         SA_CUDA(cudaStreamSynchronize(s));
         if (sqrt(hp[0]) <= tol * r0) { status = SA_OK; break; }
@@ -360,9 +387,8 @@ static int cg_eager_dev(sa_handle h, const double* b, double* x, double tol, sa_
       }
       SA_TRY(precondition(h, h->r.p, &z));
       PROF(PK_CG_VEC, 0, (flexible ? 24.0 : 16.0) * n,
-           launch_dots(s, n, h->r.p, z, flexible ? z : nullptr, flexible ? h->rprev.p : nullptr, nullptr, nullptr,
-                       h->part.p, h->dots.p));
-      SA_TRY(launch_cg_beta(s, h->cg.p, h->dots.p, flexible));
+           launch_dots(s, n, h->r.p, z, flexible ? z : nullptr, flexible ? h->rprev.p : nullptr, h->part.p,
+                       fin_one(h, FIN_BETA, h->dots.p, flexible)));
       PROF(PK_CG_VEC, 0, 24.0 * n, launch_cg_pupdate(s, n, h->cg.p, z, h->p.p, 0));
     }
     if (it > maxit) it = maxit;
@@ -371,7 +397,7 @@ static int cg_eager_dev(sa_handle h, const double* b, double* x, double tol, sa_
   }
   // true residual at exit
   SA_TRY(op_residual(h, b, x, h->t.p));
-  SA_TRY(launch_dots(s, n, h->t.p, h->t.p, nullptr, nullptr, nullptr, nullptr, h->part.p, h->dots.p + 4));
+  SA_TRY(norm2(h, h->t.p, h->dots.p + 4));
   SA_CUDA(cudaMemcpyAsync(hp, h->dots.p + 4, sizeof(double), cudaMemcpyDeviceToHost, s));
   SA_CUDA(cudaStreamSynchronize(s));
   auto t1 = std::chrono::steady_clock::now();
@@ -386,16 +412,6 @@ static int cg_eager_dev(sa_handle h, const double* b, double* x, double tol, sa_
 }
 
 
-// loop control inside the captured CG body: count the iteration and decide
-// whether the WHILE node runs the body again
-__global__ void k_loop_ctrl(cudaGraphConditionalHandle ch, int* __restrict__ it, const CgScalars* __restrict__ s,
-                            const double* __restrict__ rr, const double* __restrict__ ctl, int maxit) {
-  int k = *it + 1;
-  *it = k;
-  int cont = !s->breakdown && !(sqrt(*rr) <= ctl[0]) && k < maxit;
-  cudaGraphSetConditional(ch, cont ? 1u : 0u);
-}
-
 // the second half of one CG iteration followed by the first half of the next:
 // z = M r, beta, p = z + beta p, q = A p, alpha, x/r update, ||r||^2, control
 static int cg_body(sa_handle h, cudaGraphConditionalHandle ch) {
@@ -405,19 +421,17 @@ static int cg_body(sa_handle h, cudaGraphConditionalHandle ch) {
   const int flexible = h->opt.precision == SA_PREC_FP32_VCYCLE;
   double* z = nullptr;
   SA_TRY(precondition(h, h->r.p, &z));
-  SA_TRY(launch_dots(s, n, h->r.p, z, flexible ? z : nullptr, flexible ? h->rprev.p : nullptr, nullptr, nullptr,
-                     h->part.p, h->dots.p));
-  SA_TRY(launch_cg_beta(s, h->cg.p, h->dots.p, flexible));
+  SA_TRY(launch_dots(s, n, h->r.p, z, flexible ? z : nullptr, flexible ? h->rprev.p : nullptr, h->part.p,
+                     fin_one(h, FIN_BETA, h->dots.p, flexible)));
   SA_TRY(launch_cg_pupdate(s, n, h->cg.p, z, h->p.p, 0));
-  int np = 0;
-  SA_TRY(op_spmv_dot(h, h->p.p, h->q.p, h->part.p, &np));
-  SA_TRY(launch_finish(s, h->part.p, np, h->dots.p));
-  SA_TRY(launch_cg_alpha(s, h->cg.p, h->dots.p));
-  SA_TRY(launch_cg_update(s, n, h->cg.p, h->p.p, h->q.p, h->xb.p, h->r.p, flexible ? h->rprev.p : nullptr,
-                          h->part.p));
-  SA_TRY(launch_finish(s, h->part.p, RED_BLOCKS, h->dots.p + 4));
-  k_loop_ctrl<<<1, 1, 0, s>>>(ch, h->it_dev.p, h->cg.p, h->dots.p + 4, h->ctl.p, h->opt.maxit);
-  SA_LAUNCHED();
+  SA_TRY(op_spmv_alpha(h, h->p.p, h->q.p));
+  Fin f = fin_one(h, FIN_LOOP, h->dots.p + 4);
+  f.loop = (unsigned long long)ch;
+  f.it = h->it_dev.p;
+  f.ctl = h->ctl.p;
+  f.maxit = h->opt.maxit;
+  SA_TRY(launch_cg_update(s, n, h->cg.p, h->p.p, h->q.p, h->xb.p, h->r.p, flexible ? h->rprev.p : nullptr, h->part.p,
+                          f));
   return SA_OK;
 }
 
@@ -497,7 +511,7 @@ static int cg_graph(sa_handle h, const double* b, double* x, double tol, sa_solv
   SA_TRY(copy_in_guess(h, h->xb.p, x, sizeof(double) * n));
   int status = SA_ERR_NO_CONVERGENCE, it = 0;
   SA_TRY(op_residual(h, h->bb.p, h->xb.p, h->r.p));
-  SA_TRY(launch_dots(s, n, h->r.p, h->r.p, nullptr, nullptr, nullptr, nullptr, h->part.p, h->dots.p));
+  SA_TRY(norm2(h, h->r.p, h->dots.p));
   SA_CUDA(cudaMemcpyAsync(hp, h->dots.p, sizeof(double), cudaMemcpyDeviceToHost, s));
   SA_CUDA(cudaStreamSynchronize(s));
   const double r0 = sqrt(hp[0]);
@@ -508,15 +522,10 @@ static int cg_graph(sa_handle h, const double* b, double* x, double tol, sa_solv
     double* z = nullptr;
     SA_TRY(precondition(h, h->r.p, &z));
     SA_TRY(launch_cg_pupdate(s, n, h->cg.p, z, h->p.p, 1));
-    SA_TRY(launch_dots(s, n, h->r.p, z, nullptr, nullptr, nullptr, nullptr, h->part.p, h->dots.p));
-    SA_TRY(launch_cg_beta(s, h->cg.p, h->dots.p, -1));
-    int np = 0;
-    SA_TRY(op_spmv_dot(h, h->p.p, h->q.p, h->part.p, &np));
-    SA_TRY(launch_finish(s, h->part.p, np, h->dots.p));
-    SA_TRY(launch_cg_alpha(s, h->cg.p, h->dots.p));
+    SA_TRY(launch_dots(s, n, h->r.p, z, nullptr, nullptr, h->part.p, fin_one(h, FIN_BETA, h->dots.p, -1)));
+    SA_TRY(op_spmv_alpha(h, h->p.p, h->q.p));
     SA_TRY(launch_cg_update(s, n, h->cg.p, h->p.p, h->q.p, h->xb.p, h->r.p, flexible ? h->rprev.p : nullptr,
-                            h->part.p));
-    SA_TRY(launch_finish(s, h->part.p, RED_BLOCKS, h->dots.p + 4));
+                            h->part.p, fin_one(h, FIN_STORE, h->dots.p + 4)));
     int one = 1;
     SA_CUDA(cudaMemcpyAsync(h->it_dev.p, &one, sizeof(int), cudaMemcpyHostToDevice, s));
     bool graph_launched = false;
@@ -531,7 +540,7 @@ static int cg_graph(sa_handle h, const double* b, double* x, double tol, sa_solv
       if (brk) { status = SA_ERR_BREAKDOWN; break; }
       if (sqrt(hp[0]) <= tol * r0) {
         SA_TRY(op_residual(h, h->bb.p, h->xb.p, h->t.p));
-        SA_TRY(launch_dots(s, n, h->t.p, h->t.p, nullptr, nullptr, nullptr, nullptr, h->part.p, h->dots.p + 6));
+        SA_TRY(norm2(h, h->t.p, h->dots.p + 6));
         SA_CUDA(cudaMemcpyAsync(hp + 3, h->dots.p + 6, sizeof(double), cudaMemcpyDeviceToHost, s));
         SA_CUDA(cudaStreamSynchronize(s));
         if (sqrt(hp[3]) <= tol * r0) { status = SA_OK; break; }
@@ -546,7 +555,7 @@ static int cg_graph(sa_handle h, const double* b, double* x, double tol, sa_solv
     status = SA_OK;
   }
   SA_TRY(op_residual(h, h->bb.p, h->xb.p, h->t.p));
-  SA_TRY(launch_dots(s, n, h->t.p, h->t.p, nullptr, nullptr, nullptr, nullptr, h->part.p, h->dots.p + 6));
+  SA_TRY(norm2(h, h->t.p, h->dots.p + 6));
   SA_CUDA(cudaMemcpyAsync(hp + 3, h->dots.p + 6, sizeof(double), cudaMemcpyDeviceToHost, s));
   SA_CUDA(cudaMemcpyAsync(x, h->xb.p, sizeof(double) * n, cudaMemcpyDefault, s));
   SA_CUDA(cudaStreamSynchronize(s));
@@ -640,7 +649,7 @@ static int cg_block(sa_handle h, int k, const double* B, double* X, double tol, 
   int act[KMAX_BLOCK], its[KMAX_BLOCK], st[KMAX_BLOCK];
   struct { double rr[KMAX_BLOCK]; CgScalars S[KMAX_BLOCK]; } hr;
   SA_TRY(launch_bsell_residual64(s, h->A0s, K, Bb, Xb, R));
-  PROF(PK_B_CG_VEC, 0, 2 * vb, launch_bdots(s, n, K, R, R, nullptr, nullptr, part, dots));
+  PROF(PK_B_CG_VEC, 0, 2 * vb, launch_bdots(s, n, K, R, R, nullptr, nullptr, part, fin_block(h, K, FIN_STORE, dots)));
   SA_CUDA(cudaMemcpyAsync(hb, dots, sizeof(double) * K, cudaMemcpyDeviceToHost, s));
   SA_CUDA(cudaStreamSynchronize(s));
   int nact = 0;
@@ -657,16 +666,13 @@ static int cg_block(sa_handle h, int k, const double* B, double* X, double tol, 
     double* Z = nullptr;
     SA_TRY(precondition_block(h, K, R, &Z));
     PROF(PK_B_CG_VEC, 0, 2 * vb, launch_bcg_pupdate(s, n, K, h->kS.p, h->kact.p, Z, P, 1));
-    PROF(PK_B_CG_VEC, 0, 2 * vb, launch_bdots(s, n, K, R, Z, nullptr, nullptr, part, dots));
-    SA_TRY(launch_bcg_beta(s, K, h->kS.p, dots, -1, h->kact.p));
+    PROF(PK_B_CG_VEC, 0, 2 * vb,
+         launch_bdots(s, n, K, R, Z, nullptr, nullptr, part, fin_block(h, K, FIN_BETA, dots, -1)));
     for (int it = 1;; ++it) {
-      int np = 0;
-      SA_TRY(launch_bsell_spmv_dot(s, h->A0s, K, P, Q, part, &np));
-      SA_TRY(launch_bfinish(s, part, np, K, dots));
-      SA_TRY(launch_bcg_alpha(s, K, h->kS.p, dots, h->kact.p));
+      SA_TRY(launch_bsell_spmv_dot(s, h->A0s, K, P, Q, part, fin_block(h, K, FIN_ALPHA, dots)));
       PROF(PK_B_CG_VEC, 0, (flexible ? 7 : 6) * vb,
-           launch_bcg_update(s, n, K, h->kS.p, h->kact.p, P, Q, Xb, R, flexible ? Rp : nullptr, part));
-      SA_TRY(launch_bfinish(s, part, RED_BLOCKS, K, dots + 2 * KMAX_BLOCK));
+           launch_bcg_update(s, n, K, h->kS.p, h->kact.p, P, Q, Xb, R, flexible ? Rp : nullptr, part,
+                             fin_block(h, K, FIN_STORE, dots + 2 * KMAX_BLOCK)));
       SA_CUDA(cudaMemcpyAsync(hr.rr, dots + 2 * KMAX_BLOCK, sizeof(double) * K, cudaMemcpyDeviceToHost, s));
       SA_CUDA(cudaMemcpyAsync(hr.S, h->kS.p, sizeof(CgScalars) * K, cudaMemcpyDeviceToHost, s));
       SA_CUDA(cudaStreamSynchronize(s));
@@ -681,7 +687,7 @@ static int cg_block(sa_handle h, int k, const double* B, double* X, double tol, 
       }
       if (cand) {
         SA_TRY(launch_bsell_residual64(s, h->A0s, K, Bb, Xb, T));
-        SA_TRY(launch_bdots(s, n, K, T, T, nullptr, nullptr, part, dots + 3 * KMAX_BLOCK));
+        SA_TRY(launch_bdots(s, n, K, T, T, nullptr, nullptr, part, fin_block(h, K, FIN_STORE, dots + 3 * KMAX_BLOCK)));
         SA_CUDA(cudaMemcpyAsync(hb, dots + 3 * KMAX_BLOCK, sizeof(double) * K, cudaMemcpyDeviceToHost, s));
         SA_CUDA(cudaStreamSynchronize(s));
         for (int c = 0; c < K; ++c) {
@@ -704,14 +710,14 @@ static int cg_block(sa_handle h, int k, const double* B, double* X, double tol, 
       if (nact == 0) break;
       SA_TRY(precondition_block(h, K, R, &Z));
       PROF(PK_B_CG_VEC, 0, (flexible ? 3 : 2) * vb,
-           launch_bdots(s, n, K, R, Z, flexible ? Z : nullptr, flexible ? Rp : nullptr, part, dots));
-      SA_TRY(launch_bcg_beta(s, K, h->kS.p, dots, flexible, h->kact.p));
+           launch_bdots(s, n, K, R, Z, flexible ? Z : nullptr, flexible ? Rp : nullptr, part,
+                        fin_block(h, K, FIN_BETA, dots, flexible)));
       PROF(PK_B_CG_VEC, 0, 3 * vb, launch_bcg_pupdate(s, n, K, h->kS.p, h->kact.p, Z, P, 0));
     }
   }
   // true residuals at exit and the solutions
   SA_TRY(launch_bsell_residual64(s, h->A0s, K, Bb, Xb, T));
-  SA_TRY(launch_bdots(s, n, K, T, T, nullptr, nullptr, part, dots + 3 * KMAX_BLOCK));
+  SA_TRY(launch_bdots(s, n, K, T, T, nullptr, nullptr, part, fin_block(h, K, FIN_STORE, dots + 3 * KMAX_BLOCK)));
   SA_CUDA(cudaMemcpyAsync(hb, dots + 3 * KMAX_BLOCK, sizeof(double) * K, cudaMemcpyDeviceToHost, s));
   SA_TRY(launch_interleave(s, n, k, K, Xb, h->kStage.p, 0));
   SA_CUDA(cudaMemcpyAsync(X, h->kStage.p, sizeof(double) * n * k, cudaMemcpyDefault, s));
@@ -942,7 +948,7 @@ int sa_setup(const sa_problem* prob, const sa_options* opt, sa_handle* out) {
   h->al.fn_alloc = opt->alloc;
   h->al.fn_free = opt->dealloc;
   h->al.ctx = opt->alloc_ctx;
-  if (cudaMallocHost(&h->host_pin, 64) != cudaSuccess) {
+  if (cudaMallocHost(&h->host_pin, 16 * sa::GROUP_MAX) != cudaSuccess) {
     cudaGetLastError();
     delete h;
     return SA_ERR_OOM;
@@ -1386,7 +1392,7 @@ int sa_deserialize(const void* buf, uint64_t bytes, const sa_options* opt, sa_ha
   h->al.fn_alloc = opt->alloc;
   h->al.fn_free = opt->dealloc;
   h->al.ctx = opt->alloc_ctx;
-  if (cudaMallocHost(&h->host_pin, 64) != cudaSuccess) {
+  if (cudaMallocHost(&h->host_pin, 16 * sa::GROUP_MAX) != cudaSuccess) {
     cudaGetLastError();
     delete h;
     return SA_ERR_OOM;
@@ -1792,7 +1798,6 @@ static int cg_group(std::vector<sa_handle>& hs, std::vector<VHier<T>*>& vh, cons
   ar.al = &hs[0]->al;
   Buf<double> gath;
   SA_TRY(gath.alloc(&hs[0]->al, 2 * GROUP_MAX));
-  std::vector<double> hg(2 * GROUP_MAX);
   GroupVcycle<T> V;
   V.hs = hs;
   V.vh = vh;
@@ -1803,9 +1808,8 @@ static int cg_group(std::vector<sa_handle>& hs, std::vector<VHier<T>*>& vh, cons
   }
   // descriptor arrays for a set of problems
   struct Ops {
-    size_t resid_r, resid_t, dots_rr, fin_dots, dots_tt, fin_dots4, spmv, fin_spmv, alpha, update, fin_upd, beta0,
-        beta, pup1, pup, dots_rz, gather;
-    unsigned rows;
+    size_t resid_r, resid_t, dots_rr, dots_tt, spmv, update, beta0, beta, pup1, pup;
+    unsigned rows, red;
     int m;
   };
   auto build = [&](const std::vector<int>& set, Ops& o) {
@@ -1814,53 +1818,65 @@ static int cg_group(std::vector<sa_handle>& hs, std::vector<VHier<T>*>& vh, cons
     for (int i : set) {
       sa_handle h = hs[i];
       GCg g = {};
-      g.blk0 = blk;
       g.n = h->n;
       g.sp = h->A0s.sp.p; g.ci = h->A0s.ci.p; g.v = h->A0s.v.p;
       g.base = h->A0s.idx16 ? h->A0s.base.p : nullptr;
       g.c16 = h->A0s.idx16 ? h->A0s.c16.p : nullptr;
       g.cg = h->cg.p;
       g.part = h->part.p;
+      g.tick = h->tick.p;
+      g.gather = gath.p + 2 * base.size();
+      g.blk0 = blk;
+      g.nblk = g256(h->n);
       base.push_back(g);
-      blk += g256(h->n);
+      blk += g.nblk;
     }
     o.rows = blk;
     o.m = (int)set.size();
-    auto var = [&](auto fn) {
-      std::vector<GCg> v = base;
+    std::vector<GCg> rbase = base;  // reduction geometry
+    o.red = 0;
+    for (GCg& g : rbase) {
+      g.blk0 = o.red;
+      g.nblk = red_blocks(g.n);
+      o.red += g.nblk;
+    }
+    auto var = [&](const std::vector<GCg>& from, auto fn) {
+      std::vector<GCg> v = from;
       for (size_t k = 0; k < set.size(); ++k) fn(v[k], hs[set[k]], vh[set[k]]);
       return ar.put(v);
     };
-    o.resid_r = var([](GCg& g, sa_handle h, VHier<T>*) { g.in = h->xb.p; g.bvec = h->bb.p; g.out = h->r.p; });
-    o.resid_t = var([](GCg& g, sa_handle h, VHier<T>*) { g.in = h->xb.p; g.bvec = h->bb.p; g.out = h->t.p; });
-    o.dots_rr = var([](GCg& g, sa_handle h, VHier<T>*) { g.a0 = h->r.p; g.b0 = h->r.p; });
-    o.dots_tt = var([](GCg& g, sa_handle h, VHier<T>*) { g.a0 = h->t.p; g.b0 = h->t.p; });
-    o.dots_rz = var([&](GCg& g, sa_handle h, VHier<T>* w) {
+    o.resid_r = var(base, [](GCg& g, sa_handle h, VHier<T>*) { g.in = h->xb.p; g.bvec = h->bb.p; g.out = h->r.p; });
+    o.resid_t = var(base, [](GCg& g, sa_handle h, VHier<T>*) { g.in = h->xb.p; g.bvec = h->bb.p; g.out = h->t.p; });
+    o.spmv = var(base, [](GCg& g, sa_handle h, VHier<T>*) { g.in = h->p.p; g.out = h->q.p; g.tail = GT_ALPHA; });
+    o.dots_rr = var(rbase, [](GCg& g, sa_handle h, VHier<T>*) { g.a0 = h->r.p; g.b0 = h->r.p; g.tail = GT_GATHER; });
+    o.dots_tt = var(rbase, [](GCg& g, sa_handle h, VHier<T>*) { g.a0 = h->t.p; g.b0 = h->t.p; g.tail = GT_GATHER; });
+    auto rz = [&](GCg& g, sa_handle h, VHier<T>* w) {
       g.a0 = h->r.p; g.b0 = w->z.p;
       if (flexible) { g.a1 = w->z.p; g.b1 = h->rprev.p; }
+      g.tail = GT_BETA;
+      g.flexible = flexible;
+    };
+    o.beta0 = var(rbase, [&](GCg& g, sa_handle h, VHier<T>* w) {
+      rz(g, h, w);
+      g.a1 = g.b1 = nullptr;
+      g.flexible = -1;
     });
-    o.fin_dots = var([](GCg& g, sa_handle h, VHier<T>*) { g.np = RED_BLOCKS; g.stride = RED_BLOCKS; g.dots = h->dots.p; });
-    o.fin_dots4 = var([](GCg& g, sa_handle h, VHier<T>*) { g.np = RED_BLOCKS; g.stride = RED_BLOCKS; g.dots = h->dots.p + 4; });
-    o.spmv = var([](GCg& g, sa_handle h, VHier<T>*) { g.in = h->p.p; g.out = h->q.p; });
-    o.fin_spmv = var([](GCg& g, sa_handle h, VHier<T>*) { g.np = (int)g256(h->n); g.stride = 0; g.dots = h->dots.p; });
-    o.alpha = var([](GCg& g, sa_handle h, VHier<T>*) { g.dots = h->dots.p; });
-    o.update = var([&](GCg& g, sa_handle h, VHier<T>*) {
+    o.beta = var(rbase, rz);
+    o.update = var(rbase, [&](GCg& g, sa_handle h, VHier<T>*) {
       g.x = h->xb.p; g.r = h->r.p; g.rprev = flexible ? h->rprev.p : nullptr; g.p = h->p.p; g.q = h->q.p;
+      g.tail = GT_GATHER;
     });
-    o.fin_upd = var([](GCg& g, sa_handle h, VHier<T>*) { g.np = RED_BLOCKS; g.stride = 0; g.dots = h->dots.p + 4; });
-    o.beta0 = var([](GCg& g, sa_handle h, VHier<T>*) { g.dots = h->dots.p; g.flexible = -1; });
-    o.beta = var([&](GCg& g, sa_handle h, VHier<T>*) { g.dots = h->dots.p; g.flexible = flexible; });
-    o.pup1 = var([](GCg& g, sa_handle h, VHier<T>* w) { g.in = w->z.p; g.out = h->p.p; g.first = 1; });
-    o.pup = var([](GCg& g, sa_handle h, VHier<T>* w) { g.in = w->z.p; g.out = h->p.p; g.first = 0; });
-    o.gather = var([&](GCg& g, sa_handle h, VHier<T>*) { g.dots = h->dots.p + 4; g.gather = gath.p; });
+    o.pup1 = var(rbase, [](GCg& g, sa_handle h, VHier<T>* w) { g.in = w->z.p; g.out = h->p.p; g.first = 1; });
+    o.pup = var(rbase, [](GCg& g, sa_handle h, VHier<T>* w) { g.in = w->z.p; g.out = h->p.p; g.first = 0; });
   };
-  auto L = [&](int op, size_t off, const Ops& o, unsigned blocks) {
+  auto L = [&](int op, size_t off, const Ops& o) {
+    const unsigned blocks = op == GC_RESID || op == GC_SPMV_DOT ? o.rows : o.red;
     return launch_g_cg(s, op, ar.at<GCg>(off), o.m, blocks);
   };
-  // host copy of the gathered (r.r, breakdown) pairs of the problems in `set`
-  auto gather = [&](const Ops& o, size_t off) -> int {
-    SA_TRY(L(GC_GATHER, off, o, 0));
-    SA_CUDA(cudaMemcpyAsync(hg.data(), gath.p, sizeof(double) * 2 * o.m, cudaMemcpyDeviceToHost, s));
+  // host copy of the (sum, breakdown) pairs the last launch gathered
+  double* hg = hs[0]->host_pin;
+  auto gather = [&](const Ops& o) -> int {
+    SA_CUDA(cudaMemcpyAsync(hg, gath.p, sizeof(double) * 2 * o.m, cudaMemcpyDeviceToHost, s));
     SA_CUDA(cudaStreamSynchronize(s));
     return SA_OK;
   };
@@ -1873,13 +1889,9 @@ static int cg_group(std::vector<sa_handle>& hs, std::vector<VHier<T>*>& vh, cons
   ar.clear();
   build(all, o);
   SA_TRY(ar.upload(s));
-  SA_TRY(L(GC_RESID, o.resid_r, o, o.rows));
-  SA_TRY(L(GC_DOTS, o.dots_rr, o, 0));
-  SA_TRY(L(GC_FINISH, o.fin_dots, o, 0));
-  // gather reads dots + 4; the initial r.r sits in dots[0]: gather it by a
-  // finish into dots + 4 as well (the same sum)
-  SA_TRY(L(GC_FINISH, o.fin_dots4, o, 0));
-  SA_TRY(gather(o, o.gather));
+  SA_TRY(L(GC_RESID, o.resid_r, o));
+  SA_TRY(L(GC_DOTS, o.dots_rr, o));
+  SA_TRY(gather(o));
   for (int i = 0; i < m; ++i) {
     r0[i] = sqrt(hg[2 * i]);
     if (r0[i] > 0.0) act.push_back(i);
@@ -1892,17 +1904,12 @@ static int cg_group(std::vector<sa_handle>& hs, std::vector<VHier<T>*>& vh, cons
     V.plan(ar, act);
     SA_TRY(ar.upload(s));
     SA_TRY(V.run(ar, s));
-    SA_TRY(L(GC_PUPDATE, o.pup1, o, 0));
-    SA_TRY(L(GC_DOTS, o.dots_rz, o, 0));
-    SA_TRY(L(GC_FINISH, o.fin_dots, o, 0));
-    SA_TRY(L(GC_BETA, o.beta0, o, 0));
+    SA_TRY(L(GC_PUPDATE, o.pup1, o));
+    SA_TRY(L(GC_DOTS, o.beta0, o));
     for (it = 1; it <= maxit && !act.empty(); ++it) {
-      SA_TRY(L(GC_SPMV_DOT, o.spmv, o, o.rows));
-      SA_TRY(L(GC_FINISH, o.fin_spmv, o, 0));
-      SA_TRY(L(GC_ALPHA, o.alpha, o, 0));
-      SA_TRY(L(GC_UPDATE, o.update, o, 0));
-      SA_TRY(L(GC_FINISH, o.fin_upd, o, 0));
-      SA_TRY(gather(o, o.gather));
+      SA_TRY(L(GC_SPMV_DOT, o.spmv, o));
+      SA_TRY(L(GC_UPDATE, o.update, o));
+      SA_TRY(gather(o));
       std::vector<int> cand, keep;
       for (size_t k = 0; k < act.size(); ++k) {
         const int i = act[k];
@@ -1918,10 +1925,9 @@ static int cg_group(std::vector<sa_handle>& hs, std::vector<VHier<T>*>& vh, cons
         const size_t mark = ar.img.size();
         build(cand, oc);  // appended to the image of the iterating set and uploaded with it
         SA_TRY(ar.upload(s));
-        SA_TRY(L(GC_RESID, oc.resid_t, oc, oc.rows));
-        SA_TRY(L(GC_DOTS, oc.dots_tt, oc, 0));
-        SA_TRY(L(GC_FINISH, oc.fin_dots4, oc, 0));
-        SA_TRY(gather(oc, oc.gather));
+        SA_TRY(L(GC_RESID, oc.resid_t, oc));
+        SA_TRY(L(GC_DOTS, oc.dots_tt, oc));
+        SA_TRY(gather(oc));
         std::vector<int> still;
         for (size_t k = 0; k < cand.size(); ++k) {
           const int i = cand[k];
@@ -1945,20 +1951,17 @@ static int cg_group(std::vector<sa_handle>& hs, std::vector<VHier<T>*>& vh, cons
         SA_TRY(ar.upload(s));
       }
       SA_TRY(V.run(ar, s));
-      SA_TRY(L(GC_DOTS, o.dots_rz, o, 0));
-      SA_TRY(L(GC_FINISH, o.fin_dots, o, 0));
-      SA_TRY(L(GC_BETA, o.beta, o, 0));
-      SA_TRY(L(GC_PUPDATE, o.pup, o, 0));
+      SA_TRY(L(GC_DOTS, o.beta, o));
+      SA_TRY(L(GC_PUPDATE, o.pup, o));
     }
   }
   // true residuals at exit, the solutions
   ar.clear();
   build(all, o);
   SA_TRY(ar.upload(s));
-  SA_TRY(L(GC_RESID, o.resid_t, o, o.rows));
-  SA_TRY(L(GC_DOTS, o.dots_tt, o, 0));
-  SA_TRY(L(GC_FINISH, o.fin_dots4, o, 0));
-  SA_TRY(gather(o, o.gather));
+  SA_TRY(L(GC_RESID, o.resid_t, o));
+  SA_TRY(L(GC_DOTS, o.dots_tt, o));
+  SA_TRY(gather(o));
   for (int i = 0; i < m; ++i)
     SA_CUDA(cudaMemcpyAsync(X[i], hs[i]->xb.p, sizeof(double) * hs[i]->n, cudaMemcpyDefault, s));
   SA_CUDA(cudaStreamSynchronize(s));

@@ -7,6 +7,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "reduce.cuh"
 #include "solve.cuh"
 
 namespace sa {
@@ -69,11 +70,15 @@ __device__ __forceinline__ void block_sum_to(double (&val)[NV], double* __restri
   }
 }
 
-// partial sums of up to three dot products over a fixed grid
-__global__ void k_dots(int64_t n, const double* __restrict__ a0, const double* __restrict__ b0,
-                       const double* __restrict__ a1, const double* __restrict__ b1, const double* __restrict__ a2,
-                       const double* __restrict__ b2, double* __restrict__ part) {
-  double acc[3] = {0.0, 0.0, 0.0};
+// one or two dot products over a fixed grid, finished by the last block
+template <int NV>
+__global__ void __launch_bounds__(RED_THREADS) k_dots(int64_t n, const double* __restrict__ a0,
+                                                      const double* __restrict__ b0, const double* __restrict__ a1,
+                                                      const double* __restrict__ b1, double* __restrict__ part,
+                                                      Fin fin) {
+  double acc[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) acc[v] = 0.0;
   // two grid-stride elements per trip, their loads issued together and
   // added in the grid-stride order (the sums do not depend on the unroll)
   const int64_t st = (int64_t)gridDim.x * blockDim.x;
@@ -83,41 +88,14 @@ __global__ void k_dots(int64_t n, const double* __restrict__ a0, const double* _
     const double u0 = a0[i], v0 = b0[i], u1 = two ? a0[j] : 0.0, v1 = two ? b0[j] : 0.0;
     acc[0] = fma(u0, v0, acc[0]);
     if (two) acc[0] = fma(u1, v1, acc[0]);
-    if (a1) {
+    if constexpr (NV > 1) {
       const double e0 = a1[i], f0 = b1[i], e1 = two ? a1[j] : 0.0, f1 = two ? b1[j] : 0.0;
       acc[1] = fma(e0, f0, acc[1]);
       if (two) acc[1] = fma(e1, f1, acc[1]);
     }
-    if (a2) {
-      const double e0 = a2[i], f0 = b2[i], e1 = two ? a2[j] : 0.0, f1 = two ? b2[j] : 0.0;
-      acc[2] = fma(e0, f0, acc[2]);
-      if (two) acc[2] = fma(e1, f1, acc[2]);
-    }
   }
-  block_sum_to<3>(acc, part, RED_BLOCKS);
-}
-
-// sums `np` partials of each of 3 dots in index order -> out[0..2]
-__global__ void k_dots_finish(const double* __restrict__ part, int np, int stride, double* __restrict__ out) {
-  double acc[3] = {0.0, 0.0, 0.0};
-  for (int t = threadIdx.x; t < np; t += blockDim.x)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) acc[k] += part[(int64_t)k * stride + t];
-  __shared__ double sh[3][32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    double t = warp_sum(acc[k]);
-    if (lane == 0) sh[k][w] = t;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < 3; ++k) {
-      double s = 0.0;
-      for (int q = 0; q < nw; ++q) s += sh[k][q];
-      out[k] = s;
-    }
-  }
+  block_sum_to<NV>(acc, part, RED_BLOCKS);
+  fin_inline<NV, RED_THREADS>(fin, part, (int)gridDim.x, RED_BLOCKS, 1);
 }
 
 // ---------------------------------------------------------------------------
@@ -142,48 +120,20 @@ __global__ void k_start_vector(int64_t n, uint32_t tag, uint32_t seed, double* _
   }
 }
 
-// partial sums of w.w and v.v with v_j = X_j * sc[4]
-__global__ void k_power_dots(int64_t n, const double* __restrict__ w, const double* __restrict__ X,
-                             const double* __restrict__ sc, double* __restrict__ part) {
+// w.w and v.v with v_j = X_j * sc[4]; the last block takes the estimate and
+// the next scale from them (FIN_POWER)
+__global__ void __launch_bounds__(RED_THREADS) k_power_dots(int64_t n, const double* __restrict__ w,
+                                                            const double* __restrict__ X, const double* sc,
+                                                            double* __restrict__ part, Fin fin) {
   const double inv = sc[4];
-  double acc[3] = {0.0, 0.0, 0.0};
+  double acc[2] = {0.0, 0.0};
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const double vi = X[i] * inv;
     acc[0] += w[i] * w[i];
     acc[1] += vi * vi;
   }
-  block_sum_to<3>(acc, part, RED_BLOCKS);
-}
-
-// one CTA: sums the partials in index order, then lam = ||w|| / ||v||,
-// sc[2] = ||w|| and sc[4] = 1 / ||w|| (the scale of the next iterate).  A zero product (every
-// row unscaled) gives lam = 0 and stops the iteration (sc[3] = 1).
-__global__ void k_power_finish(const double* __restrict__ part, double* __restrict__ sc, double* __restrict__ lam) {
-  double acc[3] = {0.0, 0.0, 0.0};
-  for (int t = threadIdx.x; t < RED_BLOCKS; t += blockDim.x)
-#pragma unroll
-    for (int k = 0; k < 2; ++k) acc[k] += part[(int64_t)k * RED_BLOCKS + t];
-  __shared__ double sh[2][32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    double t = warp_sum(acc[k]);
-    if (lane == 0) sh[k][w] = t;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double ww = 0.0, vv = 0.0;
-    for (int q = 0; q < nw; ++q) { ww += sh[0][q]; vv += sh[1][q]; }
-    double nw2 = sqrt(ww);
-    if (nw2 == 0.0 || sc[3] != 0.0) {
-      sc[3] = 1.0;
-      *lam = 0.0;
-      return;
-    }
-    *lam = nw2 / sqrt(vv);
-    sc[2] = nw2;
-    sc[4] = 1.0 / nw2;
-  }
+  block_sum_to<2>(acc, part, RED_BLOCKS);
+  fin_inline<2, RED_THREADS>(fin, part, (int)gridDim.x, RED_BLOCKS, 1);
 }
 
 __global__ void k_rsqrt_scale(int64_t n, const double* __restrict__ d, double* __restrict__ out) {
@@ -221,10 +171,10 @@ int pick_sw(int64_t n, int64_t nnz) {
   } while (0)
 
 int launch_dots(cudaStream_t st, int64_t n, const double* a0, const double* b0, const double* a1,
-                const double* b1, const double* a2, const double* b2, double* part, double* out) {
-  k_dots<<<RED_BLOCKS, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, a2, b2, part);
-  SA_LAUNCHED();
-  k_dots_finish<<<1, 1024, 0, st>>>(part, RED_BLOCKS, RED_BLOCKS, out);
+                const double* b1, double* part, const Fin& fin) {
+  const unsigned g = red_blocks(n);
+  if (a1) k_dots<2><<<g, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part, fin);
+  else k_dots<1><<<g, RED_THREADS, 0, st>>>(n, a0, b0, nullptr, nullptr, part, fin);
   SA_LAUNCHED();
   return SA_OK;
 }
@@ -237,10 +187,15 @@ int run_power(Alloc& al, int64_t n, const int64_t* rp, const int32_t* ci, const 
   SA_TRY(x.alloc(&al, n));
   SA_TRY(w.alloc(&al, n));
   SA_TRY(y.alloc(&al, n));
-  SA_TRY(part.alloc(&al, 3 * RED_BLOCKS));
-  SA_TRY(sc.alloc(&al, 5));
-  const double init[5] = {0.0, 0.0, 1.0, 0.0, 1.0};
+  SA_TRY(part.alloc(&al, 2 * RED_BLOCKS));
+  SA_TRY(sc.alloc(&al, 6));  // scalars, ticket of the finishing block
+  const double init[6] = {0.0, 0.0, 1.0, 0.0, 1.0, 0.0};
   SA_CUDA(cudaMemcpyAsync(sc.p, init, sizeof(init), cudaMemcpyHostToDevice, st));
+  Fin fin;
+  fin.op = FIN_POWER;
+  fin.tick = reinterpret_cast<unsigned*>(sc.p + 5);
+  fin.sc = sc.p;
+  fin.lam = lam_dev;
   int64_t nnz = 0;
   SA_TRY(copy_d2h(&nnz, rp + n, sizeof(int64_t), st));
   const double avg = (double)nnz / (double)n;
@@ -254,9 +209,7 @@ int run_power(Alloc& al, int64_t n, const int64_t* rp, const int32_t* ci, const 
     SA_LAUNCHED();
     DISPATCH_SW(sw, k_power_spmv, n, n, rp, ci, v, s, y.p, W);
     SA_LAUNCHED();
-    k_power_dots<<<RED_BLOCKS, RED_THREADS, 0, st>>>(n, W, X, sc.p, part.p);
-    SA_LAUNCHED();
-    k_power_finish<<<1, 1024, 0, st>>>(part.p, sc.p, lam_dev);
+    k_power_dots<<<red_blocks(n), RED_THREADS, 0, st>>>(n, W, X, sc.p, part.p, fin);
     SA_LAUNCHED();
     double* t = X; X = W; W = t;
   }
@@ -271,10 +224,15 @@ int run_power_op(Alloc& al, int64_t n, int steps, uint32_t tag, uint32_t seed, d
   SA_TRY(x.alloc(&al, n));
   SA_TRY(w.alloc(&al, n));
   SA_TRY(y.alloc(&al, n));
-  SA_TRY(part.alloc(&al, 3 * RED_BLOCKS));
-  SA_TRY(sc.alloc(&al, 5));
-  const double init[5] = {0.0, 0.0, 1.0, 0.0, 1.0};
+  SA_TRY(part.alloc(&al, 2 * RED_BLOCKS));
+  SA_TRY(sc.alloc(&al, 6));  // scalars, ticket of the finishing block
+  const double init[6] = {0.0, 0.0, 1.0, 0.0, 1.0, 0.0};
   SA_CUDA(cudaMemcpyAsync(sc.p, init, sizeof(init), cudaMemcpyHostToDevice, st));
+  Fin fin;
+  fin.op = FIN_POWER;
+  fin.tick = reinterpret_cast<unsigned*>(sc.p + 5);
+  fin.sc = sc.p;
+  fin.lam = lam_dev;
   k_start_vector<<<blocks_for(n, 256), 256, 0, st>>>(n, tag, seed, x.p);
   SA_LAUNCHED();
   double* X = x.p;
@@ -283,9 +241,7 @@ int run_power_op(Alloc& al, int64_t n, int steps, uint32_t tag, uint32_t seed, d
     k_power_prep<<<blocks_for(n, 256), 256, 0, st>>>(n, X, nullptr, sc.p, y.p);
     SA_LAUNCHED();
     SA_TRY(apply(y.p, W));
-    k_power_dots<<<RED_BLOCKS, RED_THREADS, 0, st>>>(n, W, X, sc.p, part.p);
-    SA_LAUNCHED();
-    k_power_finish<<<1, 1024, 0, st>>>(part.p, sc.p, lam_dev);
+    k_power_dots<<<red_blocks(n), RED_THREADS, 0, st>>>(n, W, X, sc.p, part.p, fin);
     SA_LAUNCHED();
     double* t = X; X = W; W = t;
   }
@@ -315,19 +271,12 @@ int launch_omega(cudaStream_t s, const double* lam_dev, double omega_sym, double
 // ---------------------------------------------------------------------------
 // CG with device-resident scalars (Sec. 4)
 // ---------------------------------------------------------------------------
-// alpha = rz / pq (pq = dots[0]); flags breakdown when pq <= 0 or NaN
-__global__ void k_cg_alpha(CgScalars* __restrict__ s, const double* __restrict__ dots) {
-  double pq = dots[0];
-  s->pq = pq;
-  if (!(pq > 0.0)) { s->breakdown = 1; s->alpha = 0.0; return; }
-  s->alpha = s->rz / pq;
-}
-
-// x += alpha p; r -= alpha q; (r_prev = r before the update, if given);
-// partial sums of r.r
-__global__ void k_cg_update(int64_t n, const CgScalars* __restrict__ s, const double* __restrict__ p,
-                            const double* __restrict__ q, double* __restrict__ x, double* __restrict__ r,
-                            double* __restrict__ rprev, double* __restrict__ part) {
+// x += alpha p; r -= alpha q; (r_prev = r before the update, if given); r.r,
+// finished by the last block
+__global__ void __launch_bounds__(RED_THREADS) k_cg_update(int64_t n, const CgScalars* s, const double* __restrict__ p,
+                                                           const double* __restrict__ q, double* __restrict__ x,
+                                                           double* __restrict__ r, double* __restrict__ rprev,
+                                                           double* __restrict__ part, Fin fin) {
   const double alpha = s->alpha;
   double acc[1] = {0.0};
   // two grid-stride elements per trip (loads together; r.r added in the
@@ -361,21 +310,7 @@ __global__ void k_cg_update(int64_t n, const CgScalars* __restrict__ s, const do
     }
   }
   block_sum_to<1>(acc, part, 0);
-}
-
-// beta from the new r.z (and z.r_prev for flexible CG); flexible < 0
-// initialises rz from dots[0]
-__global__ void k_cg_beta(CgScalars* __restrict__ s, const double* __restrict__ dots, int flexible) {
-  double rz_new = dots[0];
-  if (flexible < 0) {
-    s->rz = rz_new;
-    s->beta = 0.0;
-    s->breakdown = 0;
-    return;
-  }
-  double num = flexible ? rz_new - dots[1] : rz_new;
-  s->beta = num / s->rz;
-  s->rz = rz_new;
+  fin_inline<1, RED_THREADS>(fin, part, (int)gridDim.x, 0, 0);
 }
 
 __global__ void k_cg_pupdate(int64_t n, const CgScalars* __restrict__ s, const double* __restrict__ z,
@@ -392,33 +327,24 @@ __global__ void k_cg_pupdate(int64_t n, const CgScalars* __restrict__ s, const d
   }
 }
 
-int launch_finish(cudaStream_t st, const double* part, int np, double* out) {
-  k_dots_finish<<<1, 1024, 0, st>>>(part, np, 0, out);
-  SA_LAUNCHED();
-  return SA_OK;
-}
-
-int launch_cg_alpha(cudaStream_t st, CgScalars* s, const double* dots) {
-  k_cg_alpha<<<1, 1, 0, st>>>(s, dots);
+// the sums of np partials (k columns, or one vector with k = 0) that the
+// producing launch did not finish itself
+int launch_fin_wide(cudaStream_t st, const double* part, int np, const Fin& fin) {
+  if (fin.k > 0) k_fin_wide<KMAX_BLOCK><<<32, 32 * KMAX_BLOCK, 0, st>>>(part, np, np, fin);
+  else k_fin_wide<1><<<32, 32, 0, st>>>(part, np, 0, fin);
   SA_LAUNCHED();
   return SA_OK;
 }
 
 int launch_cg_update(cudaStream_t st, int64_t n, const CgScalars* s, const double* p, const double* q, double* x,
-                     double* r, double* rprev, double* part) {
-  k_cg_update<<<RED_BLOCKS, RED_THREADS, 0, st>>>(n, s, p, q, x, r, rprev, part);
-  SA_LAUNCHED();
-  return SA_OK;
-}
-
-int launch_cg_beta(cudaStream_t st, CgScalars* s, const double* dots, int flexible) {
-  k_cg_beta<<<1, 1, 0, st>>>(s, dots, flexible);
+                     double* r, double* rprev, double* part, const Fin& fin) {
+  k_cg_update<<<red_blocks(n), RED_THREADS, 0, st>>>(n, s, p, q, x, r, rprev, part, fin);
   SA_LAUNCHED();
   return SA_OK;
 }
 
 int launch_cg_pupdate(cudaStream_t st, int64_t n, const CgScalars* s, const double* z, double* p, int first) {
-  k_cg_pupdate<<<RED_BLOCKS, RED_THREADS, 0, st>>>(n, s, z, p, first);
+  k_cg_pupdate<<<red_blocks(n), RED_THREADS, 0, st>>>(n, s, z, p, first);
   SA_LAUNCHED();
   return SA_OK;
 }
@@ -463,7 +389,8 @@ __device__ __forceinline__ void stgrp(double* p, const double (&v)[G]) {
 template <int KK, int NV>
 __global__ void __launch_bounds__(RED_THREADS, 2) k_bdots(int64_t n, const double* __restrict__ a0,
                                                           const double* __restrict__ b0, const double* __restrict__ a1,
-                                                          const double* __restrict__ b1, double* __restrict__ part) {
+                                                          const double* __restrict__ b1, double* __restrict__ part,
+                                                          Fin fin) {
   constexpr int G = KK >= 4 ? 4 : 2;
   double acc[NV];
 #pragma unroll
@@ -486,50 +413,14 @@ __global__ void __launch_bounds__(RED_THREADS, 2) k_bdots(int64_t n, const doubl
     }
   }
   block_sum_to<NV>(acc, part, RED_BLOCKS);
-}
-
-// out[v] = sum over np partials of value v (stride `stride`), in index order,
-// with the reduction of k_dots_finish
-template <int NV>
-__global__ void k_bdots_finish(const double* __restrict__ part, int np, int stride, double* __restrict__ out) {
-  double acc[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) acc[v] = 0.0;
-  for (int t = threadIdx.x; t < np; t += blockDim.x)
-#pragma unroll
-    for (int v = 0; v < NV; ++v) acc[v] += part[(int64_t)v * stride + t];
-  __shared__ double sh[NV][32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    double t = warp_sum(acc[v]);
-    if (lane == 0) sh[v][w] = t;
-  }
-  __syncthreads();
-  if (threadIdx.x < NV) {
-    double s = 0.0;
-    for (int q = 0; q < nw; ++q) s += sh[threadIdx.x][q];
-    out[threadIdx.x] = s;
-  }
-}
-
-__global__ void k_bcg_alpha(int k, CgScalars* __restrict__ s, const double* __restrict__ dots,
-                            const int* __restrict__ active) {
-  const int c = threadIdx.x;
-  if (c >= k) return;
-  CgScalars& S = s[c];
-  if (!active[c]) { S.alpha = 0.0; return; }
-  const double pq = dots[c];
-  S.pq = pq;
-  if (!(pq > 0.0)) { S.breakdown = 1; S.alpha = 0.0; return; }
-  S.alpha = S.rz / pq;
+  fin_inline<NV, RED_THREADS>(fin, part, (int)gridDim.x, RED_BLOCKS, KB);
 }
 
 template <int KK>
 __global__ void __launch_bounds__(RED_THREADS, 2)
-    k_bcg_update(const int64_t n, const CgScalars* __restrict__ s, const int* __restrict__ active,
+    k_bcg_update(const int64_t n, const CgScalars* s, const int* __restrict__ active,
                  const double* __restrict__ p, const double* __restrict__ q, double* __restrict__ x,
-                 double* __restrict__ r, double* __restrict__ rprev, double* __restrict__ part) {
+                 double* __restrict__ r, double* __restrict__ rprev, double* __restrict__ part, Fin fin) {
   constexpr int G = KK >= 4 ? 4 : 2;
   __shared__ double alpha[KB];
   __shared__ int on[KB];
@@ -574,23 +465,7 @@ __global__ void __launch_bounds__(RED_THREADS, 2)
     }
   }
   block_sum_to<KB>(acc, part, RED_BLOCKS);
-}
-
-__global__ void k_bcg_beta(int k, CgScalars* __restrict__ s, const double* __restrict__ dots, int flexible,
-                           const int* __restrict__ active) {
-  const int c = threadIdx.x;
-  if (c >= k || !active[c]) return;
-  CgScalars& S = s[c];
-  const double rz_new = dots[c];
-  if (flexible < 0) {
-    S.rz = rz_new;
-    S.beta = 0.0;
-    S.breakdown = 0;
-    return;
-  }
-  const double num = flexible ? rz_new - dots[KB + c] : rz_new;
-  S.beta = num / S.rz;
-  S.rz = rz_new;
+  fin_inline<KB, RED_THREADS>(fin, part, (int)gridDim.x, RED_BLOCKS, 0);
 }
 
 template <int KK>
@@ -637,52 +512,30 @@ __global__ void k_interleave(int64_t n, int k, int K, const double* __restrict__
 }
 
 int launch_bdots(cudaStream_t st, int64_t n, int k, const double* a0, const double* b0, const double* a1,
-                 const double* b1, double* part, double* out) {
+                 const double* b1, double* part, const Fin& fin) {
   if (k != 2 && k != 4 && k != 8) return SA_ERR_INVALID_ARG;  // whole-row vectors
+  const unsigned g = red_blocks(n);
   // one dot per column, or two (a1 . b1 into out[KB + c])
   if (a1) {
-    if (k == 2) k_bdots<2, 2 * KB><<<RED_BLOCKS, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part);
-    else if (k == 4) k_bdots<4, 2 * KB><<<RED_BLOCKS, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part);
-    else k_bdots<8, 2 * KB><<<RED_BLOCKS, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part);
-    SA_LAUNCHED();
-    k_bdots_finish<2 * KB><<<1, 1024, 0, st>>>(part, RED_BLOCKS, RED_BLOCKS, out);
+    if (k == 2) k_bdots<2, 2 * KB><<<g, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part, fin);
+    else if (k == 4) k_bdots<4, 2 * KB><<<g, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part, fin);
+    else k_bdots<8, 2 * KB><<<g, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part, fin);
   } else {
-    if (k == 2) k_bdots<2, KB><<<RED_BLOCKS, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part);
-    else if (k == 4) k_bdots<4, KB><<<RED_BLOCKS, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part);
-    else k_bdots<8, KB><<<RED_BLOCKS, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part);
-    SA_LAUNCHED();
-    k_bdots_finish<KB><<<1, 1024, 0, st>>>(part, RED_BLOCKS, RED_BLOCKS, out);
+    if (k == 2) k_bdots<2, KB><<<g, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part, fin);
+    else if (k == 4) k_bdots<4, KB><<<g, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part, fin);
+    else k_bdots<8, KB><<<g, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part, fin);
   }
   SA_LAUNCHED();
   return SA_OK;
 }
 
-// partials laid out as part[c * np + b] (c < KB)
-int launch_bfinish(cudaStream_t st, const double* part, int np, int k, double* out) {
-  if (k < 1 || k > KB) return SA_ERR_INVALID_ARG;
-  k_bdots_finish<KB><<<1, 1024, 0, st>>>(part, np, np, out);
-  SA_LAUNCHED();
-  return SA_OK;
-}
-
-int launch_bcg_alpha(cudaStream_t st, int k, CgScalars* s, const double* dots, const int* active) {
-  k_bcg_alpha<<<1, 32, 0, st>>>(k, s, dots, active);
-  SA_LAUNCHED();
-  return SA_OK;
-}
-
 int launch_bcg_update(cudaStream_t st, int64_t n, int k, const CgScalars* s, const int* active, const double* p,
-                      const double* q, double* x, double* r, double* rprev, double* part) {
+                      const double* q, double* x, double* r, double* rprev, double* part, const Fin& fin) {
   if (k != 2 && k != 4 && k != 8) return SA_ERR_INVALID_ARG;  // whole-row vectors
-  if (k == 2) k_bcg_update<2><<<RED_BLOCKS, RED_THREADS, 0, st>>>(n, s, active, p, q, x, r, rprev, part);
-  else if (k == 4) k_bcg_update<4><<<RED_BLOCKS, RED_THREADS, 0, st>>>(n, s, active, p, q, x, r, rprev, part);
-  else k_bcg_update<8><<<RED_BLOCKS, RED_THREADS, 0, st>>>(n, s, active, p, q, x, r, rprev, part);
-  SA_LAUNCHED();
-  return SA_OK;
-}
-
-int launch_bcg_beta(cudaStream_t st, int k, CgScalars* s, const double* dots, int flexible, const int* active) {
-  k_bcg_beta<<<1, 32, 0, st>>>(k, s, dots, flexible, active);
+  const unsigned g = red_blocks(n);
+  if (k == 2) k_bcg_update<2><<<g, RED_THREADS, 0, st>>>(n, s, active, p, q, x, r, rprev, part, fin);
+  else if (k == 4) k_bcg_update<4><<<g, RED_THREADS, 0, st>>>(n, s, active, p, q, x, r, rprev, part, fin);
+  else k_bcg_update<8><<<g, RED_THREADS, 0, st>>>(n, s, active, p, q, x, r, rprev, part, fin);
   SA_LAUNCHED();
   return SA_OK;
 }
@@ -690,9 +543,9 @@ int launch_bcg_beta(cudaStream_t st, int k, CgScalars* s, const double* dots, in
 int launch_bcg_pupdate(cudaStream_t st, int64_t n, int k, const CgScalars* s, const int* active, const double* z,
                        double* p, int first) {
   if (k != 2 && k != 4 && k != 8) return SA_ERR_INVALID_ARG;  // whole-row vectors
-  if (k == 2) k_bcg_pupdate<2><<<RED_BLOCKS, RED_THREADS, 0, st>>>(n, s, active, z, p, first);
-  else if (k == 4) k_bcg_pupdate<4><<<RED_BLOCKS, RED_THREADS, 0, st>>>(n, s, active, z, p, first);
-  else k_bcg_pupdate<8><<<RED_BLOCKS, RED_THREADS, 0, st>>>(n, s, active, z, p, first);
+  if (k == 2) k_bcg_pupdate<2><<<red_blocks(n), RED_THREADS, 0, st>>>(n, s, active, z, p, first);
+  else if (k == 4) k_bcg_pupdate<4><<<red_blocks(n), RED_THREADS, 0, st>>>(n, s, active, z, p, first);
+  else k_bcg_pupdate<8><<<red_blocks(n), RED_THREADS, 0, st>>>(n, s, active, z, p, first);
   SA_LAUNCHED();
   return SA_OK;
 }

@@ -24,24 +24,20 @@ struct CgScalars {
 };
 
 int pick_sw(int64_t n, int64_t nnz);
+struct Fin;  // what the last block of a reduction does (reduce.cuh)
 int launch_dots(cudaStream_t st, int64_t n, const double* a0, const double* b0, const double* a1, const double* b1,
-                const double* a2, const double* b2, double* part, double* out);
-int launch_finish(cudaStream_t st, const double* part, int np, double* out);
-int launch_cg_alpha(cudaStream_t st, CgScalars* s, const double* dots);
+                double* part, const Fin& fin);
+int launch_fin_wide(cudaStream_t st, const double* part, int np, const Fin& fin);
 int launch_cg_update(cudaStream_t st, int64_t n, const CgScalars* s, const double* p, const double* q, double* x,
-                     double* r, double* rprev, double* part);
-int launch_cg_beta(cudaStream_t st, CgScalars* s, const double* dots, int flexible);
+                     double* r, double* rprev, double* part, const Fin& fin);
 int launch_cg_pupdate(cudaStream_t st, int64_t n, const CgScalars* s, const double* z, double* p, int first);
 
 // k-column versions (k <= KMAX_BLOCK), each column summed in the one-vector
 // order so that a column of a block solve equals the one-vector solve bitwise
 int launch_bdots(cudaStream_t st, int64_t n, int k, const double* a0, const double* b0, const double* a1,
-                 const double* b1, double* part, double* out);
-int launch_bfinish(cudaStream_t st, const double* part, int np, int k, double* out);
-int launch_bcg_alpha(cudaStream_t st, int k, CgScalars* s, const double* dots, const int* active);
+                 const double* b1, double* part, const Fin& fin);
 int launch_bcg_update(cudaStream_t st, int64_t n, int k, const CgScalars* s, const int* active, const double* p,
-                      const double* q, double* x, double* r, double* rprev, double* part);
-int launch_bcg_beta(cudaStream_t st, int k, CgScalars* s, const double* dots, int flexible, const int* active);
+                      const double* q, double* x, double* r, double* rprev, double* part, const Fin& fin);
 int launch_bcg_pupdate(cudaStream_t st, int64_t n, int k, const CgScalars* s, const int* active, const double* z,
                        double* p, int first);
 // column-major n x k <-> interleaved n x K (K >= k; columns k..K-1 zero)

@@ -19,6 +19,7 @@
 #include "common.cuh"
 #include "kernels.cuh"
 #include "profile.cuh"
+#include "reduce.cuh"
 #include "solve.cuh"
 #include "vcycle.cuh"
 #include "vkern.cuh"
@@ -614,11 +615,13 @@ template void vh_free<float>(VHier<float>*);
 // ---------------------------------------------------------------------------
 // FP64 SELL kernels for the outer CG (unscaled fine operator)
 // ---------------------------------------------------------------------------
-// q = A p, partial sums of p.q per CTA (fixed order)
-__global__ void k_sell_spmv_dot(int64_t n, const int64_t* __restrict__ sp, const int32_t* __restrict__ ci,
+// q = A p, partial sums of p.q per CTA (fixed order); INLINE: the last block
+// finishes them
+template <bool INLINE>
+__global__ void __launch_bounds__(256) k_sell_spmv_dot(int64_t n, const int64_t* __restrict__ sp, const int32_t* __restrict__ ci,
                                 const int32_t* __restrict__ base, const uint16_t* __restrict__ c16,
                                 const double* __restrict__ v, const double* __restrict__ p, double* __restrict__ q,
-                                double* __restrict__ part) {
+                                double* __restrict__ part, Fin fin) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double c = 0.0;
   if (i < n) {
@@ -636,6 +639,7 @@ __global__ void k_sell_spmv_dot(int64_t n, const int64_t* __restrict__ sp, const
     t = warp_sum(t);
     if (lane == 0) part[blockIdx.x] = t;
   }
+  if constexpr (INLINE) fin_inline<1, 256>(fin, part, (int)gridDim.x, 0, 0);
 }
 
 __global__ void k_sell_res64(int64_t n, const int64_t* __restrict__ sp, const int32_t* __restrict__ ci,
@@ -648,12 +652,18 @@ __global__ void k_sell_res64(int64_t n, const int64_t* __restrict__ sp, const in
 }
 
 int launch_sell_spmv_dot(cudaStream_t st, const Sell<double>& A, const double* p, double* q, double* part,
-                         int* nparts) {
-  *nparts = (int)g256(A.n);
-  k_sell_spmv_dot<<<g256(A.n), 256, 0, st>>>(A.n, A.sp.p, A.ci.p, A.idx16 ? A.base.p : nullptr,
-                                              A.idx16 ? A.c16.p : nullptr, A.v.p, p, q, part);
+                         const Fin& fin) {
+  const unsigned g = g256(A.n);
+  const int32_t* base = A.idx16 ? A.base.p : nullptr;
+  const uint16_t* c16 = A.idx16 ? A.c16.p : nullptr;
+  if (g <= FIN_INLINE) {
+    k_sell_spmv_dot<true><<<g, 256, 0, st>>>(A.n, A.sp.p, A.ci.p, base, c16, A.v.p, p, q, part, fin);
+    SA_LAUNCHED();
+    return SA_OK;
+  }
+  k_sell_spmv_dot<false><<<g, 256, 0, st>>>(A.n, A.sp.p, A.ci.p, base, c16, A.v.p, p, q, part, fin);
   SA_LAUNCHED();
-  return SA_OK;
+  return launch_fin_wide(st, part, (int)g, fin);
 }
 
 int launch_sell_residual64(cudaStream_t st, const Sell<double>& A, const double* b, const double* x, double* r) {

@@ -126,12 +126,13 @@ template <typename T>
 int vh_vcycle_block(Alloc& al, VHier<T>* m, cudaStream_t s, int k, const double* R, double** Z);
 
 // outer CG on the unscaled fine operator in FP64 SELL
+// q = A p and p.q, summed and stepped as `fin` says
 int launch_sell_spmv_dot(cudaStream_t st, const Sell<double>& A, const double* p, double* q, double* part,
-                         int* nparts);
+                         const Fin& fin);
 int launch_sell_residual64(cudaStream_t st, const Sell<double>& A, const double* b, const double* x, double* r);
 // k-column forms (interleaved blocks); partials at part[c * np + cta]
 int launch_bsell_spmv_dot(cudaStream_t st, const Sell<double>& A, int k, const double* P, double* Q, double* part,
-                          int* nparts);
+                          const Fin& fin);
 int launch_bsell_residual64(cudaStream_t st, const Sell<double>& A, int k, const double* B, const double* X,
                             double* R);
 
