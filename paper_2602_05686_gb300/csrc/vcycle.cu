@@ -388,9 +388,18 @@ template int vh_build<float>(Alloc&, const VLevelIn*, int, int, const CoarseView
 // ---------------------------------------------------------------------------
 // kernels (one thread per row)
 // ---------------------------------------------------------------------------
+// resident blocks per SM asked of the compiler: FP32 rows of several lanes
+// gain from occupancy (6 blocks, 40 registers: 370k rows of 60 entries 55.7 ->
+// 52.3 us), FP64 ones at 5 (183k rows of 46 entries: 51.4 us at 4 blocks, 47.6
+// at 5, 47.0 at 6; 6.9k rows of 128: 21.3, 21.2, 23.7)
+template <typename T, int SW>
+struct VOcc {
+  static constexpr int B = SW > 1 ? (sizeof(T) == 4 ? 6 : 5) : 8;
+};
+
 // x_out = x_in + d,  d = first ? c2 r : c1 d + c2 r,  r = b - A~ x_in
 template <typename T, int SW>
-__global__ void k_vc_cheb(MatView<T> A, const T* __restrict__ b, const T* __restrict__ xin, T* __restrict__ xout,
+__global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_cheb(MatView<T> A, const T* __restrict__ b, const T* __restrict__ xin, T* __restrict__ xout,
                           T* __restrict__ d, T c1, T c2, int first) {
   T y;
   int64_t i;
@@ -401,21 +410,21 @@ __global__ void k_vc_cheb(MatView<T> A, const T* __restrict__ b, const T* __rest
 }
 
 template <typename T, int SW>
-__global__ void k_vc_residual(MatView<T> A, const T* __restrict__ b, const T* __restrict__ x, T* __restrict__ r) {
+__global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_residual(MatView<T> A, const T* __restrict__ b, const T* __restrict__ x, T* __restrict__ r) {
   T y;
   int64_t i;
   if (row_apply<T, SW>(A, x, y, i)) r[i] = b[i] - y;
 }
 
 template <typename T, int SW>
-__global__ void k_vc_spmv(MatView<T> A, const T* __restrict__ x, T* __restrict__ out) {
+__global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_spmv(MatView<T> A, const T* __restrict__ x, T* __restrict__ out) {
   T y;
   int64_t i;
   if (row_apply<T, SW>(A, x, y, i)) out[i] = y;
 }
 
 template <typename T, int SW>
-__global__ void k_vc_spmv_add(MatView<T> A, const T* __restrict__ x, T* __restrict__ out) {
+__global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_spmv_add(MatView<T> A, const T* __restrict__ x, T* __restrict__ out) {
   T y;
   int64_t i;
   if (row_apply<T, SW>(A, x, y, i)) out[i] += y;

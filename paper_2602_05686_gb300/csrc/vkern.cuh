@@ -144,26 +144,67 @@ constexpr int64_t SELL2_ROWS = int64_t(1) << 19;
 constexpr int CSR_UNROLL = 4;
 constexpr int LONG_UNROLL = 8;
 
-// the CSR lane sum of row i over entries b + sl, b + sl + W, ... (< e):
-// U entries loaded per round, added in entry order
+// the CSR lane sum over entries b + sl, b + sl + W, ... (< e), added in entry
+// order, in rounds of U entries.  Several lanes per row (rows of tens of
+// entries): the last round is predicated and the next round's values and
+// columns are loaded while this round's gathers are in flight; a tail of
+// single entries was a chain of dependent loads (FP64 Chebyshev step on 183k
+// rows of 46 entries 53.8 -> 47.6 us, on 6.9k rows of 128 26.1 -> 21.2 us; the
+// rest is rows of unequal length in one warp).  One lane per row (rows of a
+// few entries): full rounds and single entries, the fastest there (120^3 FP32
+// prolongation 26.7 us, 31 to 35 us with predicated or prefetched rounds).
 template <typename T, int W, int U>
 __device__ __forceinline__ T csr_lane(const MatView<T>& M, const T* __restrict__ x, int64_t b, int64_t e, int sl) {
   T acc = (T)0;
-  int64_t q = b + sl;
-  for (; q + W * (U - 1) < e; q += W * U) {
-    T vv[U], xx[U];
+  if constexpr (W == 1) {
+    int64_t q = b + sl;
+    for (; q + W * (U - 1) < e; q += W * U) {
+      T vv[U], xx[U];
+      int32_t cc[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        vv[u] = M.v[q + W * u];
+        cc[u] = M.ci[q + W * u];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) xx[u] = __ldg(&x[cc[u]]);
+#pragma unroll
+      for (int u = 0; u < U; ++u) acc += vv[u] * xx[u];
+    }
+    for (; q < e; q += W) acc += M.v[q] * __ldg(&x[M.ci[q]]);
+  } else {
+    const int len = (int)(e - b);
+    const T* __restrict__ v = M.v + b;
+    const int32_t* __restrict__ ci = M.ci + b;
+    T vv[U];
     int32_t cc[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      vv[u] = M.v[q + W * u];
-      cc[u] = M.ci[q + W * u];
+      const bool in = sl + W * u < len;
+      vv[u] = in ? v[sl + W * u] : (T)0;
+      cc[u] = in ? ci[sl + W * u] : 0;
     }
+    for (int q = sl; q < len; q += W * U) {
+      T xx[U], vn[U];
+      int32_t cn[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) xx[u] = __ldg(&x[cc[u]]);
+      for (int u = 0; u < U; ++u) xx[u] = q + W * u < len ? __ldg(&x[cc[u]]) : (T)0;
 #pragma unroll
-    for (int u = 0; u < U; ++u) acc += vv[u] * xx[u];
+      for (int u = 0; u < U; ++u) {
+        const bool in = q + W * (U + u) < len;
+        vn[u] = in ? v[q + W * (U + u)] : (T)0;
+        cn[u] = in ? ci[q + W * (U + u)] : 0;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (q + W * u < len) acc += vv[u] * xx[u];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        vv[u] = vn[u];
+        cc[u] = cn[u];
+      }
+    }
   }
-  for (; q < e; q += W) acc += M.v[q] * __ldg(&x[M.ci[q]]);
   return acc;
 }
 
