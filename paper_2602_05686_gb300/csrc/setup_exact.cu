@@ -220,111 +220,141 @@ __device__ __forceinline__ double quad_form(int dim, const double* __restrict__ 
 // (j, i) the difference vector is exactly -(x_i - x_j), and both quadratic
 // forms are even in it with sign-symmetric rounding, so w_ji computed from row
 // j would be the same bits: computing each pair once halves the FP64 work.
-// One thread per row: the FP64 pipe issues a warp instruction whatever its
-// active lanes, so the upper entries of 32 rows share each instruction.
-template <int DIM>
-__global__ void k_material_w(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                             const double* __restrict__ x, const double* __restrict__ sinv, double* __restrict__ w) {
-  constexpr int KP = DIM == 3 ? 6 : 3;
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int64_t b = rp[i], e = rp[i + 1];
-  double xi[3], si_i[KP];
-#pragma unroll
-  for (int c = 0; c < DIM; ++c) xi[c] = x[i * DIM + c];
-#pragma unroll
-  for (int c = 0; c < KP; ++c) si_i[c] = sinv[i * KP + c];
-  for (int64_t p = b; p < e; ++p) {
-    const int32_t j = ci[p];
-    if (j < (int32_t)i) continue;  // mirrored by k_material_w_mirror
-    double wv = 0.0;
-    if (j != (int32_t)i) {
-      double d[3], sj[KP];
-#pragma unroll
-      for (int c = 0; c < DIM; ++c) d[c] = xi[c] - x[(int64_t)j * DIM + c];
-#pragma unroll
-      for (int c = 0; c < KP; ++c) sj[c] = sinv[(int64_t)j * KP + c];
-      double qij = quad_form(DIM, si_i, d);
-      double qji = quad_form(DIM, sj, d);
-      double m = qij > qji ? qij : qji;
-      wv = 1.0 / m;
-    }
-    w[p] = wv;
-  }
-}
+// Bound by FP64 issue (38 FP64 instructions a pair, 16 cycles each per SM), so
+// every lane of a warp takes a pair: the pairs of PAIR_ROWS rows are
+// numbered through (offsets in shared memory), whatever the rows' lengths -- a
+// thread per row left long coarse rows as tails, a warp per row 13 of 32
+// lanes.  Where both ends carry the same tensor, bit for bit (the inside of a
+// material region), q_ji = q_ij and its twelve instructions are left out.
+// 2.1M nodes, 64 Voronoi regions: 1733 us with a thread per row; coarse
+// levels of the stretched battery stack: 251 us on average with a warp per row
+constexpr int PAIR_ROWS = 64;
+constexpr int PAIR_THREADS = 256;
 
-// the same per pair with a warp per row (lanes stride the row): on coarse
-// levels a few rows are 10-40x longer than the rest, and a thread per row
-// leaves them a long sequential tail.  Every w_ij comes from the same
-// expression, so the values equal those of the thread-per-row form.
-template <int DIM>
-__global__ void k_material_w_warp(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                                  const double* __restrict__ x, const double* __restrict__ sinv,
-                                  double* __restrict__ w) {
-  constexpr int KP = DIM == 3 ? 6 : 3;
-  const int lane = lane_id();
-  for (int64_t i = global_warp(); i < n; i += warp_stride()) {
-    double xi[3], si_i[KP];
-#pragma unroll
-    for (int c = 0; c < DIM; ++c) xi[c] = x[i * DIM + c];
-#pragma unroll
-    for (int c = 0; c < KP; ++c) si_i[c] = sinv[i * KP + c];
-    for (int64_t p = rp[i] + lane; p < rp[i + 1]; p += 32) {
-      const int32_t j = ci[p];
-      if (j < (int32_t)i) continue;  // mirrored by k_material_w_mirror
-      double wv = 0.0;
-      if (j != (int32_t)i) {
-        double d[3], sj[KP];
-#pragma unroll
-        for (int c = 0; c < DIM; ++c) d[c] = xi[c] - x[(int64_t)j * DIM + c];
-#pragma unroll
-        for (int c = 0; c < KP; ++c) sj[c] = sinv[(int64_t)j * KP + c];
-        double qij = quad_form(DIM, si_i, d);
-        double qji = quad_form(DIM, sj, d);
-        double m = qij > qji ? qij : qji;
-        wv = 1.0 / m;
+// pair numbering of the block's rows r0 .. r0 + PAIR_ROWS - 1: the entries
+// above (UPPER) or below the diagonal of row r0 + r are start[r] + 0, 1, ...
+// and pairs off[r] .. off[r + 1] - 1
+template <bool UPPER>
+__device__ __forceinline__ void pair_offsets(int64_t n, const int64_t* __restrict__ rp,
+                                             const int32_t* __restrict__ ci, int64_t r0, int64_t* start, int* off,
+                                             double* __restrict__ w) {
+  __shared__ int wsum;
+  const int t = (int)threadIdx.x, lane = t & 31;
+  int cnt = 0;
+  if (t < PAIR_ROWS) {
+    const int64_t i = r0 + t;
+    int64_t st = 0;
+    if (i < n) {
+      const int64_t b = rp[i], e = rp[i + 1];
+      // first entry with column > i (UPPER) or >= i
+      int64_t lo = b, hi = e;
+      while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        const bool left = UPPER ? ci[mid] <= (int32_t)i : ci[mid] < (int32_t)i;
+        if (left) lo = mid + 1;
+        else hi = mid;
       }
-      w[p] = wv;
+      st = UPPER ? lo : b;
+      cnt = (int)(UPPER ? e - lo : lo - b);
+      if (UPPER && lo > b && ci[lo - 1] == (int32_t)i) w[lo - 1] = 0.0;
     }
+    start[t] = st;
+  }
+  int inc = cnt;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(FULL, inc, o);
+    if (lane >= o) inc += u;
+  }
+  if (t == 31) wsum = inc;
+  __syncthreads();
+  if (t < PAIR_ROWS) off[t + 1] = inc + (t >= 32 ? wsum : 0);
+  if (t == 0) off[0] = 0;
+  __syncthreads();
+}
+
+// the row (of the block) that pair q belongs to
+__device__ __forceinline__ int pair_row(const int* off, int q) {
+  int lo = 0, hi = PAIR_ROWS - 1;
+#pragma unroll
+  for (int s = 0; s < 6; ++s) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (off[mid] <= q) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
+template <int DIM>
+__device__ __forceinline__ double pair_weight(const double* __restrict__ x, const double* __restrict__ sinv, int64_t i,
+                                              int64_t j) {
+  constexpr int KP = DIM == 3 ? 6 : 3;
+  double d[3], si[KP], sj[KP];
+#pragma unroll
+  for (int c = 0; c < DIM; ++c) d[c] = x[i * DIM + c] - x[j * DIM + c];
+  bool same = true;
+#pragma unroll
+  for (int c = 0; c < KP; ++c) {
+    si[c] = sinv[i * KP + c];
+    sj[c] = sinv[j * KP + c];
+    same &= __double_as_longlong(si[c]) == __double_as_longlong(sj[c]);
+  }
+  const double qij = quad_form(DIM, si, d);
+  double m = qij;
+  if (!same) {
+    const double qji = quad_form(DIM, sj, d);
+    m = qij > qji ? qij : qji;
+  }
+  return 1.0 / m;
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(PAIR_THREADS) k_material_w(int64_t n, const int64_t* __restrict__ rp,
+                                                             const int32_t* __restrict__ ci,
+                                                             const double* __restrict__ x,
+                                                             const double* __restrict__ sinv, double* __restrict__ w) {
+  __shared__ int64_t start[PAIR_ROWS];
+  __shared__ int off[PAIR_ROWS + 1];
+  const int64_t r0 = (int64_t)blockIdx.x * PAIR_ROWS;
+  pair_offsets<true>(n, rp, ci, r0, start, off, w);
+  const int tot = off[PAIR_ROWS];
+  for (int q = (int)threadIdx.x; q < tot; q += PAIR_THREADS) {
+    const int r = pair_row(off, q);
+    const int64_t p = start[r] + (q - off[r]);
+    w[p] = pair_weight<DIM>(x, sinv, r0 + r, ci[p]);
   }
 }
 
-// lower entries: w_ij = w_ji, the (j, i) entry found by binary search in row
-// j; a pattern without that entry (not structurally symmetric) gets w_ij
-// computed here by the same expression
+// lower entries: w_ij = w_ji.  On a symmetric stencil entry k of row i is
+// entry len - 1 - k of row j, which is tried first, then a binary search in
+// row j; a pattern without that entry (not structurally symmetric) gets w_ij
+// computed here by the same expression.
 template <int DIM>
-__global__ void k_material_w_mirror(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                                    const double* __restrict__ x, const double* __restrict__ sinv,
-                                    double* __restrict__ w) {
-  constexpr int KP = DIM == 3 ? 6 : 3;
-  const int lane = lane_id();
-  for (int64_t i = global_warp(); i < n; i += warp_stride()) {
-    for (int64_t p = rp[i] + lane; p < rp[i + 1]; p += 32) {
-      const int32_t j = ci[p];
-      if (j >= (int32_t)i) break;  // columns ascend: the rest of the row is upper
-      int64_t lo = rp[j], hi = rp[j + 1] - 1, f = -1;
+__global__ void __launch_bounds__(PAIR_THREADS) k_material_w_mirror(int64_t n, const int64_t* __restrict__ rp,
+                                                                    const int32_t* __restrict__ ci,
+                                                                    const double* __restrict__ x,
+                                                                    const double* __restrict__ sinv, double* w) {
+  __shared__ int64_t start[PAIR_ROWS];
+  __shared__ int off[PAIR_ROWS + 1];
+  const int64_t r0 = (int64_t)blockIdx.x * PAIR_ROWS;
+  pair_offsets<false>(n, rp, ci, r0, start, off, w);
+  const int tot = off[PAIR_ROWS];
+  for (int q = (int)threadIdx.x; q < tot; q += PAIR_THREADS) {
+    const int r = pair_row(off, q);
+    const int k = q - off[r];
+    const int64_t p = start[r] + k, i = r0 + r;
+    const int32_t j = ci[p];
+    int64_t lo = rp[j], hi = rp[j + 1] - 1, f = hi - k;
+    if (f < lo || ci[f] != (int32_t)i) {
+      f = -1;
       while (lo <= hi) {
         const int64_t mid = (lo + hi) >> 1;
         const int32_t c = ci[mid];
         if (c == (int32_t)i) { f = mid; break; }
         if (c < (int32_t)i) lo = mid + 1; else hi = mid - 1;
       }
-      if (f >= 0) {
-        w[p] = w[f];
-      } else {
-        double d[3], si[KP], sj[KP];
-#pragma unroll
-        for (int c = 0; c < DIM; ++c) d[c] = x[i * DIM + c] - x[(int64_t)j * DIM + c];
-#pragma unroll
-        for (int c = 0; c < KP; ++c) {
-          si[c] = sinv[i * KP + c];
-          sj[c] = sinv[(int64_t)j * KP + c];
-        }
-        double qij = quad_form(DIM, si, d);
-        double qji = quad_form(DIM, sj, d);
-        w[p] = 1.0 / (qij > qji ? qij : qji);
-      }
     }
+    w[p] = f >= 0 ? w[f] : pair_weight<DIM>(x, sinv, i, j);
   }
 }
 
@@ -352,31 +382,100 @@ __global__ void k_row_sum_ordered(int64_t n, const int64_t* __restrict__ rp, con
   D[i] = acc;
 }
 
-// keep_ij <=> w_ij*w_ij >= (theta*theta) * (D_i*D_j)
-__global__ void k_material_keep(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                                const double* __restrict__ w, const double* __restrict__ D,
-                                const uint8_t* __restrict__ dir, double t2, uint8_t* __restrict__ keep,
-                                int64_t* __restrict__ cnt) {
+// keep_ij <=> w_ij*w_ij >= (theta*theta) * (D_i*D_j), the products rounded in
+// FP64.  Four FP64 instructions a pair bound this kernel (2.1M rows 538 us), so
+// the comparison is first made on the exponents and on the leading 20 bits of
+// the significands in FP32: 1 when w w is larger by more than their error, 0
+// when it is smaller, -1 when neither is certain (or an operand's exponent is
+// outside +-330, where an FP64 product could overflow or lose bits).
+__device__ __forceinline__ int keep_sure(double w, double t2, double Di, double Dj) {
+  const int hw = __double2hiint(w), ht = __double2hiint(t2), hi = __double2hiint(Di), hj = __double2hiint(Dj);
+  // biased exponents (a set sign bit, zero, infinity and NaN fall outside)
+  const unsigned ew = (unsigned)hw >> 20, et = (unsigned)ht >> 20, ei = (unsigned)hi >> 20, ej = (unsigned)hj >> 20;
+  const unsigned lim = 660;
+  if (ew - 693u > lim || et - 693u > lim || ei - 693u > lim || ej - 693u > lim) return -1;
+  const float mw = __int_as_float(0x3f800000 | ((hw & 0xfffff) << 3));
+  const float mt = __int_as_float(0x3f800000 | ((ht & 0xfffff) << 3));
+  const float mi = __int_as_float(0x3f800000 | ((hi & 0xfffff) << 3));
+  const float mj = __int_as_float(0x3f800000 | ((hj & 0xfffff) << 3));
+  // w w = L 2^(2 ew - 2046), t2 Di Dj = R 2^(et + ei + ej - 3069); L < 4, R < 8,
+  // each low by less than 2^-18 of itself (truncated significands, FP32 rounding)
+  const int k = (int)(et + ei + ej) - 2 * (int)ew - 1023;
+  if (k > 4) return 0;
+  if (k < -4) return 1;
+  const float L = mw * mw;
+  const float R = mt * mi * mj * __int_as_float((127 + k) << 23);
+  if (L > R * 1.00001f) return 1;
+  if (R > L * 1.00001f) return 0;
+  return -1;
+}
+
+// keep flag of entry p = (i, j), j != i
+__device__ __forceinline__ int keep_entry(double wv, double t2, double Di, double Dj, bool dirichlet) {
+  if (dirichlet) return 0;
+  const int sure = keep_sure(wv, t2, Di, Dj);
+  return sure >= 0 ? sure : ((wv * wv >= t2 * (Di * Dj)) ? 1 : 0);
+}
+
+// a warp takes KEEP_ROWS consecutive rows at a time, their loads together (one
+// row after another was a chain of dependent loads: 458 us), the entries past
+// the 32nd of a row after them
+constexpr int KEEP_ROWS = 4;
+__global__ void __launch_bounds__(256) k_material_keep(int64_t n, const int64_t* __restrict__ rp,
+                                                       const int32_t* __restrict__ ci, const double* __restrict__ w,
+                                                       const double* __restrict__ D, const uint8_t* __restrict__ dir,
+                                                       double t2, uint8_t* __restrict__ keep,
+                                                       int64_t* __restrict__ cnt) {
   const int lane = lane_id();
-  for (int64_t i = global_warp(); i < n; i += warp_stride()) {
-    const int64_t b = rp[i], e = rp[i + 1];
-    const double Di = D[i];
-    const bool diri = dir && dir[i];
-    int kept = 0;
-    for (int64_t p = b + lane; p < e; p += 32) {
-      int32_t j = ci[p];
-      uint8_t k;
-      if (j == (int32_t)i) k = 1;
-      else if (diri || (dir && dir[j])) k = 0;
-      else {
-        double wv = w[p];
-        k = (wv * wv >= t2 * (Di * D[j])) ? 1 : 0;
-      }
-      keep[p] = k;
-      kept += k;
+  for (int64_t i0 = global_warp() * KEEP_ROWS; i0 < n; i0 += warp_stride() * KEEP_ROWS) {
+    const int64_t at = i0 + (lane <= KEEP_ROWS ? lane : KEEP_ROWS);
+    const int64_t rpl = rp[at < n ? at : n];
+    int64_t b[KEEP_ROWS], e[KEEP_ROWS];
+    int32_t j[KEEP_ROWS];
+    double wv[KEEP_ROWS], Di[KEEP_ROWS], Dj[KEEP_ROWS];
+    bool dd[KEEP_ROWS];
+    int kept[KEEP_ROWS];
+#pragma unroll
+    for (int u = 0; u < KEEP_ROWS; ++u) {
+      b[u] = __shfl_sync(FULL, rpl, u);
+      e[u] = __shfl_sync(FULL, rpl, u + 1);
+      const bool in = b[u] + lane < e[u];
+      j[u] = in ? ci[b[u] + lane] : -1;
+      wv[u] = in ? w[b[u] + lane] : 0.0;
+      const int64_t i = i0 + u < n ? i0 + u : n - 1;
+      Di[u] = D[i];
+      dd[u] = dir && dir[i];
     }
-    for (int o = 16; o > 0; o >>= 1) kept += __shfl_xor_sync(FULL, kept, o);
-    if (lane == 0 && cnt) cnt[i + 1] = kept;
+#pragma unroll
+    for (int u = 0; u < KEEP_ROWS; ++u) {
+      Dj[u] = j[u] >= 0 ? D[j[u]] : 0.0;
+      if (dir && j[u] >= 0) dd[u] |= dir[j[u]] != 0;
+    }
+#pragma unroll
+    for (int u = 0; u < KEEP_ROWS; ++u) {
+      int k = 0;
+      if (j[u] >= 0) {
+        k = j[u] == (int32_t)(i0 + u) ? 1 : keep_entry(wv[u], t2, Di[u], Dj[u], dd[u]);
+        keep[b[u] + lane] = (uint8_t)k;
+      }
+      kept[u] = __popc(__ballot_sync(FULL, k != 0));
+    }
+#pragma unroll
+    for (int u = 0; u < KEEP_ROWS; ++u) {
+      if (e[u] - b[u] > 32) {  // warp-uniform
+        const int64_t i = i0 + u;
+        const bool diri = dir && dir[i];
+        int c = 0;
+        for (int64_t p = b[u] + 32 + lane; p < e[u]; p += 32) {
+          const int32_t jj = ci[p];
+          const int k = jj == (int32_t)i ? 1 : keep_entry(w[p], t2, Di[u], D[jj], diri || (dir && dir[jj]));
+          keep[p] = (uint8_t)k;
+          c += k;
+        }
+        kept[u] += __reduce_add_sync(FULL, c);
+      }
+      if (lane == 0 && cnt && i0 + u < n) cnt[i0 + u + 1] = kept[u];
+    }
   }
 }
 
@@ -684,22 +783,16 @@ int launch_strength_material(cudaStream_t s, int dim, int64_t n, const int64_t* 
                              double* w, double* D, uint8_t* keep, int64_t* cnt) {
   if (n <= 0) return SA_OK;
   const double t2 = theta * theta;
-  // a thread per row on large levels (uniform rows: 32 rows share each FP64
-  // instruction), a warp per row below 2^19 rows (coarse levels, long rows)
-  if (n >= (int64_t(1) << 19)) {
-    if (dim == 3) k_material_w<3><<<blocks_for(n, 128), 128, 0, s>>>(n, rp, ci, x, sinv, w);
-    else k_material_w<2><<<blocks_for(n, 128), 128, 0, s>>>(n, rp, ci, x, sinv, w);
-  } else {
-    if (dim == 3) k_material_w_warp<3><<<warp_rows_grid(n), 256, 0, s>>>(n, rp, ci, x, sinv, w);
-    else k_material_w_warp<2><<<warp_rows_grid(n), 256, 0, s>>>(n, rp, ci, x, sinv, w);
-  }
+  const unsigned g = blocks_for(n, PAIR_ROWS);
+  if (dim == 3) k_material_w<3><<<g, PAIR_THREADS, 0, s>>>(n, rp, ci, x, sinv, w);
+  else k_material_w<2><<<g, PAIR_THREADS, 0, s>>>(n, rp, ci, x, sinv, w);
   SA_LAUNCHED();
-  if (dim == 3) k_material_w_mirror<3><<<warp_rows_grid(n), 256, 0, s>>>(n, rp, ci, x, sinv, w);
-  else k_material_w_mirror<2><<<warp_rows_grid(n), 256, 0, s>>>(n, rp, ci, x, sinv, w);
+  if (dim == 3) k_material_w_mirror<3><<<g, PAIR_THREADS, 0, s>>>(n, rp, ci, x, sinv, w);
+  else k_material_w_mirror<2><<<g, PAIR_THREADS, 0, s>>>(n, rp, ci, x, sinv, w);
   SA_LAUNCHED();
   k_row_sum_ordered<<<blocks_for(n, 128), 128, 0, s>>>(n, rp, w, D);
   SA_LAUNCHED();
-  k_material_keep<<<warp_rows_grid(n), 256, 0, s>>>(n, rp, ci, w, D, dir, t2, keep, cnt);
+  k_material_keep<<<warp_rows_grid((n + KEEP_ROWS - 1) / KEEP_ROWS), 256, 0, s>>>(n, rp, ci, w, D, dir, t2, keep, cnt);
   SA_LAUNCHED();
   return SA_OK;
 }
