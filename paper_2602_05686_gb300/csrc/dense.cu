@@ -74,17 +74,18 @@ struct CholView {
   const uint32_t* task;
   int ntask;
   double *M, *LT, *W, *WT, *Dinv;
-  int* flag;             // 1: the tile of L is written (and, on the diagonal, its inverse)
+  int* flag;             // 1: the tile of L is written; on the diagonal: chunks of its inverse written
   int* ticket;
   int* err;              // 1: pivot not positive; 2: a wait ran out
 };
 
-// bounded wait of one thread for *p: false when it ran out or another wait did
-__device__ bool ch_poll(const int* p, int* err) {
+// bounded wait of one thread for *p >= want: false when it ran out or another
+// wait did
+__device__ bool ch_poll(const int* p, int want, int* err) {
   for (int it = 0; it < (1 << 24); ++it) {
     int v;
     asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    if (v) return true;
+    if (v >= want) return true;
     if (it > 64) {
       __nanosleep(64);
       if ((it & 1023) == 0 && (*(volatile int*)err & 2)) return false;
@@ -94,87 +95,202 @@ __device__ bool ch_poll(const int* p, int* err) {
   return false;
 }
 
-__device__ __forceinline__ void ch_publish(int* p) {
-  // the block's writes are ordered before the flag: barrier (by the caller),
+__device__ __forceinline__ void ch_publish(int* p, int v) {
+  // the writers' stores are ordered before the flag: barrier (by the caller),
   // then this thread's fence and release
   __threadfence();
-  asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(1) : "memory");
+  asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// s = sqrt(d) and r = 1 / s, both rounded to nearest, for a positive normal d,
+// in integer arithmetic: Newton's iteration for the reciprocal square root of
+// the significand in fixed point (two steps from the FP32 approximation: 2^-60),
+// then the integer square root and quotient settled by their exact remainders
+// (taken modulo 2^64, where they fit).  No FP64 instruction: a dependent one
+// takes 65 cycles here, and this pair is the chain of a Cholesky pivot (574
+// cycles, 954 as sqrt() and a divide).  Equal to sqrt() and 1.0 / s on 5e8
+// operands of every exponent on the GPU, and on 6e7 on the host with the
+// starting value off by up to four units.
+__device__ __forceinline__ void sqrt_rcp(double d, double& s, double& r) {
+  const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+  const int ex = (int)(hi >> 20);
+  if (ex == 0 || ex >= 2047) {  // zero exponent, infinity, NaN, negative
+    s = sqrt(d);
+    r = 1.0 / s;
+    return;
+  }
+  // d = m 2^p, p even, m in [2^52, 2^54); mu = m 2^-52 in [1, 4)
+  uint64_t m = (((uint64_t)hi << 32) | lo) & 0xfffffffffffffull | 0x10000000000000ull;
+  int p = ex - 1075;
+  const int odd = p & 1;
+  m <<= odd;
+  p -= odd;
+  const float f = __int_as_float(((127 + odd) << 23) | ((hi & 0xfffff) << 3) | (lo >> 29));
+  float yf;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(f));
+  const uint32_t yb = (uint32_t)__float_as_int(yf);
+  // y in [0.5, 1] as Q0.32
+  uint32_t y0 = yb >= 0x3f800000u ? 0xffffffffu : (((yb & 0x7fffff) | 0x800000) << 8);
+  if (yb < 0x3f000000u) y0 = 0x80000000u;
+  const uint64_t mf = m << 10;  // mu, Q2.62
+  uint64_t t = (uint64_t)y0 * y0;
+  const int64_t e1 = (int64_t)((1ull << 62) - __umul64hi(mf, t));        // 1 - mu y^2, Q.62
+  const uint64_t y1 = ((uint64_t)y0 << 31) + (uint64_t)(((int64_t)(uint64_t)y0 * (int32_t)(e1 >> 12)) >> 20);  // Q1.63
+  t = __umul64hi(y1, y1);
+  const int32_t e2 = (int32_t)((1ull << 60) - __umul64hi(mf, t));        // Q.60
+  const uint64_t y2 = y1 + (uint64_t)(((int64_t)(y1 >> 32) * e2) >> 29);
+  // S = sqrt(m 2^52) rounded: at most one off before the remainder says so
+  uint64_t S = __umul64hi(mf, y2) >> 9;
+  int64_t rem = (int64_t)((m << 52) - S * S);
+  if (rem < 0) {
+    S -= 1;
+    rem += (int64_t)(2 * S + 1);
+  } else if (rem > (int64_t)(2 * S)) {
+    rem -= (int64_t)(2 * S + 1);
+    S += 1;
+  }
+  S += rem > (int64_t)S;
+  const int e = (p - 52) / 2;
+  s = __longlong_as_double((long long)(((uint64_t)(e + 1074) << 52) + S));
+  // Q = 2^105 / S rounded (no ties: 2^106 has no odd factor)
+  uint64_t Q = y2 >> 10;
+  int64_t q = (int64_t)(0 - S * Q);
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+    if (q < 0) {
+      Q -= 1;
+      q += (int64_t)S;
+    }
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+    if (q >= (int64_t)S) {
+      Q += 1;
+      q -= (int64_t)S;
+    }
+  Q += 2 * q > (int64_t)S;
+  r = __longlong_as_double((long long)(((uint64_t)(969 - e) << 52) + Q));
 }
 
 // factor the tile in T (rows and columns < bs) in place and form its inverse
-// in Y (lower triangular, zero elsewhere).  What bounds it is the chain
-// sqrt -> 1/x -> scale -> update of the next pivot, about 1490 cycles per
-// column of FP64 latency (dependent DFMA 65 cycles, sqrt 640, divide 606,
-// measured), so warp 0 runs only that chain (a row per lane) while the other
-// warps apply the previous column to the columns right of the next one and
-// form the previous row of the inverse; one barrier per column.  Warp 4
-// shares warp 0's scheduler (and its FP64 issue) and stays idle.
-__device__ __forceinline__ void potrf_inv(int bs, double (*T)[NB + 1], double (*Y)[NB + 1], double* rinv, int* err) {
+// in Y (lower triangular, zero elsewhere), published to D in CH_CHUNKS chunks
+// of rows.  The chain is sqrt -> 1/x -> scale -> update of the next pivot; FP64
+// issue (64 cycles an instruction on each of the four schedulers) is the next
+// bound.  Warp 0 runs the chain alone (a row per lane); warps 1-3 apply the
+// previous column to the columns right of the next one, one barrier of these
+// four per column; warps 4-7 form the inverse's rows behind them at their own
+// pace (a column of the inverse needs no other column).
+// 32 columns with the inverse: 45 us as one block's loop over columns, 31 us
+// with the inverse inside the per-column barrier, 27 us now (22 us for the
+// columns; 14 us is the FP64 issue of both on one SM).
+constexpr int CH_CHUNKS = 4;
+__device__ __forceinline__ void potrf_inv(int bs, double (*T)[NB + 1], double (*Y)[NB + 1], double* rinv, int* ready,
+                                          double* __restrict__ D, int* dflag, int* err) {
   const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
-  double l = 0.0;  // warp 0: row `lane` of the previous column of L
-  for (int j = 0; j <= bs; ++j) {
-    if (warp == 0) {
-      if (j < bs) {
+  if (warp < 4) {
+    double l = 0.0;  // warp 0: row `lane` of the previous column of L
+    for (int j = 0; j < bs; ++j) {
+      if (warp == 0) {
         double t = T[lane][j];
         if (j > 0) {
           const double lj = __shfl_sync(FULL, l, j);
           if (lane >= j) t = fma(-l, lj, t);
         }
         double d = __shfl_sync(FULL, t, j);
-        if (!(d > 0.0)) {
+        // !(d > 0), as integers (an FP64 comparison is 65 cycles of the chain)
+        const long long db = __double_as_longlong(d);
+        if (db <= 0 || db > 0x7ff0000000000000ll) {
           if (lane == 0) atomicOr(err, 1);
           d = 1.0;
         }
-        d = sqrt(d);
-        const double ri = 1.0 / d;
-        l = lane == j ? d : (lane > j ? t * ri : 0.0);
+        double dr, ri;
+        sqrt_rcp(d, dr, ri);
+        l = lane == j ? dr : (lane > j ? t * ri : 0.0);
         if (lane >= j) T[lane][j] = l;
         if (lane == 0) rinv[j] = ri;
-      }
-    } else if (warp != 4 && j > 0) {
-      const int m = j - 1, wi = warp < 4 ? warp - 1 : warp - 2;
-      const int nd = (m >> 2) + 1;                      // groups of four columns of the inverse's row m
-      const int nu = bs - (j + 1) > 0 ? bs - (j + 1) : 0;  // columns j + 1 ... of the update
-      for (int it = wi; it < nd + nu; it += 6) {
-        if (it < nd) {
-          // row m of the inverse by forward substitution, L y = e_c: eight
-          // lanes per column split the dot product
-          const int c = it * 4 + (lane >> 3), g = lane & 7;
-          double part = 0.0;
-          if (m > c)
-            for (int q = c + g; q < m; q += 8) part = fma(T[m][q], Y[q][c], part);
-          part += __shfl_xor_sync(FULL, part, 4, 8);
-          part += __shfl_xor_sync(FULL, part, 2, 8);
-          part += __shfl_xor_sync(FULL, part, 1, 8);
-          if (g == 0 && c <= m) Y[m][c] = ((m == c ? 1.0 : 0.0) - part) * rinv[m];
-        } else {
-          const int q = j + 1 + (it - nd);
-          if (lane >= q && lane < bs) T[lane][q] = fma(-T[lane][m], T[q][m], T[lane][q]);
+      } else if (j > 0) {
+        const int m = j - 1;
+        const double lm = T[lane][m];
+        for (int q0 = j + warp; q0 < bs; q0 += 15) {
+          double a[5], b[5];
+#pragma unroll
+          for (int u = 0; u < 5; ++u) {
+            const int q = q0 + 3 * u;
+            const bool in = q < bs && lane >= q && lane < bs;
+            a[u] = in ? T[lane][q] : 0.0;
+            b[u] = in ? T[q][m] : 0.0;
+          }
+#pragma unroll
+          for (int u = 0; u < 5; ++u) {
+            const int q = q0 + 3 * u;
+            if (q < bs && lane >= q && lane < bs) T[lane][q] = fma(-lm, b[u], a[u]);
+          }
         }
       }
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      // column j is written (the barrier): tell the inverse's warps
+      if (threadIdx.x == 32) *(volatile int*)ready = j + 1;
     }
-    __syncthreads();
+  } else {
+    // eight lanes per column split each row's dot product; two columns a lane
+    const int c0 = (warp - 4) * 4 + (lane >> 3), c1 = c0 + 16, g = lane & 7;
+    for (int m = 0; m < NB; ++m) {
+      if (m < bs) {
+        // (the column warps end without waiting for these; bounded all the same)
+        int it = 0;
+        while (*(volatile int*)ready <= m && ++it < (1 << 22)) __nanosleep(20);
+        if (it >= (1 << 22)) atomicOr(err, 2);
+        asm volatile("" ::: "memory");
+        double p0 = 0.0, p1 = 0.0;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const int q0 = c0 + g + 8 * t, q1 = c1 + g + 8 * t;
+          if (q0 < m) p0 = fma(T[m][q0], Y[q0][c0], p0);
+          if (q1 < m) p1 = fma(T[m][q1], Y[q1][c1], p1);
+        }
+        // the butterfly over the eight lanes (4, 2, 1), lanes 0-3 keeping
+        // column c0 after the first exchange and lanes 4-7 column c1
+        const bool up = (lane & 4) != 0;
+        double part = (up ? p1 : p0) + __shfl_xor_sync(FULL, up ? p0 : p1, 4, 8);
+        part += __shfl_xor_sync(FULL, part, 2, 8);
+        part += __shfl_xor_sync(FULL, part, 1, 8);
+        const int c = up ? c1 : c0;
+        const double y = ((m == c ? 1.0 : 0.0) - part) * rinv[m];
+        if ((g & 3) == 0 && c <= m) Y[m][c] = y;
+        __syncwarp();
+      }
+      if ((m + 1) % (NB / CH_CHUNKS) == 0) {
+        const int r0 = m + 1 - NB / CH_CHUNKS, t = (int)threadIdx.x - 128;
+        asm volatile("bar.sync 2, 128;" ::: "memory");
+        for (int e = t; e < NB * NB / CH_CHUNKS; e += 128) D[r0 * NB + e] = Y[r0 + e / NB][e % NB];
+        asm volatile("bar.sync 2, 128;" ::: "memory");
+        if (t == 0) ch_publish(dflag, (m + 1) / (NB / CH_CHUNKS));
+      }
+    }
   }
+  __syncthreads();
 }
 
 // One launch factors the matrix and inverts its diagonal blocks.  A task is
 // one tile of L (left-looking: all its products, then its solve or its own
-// factor) or a strip of CH_STRIP columns of one W_KK; tasks are numbered so
-// that a task reads only tiles of lower-numbered tasks, CTAs draw tickets in
-// that order and wait (bounded) on the tiles' flags.  The lowest unfinished
+// factor) or a strip of CH_STRIP columns of one W_KK; the tile left of a
+// diagonal tile is part of the diagonal tile's task (the factor's chain is
+// L_jj -> L_(j+1)j -> L_(j+1)(j+1), one hop between CTAs per tile column).
+// Tasks are numbered so that a task reads only tiles of lower-numbered tasks,
+// CTAs draw tickets in that order and wait (bounded) on the tiles' flags.  The lowest unfinished
 // task never waits for one that no CTA has drawn, so the launch makes
 // progress with any number of resident CTAs.
 // Every tile sees the products of the blocked right-looking form in the same
 // order (per product a sum over the tile's 32 columns, subtracted from the
 // tile; tile columns ascending), so the factor is bitwise that form's.
-// Before: one launch per panel step and two more streams, a diagonal tile in
-// a single CTA's 45 us; 4225-row square 34.4 ms, 814 rows 3.9 ms, 3528 rows
-// 35.1 ms.
+// Bound by the chain of diagonal tiles (32 us a tile column) on narrow
+// skylines, by FP64 issue (8 us a tile product and SM) on wide ones.  4225-row
+// square 34.4 ms as launches per panel over the whole triangle, 4.6 ms now;
+// 2210-row 3D level (skyline 0.26) 10.7 ms, 2.6 ms.
 __global__ void __launch_bounds__(CH_THREADS) k_chol(CholView C) {
   __shared__ double As[2][NB][NB + 1];
   __shared__ double Bs[2][NB][NB + 1];
   __shared__ double rinv[NB];
-  __shared__ int s_task;
+  __shared__ int s_task, s_ready;
   const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t n = C.n;
   for (;;) {
@@ -200,7 +316,7 @@ __global__ void __launch_bounds__(CH_THREADS) k_chol(CholView C) {
         const int fi = C.f[i];
         double x0 = c0 + c == oi + r ? 1.0 : 0.0, x1 = c0 + c == oi + r + 16 ? 1.0 : 0.0;
         for (int m = fi > jt ? fi : jt; m < i; ++m) {
-          const bool ok = tid != 0 || ch_poll(&C.flag[C.off[i] + m - fi], C.err);
+          const bool ok = tid != 0 || ch_poll(&C.flag[C.off[i] + m - fi], 1, C.err);
           if (!__syncthreads_and(ok)) return;
           const int64_t om = (int64_t)m * NB;
           for (int t = tid; t < NB * NB; t += CH_THREADS) {
@@ -223,7 +339,7 @@ __global__ void __launch_bounds__(CH_THREADS) k_chol(CholView C) {
           x1 -= s1;
           buf ^= 1;
         }
-        const bool ok = tid != 0 || ch_poll(&C.flag[C.off[i] + i - fi], C.err);
+        const bool ok = tid != 0 || ch_poll(&C.flag[C.off[i] + i - fi], CH_CHUNKS, C.err);
         if (!__syncthreads_and(ok)) return;
         const double* D = C.Dinv + (int64_t)i * NB * NB;
         for (int t = tid; t < NB * NB; t += CH_THREADS) As[buf][t / NB][t % NB] = __ldcg(&D[t]);
@@ -249,52 +365,50 @@ __global__ void __launch_bounds__(CH_THREADS) k_chol(CholView C) {
       continue;
     }
     const int i = (int)(tw >> 15), j = (int)(tw & 0x7fff);
-    const int fi = C.f[i], fj = C.f[j];
-    const int64_t oi = (int64_t)i * NB, oj = (int64_t)j * NB;
-    const int bi = (int)(n - oi < NB ? n - oi : NB), bj = (int)(n - oj < NB ? n - oj : NB);
     const bool diag = i == j;
-    // this thread's elements of the tile: off the diagonal rows warp + 8u of
-    // column `lane`; on it the lower triangle's 528 elements in order
-    int er[4], ec[4];
-    double acc[4];
+    const int fi = C.f[i];
+    // the off-diagonal tile of this task: (i, j), or (i, i - 1) on the diagonal
+    const int jo = diag ? i - 1 : j;
+    const bool off = !diag || fi < i;
+    const int fo = off ? C.f[jo] : 0;
+    const int64_t oi = (int64_t)i * NB, oj = (int64_t)jo * NB;
+    const int bi = (int)(n - oi < NB ? n - oi : NB);  // column tiles left of the diagonal are full
+    // this thread's elements: rows warp + 8u of column `lane`; of the diagonal
+    // tile the lower triangle's 528 elements in order
+    double acc[4] = {0.0, 0.0, 0.0, 0.0}, dac[3] = {0.0, 0.0, 0.0};
+    int er[3], ec[3];
+    if (off) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      er[u] = warp + 8 * u;
-      ec[u] = lane;
-      if (diag) {
-        const int t = tid + CH_THREADS * u;
-        int a = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-        while ((a + 1) * (a + 2) / 2 <= t) ++a;
-        while (a * (a + 1) / 2 > t) --a;
-        er[u] = a;
-        ec[u] = t - a * (a + 1) / 2;
+      for (int u = 0; u < 4; ++u) {
+        const int a = warp + 8 * u;
+        acc[u] = a < bi ? __ldcg(&C.M[(oi + a) * n + oj + lane]) : 0.0;
       }
-      acc[u] = er[u] < bi && ec[u] < bj ? __ldcg(&C.M[(oi + er[u]) * n + oj + ec[u]]) : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+      const int t = tid + CH_THREADS * u;
+      int a = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+      while ((a + 1) * (a + 2) / 2 <= t) ++a;
+      while (a * (a + 1) / 2 > t) --a;
+      er[u] = a;
+      ec[u] = t - a * (a + 1) / 2;
+      if (diag && a < bi) dac[u] = __ldcg(&C.M[(oi + a) * n + oi + ec[u]]);
     }
     int buf = 0;
-    for (int k = fi > fj ? fi : fj; k < j; ++k) {
+    for (int k = diag || fi > fo ? fi : fo; k < jo; ++k) {
+      const bool prod = k >= fo;  // (diagonal tasks: the off-diagonal tile's skyline may start later)
       bool ok = true;
-      if (tid == 0) ok = ch_poll(&C.flag[C.off[i] + k - fi], C.err);
-      if (tid == 32 && !diag) ok = ch_poll(&C.flag[C.off[j] + k - fj], C.err);
+      if (tid == 0) ok = ch_poll(&C.flag[C.off[i] + k - fi], 1, C.err);
+      if (tid == 32 && prod) ok = ch_poll(&C.flag[C.off[jo] + k - fo], 1, C.err);
       if (!__syncthreads_and(ok)) return;
-      const int64_t ok_ = (int64_t)k * NB;
+      const int64_t kc = (int64_t)k * NB;
       for (int t = tid; t < NB * NB; t += CH_THREADS) {
         const int a = t / NB, b = t % NB;
-        As[buf][a][b] = a < bi ? __ldcg(&C.M[(oi + a) * n + ok_ + b]) : 0.0;
-        if (!diag) Bs[buf][a][b] = a < bj ? __ldcg(&C.M[(oj + a) * n + ok_ + b]) : 0.0;
+        As[buf][a][b] = a < bi ? __ldcg(&C.M[(oi + a) * n + kc + b]) : 0.0;
+        if (prod) Bs[buf][a][b] = __ldcg(&C.M[(oj + a) * n + kc + b]);
       }
       __syncthreads();
-      if (diag) {
-#pragma unroll
-        for (int u = 0; u < 3; ++u) {
-          if (er[u] < NB) {
-            double s = 0.0;
-#pragma unroll 8
-            for (int m = 0; m < NB; ++m) s = fma(As[buf][er[u]][m], As[buf][ec[u]][m], s);
-            acc[u] -= s;
-          }
-        }
-      } else {
+      if (prod) {
         double s[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 8
         for (int m = 0; m < NB; ++m) {
@@ -305,59 +419,81 @@ __global__ void __launch_bounds__(CH_THREADS) k_chol(CholView C) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) acc[u] -= s[u];
       }
+      if (diag) {
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+          if (er[u] < NB) {
+            double s = 0.0;
+#pragma unroll 8
+            for (int m = 0; m < NB; ++m) s = fma(As[buf][er[u]][m], As[buf][ec[u]][m], s);
+            dac[u] -= s;
+          }
+        }
+      }
       buf ^= 1;
     }
     double(*T)[NB + 1] = As[buf];
     double(*Y)[NB + 1] = Bs[buf];
+    if (off) {
+      // L_ij = X L_jj^-T, (L^-T)_qc = (L^-1)_cq, nonzero for q <= c: columns by
+      // chunks as the inverse's rows arrive, row `lane`, column c0 + warp; on
+      // the diagonal each chunk's part of the tile's last product follows
+      double(*Lb)[NB + 1] = As[buf ^ 1];
+      double s[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) T[warp + 8 * u][lane] = acc[u];
+      const double* D = C.Dinv + (int64_t)jo * NB * NB;
+      for (int ch = 0; ch < CH_CHUNKS; ++ch) {
+        const int r0 = ch * (NB / CH_CHUNKS);
+        const bool ok = tid != 0 || ch_poll(&C.flag[C.off[jo] + jo - fo], ch + 1, C.err);
+        if (!__syncthreads_and(ok)) return;
+        Y[r0 + warp][lane] = __ldcg(&D[(r0 + warp) * NB + lane]);
+        __syncthreads();
+        const int c = r0 + warp;
+        double o = 0.0;
+        for (int q = 0; q <= c; ++q) o = fma(T[lane][q], Y[c][q], o);
+        Lb[lane][c] = o;
+        if (diag) {
+          __syncthreads();
+#pragma unroll
+          for (int u = 0; u < 3; ++u)
+            if (er[u] < NB)
+#pragma unroll
+              for (int m = 0; m < NB / CH_CHUNKS; ++m) s[u] = fma(Lb[er[u]][r0 + m], Lb[ec[u]][r0 + m], s[u]);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 3; ++u) dac[u] -= s[u];
+      __syncthreads();
+      for (int t = tid; t < NB * NB; t += CH_THREADS) {
+        const int a = t / NB, b = t % NB;
+        if (a < bi) C.M[(oi + a) * n + oj + b] = Lb[a][b];
+        if (b < bi) C.LT[(oj + a) * n + oi + b] = Lb[b][a];
+      }
+    }
     if (diag) {
       for (int t = tid; t < NB * NB; t += CH_THREADS) {
         T[t / NB][t % NB] = 0.0;
         Y[t / NB][t % NB] = 0.0;
       }
-      __syncthreads();
+      if (tid == 0) s_ready = 0;
+    }
+    __syncthreads();
+    if (off && tid == 128) ch_publish(&C.flag[C.off[i] + jo - fi], 1);
+    if (diag) {
 #pragma unroll
       for (int u = 0; u < 3; ++u)
-        if (er[u] < NB) T[er[u]][ec[u]] = acc[u];
+        if (er[u] < NB) T[er[u]][ec[u]] = dac[u];
       __syncthreads();
-      potrf_inv(bi, T, Y, rinv, C.err);
-      double* D = C.Dinv + (int64_t)i * NB * NB;
+      potrf_inv(bi, T, Y, rinv, &s_ready, C.Dinv + (int64_t)i * NB * NB, &C.flag[C.off[i] + i - fi], C.err);
       for (int t = tid; t < NB * NB; t += CH_THREADS) {
         const int a = t / NB, b = t % NB;
-        D[t] = Y[a][b];
         if (a < bi && b < bi) {
           C.M[(oi + a) * n + oi + b] = b <= a ? T[a][b] : 0.0;
           C.LT[(oi + a) * n + oi + b] = a <= b ? T[b][a] : 0.0;
         }
       }
-    } else {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) T[er[u]][ec[u]] = acc[u];
-      const bool ok = tid != 0 || ch_poll(&C.flag[C.off[j] + j - fj], C.err);
-      if (!__syncthreads_and(ok)) return;
-      const double* D = C.Dinv + (int64_t)j * NB * NB;
-      for (int t = tid; t < NB * NB; t += CH_THREADS) Y[t / NB][t % NB] = __ldcg(&D[t]);
-      __syncthreads();
-      // L_ij = X L_jj^-T: row `lane`, columns warp + 8u (uniform trip counts)
-      double o[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int c = warp + 8 * u;
-        double a = 0.0;  // (L^-T)_qc = (L^-1)_cq, nonzero for q <= c
-        for (int q = 0; q <= c; ++q) a = fma(T[lane][q], Y[c][q], a);
-        o[u] = a;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int u = 0; u < 4; ++u) T[lane][warp + 8 * u] = o[u];
-      __syncthreads();
-      for (int t = tid; t < NB * NB; t += CH_THREADS) {
-        const int a = t / NB, b = t % NB;
-        if (a < bi && b < bj) C.M[(oi + a) * n + oj + b] = T[a][b];
-        if (b < bi && a < bj) C.LT[(oj + a) * n + oi + b] = T[b][a];
-      }
     }
-    __syncthreads();
-    if (tid == 0) ch_publish(&C.flag[C.off[i] + j - fi]);
   }
 }
 
@@ -409,12 +545,15 @@ int dense_start(Alloc& al, int64_t n, const int64_t* rp, const int32_t* ci, cons
       if (env[j] < env[j - 1]) env[j] = env[j - 1];
     ntile = off[nb];
   }
-  // tasks: tiles by columns; a diagonal block's inverse strips once its last
-  // column is numbered
+  // tasks: tiles by columns, a diagonal tile (with the tile left of it) where
+  // the tile left of it stands; a diagonal block's inverse strips once its
+  // last column is numbered
   tab.reserve(tab.size() + (size_t)ntile + (size_t)(n / CH_STRIP) + 1);
   for (int j = 0; j < nb; ++j) {
     const int e = tab[nb + j];
-    for (int i = j; i < e; ++i)
+    if (tab[j] == j) tab.push_back((j << 15) | j);  // no tile left of it
+    if (j + 1 < nb && tab[j + 1] <= j) tab.push_back(((j + 1) << 15) | (j + 1));
+    for (int i = j + 2; i < e; ++i)
       if (tab[i] <= j) tab.push_back((i << 15) | j);
     if ((j + 1) % CH_BT == 0 || j + 1 == nb) {
       const int q = j / CH_BT;
