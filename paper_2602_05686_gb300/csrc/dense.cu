@@ -548,13 +548,17 @@ int dense_start(Alloc& al, int64_t n, const int64_t* rp, const int32_t* ci, cons
   // tasks: tiles by columns, a diagonal tile (with the tile left of it) where
   // the tile left of it stands; a diagonal block's inverse strips once its
   // last column is numbered
+  int64_t nprod = 0;  // tile products of the factor
   tab.reserve(tab.size() + (size_t)ntile + (size_t)(n / CH_STRIP) + 1);
   for (int j = 0; j < nb; ++j) {
     const int e = tab[nb + j];
     if (tab[j] == j) tab.push_back((j << 15) | j);  // no tile left of it
     if (j + 1 < nb && tab[j + 1] <= j) tab.push_back(((j + 1) << 15) | (j + 1));
     for (int i = j + 2; i < e; ++i)
-      if (tab[i] <= j) tab.push_back((i << 15) | j);
+      if (tab[i] <= j) {
+        tab.push_back((i << 15) | j);
+        nprod += j - (tab[i] > tab[j] ? tab[i] : tab[j]);
+      }
     if ((j + 1) % CH_BT == 0 || j + 1 == nb) {
       const int q = j / CH_BT;
       const int64_t r0 = (int64_t)q * COARSE_BS, r1 = (int64_t)(j + 1) * NB < n ? (int64_t)(j + 1) * NB : n;
@@ -602,7 +606,11 @@ int dense_start(Alloc& al, int64_t n, const int64_t* rp, const int32_t* ci, cons
   C.task = reinterpret_cast<const uint32_t*>(F.sky.p + 3 * nb + 1); C.ntask = (int)nt;
   C.M = F.L.p; C.LT = F.LT.p; C.W = F.W.p; C.WT = F.WT.p; C.Dinv = job.Dinv.p;
   C.flag = job.flag.p; C.ticket = job.err.p + 1; C.err = job.err.p;
-  const int64_t g = 2 * (int64_t)num_sms();
+  // one block per SM where the chain of diagonal tiles is the time (a second
+  // block takes FP64 issue from it: 2210 rows, 41 products a tile column, 3.3
+  // against 3.8 ms), two where the products are (1039 rows, 48 a column, 3.9
+  // against 4.4 ms; 3989 rows, 410 a column, 18 against 27 ms)
+  const int64_t g = (nprod < 45 * (int64_t)nb ? 1 : 2) * (int64_t)num_sms();
   k_chol<<<(unsigned)(nt < g ? nt : g), CH_THREADS, 0, m>>>(C);
   SA_LAUNCHED();
   prof_end(m, ph);
