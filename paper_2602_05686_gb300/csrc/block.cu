@@ -122,40 +122,6 @@ __device__ __forceinline__ void ldvec(const T* __restrict__ p, T (&v)[K]) {
   }
 }
 
-// Reduction of the K per-lane partial sums over the W lanes of one row.  The
-// one-vector kernels add a row's lane sums by the butterfly xor W/2, ..., 1;
-// here every exchange also halves the columns a lane carries (a lane keeps
-// the lower or upper half and receives its partner's values of that half),
-// so each column is added in exactly the butterfly's tree -- bitwise the
-// one-vector sum -- with K/2 + K/4 + ... additions per lane instead of
-// K log2(W).  On return the lane holds the sums of columns c0 .. c0+V-1 in
-// acc[0 .. V); V = K/W when K >= W, else 1 (then lanes whose low bits
-// (lane mod W/K) are not zero hold copies).
-template <typename T, int K, int W>
-__device__ __forceinline__ int lane_reduce(T (&acc)[K], int lane, int& c0) {
-  int V = K;
-  c0 = 0;
-#pragma unroll
-  for (int o = W / 2; o > 0; o >>= 1) {
-    if (V > 1) {
-      const bool up = (lane & o) != 0;
-#pragma unroll
-      for (int j = 0; j < K / 2; ++j) {
-        if (j < V / 2) {
-          const T send = up ? acc[j] : acc[j + V / 2];
-          const T keep = up ? acc[j + V / 2] : acc[j];
-          acc[j] = keep + __shfl_xor_sync(FULL, send, o, W);
-        }
-      }
-      if (up) c0 += V / 2;
-      V /= 2;
-    } else {
-      acc[0] += __shfl_xor_sync(FULL, acc[0], o, W);
-    }
-  }
-  return V;
-}
-
 // the row product of this thread's row for K interleaved columns; returns the
 // number of columns this thread writes (0: none), their sums in acc[0 .. nw)
 // being columns c0 .. c0+nw-1 of `row`.  Entries are loaded U at a time
@@ -741,13 +707,6 @@ __global__ void k_bcoarse_in(int64_t n, int K, const T* __restrict__ b, const do
   if (e < n * K) t[e] = sq[e / K] * (double)b[e];
 }
 
-template <typename T>
-__global__ void k_bcoarse_out(int64_t n, int K, const double* __restrict__ x, const double* __restrict__ sq,
-                              T* __restrict__ xo) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < n * K) xo[e] = (T)(sq[e / K] * x[e]);
-}
-
 // launch `Kern<T, sw, K>` over the rows of M
 #define BMAT_SW(Kern, KK, M, st, ...)                                                    \
   do {                                                                                   \
@@ -848,10 +807,9 @@ static int mv_block(VHier<T>* m, cudaStream_t st, int l, int K, const double* r6
     int pi = prof_begin(st, PK_B_COARSE, l, 8.0 * n * n + 48.0 * n * K);
     k_bcoarse_in<T><<<g256(nk), 256, 0, st>>>(n, K, L->kb.p, L->sq.p, m->kct.p);
     SA_LAUNCHED();
-    SA_TRY(launch_coarse_solve_block(st, m->cf, K, m->kct.p, m->kcs.p, m->kcy.p, m->kcx.p));
-    k_bcoarse_out<T><<<g256(nk), 256, 0, st>>>(n, K, m->kcx.p, L->sq.p, L->kx.p);
+    SA_TRY(launch_coarse_solve(st, K, coarse_prob(m->cf, m->kct.p, m->kcs.p, m->kcy.p, m->kcx.p, L->sq.p, L->kx.p,
+                                                  sizeof(T) == 4)));
     prof_end(st, pi);
-    SA_LAUNCHED();
     *xo = L->kx.p;
     return SA_OK;
   }
@@ -930,7 +888,7 @@ int vh_vcycle_block(Alloc& al, VHier<T>* m, cudaStream_t st, int K, const double
   SA_TRY(block_alloc(al, m));
   if (m->lev.size() == 1) {
     const int64_t n = m->lev[0]->n;
-    SA_TRY(launch_coarse_solve_block(st, m->cf, K, R, m->kcs.p, m->kcy.p, m->kz.p));
+    SA_TRY(launch_coarse_solve(st, K, coarse_prob(m->cf, R, m->kcs.p, m->kcy.p, m->kz.p)));
     *Z = m->kz.p;
     return SA_OK;
   }

@@ -123,6 +123,40 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// Reduction of the K per-lane partial sums over the W lanes of one row.  The
+// one-vector kernels add a row's lane sums by the butterfly xor W/2, ..., 1;
+// here every exchange also halves the columns a lane carries (a lane keeps
+// the lower or upper half and receives its partner's values of that half),
+// so each column is added in exactly the butterfly's tree -- bitwise the
+// one-vector sum -- with K/2 + K/4 + ... additions per lane instead of
+// K log2(W).  On return the lane holds the sums of columns c0 .. c0+V-1 in
+// acc[0 .. V); V = K/W when K >= W, else 1 (then lanes whose low bits
+// (lane mod W/K) are not zero hold copies).
+template <typename T, int K, int W>
+__device__ __forceinline__ int lane_reduce(T (&acc)[K], int lane, int& c0) {
+  int V = K;
+  c0 = 0;
+#pragma unroll
+  for (int o = W / 2; o > 0; o >>= 1) {
+    if (V > 1) {
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int j = 0; j < K / 2; ++j) {
+        if (j < V / 2) {
+          const T send = up ? acc[j] : acc[j + V / 2];
+          const T keep = up ? acc[j + V / 2] : acc[j];
+          acc[j] = keep + __shfl_xor_sync(FULL, send, o, W);
+        }
+      }
+      if (up) c0 += V / 2;
+      V /= 2;
+    } else {
+      acc[0] += __shfl_xor_sync(FULL, acc[0], o, W);
+    }
+  }
+  return V;
+}
+
 // ---------------------------------------------------------------------------
 // primitives (prim.cu)
 // ---------------------------------------------------------------------------

@@ -572,6 +572,8 @@ int dense_start(Alloc& al, int64_t n, const int64_t* rp, const int32_t* ci, cons
   SA_TRY(job.Dinv.alloc(&al, (int64_t)nb * NB * NB));
   // (pageable source: the copy has left it when the call returns)
   SA_TRY(copy_h2d(F.sky.p, tab.data(), sizeof(int32_t) * tab.size(), s));
+  F.steps.clear();  // the solve's steps
+  coarse_steps(n, tab.data(), tab.data() + nb, F.steps);
   SA_TRY(memset_d(job.flag.p, 0, job.flag.bytes(), s));
   // L^T rows are read up to the last tile row that reaches them; tiles of
   // that range outside another row's skyline stay zero
@@ -638,164 +640,199 @@ int dense_finish(DenseJob& job) {
 // blocks K (rows [r0, r1) of COARSE_BS):
 //   forward   t_K = b_K - L_{K,<K} y_{<K};  y_K = W_KK t_K   (W_KK = L_KK^-1)
 //   backward  t_K = y_K - (L^T)_{K,>K} x_{>K};  x_K = W_KK^T t_K
-// Each step is a row-parallel product over one row range: one CTA of
-// TRI_WARPS warps per row, warp q taking the q-th of TRI_WARPS consecutive
-// column segments of the row's range (segments of a multiple of 32 columns;
-// lanes stride the segment with four loads in flight, each lane summing in
-// column order; a shuffle tree adds the lanes), the warps' sums added in warp
-// order.  MODE: 0 sum over [r0, i] (lower triangle of a diagonal block),
-// 1 over [i, r1) (upper), 2 rhs_i minus the sum over [0, r0), 3 rhs_i minus
-// the sum over [r1, n).  The K-column forms run the same sums for every
-// column as the one-column form (bitwise equal columns).
+// Each step is a row-parallel product over one row range: TRI_WARPS warps per
+// row, warp q taking the q-th of TRI_WARPS consecutive column segments of the
+// row's range (segments of a multiple of 32 columns; lanes stride the segment,
+// each lane summing in column order; a shuffle tree adds the lanes), the
+// warps' sums added in warp order.  CS_W sums over [r0, i] (lower triangle of a
+// diagonal block), CS_WT over [i, r1) (upper), CS_L rhs_i minus the sum over
+// [0, r0), CS_LT rhs_i minus the sum over [r1, n); the last two leave out the
+// columns outside the skyline (a lane starts at the first of its own columns
+// inside it, so the sums are those over the whole range) and are taken for
+// the rows whose skyline leaves the block only -- the others' t is the right-
+// hand side itself.  The K-column forms run the same sums for every column as
+// the one-column form (bitwise equal columns).
+//
+// One launch per step, for one problem or for all of a group that have it; a
+// warp takes a row with its four segment sums side by side, all its loads in
+// flight, and the exchanging butterfly over them (6 FP64 additions a row; a
+// warp per segment took 20, and FP64 issue was half of a step's time).  Bound by
+// the chain of steps, up to 4 per diagonal block: 3989 rows, 14 steps: 124 us
+// with a block per row and a warp per segment, 97 us of kernels now (8 columns
+// of 2062 rows, 10 steps: 165 -> 143 us).  (All steps in one launch, tasks on
+// tickets and step counters, took 105 to 147 us: release, acquire and the
+// uneven spread of the tasks cost more than the launches.)
 // ---------------------------------------------------------------------------
-constexpr int TRI_WARPS = 4;
+constexpr int CS_SEG = 4;       // column segments of a row
+constexpr int CS_ROWS = 4;      // rows of a block, a warp each
+constexpr int CS_THREADS = CS_ROWS * 32;
 
-// The products with L and L^T (MODE 2, 3) leave out the columns outside the
-// skyline (`sky`: the first tile column of each tile row, or the end of the
-// tile rows that reach each tile column): a lane starts at the first of its
-// own columns inside it, so the sums are those over the whole range.
-// the row i of one step (a block of TRI_WARPS warps per row)
-template <int MODE, int K>
-__device__ __forceinline__ void tri_row_at(int64_t n, int64_t r0, int64_t r1, const double* __restrict__ M,
-                                           const int32_t* __restrict__ sky, const double* __restrict__ v,
-                                           const double* __restrict__ rhs, double* __restrict__ out, int64_t i) {
-  __shared__ double sh[TRI_WARPS][K];
-  const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
-  const int64_t lo = MODE == 0 ? r0 : (MODE == 1 ? i : (MODE == 2 ? 0 : r1));
-  const int64_t hi = MODE == 0 ? i + 1 : (MODE == 1 ? r1 : (MODE == 2 ? r0 : n));
-  const int64_t seg = (((hi - lo) + TRI_WARPS - 1) / TRI_WARPS + 31) & ~(int64_t)31;
-  const int64_t b = lo + warp * seg;
-  int64_t e = b + seg < hi ? b + seg : hi;
-  const double* __restrict__ Mi = M + i * n;
-  double sum[K];
+template <int K>
+__device__ __forceinline__ void coarse_rows(const CoarseEnt& E, const CoarseProb& P, unsigned blk) {
+  constexpr int PF = K == 1 ? 8 : (K == 2 ? 4 : 2);  // entries per segment loaded together
+  const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n = (int)P.n;
+  const int i = E.rb + (int)blk * CS_ROWS + warp;
+  if (i >= E.re) return;  // warp-uniform
+  const int lo = E.mode == CS_W ? E.r0 : (E.mode == CS_WT ? i : (E.mode == CS_L ? 0 : E.r1));
+  const int hi = E.mode == CS_W ? i + 1 : (E.mode == CS_WT ? E.r1 : (E.mode == CS_L ? E.r0 : n));
+  const int seg = (((hi - lo) + CS_SEG - 1) / CS_SEG + 31) & ~31;
+  int js[CS_SEG], je[CS_SEG];
+  int top = hi, bot = 0;
+  if (E.mode == CS_L) bot = P.F.first[i / NB] * NB;
+  if (E.mode == CS_LT) top = min(hi, P.F.end[i / NB] * NB);
 #pragma unroll
-  for (int c = 0; c < K; ++c) sum[c] = 0.0;
-  int64_t j = b + lane;
-  if (MODE == 2) {
-    const int64_t f = (int64_t)sky[i / NB] * NB;
-    if (j < f) j += (f - j + 31) & ~(int64_t)31;
+  for (int q = 0; q < CS_SEG; ++q) {
+    const int b = lo + q * seg;
+    je[q] = min(b + seg, top);
+    js[q] = b + lane;
+    if (js[q] < bot) js[q] += (bot - js[q] + 31) & ~31;
   }
-  if (MODE == 3) {
-    const int64_t g = (int64_t)sky[i / NB] * NB;
-    if (e > g) e = g;
-  }
-  for (; j + 96 < e; j += 128) {
-    const double w0 = __ldcs(&Mi[j]), w1 = __ldcs(&Mi[j + 32]), w2 = __ldcs(&Mi[j + 64]), w3 = __ldcs(&Mi[j + 96]);
+  const double* M = E.mode == CS_W ? P.F.W : (E.mode == CS_WT ? P.F.WT : (E.mode == CS_L ? P.F.L : P.F.LT));
+  const double* __restrict__ Mi = M + (int64_t)i * n;
+  // columns below `split` come from va, the others from vb
+  const double* __restrict__ va = E.mode == CS_W ? P.t : (E.mode == CS_LT ? P.x : P.y);
+  const double* __restrict__ vb = E.mode == CS_W ? P.bin : P.t;
+  double sum[CS_SEG * K];
 #pragma unroll
-    for (int c = 0; c < K; ++c) {
-      sum[c] += w0 * v[j * K + c];
-      sum[c] += w1 * v[(j + 32) * K + c];
-      sum[c] += w2 * v[(j + 64) * K + c];
-      sum[c] += w3 * v[(j + 96) * K + c];
+  for (int c = 0; c < CS_SEG * K; ++c) sum[c] = 0.0;
+  {
+    double w[CS_SEG][PF];
+#pragma unroll
+    for (int q = 0; q < CS_SEG; ++q)
+#pragma unroll
+      for (int u = 0; u < PF; ++u) w[q][u] = js[q] + 32 * u < je[q] ? __ldcs(&Mi[js[q] + 32 * u]) : 0.0;
+    if constexpr (K == 1) {
+      double v[CS_SEG][PF];
+#pragma unroll
+      for (int q = 0; q < CS_SEG; ++q)
+#pragma unroll
+        for (int u = 0; u < PF; ++u) {
+          const int p = js[q] + 32 * u;
+          v[q][u] = p < je[q] ? (p < E.split ? va : vb)[p] : 0.0;
+        }
+#pragma unroll
+      for (int u = 0; u < PF; ++u)
+#pragma unroll
+        for (int q = 0; q < CS_SEG; ++q)
+          if (js[q] + 32 * u < je[q]) sum[q] = fma(w[q][u], v[q][u], sum[q]);
+    } else {
+#pragma unroll
+      for (int u = 0; u < PF; ++u)
+#pragma unroll
+        for (int q = 0; q < CS_SEG; ++q) {
+          const int p = js[q] + 32 * u;
+          if (p < je[q]) {
+            const double* v = (p < E.split ? va : vb) + (int64_t)p * K;
+#pragma unroll
+            for (int c = 0; c < K; ++c) sum[q * K + c] = fma(w[q][u], v[c], sum[q * K + c]);
+          }
+        }
     }
   }
-  for (; j < e; j += 32) {
-    const double w = Mi[j];
+  // the rest of the segments, four entries of one segment at a time
 #pragma unroll
-    for (int c = 0; c < K; ++c) sum[c] += w * v[j * K + c];
-  }
+  for (int q = 0; q < CS_SEG; ++q)
+    for (int p = js[q] + 32 * PF; p < je[q]; p += 128) {
+      double a[4];
 #pragma unroll
-  for (int c = 0; c < K; ++c) {
-    const double t = warp_sum(sum[c]);
-    if (lane == 0) sh[warp][c] = t;
-  }
-  __syncthreads();
-  if (threadIdx.x < K) {
-    const int c = (int)threadIdx.x;
-    double t = sh[0][c];
+      for (int u = 0; u < 4; ++u) a[u] = p + 32 * u < je[q] ? __ldcs(&Mi[p + 32 * u]) : 0.0;
 #pragma unroll
-    for (int q = 1; q < TRI_WARPS; ++q) t += sh[q][c];
-    out[i * K + c] = MODE >= 2 ? rhs[i * K + c] - t : t;
-  }
-}
-
-template <int MODE, int K>
-__global__ void __launch_bounds__(TRI_WARPS * 32) k_tri_row(int64_t n, int64_t r0, int64_t r1,
-                                                            const double* __restrict__ M,
-                                                            const int32_t* __restrict__ sky,
-                                                            const double* __restrict__ v,
-                                                            const double* __restrict__ rhs,
-                                                            double* __restrict__ out) {
-  tri_row_at<MODE, K>(n, r0, r1, M, sky, v, rhs, out, r0 + blockIdx.x);
-}
-
-// the same step for several problems in one launch (group solve): block
-// blockIdx.x - blk0 of a segment takes that segment's row r0 + (blockIdx.x -
-// blk0), as its own launch would
-template <int MODE>
-__global__ void __launch_bounds__(TRI_WARPS * 32) k_g_tri(const GTri* __restrict__ d, int m) {
-  __shared__ int s_seg;
-  if (threadIdx.x == 0) {
-    int lo = 0, hi = m - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (d[mid].blk0 <= blockIdx.x) lo = mid;
-      else hi = mid - 1;
+      for (int u = 0; u < 4; ++u)
+        if (p + 32 * u < je[q]) {
+          const double* v = (p + 32 * u < E.split ? va : vb) + (int64_t)(p + 32 * u) * K;
+#pragma unroll
+          for (int c = 0; c < K; ++c) sum[q * K + c] = fma(a[u], v[c], sum[q * K + c]);
+        }
     }
-    s_seg = lo;
+  // value q K + c ends in lane 8 q + (8 / K) c; the segments in order
+  int c0;
+  lane_reduce<double, CS_SEG * K, 32>(sum, lane, c0);
+  double s = sum[0];
+#pragma unroll
+  for (int q = 1; q < CS_SEG; ++q) s += __shfl_down_sync(FULL, sum[0], 8 * q);
+  if (lane < 8 && lane % (8 / K) == 0) {
+    const int64_t o = (int64_t)i * K + lane / (8 / K);
+    if (E.mode == CS_L) s = P.bin[o] - s;
+    if (E.mode == CS_LT) s = P.y[o] - s;
+    (E.mode == CS_W ? P.y : (E.mode == CS_WT ? P.x : P.t))[o] = s;
+    if (E.mode == CS_WT && P.xo) {
+      if (P.xo_f32) static_cast<float*>(P.xo)[o] = (float)(P.sq[i] * s);
+      else static_cast<double*>(P.xo)[o] = P.sq[i] * s;
+    }
   }
-  __syncthreads();
-  const GTri& D = d[s_seg];
-  tri_row_at<MODE, 1>(D.n, D.r0, D.r1, D.M, D.sky, D.v, D.rhs, D.out, D.r0 + (int64_t)(blockIdx.x - D.blk0));
 }
 
-int launch_g_tri(cudaStream_t st, int mode, const GTri* d, int m, unsigned blocks) {
-  if (m <= 0 || blocks == 0) return SA_OK;
-  const unsigned T = TRI_WARPS * 32;
-  switch (mode) {
-    case 0: k_g_tri<0><<<blocks, T, 0, st>>>(d, m); break;
-    case 1: k_g_tri<1><<<blocks, T, 0, st>>>(d, m); break;
-    case 2: k_g_tri<2><<<blocks, T, 0, st>>>(d, m); break;
-    default: k_g_tri<3><<<blocks, T, 0, st>>>(d, m); break;
+template <int K>
+__global__ void __launch_bounds__(CS_THREADS) k_coarse(CoarseEnt E, CoarseProb P) {
+  coarse_rows<K>(E, P, blockIdx.x);
+}
+
+// the same step of several problems (group solve): blocks blk0 ... of entry k
+__global__ void __launch_bounds__(CS_THREADS) k_g_coarse(const CoarseEnt* __restrict__ ent, int nent,
+                                                         const CoarseProb* __restrict__ probs) {
+  int lo = 0, hi = nent - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (ent[mid].blk0 <= (int)blockIdx.x) lo = mid;
+    else hi = mid - 1;
   }
+  const CoarseEnt E = ent[lo];
+  coarse_rows<1>(E, probs[E.prob], blockIdx.x - E.blk0);
+}
+
+// the steps of one problem's solve, in order
+void coarse_steps(int64_t n, const int32_t* first, const int32_t* end, std::vector<CoarseEnt>& out) {
+  const int nbk = (int)((n + COARSE_BS - 1) / COARSE_BS);
+  auto push = [&](int mode, int64_t rb, int64_t re, int64_t r0, int64_t r1, int64_t split) {
+    if (re <= rb) return;
+    CoarseEnt E = {};
+    E.mode = mode;
+    E.rb = (int)rb; E.re = (int)re; E.r0 = (int)r0; E.r1 = (int)r1; E.split = (int)split;
+    out.push_back(E);
+  };
+  for (int q = 0; q < nbk; ++q) {
+    const int64_t r0 = q * COARSE_BS, r1 = r0 + COARSE_BS < n ? r0 + COARSE_BS : n;
+    int64_t ek = r0;  // rows [r0, ek) reach left of the block
+    for (int64_t i = r0 / NB; i * NB < r1; ++i)
+      if ((int64_t)first[i] * NB < r0) ek = (i + 1) * NB < r1 ? (i + 1) * NB : r1;
+    push(CS_L, r0, ek, r0, r1, n);
+    push(CS_W, r0, r1, r0, r1, ek);
+  }
+  for (int q = nbk - 1; q >= 0; --q) {
+    const int64_t r0 = q * COARSE_BS, r1 = r0 + COARSE_BS < n ? r0 + COARSE_BS : n;
+    int64_t sk = r1;  // rows [sk, r1) are reached from below the block
+    if (r1 < n)
+      for (int64_t i = (r1 - 1) / NB; i * NB >= r0 && i >= 0; --i)
+        if ((int64_t)end[i] * NB > r1) sk = i * NB;
+    push(CS_LT, sk, r1, r0, r1, n);
+    push(CS_WT, r0, r1, r0, r1, sk);
+  }
+}
+
+int coarse_blocks(const CoarseEnt& E) { return (E.re - E.rb + CS_ROWS - 1) / CS_ROWS; }
+
+int launch_coarse_group(cudaStream_t st, const CoarseEnt* ent, int nent, int blocks, const CoarseProb* probs) {
+  if (blocks <= 0) return SA_OK;
+  k_g_coarse<<<(unsigned)blocks, CS_THREADS, 0, st>>>(ent, nent, probs);
   SA_LAUNCHED();
   return SA_OK;
 }
 
-int tri_threads() { return TRI_WARPS * 32; }
-
-template <int K>
-static int coarse_solve_k(cudaStream_t st, const CoarseView& F, const double* b, double* t, double* y, double* x) {
-  const int64_t n = F.n;
-  const int nbk = (int)((n + COARSE_BS - 1) / COARSE_BS);
-  const unsigned T = TRI_WARPS * 32;
-  for (int q = 0; q < nbk; ++q) {
-    const int64_t r0 = q * COARSE_BS, r1 = r0 + COARSE_BS < n ? r0 + COARSE_BS : n;
-    const unsigned g = (unsigned)(r1 - r0);
-    if (q > 0) {
-      k_tri_row<2, K><<<g, T, 0, st>>>(n, r0, r1, F.L, F.first, y, b, t);
-      SA_LAUNCHED();
+int launch_coarse_solve(cudaStream_t st, int k, const CoarseProb& P) {
+  if (P.n <= 0) return SA_OK;
+  for (const CoarseEnt& E : *P.F.steps) {
+    const unsigned g = (unsigned)coarse_blocks(E);
+    switch (k) {
+      case 1: k_coarse<1><<<g, CS_THREADS, 0, st>>>(E, P); break;
+      case 2: k_coarse<2><<<g, CS_THREADS, 0, st>>>(E, P); break;
+      case 4: k_coarse<4><<<g, CS_THREADS, 0, st>>>(E, P); break;
+      case 8: k_coarse<8><<<g, CS_THREADS, 0, st>>>(E, P); break;
+      default: return SA_ERR_INVALID_ARG;
     }
-    k_tri_row<0, K><<<g, T, 0, st>>>(n, r0, r1, F.W, nullptr, q > 0 ? t : b, nullptr, y);
-    SA_LAUNCHED();
-  }
-  for (int q = nbk - 1; q >= 0; --q) {
-    const int64_t r0 = q * COARSE_BS, r1 = r0 + COARSE_BS < n ? r0 + COARSE_BS : n;
-    const unsigned g = (unsigned)(r1 - r0);
-    if (q < nbk - 1) {
-      k_tri_row<3, K><<<g, T, 0, st>>>(n, r0, r1, F.LT, F.end, x, y, t);
-      SA_LAUNCHED();
-    }
-    k_tri_row<1, K><<<g, T, 0, st>>>(n, r0, r1, F.WT, nullptr, q < nbk - 1 ? t : y, nullptr, x);
     SA_LAUNCHED();
   }
   return SA_OK;
-}
-
-int launch_coarse_solve(cudaStream_t st, const CoarseView& F, const double* b, double* t, double* y, double* x) {
-  if (F.n <= 0) return SA_OK;
-  return coarse_solve_k<1>(st, F, b, t, y, x);
-}
-
-int launch_coarse_solve_block(cudaStream_t st, const CoarseView& F, int k, const double* b, double* t, double* y,
-                              double* x) {
-  if (F.n <= 0) return SA_OK;
-  switch (k) {
-    case 2: return coarse_solve_k<2>(st, F, b, t, y, x);
-    case 4: return coarse_solve_k<4>(st, F, b, t, y, x);
-    case 8: return coarse_solve_k<8>(st, F, b, t, y, x);
-    default: return SA_ERR_INVALID_ARG;
-  }
 }
 
 }  // namespace sa

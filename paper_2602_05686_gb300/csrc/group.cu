@@ -98,11 +98,8 @@ __global__ void __launch_bounds__(256) k_g_vec(int op, const GVec<T>* __restrict
       D.x[i] = dn;
       return;
     }
-    case GV_COARSE_IN:
+    default:  // GV_COARSE_IN
       D.t[i] = D.s[i] * (double)D.b[i];
-      return;
-    default:  // GV_COARSE_OUT
-      D.x[i] = (T)(D.s[i] * D.t[i]);
       return;
   }
 }

@@ -37,30 +37,19 @@ struct GMat {
 };
 
 // elementwise kernels of the V-cycle
-enum GVecOp { GV_FINE_IN = 0, GV_FIRST = 1, GV_COARSE_IN = 2, GV_COARSE_OUT = 3 };
+enum GVecOp { GV_FINE_IN = 0, GV_FIRST = 1, GV_COARSE_IN = 2 };
 
 template <typename T>
 struct GVec {
   uint32_t blk0;
   int64_t n;
   const double* r64;  // fine entry: FP64 residual
-  const double* s;    // fine entry: D^-1/2; coarse in/out: sqrt(diag)
+  const double* s;    // fine entry: D^-1/2; coarse in: sqrt(diag)
   T c2;
   T* b;
   T* x;
   T* d;
-  double* t;          // coarse in: t = sq * b; coarse out: x = (T)(sq * t)
-};
-
-// one row range of the coarse block substitution
-struct GTri {
-  uint32_t blk0;
-  int64_t n, r0, r1;
-  const double* M;
-  const int32_t* sky;  // modes 2 and 3: the factor's skyline (CoarseView first / end)
-  const double* v;
-  const double* rhs;
-  double* out;
+  double* t;          // coarse in: t = sq * b
 };
 
 // outer FP64 CG of one problem
@@ -115,7 +104,6 @@ template <typename T>
 int launch_g_mat(cudaStream_t st, int op, const GMat<T>* d, int m, unsigned blocks);
 template <typename T>
 int launch_g_vec(cudaStream_t st, int op, const GVec<T>* d, int m, unsigned blocks);
-int launch_g_tri(cudaStream_t st, int mode, const GTri* d, int m, unsigned blocks);
 int launch_g_cg(cudaStream_t st, int op, const GCg* d, int m, unsigned blocks);
 
 // launch geometry of one problem's matrix kernel (blocks of 256) and format code
@@ -126,7 +114,5 @@ inline int g_mat_fmt(const Mat<T>& M) {
   if (M.sw == 0) return M.sell_lanes == 2 ? -2 : 0;
   return M.sw == 1 ? 1 : CSR_LANES;
 }
-// the coarse solve's row kernels use blocks of this many threads
-int tri_threads();
 
 }  // namespace sa

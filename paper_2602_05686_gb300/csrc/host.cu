@@ -1535,7 +1535,7 @@ struct GArena {
 
 struct GLaunch {
   int kind;  // 0 matrix rows, 1 elementwise, 2 coarse substitution
-  int op;    // op or substitution mode
+  int op;    // op
   size_t off;
   int m;
   unsigned blocks;
@@ -1548,6 +1548,7 @@ struct GroupVcycle {
   std::vector<const double*> r64;  // cycle input per problem (the outer residual)
   std::vector<GLaunch> launches;
   std::vector<std::pair<int, int>> pending;  // (problem, coarsest level) waiting for the shared coarse solve
+  size_t coarse_probs = 0;                   // arena offset of its problems
 
   // level l for the problems `segs` that have it; returns per problem the
   // level's output vector
@@ -1689,81 +1690,43 @@ struct GroupVcycle {
   // of dense.cu, one launch per step for all problems that have the step)
   void flush_coarse(GArena& ar) {
     if (pending.empty()) return;
-    struct C { int i, l; bool direct; int64_t n; int nbk; const double* bin; double *t, *y, *x; CoarseView F; };
-    std::vector<C> cs;
-    int maxnbk = 0;
+    std::vector<CoarseProb> probs;
+    std::vector<const std::vector<CoarseEnt>*> steps;
+    size_t most = 0;
     {
       std::vector<GVec<T>> v;
       uint32_t blk = 0;
       for (auto& pr : pending) {
         const int i = pr.first, l = pr.second;
         VHier<T>* m = vh[i];
-        C c;
-        c.i = i; c.l = l; c.direct = (m->lev.size() == 1); c.F = m->cf; c.n = m->cf.n;
-        c.nbk = (int)((c.n + COARSE_BS - 1) / COARSE_BS);
-        c.bin = c.direct ? r64[i] : m->ct.p;
-        c.t = m->cs.p; c.y = m->cy.p; c.x = c.direct ? m->z.p : m->cx.p;
-        cs.push_back(c);
-        maxnbk = c.nbk > maxnbk ? c.nbk : maxnbk;
-        if (!c.direct) {
-          VLevel<T>* L = m->lev[l];
+        VLevel<T>* L = m->lev[l];
+        if (m->lev.size() == 1) {  // one level: the dense solve on r directly
+          probs.push_back(coarse_prob(m->cf, r64[i], m->cs.p, m->cy.p, m->z.p));
+        } else {
+          probs.push_back(coarse_prob(m->cf, m->ct.p, m->cs.p, m->cy.p, m->cx.p, L->sq.p, L->x.p, sizeof(T) == 4));
           GVec<T> g = {};
           g.blk0 = blk; g.n = L->n; g.s = L->sq.p; g.b = L->b.p; g.t = m->ct.p;
           v.push_back(g);
           blk += g256(L->n);
         }
+        steps.push_back(m->cf.steps);
+        most = std::max(most, steps.back()->size());
       }
       launches.push_back({1, GV_COARSE_IN, ar.put(v), (int)v.size(), blk});
     }
-    for (int q = 0; q < maxnbk; ++q) {   // forward: t_K = b_K - L_{K,<K} y; y_K = W_KK t_K
-      for (int mode : {2, 0}) {
-        if (mode == 2 && q == 0) continue;
-        std::vector<GTri> v;
-        uint32_t blk = 0;
-        for (auto& c : cs) {
-          if (c.nbk <= q) continue;
-          const int64_t r0 = q * COARSE_BS, r1 = r0 + COARSE_BS < c.n ? r0 + COARSE_BS : c.n;
-          GTri g = {};
-          g.blk0 = blk; g.n = c.n; g.r0 = r0; g.r1 = r1;
-          if (mode == 2) { g.M = c.F.L; g.sky = c.F.first; g.v = c.y; g.rhs = c.bin; g.out = c.t; }
-          else { g.M = c.F.W; g.v = q > 0 ? c.t : c.bin; g.rhs = nullptr; g.out = c.y; }
-          v.push_back(g);
-          blk += (uint32_t)(r1 - r0);
-        }
-        launches.push_back({2, mode, ar.put(v), (int)v.size(), blk});
-      }
-    }
-    for (int t = 0; t < maxnbk; ++t) {   // backward: t_K = y_K - L^T_{K,>K} x; x_K = W_KK^T t_K
-      for (int mode : {3, 1}) {
-        if (mode == 3 && t == 0) continue;
-        std::vector<GTri> v;
-        uint32_t blk = 0;
-        for (auto& c : cs) {
-          if (c.nbk <= t) continue;
-          const int q = c.nbk - 1 - t;
-          const int64_t r0 = q * COARSE_BS, r1 = r0 + COARSE_BS < c.n ? r0 + COARSE_BS : c.n;
-          GTri g = {};
-          g.blk0 = blk; g.n = c.n; g.r0 = r0; g.r1 = r1;
-          if (mode == 3) { g.M = c.F.LT; g.sky = c.F.end; g.v = c.x; g.rhs = c.y; g.out = c.t; }
-          else { g.M = c.F.WT; g.v = t > 0 ? c.t : c.y; g.rhs = nullptr; g.out = c.x; }
-          v.push_back(g);
-          blk += (uint32_t)(r1 - r0);
-        }
-        launches.push_back({2, mode, ar.put(v), (int)v.size(), blk});
-      }
-    }
-    {
-      std::vector<GVec<T>> v;
+    coarse_probs = ar.put(probs);
+    for (size_t s = 0; s < most; ++s) {
+      std::vector<CoarseEnt> ent;
       uint32_t blk = 0;
-      for (auto& c : cs) {
-        if (c.direct) continue;
-        VLevel<T>* L = vh[c.i]->lev[c.l];
-        GVec<T> g = {};
-        g.blk0 = blk; g.n = L->n; g.s = L->sq.p; g.x = L->x.p; g.t = vh[c.i]->cx.p;
-        v.push_back(g);
-        blk += g256(L->n);
+      for (size_t p = 0; p < probs.size(); ++p) {
+        if (s >= steps[p]->size()) continue;
+        CoarseEnt E = (*steps[p])[s];
+        E.prob = (int)p;
+        E.blk0 = (int)blk;
+        blk += (uint32_t)coarse_blocks(E);
+        ent.push_back(E);
       }
-      launches.push_back({1, GV_COARSE_OUT, ar.put(v), (int)v.size(), blk});
+      launches.push_back({2, 0, ar.put(ent), (int)ent.size(), blk});
     }
     pending.clear();
   }
@@ -1780,7 +1743,8 @@ struct GroupVcycle {
       if (g.m == 0) continue;
       if (g.kind == 0) SA_TRY(launch_g_mat<T>(st, g.op, ar.at<GMat<T>>(g.off), g.m, g.blocks));
       else if (g.kind == 1) SA_TRY(launch_g_vec<T>(st, g.op, ar.at<GVec<T>>(g.off), g.m, g.blocks));
-      else SA_TRY(launch_g_tri(st, g.op, ar.at<GTri>(g.off), g.m, g.blocks));
+      else SA_TRY(launch_coarse_group(st, ar.at<CoarseEnt>(g.off), g.m, (int)g.blocks,
+                                      ar.at<CoarseProb>(coarse_probs)));
     }
     return SA_OK;
   }

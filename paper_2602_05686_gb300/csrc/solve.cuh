@@ -1,6 +1,8 @@
 // Solve-phase launchers and the device-resident CG scalars.
 #pragma once
 
+#include <vector>
+
 #include "common.cuh"
 
 namespace sa {
@@ -53,12 +55,24 @@ constexpr int64_t COARSE_BS = 1024;
 
 // Only the skyline of L is stored (tiles of 32 x 32 from each tile row's
 // first nonzero tile column on), the rest of L is unset.
+
+// one step of a coarse solve: rows [rb, re) of the diagonal block [r0, r1)
+enum CoarseMode { CS_W = 0, CS_WT = 1, CS_L = 2, CS_LT = 3 };
+struct CoarseEnt {
+  int blk0;      // first block in a launch of several problems
+  int prob;      // and its problem
+  int mode;
+  int rb, re, r0, r1;
+  int split;     // columns below it come from the first operand (dense.cu)
+};
+
 struct CoarseFactor {
   Buf<double> L, LT, W, WT;
   // per tile row of 32: the first tile column of its skyline; then per tile
   // column the end of the tile rows that reach it; then the factorisation's
   // own tables
   Buf<int32_t> sky;
+  std::vector<CoarseEnt> steps;  // of the solve
 };
 
 struct CoarseView {
@@ -69,13 +83,33 @@ struct CoarseView {
   const double* WT = nullptr;
   const int32_t* first = nullptr;  // skyline: first tile column per tile row
   const int32_t* end = nullptr;    // ... and end of the tile rows per tile column
+  const std::vector<CoarseEnt>* steps = nullptr;  // host (the factor's)
 };
 
 inline CoarseView coarse_view(const CoarseFactor& F, int64_t n) {
   CoarseView v;
   v.n = n; v.L = F.L.p; v.LT = F.LT.p; v.W = F.W.p; v.WT = F.WT.p;
   v.first = F.sky.p; v.end = F.sky.p + (n + 31) / 32;
+  v.steps = &F.steps;
   return v;
+}
+
+// one coarse solve: x = A_c^-1 bin; t and y: n-vector workspaces (no two of
+// bin, t, y, x alias); xo (may be NULL) also receives sq_i x_i in FP32 or FP64
+struct CoarseProb {
+  int64_t n = 0;
+  CoarseView F;
+  const double* bin = nullptr;
+  double *t = nullptr, *y = nullptr, *x = nullptr;
+  void* xo = nullptr;
+  const double* sq = nullptr;
+  int xo_f32 = 0;
+};
+inline CoarseProb coarse_prob(const CoarseView& F, const double* b, double* t, double* y, double* x,
+                              const double* sq = nullptr, void* xo = nullptr, int xo_f32 = 0) {
+  CoarseProb p;
+  p.n = F.n; p.F = F; p.bin = b; p.t = t; p.y = y; p.x = x; p.sq = sq; p.xo = xo; p.xo_f32 = xo_f32;
+  return p;
 }
 
 // dense_start enqueues the whole factorisation on a stream of its own, forked
@@ -99,10 +133,12 @@ struct DenseJob {
 int dense_start(Alloc& al, int64_t n, const int64_t* rp, const int32_t* ci, const double* v, CoarseFactor& F,
                 DenseJob& job);
 int dense_finish(DenseJob& job);
-// x = A_c^-1 b = L^-T (L^-1 b); t and y: n-vector workspaces (t may not
-// alias b, y or x).  The block form takes k in {2, 4, 8} interleaved columns.
-int launch_coarse_solve(cudaStream_t st, const CoarseView& F, const double* b, double* t, double* y, double* x);
-int launch_coarse_solve_block(cudaStream_t st, const CoarseView& F, int k, const double* b, double* t, double* y,
-                              double* x);
+// one solve with k in {1, 2, 4, 8} interleaved columns
+int launch_coarse_solve(cudaStream_t st, int k, const CoarseProb& P);
+// the steps of one solve (first, end: the skyline on the host); one step of
+// several problems in one launch (entries in the order of their blocks)
+void coarse_steps(int64_t n, const int32_t* first, const int32_t* end, std::vector<CoarseEnt>& out);
+int coarse_blocks(const CoarseEnt& E);
+int launch_coarse_group(cudaStream_t st, const CoarseEnt* ent, int nent, int blocks, const CoarseProb* probs);
 
 }  // namespace sa

@@ -498,13 +498,6 @@ __global__ void k_coarse_in(int64_t n, const T* __restrict__ b, const double* __
   if (i < n) t[i] = sq[i] * (double)b[i];
 }
 
-template <typename T>
-__global__ void k_coarse_out(int64_t n, const double* __restrict__ x, const double* __restrict__ sq,
-                             T* __restrict__ xo) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) xo[i] = (T)(sq[i] * x[i]);
-}
-
 // ---------------------------------------------------------------------------
 // the cycle
 // ---------------------------------------------------------------------------
@@ -531,10 +524,9 @@ static int mv(VHier<T>* m, cudaStream_t st, int l, const double* r64, T** xo) {
     int pi = prof_begin(st, PK_COARSE, l, 8.0 * n * n + 48.0 * n);
     k_coarse_in<T><<<g256(n), 256, 0, st>>>(n, L->b.p, L->sq.p, m->ct.p);
     SA_LAUNCHED();
-    SA_TRY(launch_coarse_solve(st, m->cf, m->ct.p, m->cs.p, m->cy.p, m->cx.p));
-    k_coarse_out<T><<<g256(n), 256, 0, st>>>(n, m->cx.p, L->sq.p, L->x.p);
+    SA_TRY(launch_coarse_solve(st, 1, coarse_prob(m->cf, m->ct.p, m->cs.p, m->cy.p, m->cx.p, L->sq.p, L->x.p,
+                                                  sizeof(T) == 4)));
     prof_end(st, pi);
-    SA_LAUNCHED();
     *xo = L->x.p;
     return SA_OK;
   }
@@ -596,7 +588,7 @@ int vh_vcycle(VHier<T>* m, cudaStream_t st, const double* r, double** z) {
     // one level: the dense solve on r directly
     const int64_t n = m->lev[0]->n;
     int pi = prof_begin(st, PK_COARSE, 0, 8.0 * n * n + 32.0 * n);
-    int s = launch_coarse_solve(st, m->cf, r, m->cs.p, m->cy.p, m->z.p);
+    int s = launch_coarse_solve(st, 1, coarse_prob(m->cf, r, m->cs.p, m->cy.p, m->z.p));
     prof_end(st, pi);
     SA_TRY(s);
     *z = m->z.p;
