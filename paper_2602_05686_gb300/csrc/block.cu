@@ -537,6 +537,7 @@ template <typename T, int SW, int K>
 // d_in may also be x_in's buffer (after the first step, where x_1 = d_1)
 __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_cheb(MatView<T> A, const T* __restrict__ b, const T* __restrict__ xin, T* __restrict__ xout,
                            const T* din, T* dout, T c1, T c2, int first) {
+  pdl_sync();
   T y[K];
   int64_t i;
   int c0;
@@ -576,6 +577,7 @@ __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_cheb(MatView<T> A, 
 
 template <typename T, int SW, int K>
 __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_residual(MatView<T> A, const T* __restrict__ b, const T* __restrict__ x, T* __restrict__ r) {
+  pdl_sync();
   T y[K];
   int64_t i;
   int c0;
@@ -599,6 +601,7 @@ __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_residual(MatView<T>
 
 template <typename T, int SW, int K>
 __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_spmv(MatView<T> A, const T* __restrict__ x, T* __restrict__ out) {
+  pdl_sync();
   T y[K];
   int64_t i;
   int c0;
@@ -621,6 +624,7 @@ __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_spmv(MatView<T> A, 
 
 template <typename T, int SW, int K>
 __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_spmv_add(MatView<T> A, const T* __restrict__ x, T* __restrict__ out) {
+  pdl_sync();
   T y[K];
   int64_t i;
   int c0;
@@ -646,6 +650,7 @@ template <typename T, int SW, int K>
 __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_cheb_out(MatView<T> A, const T* __restrict__ b, const T* __restrict__ xin,
                                const T* __restrict__ d, T c1, T c2, int first, const double* __restrict__ s,
                                double* __restrict__ z) {
+  pdl_sync();
   T y[K];
   int64_t i;
   int c0;
@@ -686,6 +691,7 @@ __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_cheb_out(MatView<T>
 template <typename T>
 __global__ void k_bvc_fine_in(int64_t n, int K, const double* __restrict__ r, const double* __restrict__ s, T c2,
                               T* __restrict__ b, T* __restrict__ d) {
+  pdl_sync();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e < n * K) {
     const T bi = (T)(s[e / K] * r[e]);
@@ -696,6 +702,7 @@ __global__ void k_bvc_fine_in(int64_t n, int K, const double* __restrict__ r, co
 
 template <typename T>
 __global__ void k_bvc_first(int64_t nk, const T* __restrict__ b, T c2, T* __restrict__ d) {
+  pdl_sync();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e < nk) d[e] = c2 * b[e];
 }
@@ -703,6 +710,7 @@ __global__ void k_bvc_first(int64_t nk, const T* __restrict__ b, T c2, T* __rest
 template <typename T>
 __global__ void k_bcoarse_in(int64_t n, int K, const T* __restrict__ b, const double* __restrict__ sq,
                              double* __restrict__ t) {
+  pdl_sync();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e < n * K) t[e] = sq[e / K] * (double)b[e];
 }
@@ -713,11 +721,11 @@ __global__ void k_bcoarse_in(int64_t n, int K, const T* __restrict__ b, const do
     const MatView<T> _mv = view(M);                                                      \
     const unsigned _g = bmat_grid(M, KK);                                                \
     if (staged_form(M))                                                                  \
-      Kern<T, staged_code<T>(), KK><<<stage_grid(M), STAGE_WPB * 32, stage_smem_bytes(), st>>>(_mv, __VA_ARGS__); \
-    else if ((M).sw == 0 && (M).sell_lanes == 2) Kern<T, -2, KK><<<_g, 256, 0, st>>>(_mv, __VA_ARGS__); \
-    else if ((M).sw == 0) Kern<T, 0, KK><<<_g, 256, 0, st>>>(_mv, __VA_ARGS__);          \
-    else if ((M).sw == 1) Kern<T, 1, KK><<<_g, 256, 0, st>>>(_mv, __VA_ARGS__);          \
-    else Kern<T, CSR_LANES, KK><<<_g, 256, 0, st>>>(_mv, __VA_ARGS__);                   \
+      launch_pdl(Kern<T, staged_code<T>(), KK>, stage_grid(M), STAGE_WPB * 32, stage_smem_bytes(), st, _mv, __VA_ARGS__); \
+    else if ((M).sw == 0 && (M).sell_lanes == 2) launch_pdl(Kern<T, -2, KK>, _g, 256, 0, st, _mv, __VA_ARGS__); \
+    else if ((M).sw == 0) launch_pdl(Kern<T, 0, KK>, _g, 256, 0, st, _mv, __VA_ARGS__);          \
+    else if ((M).sw == 1) launch_pdl(Kern<T, 1, KK>, _g, 256, 0, st, _mv, __VA_ARGS__);          \
+    else launch_pdl(Kern<T, CSR_LANES, KK>, _g, 256, 0, st, _mv, __VA_ARGS__);                   \
   } while (0)
 
 #define LAUNCH_BMAT(Kern, M, st, K, ...)                                                 \
@@ -805,7 +813,7 @@ static int mv_block(VHier<T>* m, cudaStream_t st, int l, int K, const double* r6
   const int64_t n = L->n, nk = n * K;
   if (l == nl - 1) {
     int pi = prof_begin(st, PK_B_COARSE, l, 8.0 * n * n + 48.0 * n * K);
-    k_bcoarse_in<T><<<g256(nk), 256, 0, st>>>(n, K, L->kb.p, L->sq.p, m->kct.p);
+    launch_pdl(k_bcoarse_in<T>, g256(nk), 256, 0, st, n, K, L->kb.p, L->sq.p, m->kct.p);
     SA_LAUNCHED();
     SA_TRY(launch_coarse_solve(st, K, coarse_prob(m->cf, m->kct.p, m->kcs.p, m->kcy.p, m->kcx.p, L->sq.p, L->kx.p,
                                                   sizeof(T) == 4)));
@@ -821,9 +829,9 @@ static int mv_block(VHier<T>* m, cudaStream_t st, int l, int K, const double* r6
   // from there and writes d into kx2 and x into kx (then in place / ping-pong)
   if (l == 0) {
     BPROF(K_FST, l, 8.0 * K * n + 8.0 * n + 2.0 * S * K * n,
-          (k_bvc_fine_in<T><<<g256(nk), 256, 0, st>>>(n, K, r64, m->s0.p, (T)(1.0 / th), L->kb.p, L->kd.p)));
+          (launch_pdl(k_bvc_fine_in<T>, g256(nk), 256, 0, st, n, K, r64, m->s0.p, (T)(1.0 / th), L->kb.p, L->kd.p)));
   } else {
-    BPROF(K_FST, l, 2.0 * S * K * n, (k_bvc_first<T><<<g256(nk), 256, 0, st>>>(nk, L->kb.p, (T)(1.0 / th), L->kd.p)));
+    BPROF(K_FST, l, 2.0 * S * K * n, (launch_pdl(k_bvc_first<T>, g256(nk), 256, 0, st, nk, L->kb.p, (T)(1.0 / th), L->kd.p)));
   }
   SA_LAUNCHED();
   T* x = L->kd.p;  // the iterate
@@ -908,6 +916,7 @@ template int vh_vcycle_block<float>(Alloc&, VHier<float>*, cudaStream_t, int, co
 template <int K>
 __global__ void k_bsell_spmv_dot(MatView<double> A, const double* __restrict__ P, double* __restrict__ Q,
                                  double* __restrict__ part) {
+  pdl_sync();
   double y[K], c[K];
   int64_t i;
   int c0;
@@ -948,6 +957,7 @@ __global__ void k_bsell_spmv_dot(MatView<double> A, const double* __restrict__ P
 template <int K>
 __global__ void k_bsell_res64(MatView<double> A, const double* __restrict__ B, const double* __restrict__ X,
                               double* __restrict__ R) {
+  pdl_sync();
   double y[K];
   int64_t i;
   int c0;
@@ -984,9 +994,9 @@ int launch_bsell_spmv_dot(cudaStream_t st, const Sell<double>& A, int K, const d
                        16.0 * K * A.n;
   if (K != 2 && K != 4 && K != 8) return SA_ERR_INVALID_ARG;
   const int pi = prof_begin(st, PK_B_CG_SPMV, 0, bytes);
-  if (K == 2) k_bsell_spmv_dot<2><<<g256(A.n), 256, 0, st>>>(mv, P, Q, part);
-  else if (K == 4) k_bsell_spmv_dot<4><<<g256(A.n), 256, 0, st>>>(mv, P, Q, part);
-  else k_bsell_spmv_dot<8><<<g256(A.n), 256, 0, st>>>(mv, P, Q, part);
+  if (K == 2) launch_pdl(k_bsell_spmv_dot<2>, g256(A.n), 256, 0, st, mv, P, Q, part);
+  else if (K == 4) launch_pdl(k_bsell_spmv_dot<4>, g256(A.n), 256, 0, st, mv, P, Q, part);
+  else launch_pdl(k_bsell_spmv_dot<8>, g256(A.n), 256, 0, st, mv, P, Q, part);
   prof_end(st, pi);
   SA_LAUNCHED();
   return launch_fin_wide(st, part, (int)g256(A.n), fin);
@@ -995,9 +1005,9 @@ int launch_bsell_spmv_dot(cudaStream_t st, const Sell<double>& A, int K, const d
 int launch_bsell_residual64(cudaStream_t st, const Sell<double>& A, int K, const double* B, const double* X,
                             double* R) {
   const MatView<double> mv = sell_view(A);
-  if (K == 2) k_bsell_res64<2><<<g256(A.n), 256, 0, st>>>(mv, B, X, R);
-  else if (K == 4) k_bsell_res64<4><<<g256(A.n), 256, 0, st>>>(mv, B, X, R);
-  else if (K == 8) k_bsell_res64<8><<<g256(A.n), 256, 0, st>>>(mv, B, X, R);
+  if (K == 2) launch_pdl(k_bsell_res64<2>, g256(A.n), 256, 0, st, mv, B, X, R);
+  else if (K == 4) launch_pdl(k_bsell_res64<4>, g256(A.n), 256, 0, st, mv, B, X, R);
+  else if (K == 8) launch_pdl(k_bsell_res64<8>, g256(A.n), 256, 0, st, mv, B, X, R);
   else return SA_ERR_INVALID_ARG;
   SA_LAUNCHED();
   return SA_OK;

@@ -106,6 +106,31 @@ inline unsigned warp_rows_grid(int64_t rows, int block = 256) {
   return blocks_for(warps * 32, block);
 }
 
+// Programmatic dependent launch: a kernel launched by launch_pdl may start while
+// its predecessor in the stream drains, and waits in pdl_sync() for that
+// predecessor's completion before it touches anything the stream writes (it
+// may read matrices built before the solve earlier).  The trigger follows the
+// wait, so no kernel starts before the one before its predecessor has ended.
+// Every kernel launched this way calls pdl_sync() first.  The launches of one
+// V-cycle on small levels are 2 to 4 us of work with 1.3 us between them.
+template <typename... P, typename... A>
+inline void launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(block);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+__device__ __forceinline__ void pdl_sync() {
+  asm volatile("griddepcontrol.wait;\ngriddepcontrol.launch_dependents;" ::: "memory");
+}
+
 constexpr unsigned FULL = 0xffffffffu;
 
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }

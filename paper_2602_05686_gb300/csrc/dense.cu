@@ -673,7 +673,10 @@ __device__ __forceinline__ void coarse_rows(const CoarseEnt& E, const CoarseProb
   const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = (int)P.n;
   const int i = E.rb + (int)blk * CS_ROWS + warp;
-  if (i >= E.re) return;  // warp-uniform
+  if (i >= E.re) {  // warp-uniform
+    pdl_sync();
+    return;
+  }
   const int lo = E.mode == CS_W ? E.r0 : (E.mode == CS_WT ? i : (E.mode == CS_L ? 0 : E.r1));
   const int hi = E.mode == CS_W ? i + 1 : (E.mode == CS_WT ? E.r1 : (E.mode == CS_L ? E.r0 : n));
   const int seg = (((hi - lo) + CS_SEG - 1) / CS_SEG + 31) & ~31;
@@ -702,6 +705,7 @@ __device__ __forceinline__ void coarse_rows(const CoarseEnt& E, const CoarseProb
     for (int q = 0; q < CS_SEG; ++q)
 #pragma unroll
       for (int u = 0; u < PF; ++u) w[q][u] = js[q] + 32 * u < je[q] ? __ldcs(&Mi[js[q] + 32 * u]) : 0.0;
+    pdl_sync();  // the matrix is not written by this stream's solves
     if constexpr (K == 1) {
       double v[CS_SEG][PF];
 #pragma unroll
@@ -814,7 +818,7 @@ int coarse_blocks(const CoarseEnt& E) { return (E.re - E.rb + CS_ROWS - 1) / CS_
 
 int launch_coarse_group(cudaStream_t st, const CoarseEnt* ent, int nent, int blocks, const CoarseProb* probs) {
   if (blocks <= 0) return SA_OK;
-  k_g_coarse<<<(unsigned)blocks, CS_THREADS, 0, st>>>(ent, nent, probs);
+  launch_pdl(k_g_coarse, (unsigned)blocks, CS_THREADS, 0, st, ent, nent, probs);
   SA_LAUNCHED();
   return SA_OK;
 }
@@ -824,10 +828,10 @@ int launch_coarse_solve(cudaStream_t st, int k, const CoarseProb& P) {
   for (const CoarseEnt& E : *P.F.steps) {
     const unsigned g = (unsigned)coarse_blocks(E);
     switch (k) {
-      case 1: k_coarse<1><<<g, CS_THREADS, 0, st>>>(E, P); break;
-      case 2: k_coarse<2><<<g, CS_THREADS, 0, st>>>(E, P); break;
-      case 4: k_coarse<4><<<g, CS_THREADS, 0, st>>>(E, P); break;
-      case 8: k_coarse<8><<<g, CS_THREADS, 0, st>>>(E, P); break;
+      case 1: launch_pdl(k_coarse<1>, g, CS_THREADS, 0, st, E, P); break;
+      case 2: launch_pdl(k_coarse<2>, g, CS_THREADS, 0, st, E, P); break;
+      case 4: launch_pdl(k_coarse<4>, g, CS_THREADS, 0, st, E, P); break;
+      case 8: launch_pdl(k_coarse<8>, g, CS_THREADS, 0, st, E, P); break;
       default: return SA_ERR_INVALID_ARG;
     }
     SA_LAUNCHED();

@@ -62,6 +62,7 @@ __device__ __forceinline__ void g_mat_row(int op, const GMat<T>& D, unsigned blk
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_g_mat(int op, const GMat<T>* __restrict__ d, int m) {
+  pdl_sync();
   const int k = seg_of(d, m);
   const GMat<T> D = d[k];
   const unsigned blk = blockIdx.x - D.blk0;
@@ -79,6 +80,7 @@ __global__ void __launch_bounds__(256) k_g_mat(int op, const GMat<T>* __restrict
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256) k_g_vec(int op, const GVec<T>* __restrict__ d, int m) {
+  pdl_sync();
   const int k = seg_of(d, m);
   const GVec<T>& D = d[k];
   const int64_t i = (int64_t)(blockIdx.x - D.blk0) * blockDim.x + threadIdx.x;
@@ -107,7 +109,7 @@ __global__ void __launch_bounds__(256) k_g_vec(int op, const GVec<T>* __restrict
 template <typename T>
 int launch_g_mat(cudaStream_t st, int op, const GMat<T>* d, int m, unsigned blocks) {
   if (m <= 0 || blocks == 0) return SA_OK;
-  k_g_mat<T><<<blocks, 256, 0, st>>>(op, d, m);
+  launch_pdl(k_g_mat<T>, blocks, 256, 0, st, op, d, m);
   SA_LAUNCHED();
   return SA_OK;
 }
@@ -115,7 +117,7 @@ int launch_g_mat(cudaStream_t st, int op, const GMat<T>* d, int m, unsigned bloc
 template <typename T>
 int launch_g_vec(cudaStream_t st, int op, const GVec<T>* d, int m, unsigned blocks) {
   if (m <= 0 || blocks == 0) return SA_OK;
-  k_g_vec<T><<<blocks, 256, 0, st>>>(op, d, m);
+  launch_pdl(k_g_vec<T>, blocks, 256, 0, st, op, d, m);
   SA_LAUNCHED();
   return SA_OK;
 }
@@ -174,6 +176,7 @@ __device__ __forceinline__ void g_tail(const GCg& D) {
 
 // rows geometry (blocks of 256): residual, operator product with p.q
 __global__ void __launch_bounds__(256) k_g_cg_rows(int op, const GCg* __restrict__ d, int m) {
+  pdl_sync();
   const int k = seg_of(d, m);
   const GCg& D = d[k];
   const unsigned blk = blockIdx.x - D.blk0;
@@ -206,6 +209,7 @@ __global__ void __launch_bounds__(256) k_g_cg_rows(int op, const GCg* __restrict
 // elements; sixteen small problems in full grids spent 25 us a launch on
 // block sums of zeros)
 __global__ void __launch_bounds__(RED_THREADS) k_g_cg_red(int op, const GCg* __restrict__ d, int m) {
+  pdl_sync();
   const int k = seg_of(d, m);
   const GCg& D = d[k];
   const unsigned blk = blockIdx.x - D.blk0;
@@ -241,8 +245,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_g_cg_red(int op, const GCg* __r
 
 int launch_g_cg(cudaStream_t st, int op, const GCg* d, int m, unsigned blocks) {
   if (m <= 0 || blocks == 0) return SA_OK;
-  if (op == GC_RESID || op == GC_SPMV_DOT) k_g_cg_rows<<<blocks, 256, 0, st>>>(op, d, m);
-  else k_g_cg_red<<<blocks, RED_THREADS, 0, st>>>(op, d, m);
+  if (op == GC_RESID || op == GC_SPMV_DOT) launch_pdl(k_g_cg_rows, blocks, 256, 0, st, op, d, m);
+  else launch_pdl(k_g_cg_red, blocks, RED_THREADS, 0, st, op, d, m);
   SA_LAUNCHED();
   return SA_OK;
 }

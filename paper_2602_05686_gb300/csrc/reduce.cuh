@@ -177,6 +177,7 @@ __device__ __forceinline__ void fin_inline(const Fin& f, const double* part, int
 template <int NV>
 __global__ void __launch_bounds__(32 * NV) k_fin_wide(const double* __restrict__ part, int np, int64_t stride,
                                                       Fin f) {
+  pdl_sync();
   __shared__ double res[NV];
   const int lane = (int)(threadIdx.x & 31), v = (int)(threadIdx.x >> 5);
   const int q = (int)blockIdx.x;

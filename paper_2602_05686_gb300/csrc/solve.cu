@@ -27,6 +27,7 @@ namespace sa {
 // step so that the product below costs one FP64 FMA per stored entry
 __global__ void k_power_prep(int64_t n, const double* __restrict__ X, const double* __restrict__ s,
                              const double* __restrict__ sc, double* __restrict__ y) {
+  pdl_sync();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) y[i] = s ? s[i] * (X[i] * sc[4]) : X[i] * sc[4];  // s NULL: a pre-scaled operator
 }
@@ -36,6 +37,7 @@ template <int SW>
 __global__ void k_power_spmv(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
                              const double* __restrict__ v, const double* __restrict__ s, const double* __restrict__ y,
                              double* __restrict__ w) {
+  pdl_sync();
   ROW_SETUP(SW)
   double acc = 0.0;
   if (valid) {
@@ -76,6 +78,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_dots(int64_t n, const double* _
                                                       const double* __restrict__ b0, const double* __restrict__ a1,
                                                       const double* __restrict__ b1, double* __restrict__ part,
                                                       Fin fin) {
+  pdl_sync();
   double acc[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) acc[v] = 0.0;
@@ -125,6 +128,7 @@ __global__ void k_start_vector(int64_t n, uint32_t tag, uint32_t seed, double* _
 __global__ void __launch_bounds__(RED_THREADS) k_power_dots(int64_t n, const double* __restrict__ w,
                                                             const double* __restrict__ X, const double* sc,
                                                             double* __restrict__ part, Fin fin) {
+  pdl_sync();
   const double inv = sc[4];
   double acc[2] = {0.0, 0.0};
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -163,18 +167,18 @@ int pick_sw(int64_t n, int64_t nnz) {
     const int _sw = (sw);                                                                    \
     const unsigned _g = blocks_for((GRIDN) * (int64_t)_sw, 256);                             \
     switch (_sw) {                                                                           \
-      case 4: KERNEL<4><<<_g, 256, 0, st>>>(__VA_ARGS__); break;                             \
-      case 8: KERNEL<8><<<_g, 256, 0, st>>>(__VA_ARGS__); break;                             \
-      case 16: KERNEL<16><<<_g, 256, 0, st>>>(__VA_ARGS__); break;                           \
-      default: KERNEL<32><<<_g, 256, 0, st>>>(__VA_ARGS__); break;                           \
+      case 4: launch_pdl(KERNEL<4>, _g, 256, 0, st, __VA_ARGS__); break;                             \
+      case 8: launch_pdl(KERNEL<8>, _g, 256, 0, st, __VA_ARGS__); break;                             \
+      case 16: launch_pdl(KERNEL<16>, _g, 256, 0, st, __VA_ARGS__); break;                           \
+      default: launch_pdl(KERNEL<32>, _g, 256, 0, st, __VA_ARGS__); break;                           \
     }                                                                                        \
   } while (0)
 
 int launch_dots(cudaStream_t st, int64_t n, const double* a0, const double* b0, const double* a1,
                 const double* b1, double* part, const Fin& fin) {
   const unsigned g = red_blocks(n);
-  if (a1) k_dots<2><<<g, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part, fin);
-  else k_dots<1><<<g, RED_THREADS, 0, st>>>(n, a0, b0, nullptr, nullptr, part, fin);
+  if (a1) launch_pdl(k_dots<2>, g, RED_THREADS, 0, st, n, a0, b0, a1, b1, part, fin);
+  else launch_pdl(k_dots<1>, g, RED_THREADS, 0, st, n, a0, b0, nullptr, nullptr, part, fin);
   SA_LAUNCHED();
   return SA_OK;
 }
@@ -205,11 +209,11 @@ int run_power(Alloc& al, int64_t n, const int64_t* rp, const int32_t* ci, const 
   double* X = x.p;  // previous product (the start vector at first)
   double* W = w.p;
   for (int it = 0; it < steps; ++it) {
-    k_power_prep<<<blocks_for(n, 256), 256, 0, st>>>(n, X, s, sc.p, y.p);
+    launch_pdl(k_power_prep, blocks_for(n, 256), 256, 0, st, n, X, s, sc.p, y.p);
     SA_LAUNCHED();
     DISPATCH_SW(sw, k_power_spmv, n, n, rp, ci, v, s, y.p, W);
     SA_LAUNCHED();
-    k_power_dots<<<red_blocks(n), RED_THREADS, 0, st>>>(n, W, X, sc.p, part.p, fin);
+    launch_pdl(k_power_dots, red_blocks(n), RED_THREADS, 0, st, n, W, X, sc.p, part.p, fin);
     SA_LAUNCHED();
     double* t = X; X = W; W = t;
   }
@@ -238,10 +242,10 @@ int run_power_op(Alloc& al, int64_t n, int steps, uint32_t tag, uint32_t seed, d
   double* X = x.p;
   double* W = w.p;
   for (int it = 0; it < steps; ++it) {
-    k_power_prep<<<blocks_for(n, 256), 256, 0, st>>>(n, X, nullptr, sc.p, y.p);
+    launch_pdl(k_power_prep, blocks_for(n, 256), 256, 0, st, n, X, nullptr, sc.p, y.p);
     SA_LAUNCHED();
     SA_TRY(apply(y.p, W));
-    k_power_dots<<<red_blocks(n), RED_THREADS, 0, st>>>(n, W, X, sc.p, part.p, fin);
+    launch_pdl(k_power_dots, red_blocks(n), RED_THREADS, 0, st, n, W, X, sc.p, part.p, fin);
     SA_LAUNCHED();
     double* t = X; X = W; W = t;
   }
@@ -277,6 +281,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_cg_update(int64_t n, const CgSc
                                                            const double* __restrict__ q, double* __restrict__ x,
                                                            double* __restrict__ r, double* __restrict__ rprev,
                                                            double* __restrict__ part, Fin fin) {
+  pdl_sync();
   const double alpha = s->alpha;
   double acc[1] = {0.0};
   // two grid-stride elements per trip (loads together; r.r added in the
@@ -315,6 +320,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_cg_update(int64_t n, const CgSc
 
 __global__ void k_cg_pupdate(int64_t n, const CgScalars* __restrict__ s, const double* __restrict__ z,
                              double* __restrict__ p, int first) {
+  pdl_sync();
   const double beta = s->beta;
   const int64_t st = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += 2 * st) {
@@ -330,21 +336,21 @@ __global__ void k_cg_pupdate(int64_t n, const CgScalars* __restrict__ s, const d
 // the sums of np partials (k columns, or one vector with k = 0) that the
 // producing launch did not finish itself
 int launch_fin_wide(cudaStream_t st, const double* part, int np, const Fin& fin) {
-  if (fin.k > 0) k_fin_wide<KMAX_BLOCK><<<32, 32 * KMAX_BLOCK, 0, st>>>(part, np, np, fin);
-  else k_fin_wide<1><<<32, 32, 0, st>>>(part, np, 0, fin);
+  if (fin.k > 0) launch_pdl(k_fin_wide<KMAX_BLOCK>, 32, 32 * KMAX_BLOCK, 0, st, part, np, np, fin);
+  else launch_pdl(k_fin_wide<1>, 32, 32, 0, st, part, np, 0, fin);
   SA_LAUNCHED();
   return SA_OK;
 }
 
 int launch_cg_update(cudaStream_t st, int64_t n, const CgScalars* s, const double* p, const double* q, double* x,
                      double* r, double* rprev, double* part, const Fin& fin) {
-  k_cg_update<<<red_blocks(n), RED_THREADS, 0, st>>>(n, s, p, q, x, r, rprev, part, fin);
+  launch_pdl(k_cg_update, red_blocks(n), RED_THREADS, 0, st, n, s, p, q, x, r, rprev, part, fin);
   SA_LAUNCHED();
   return SA_OK;
 }
 
 int launch_cg_pupdate(cudaStream_t st, int64_t n, const CgScalars* s, const double* z, double* p, int first) {
-  k_cg_pupdate<<<red_blocks(n), RED_THREADS, 0, st>>>(n, s, z, p, first);
+  launch_pdl(k_cg_pupdate, red_blocks(n), RED_THREADS, 0, st, n, s, z, p, first);
   SA_LAUNCHED();
   return SA_OK;
 }
@@ -391,6 +397,7 @@ __global__ void __launch_bounds__(RED_THREADS, 2) k_bdots(int64_t n, const doubl
                                                           const double* __restrict__ b0, const double* __restrict__ a1,
                                                           const double* __restrict__ b1, double* __restrict__ part,
                                                           Fin fin) {
+  pdl_sync();
   constexpr int G = KK >= 4 ? 4 : 2;
   double acc[NV];
 #pragma unroll
@@ -421,6 +428,7 @@ __global__ void __launch_bounds__(RED_THREADS, 2)
     k_bcg_update(const int64_t n, const CgScalars* s, const int* __restrict__ active,
                  const double* __restrict__ p, const double* __restrict__ q, double* __restrict__ x,
                  double* __restrict__ r, double* __restrict__ rprev, double* __restrict__ part, Fin fin) {
+  pdl_sync();
   constexpr int G = KK >= 4 ? 4 : 2;
   __shared__ double alpha[KB];
   __shared__ int on[KB];
@@ -472,6 +480,7 @@ template <int KK>
 __global__ void __launch_bounds__(RED_THREADS, 2)
     k_bcg_pupdate(int64_t n, const CgScalars* __restrict__ s, const int* __restrict__ active,
                   const double* __restrict__ z, double* __restrict__ p, int first) {
+  pdl_sync();
   constexpr int G = KK >= 4 ? 4 : 2;
   __shared__ double beta[KB];
   __shared__ int on[KB];
@@ -517,13 +526,13 @@ int launch_bdots(cudaStream_t st, int64_t n, int k, const double* a0, const doub
   const unsigned g = red_blocks(n);
   // one dot per column, or two (a1 . b1 into out[KB + c])
   if (a1) {
-    if (k == 2) k_bdots<2, 2 * KB><<<g, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part, fin);
-    else if (k == 4) k_bdots<4, 2 * KB><<<g, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part, fin);
-    else k_bdots<8, 2 * KB><<<g, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part, fin);
+    if (k == 2) launch_pdl(k_bdots<2, 2 * KB>, g, RED_THREADS, 0, st, n, a0, b0, a1, b1, part, fin);
+    else if (k == 4) launch_pdl(k_bdots<4, 2 * KB>, g, RED_THREADS, 0, st, n, a0, b0, a1, b1, part, fin);
+    else launch_pdl(k_bdots<8, 2 * KB>, g, RED_THREADS, 0, st, n, a0, b0, a1, b1, part, fin);
   } else {
-    if (k == 2) k_bdots<2, KB><<<g, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part, fin);
-    else if (k == 4) k_bdots<4, KB><<<g, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part, fin);
-    else k_bdots<8, KB><<<g, RED_THREADS, 0, st>>>(n, a0, b0, a1, b1, part, fin);
+    if (k == 2) launch_pdl(k_bdots<2, KB>, g, RED_THREADS, 0, st, n, a0, b0, a1, b1, part, fin);
+    else if (k == 4) launch_pdl(k_bdots<4, KB>, g, RED_THREADS, 0, st, n, a0, b0, a1, b1, part, fin);
+    else launch_pdl(k_bdots<8, KB>, g, RED_THREADS, 0, st, n, a0, b0, a1, b1, part, fin);
   }
   SA_LAUNCHED();
   return SA_OK;
@@ -533,9 +542,9 @@ int launch_bcg_update(cudaStream_t st, int64_t n, int k, const CgScalars* s, con
                       const double* q, double* x, double* r, double* rprev, double* part, const Fin& fin) {
   if (k != 2 && k != 4 && k != 8) return SA_ERR_INVALID_ARG;  // whole-row vectors
   const unsigned g = red_blocks(n);
-  if (k == 2) k_bcg_update<2><<<g, RED_THREADS, 0, st>>>(n, s, active, p, q, x, r, rprev, part, fin);
-  else if (k == 4) k_bcg_update<4><<<g, RED_THREADS, 0, st>>>(n, s, active, p, q, x, r, rprev, part, fin);
-  else k_bcg_update<8><<<g, RED_THREADS, 0, st>>>(n, s, active, p, q, x, r, rprev, part, fin);
+  if (k == 2) launch_pdl(k_bcg_update<2>, g, RED_THREADS, 0, st, n, s, active, p, q, x, r, rprev, part, fin);
+  else if (k == 4) launch_pdl(k_bcg_update<4>, g, RED_THREADS, 0, st, n, s, active, p, q, x, r, rprev, part, fin);
+  else launch_pdl(k_bcg_update<8>, g, RED_THREADS, 0, st, n, s, active, p, q, x, r, rprev, part, fin);
   SA_LAUNCHED();
   return SA_OK;
 }
@@ -543,9 +552,9 @@ int launch_bcg_update(cudaStream_t st, int64_t n, int k, const CgScalars* s, con
 int launch_bcg_pupdate(cudaStream_t st, int64_t n, int k, const CgScalars* s, const int* active, const double* z,
                        double* p, int first) {
   if (k != 2 && k != 4 && k != 8) return SA_ERR_INVALID_ARG;  // whole-row vectors
-  if (k == 2) k_bcg_pupdate<2><<<red_blocks(n), RED_THREADS, 0, st>>>(n, s, active, z, p, first);
-  else if (k == 4) k_bcg_pupdate<4><<<red_blocks(n), RED_THREADS, 0, st>>>(n, s, active, z, p, first);
-  else k_bcg_pupdate<8><<<red_blocks(n), RED_THREADS, 0, st>>>(n, s, active, z, p, first);
+  if (k == 2) launch_pdl(k_bcg_pupdate<2>, red_blocks(n), RED_THREADS, 0, st, n, s, active, z, p, first);
+  else if (k == 4) launch_pdl(k_bcg_pupdate<4>, red_blocks(n), RED_THREADS, 0, st, n, s, active, z, p, first);
+  else launch_pdl(k_bcg_pupdate<8>, red_blocks(n), RED_THREADS, 0, st, n, s, active, z, p, first);
   SA_LAUNCHED();
   return SA_OK;
 }

@@ -401,6 +401,7 @@ struct VOcc {
 template <typename T, int SW>
 __global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_cheb(MatView<T> A, const T* __restrict__ b, const T* __restrict__ xin, T* __restrict__ xout,
                           T* __restrict__ d, T c1, T c2, int first) {
+  pdl_sync();
   T y;
   int64_t i;
   if (!row_apply<T, SW>(A, xin, y, i)) return;
@@ -411,6 +412,7 @@ __global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_cheb(MatView<T> A, c
 
 template <typename T, int SW>
 __global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_residual(MatView<T> A, const T* __restrict__ b, const T* __restrict__ x, T* __restrict__ r) {
+  pdl_sync();
   T y;
   int64_t i;
   if (row_apply<T, SW>(A, x, y, i)) r[i] = b[i] - y;
@@ -418,6 +420,7 @@ __global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_residual(MatView<T> 
 
 template <typename T, int SW>
 __global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_spmv(MatView<T> A, const T* __restrict__ x, T* __restrict__ out) {
+  pdl_sync();
   T y;
   int64_t i;
   if (row_apply<T, SW>(A, x, y, i)) out[i] = y;
@@ -425,6 +428,7 @@ __global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_spmv(MatView<T> A, c
 
 template <typename T, int SW>
 __global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_spmv_add(MatView<T> A, const T* __restrict__ x, T* __restrict__ out) {
+  pdl_sync();
   T y;
   int64_t i;
   if (row_apply<T, SW>(A, x, y, i)) out[i] += y;
@@ -435,6 +439,7 @@ template <typename T, int SW>
 __global__ void k_vc_cheb_out(MatView<T> A, const T* __restrict__ b, const T* __restrict__ xin,
                               const T* __restrict__ d, T c1, T c2, int first, const double* __restrict__ s,
                               double* __restrict__ z) {
+  pdl_sync();
   T y;
   int64_t i;
   if (!row_apply<T, SW>(A, xin, y, i)) return;
@@ -444,6 +449,7 @@ __global__ void k_vc_cheb_out(MatView<T> A, const T* __restrict__ b, const T* __
 
 template <typename T>
 __global__ void k_vc_first(int64_t n, const T* __restrict__ b, T c2, T* __restrict__ x, T* __restrict__ d) {
+  pdl_sync();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) {
     T dn = c2 * b[i];
@@ -456,6 +462,7 @@ __global__ void k_vc_first(int64_t n, const T* __restrict__ b, T c2, T* __restri
 template <typename T>
 __global__ void k_vc_fine_in(int64_t n, const double* __restrict__ r, const double* __restrict__ s, T c2,
                              T* __restrict__ b, T* __restrict__ x, T* __restrict__ d) {
+  pdl_sync();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) {
     T bi = (T)(s[i] * r[i]);
@@ -471,10 +478,10 @@ __global__ void k_vc_fine_in(int64_t n, const double* __restrict__ r, const doub
   do {                                                                                   \
     const MatView<T> _mv = view(M);                                                      \
     const unsigned _g = mat_grid(M);                                                     \
-    if ((M).sw == 0 && (M).sell_lanes == 2) K<T, -2><<<_g, 256, 0, st>>>(_mv, __VA_ARGS__); \
-    else if ((M).sw == 0) K<T, 0><<<_g, 256, 0, st>>>(_mv, __VA_ARGS__);                 \
-    else if ((M).sw == 1) K<T, 1><<<_g, 256, 0, st>>>(_mv, __VA_ARGS__);                 \
-    else K<T, CSR_LANES><<<_g, 256, 0, st>>>(_mv, __VA_ARGS__);                          \
+    if ((M).sw == 0 && (M).sell_lanes == 2) launch_pdl(K<T, -2>, _g, 256, 0, st, _mv, __VA_ARGS__); \
+    else if ((M).sw == 0) launch_pdl(K<T, 0>, _g, 256, 0, st, _mv, __VA_ARGS__);                 \
+    else if ((M).sw == 1) launch_pdl(K<T, 1>, _g, 256, 0, st, _mv, __VA_ARGS__);                 \
+    else launch_pdl(K<T, CSR_LANES>, _g, 256, 0, st, _mv, __VA_ARGS__);                          \
   } while (0)
 
 // spectral-radius estimate of level l's operator D^-1/2 A D^-1/2 by `steps`
@@ -494,6 +501,7 @@ int vh_power(Alloc& al, VHier<double>* m, int l, int steps, uint32_t tag, uint32
 template <typename T>
 __global__ void k_coarse_in(int64_t n, const T* __restrict__ b, const double* __restrict__ sq,
                             double* __restrict__ t) {
+  pdl_sync();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) t[i] = sq[i] * (double)b[i];
 }
@@ -522,7 +530,7 @@ static int mv(VHier<T>* m, cudaStream_t st, int l, const double* r64, T** xo) {
   const int64_t n = L->n;
   if (l == nl - 1) {
     int pi = prof_begin(st, PK_COARSE, l, 8.0 * n * n + 48.0 * n);
-    k_coarse_in<T><<<g256(n), 256, 0, st>>>(n, L->b.p, L->sq.p, m->ct.p);
+    launch_pdl(k_coarse_in<T>, g256(n), 256, 0, st, n, L->b.p, L->sq.p, m->ct.p);
     SA_LAUNCHED();
     SA_TRY(launch_coarse_solve(st, 1, coarse_prob(m->cf, m->ct.p, m->cs.p, m->cy.p, m->cx.p, L->sq.p, L->x.p,
                                                   sizeof(T) == 4)));
@@ -538,9 +546,9 @@ static int mv(VHier<T>* m, cudaStream_t st, int l, const double* r64, T** xo) {
   const Mat<T>& A = L->A;
   if (l == 0) {
     PROFK(K_FST, l, 16.0 * n + 3.0 * S * n,
-          (k_vc_fine_in<T><<<g256(n), 256, 0, st>>>(n, r64, m->s0.p, (T)(1.0 / th), L->b.p, xa, L->d.p)));
+          (launch_pdl(k_vc_fine_in<T>, g256(n), 256, 0, st, n, r64, m->s0.p, (T)(1.0 / th), L->b.p, xa, L->d.p)));
   } else {
-    PROFK(K_FST, l, 3.0 * S * n, (k_vc_first<T><<<g256(n), 256, 0, st>>>(n, L->b.p, (T)(1.0 / th), xa, L->d.p)));
+    PROFK(K_FST, l, 3.0 * S * n, (launch_pdl(k_vc_first<T>, g256(n), 256, 0, st, n, L->b.p, (T)(1.0 / th), xa, L->d.p)));
   }
   double rho = 1.0 / s1;
   for (int k = 1; k < deg; ++k) {
@@ -623,6 +631,7 @@ __global__ void __launch_bounds__(256) k_sell_spmv_dot(int64_t n, const int64_t*
                                 const int32_t* __restrict__ base, const uint16_t* __restrict__ c16,
                                 const double* __restrict__ v, const double* __restrict__ p, double* __restrict__ q,
                                 double* __restrict__ part, Fin fin) {
+  pdl_sync();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double c = 0.0;
   if (i < n) {
@@ -647,6 +656,7 @@ __global__ void k_sell_res64(int64_t n, const int64_t* __restrict__ sp, const in
                              const int32_t* __restrict__ base, const uint16_t* __restrict__ c16,
                              const double* __restrict__ v, const double* __restrict__ b,
                              const double* __restrict__ x, double* __restrict__ r) {
+  pdl_sync();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n)
     r[i] = b[i] - (c16 ? sell_row16<double>(sp, base, c16, v, x, i) : sell_row<double>(sp, ci, v, x, i));
@@ -658,17 +668,17 @@ int launch_sell_spmv_dot(cudaStream_t st, const Sell<double>& A, const double* p
   const int32_t* base = A.idx16 ? A.base.p : nullptr;
   const uint16_t* c16 = A.idx16 ? A.c16.p : nullptr;
   if (g <= FIN_INLINE) {
-    k_sell_spmv_dot<true><<<g, 256, 0, st>>>(A.n, A.sp.p, A.ci.p, base, c16, A.v.p, p, q, part, fin);
+    launch_pdl(k_sell_spmv_dot<true>, g, 256, 0, st, A.n, A.sp.p, A.ci.p, base, c16, A.v.p, p, q, part, fin);
     SA_LAUNCHED();
     return SA_OK;
   }
-  k_sell_spmv_dot<false><<<g, 256, 0, st>>>(A.n, A.sp.p, A.ci.p, base, c16, A.v.p, p, q, part, fin);
+  launch_pdl(k_sell_spmv_dot<false>, g, 256, 0, st, A.n, A.sp.p, A.ci.p, base, c16, A.v.p, p, q, part, fin);
   SA_LAUNCHED();
   return launch_fin_wide(st, part, (int)g, fin);
 }
 
 int launch_sell_residual64(cudaStream_t st, const Sell<double>& A, const double* b, const double* x, double* r) {
-  k_sell_res64<<<g256(A.n), 256, 0, st>>>(A.n, A.sp.p, A.ci.p, A.idx16 ? A.base.p : nullptr,
+  launch_pdl(k_sell_res64, g256(A.n), 256, 0, st, A.n, A.sp.p, A.ci.p, A.idx16 ? A.base.p : nullptr,
                                            A.idx16 ? A.c16.p : nullptr, A.v.p, b, x, r);
   SA_LAUNCHED();
   return SA_OK;
