@@ -62,7 +62,6 @@ __device__ __forceinline__ void g_mat_row(int op, const GMat<T>& D, unsigned blk
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_g_mat(int op, const GMat<T>* __restrict__ d, int m) {
-  pdl_sync();
   const int k = seg_of(d, m);
   const GMat<T> D = d[k];
   const unsigned blk = blockIdx.x - D.blk0;
@@ -80,8 +79,8 @@ __global__ void __launch_bounds__(256) k_g_mat(int op, const GMat<T>* __restrict
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256) k_g_vec(int op, const GVec<T>* __restrict__ d, int m) {
-  pdl_sync();
   const int k = seg_of(d, m);
+  pdl_sync();
   const GVec<T>& D = d[k];
   const int64_t i = (int64_t)(blockIdx.x - D.blk0) * blockDim.x + threadIdx.x;
   if (i >= D.n) return;
@@ -176,8 +175,8 @@ __device__ __forceinline__ void g_tail(const GCg& D) {
 
 // rows geometry (blocks of 256): residual, operator product with p.q
 __global__ void __launch_bounds__(256) k_g_cg_rows(int op, const GCg* __restrict__ d, int m) {
-  pdl_sync();
   const int k = seg_of(d, m);
+  pdl_sync();
   const GCg& D = d[k];
   const unsigned blk = blockIdx.x - D.blk0;
   const int64_t i = (int64_t)blk * blockDim.x + threadIdx.x;
@@ -209,8 +208,8 @@ __global__ void __launch_bounds__(256) k_g_cg_rows(int op, const GCg* __restrict
 // elements; sixteen small problems in full grids spent 25 us a launch on
 // block sums of zeros)
 __global__ void __launch_bounds__(RED_THREADS) k_g_cg_red(int op, const GCg* __restrict__ d, int m) {
-  pdl_sync();
   const int k = seg_of(d, m);
+  pdl_sync();
   const GCg& D = d[k];
   const unsigned blk = blockIdx.x - D.blk0;
   const int64_t n = D.n;

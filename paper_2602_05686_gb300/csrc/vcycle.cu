@@ -401,7 +401,6 @@ struct VOcc {
 template <typename T, int SW>
 __global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_cheb(MatView<T> A, const T* __restrict__ b, const T* __restrict__ xin, T* __restrict__ xout,
                           T* __restrict__ d, T c1, T c2, int first) {
-  pdl_sync();
   T y;
   int64_t i;
   if (!row_apply<T, SW>(A, xin, y, i)) return;
@@ -412,7 +411,6 @@ __global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_cheb(MatView<T> A, c
 
 template <typename T, int SW>
 __global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_residual(MatView<T> A, const T* __restrict__ b, const T* __restrict__ x, T* __restrict__ r) {
-  pdl_sync();
   T y;
   int64_t i;
   if (row_apply<T, SW>(A, x, y, i)) r[i] = b[i] - y;
@@ -420,7 +418,6 @@ __global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_residual(MatView<T> 
 
 template <typename T, int SW>
 __global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_spmv(MatView<T> A, const T* __restrict__ x, T* __restrict__ out) {
-  pdl_sync();
   T y;
   int64_t i;
   if (row_apply<T, SW>(A, x, y, i)) out[i] = y;
@@ -428,7 +425,6 @@ __global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_spmv(MatView<T> A, c
 
 template <typename T, int SW>
 __global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_spmv_add(MatView<T> A, const T* __restrict__ x, T* __restrict__ out) {
-  pdl_sync();
   T y;
   int64_t i;
   if (row_apply<T, SW>(A, x, y, i)) out[i] += y;
@@ -439,7 +435,6 @@ template <typename T, int SW>
 __global__ void k_vc_cheb_out(MatView<T> A, const T* __restrict__ b, const T* __restrict__ xin,
                               const T* __restrict__ d, T c1, T c2, int first, const double* __restrict__ s,
                               double* __restrict__ z) {
-  pdl_sync();
   T y;
   int64_t i;
   if (!row_apply<T, SW>(A, xin, y, i)) return;

@@ -82,18 +82,32 @@ __device__ __forceinline__ T sell2_lane(const int64_t* __restrict__ sp, const in
   const T* __restrict__ xs = C16 ? x + base[sl] : x;
   T acc = (T)0;
   int64_t p = b + 32 * h + r;
-  for (; p + 64 * (U - 1) < e; p += 64 * U) {
-    T vv[U], xx[U];
-    unsigned cc[U];
+  // the first round's values and columns before the wait for the vector
+  T vv[U], xx[U];
+  unsigned cc[U];
+  const bool full = p + 64 * (U - 1) < e;
+  if (full) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       vv[u] = __ldcs(&v[p + 64 * u]);
       cc[u] = C16 ? (unsigned)__ldcs(&c16[p + 64 * u]) : (unsigned)__ldcs(&ci[p + 64 * u]);
     }
+  }
+  pdl_sync();
+  if (full) {
+    for (;;) {
 #pragma unroll
-    for (int u = 0; u < U; ++u) xx[u] = __ldg(&xs[cc[u]]);
+      for (int u = 0; u < U; ++u) xx[u] = __ldg(&xs[cc[u]]);
 #pragma unroll
-    for (int u = 0; u < U; ++u) acc += vv[u] * xx[u];
+      for (int u = 0; u < U; ++u) acc += vv[u] * xx[u];
+      p += 64 * U;
+      if (p + 64 * (U - 1) >= e) break;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        vv[u] = __ldcs(&v[p + 64 * u]);
+        cc[u] = C16 ? (unsigned)__ldcs(&c16[p + 64 * u]) : (unsigned)__ldcs(&ci[p + 64 * u]);
+      }
+    }
   }
   for (; p < e; p += 64) {
     const unsigned c = C16 ? (unsigned)__ldcs(&c16[p]) : (unsigned)__ldcs(&ci[p]);
@@ -157,6 +171,7 @@ template <typename T, int W, int U>
 __device__ __forceinline__ T csr_lane(const MatView<T>& M, const T* __restrict__ x, int64_t b, int64_t e, int sl) {
   T acc = (T)0;
   if constexpr (W == 1) {
+    pdl_sync();
     int64_t q = b + sl;
     for (; q + W * (U - 1) < e; q += W * U) {
       T vv[U], xx[U];
@@ -184,6 +199,7 @@ __device__ __forceinline__ T csr_lane(const MatView<T>& M, const T* __restrict__
       vv[u] = in ? v[sl + W * u] : (T)0;
       cc[u] = in ? ci[sl + W * u] : 0;
     }
+    pdl_sync();  // the matrix is not written by the stream's solves, the vector is
     for (int q = sl; q < len; q += W * U) {
       T xx[U], vn[U];
       int32_t cn[U];
@@ -249,7 +265,10 @@ static unsigned mat_grid(const Mat<T>& M) {
 // SW = -2: SELL-32, two lanes per row; SW > 0: CSR, SW lanes per row,
 // reduced by shuffles (every lane of the warp reaches the shuffles), rows of
 // the long-row bin by a warp each.  The sums do not depend on the unroll.
-// Returns true for the thread that owns the row.
+// Returns true for the thread that owns the row.  Calls pdl_sync() on the way
+// to the vector (the row's pointers, and where rows are spread over lanes
+// their first values and columns, are read before): every thread that returns
+// true has called it.
 // row_apply_at takes the launch-local block index explicitly (blk), so a
 // launch that covers several matrices one after another (the group solve)
 // gives every row exactly the threads and arithmetic of its own launch.
@@ -273,6 +292,7 @@ __device__ __forceinline__ bool row_apply_at(const MatView<T>& M, const T* __res
     const int64_t gt = (int64_t)blk * blockDim.x + threadIdx.x;
     row = gt;
     if (gt >= M.n) return false;
+    pdl_sync();
     out = M.c16 ? sell_row16<T>(M.p, M.base, M.c16, M.v, x, gt) : sell_row<T>(M.p, M.ci, M.v, x, gt);
     return true;
   } else {
