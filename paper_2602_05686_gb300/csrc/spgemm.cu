@@ -51,31 +51,84 @@ __device__ __forceinline__ int hfind(const int32_t* keys, int32_t j) {
   return -1;
 }
 
+// The products of a row of A B, flattened: 32 entries of A at a time (a lane
+// each: column, value, bounds of its B row), their B rows numbered through,
+// lane t of a round taking product t.  One gather of row bounds per 32 entries
+// and full lanes, where an entry at a time was a chain of three dependent loads
+// with half the lanes idle (B rows of about 15 entries).
+struct ProdChunk {
+  int32_t k = 0;          // this lane's A column
+  double a = 0.0;
+  int64_t qb = 0;         // start of its B row
+  int off = 0, tot = 0;   // first product of this lane's B row in the chunk; products of the chunk
+};
+
+__device__ __forceinline__ ProdChunk chunk_load(int64_t p0, int64_t e, const int32_t* __restrict__ Aci,
+                                                const double* __restrict__ Av, const int64_t* __restrict__ Brp) {
+  const int lane = lane_id();
+  ProdChunk c;
+  int len = 0;
+  if (p0 + lane < e) {
+    c.k = Aci[p0 + lane];
+    if (Av) c.a = Av[p0 + lane];
+    c.qb = Brp[c.k];
+    len = (int)(Brp[c.k + 1] - c.qb);
+  }
+  int inc = len;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(FULL, inc, o);
+    if (lane >= o) inc += u;
+  }
+  c.off = inc - len;
+  c.tot = __shfl_sync(FULL, inc, 31);
+  return c;
+}
+
+// the lane whose B row holds product t (< tot): the last with off <= t (of
+// equal offsets the last one: empty rows share their successor's)
+__device__ __forceinline__ int chunk_owner(const ProdChunk& c, int t) {
+  int lo = 0;
+#pragma unroll
+  for (int st = 16; st > 0; st >>= 1) {
+    const int o = __shfl_sync(FULL, c.off, lo + st);
+    if (o <= t) lo += st;
+  }
+  return lo;
+}
+
 // inserts every column of row i of A*B; returns the distinct count, or -1 on
 // overflow (more than HCAP distinct columns)
 __device__ int warp_build_row(int64_t i, const int64_t* __restrict__ Arp, const int32_t* __restrict__ Aci,
-                              const int64_t* __restrict__ Brp, const int32_t* __restrict__ Bci, int32_t* keys,
-                              int* wcount) {
+                              const int64_t* __restrict__ Brp, const int32_t* __restrict__ Bci, int32_t* keys) {
   const int lane = lane_id();
   for (int t = lane; t < HB; t += 32) keys[t] = -1;
-  if (lane == 0) *wcount = 0;
   __syncwarp();
   const int64_t b = Arp[i], e = Arp[i + 1];
-  bool over = false;
-  for (int64_t p = b; p < e && !over; ++p) {
-    const int32_t k = Aci[p];
-    const int64_t qb = Brp[k], qe = Brp[k + 1];
-    for (int64_t q = qb + lane; q < qe; q += 32) {
-      int r = hinsert(keys, Bci[q]);
-      if (r == 1) atomicAdd(wcount, 1);
-      if (r < 0) atomicAdd(wcount, HCAP + 1);
+  int total = 0;
+  for (int64_t p0 = b; p0 < e && total <= HCAP; p0 += 32) {
+    const ProdChunk c = chunk_load(p0, e, Aci, nullptr, Brp);
+    for (int t0 = 0; t0 < c.tot && total <= HCAP; t0 += 64) {
+      // two rounds' loads together
+      int32_t j[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int t = t0 + 32 * u + lane;
+        const int o = chunk_owner(c, t < c.tot ? t : c.tot - 1);
+        const int64_t q = __shfl_sync(FULL, c.qb, o) + (t - __shfl_sync(FULL, c.off, o));
+        j[u] = t < c.tot ? Bci[q] : -1;
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        // at most HCAP + 32 columns before the check: the table holds them
+        int r = 0;
+        if (total <= HCAP && j[u] >= 0) r = hinsert(keys, j[u]);
+        total += __popc(__ballot_sync(FULL, r == 1)) + (__any_sync(FULL, r < 0) ? HCAP + 1 : 0);
+      }
     }
-    __syncwarp();
-    over = *((volatile int*)wcount) > HCAP;
   }
   __syncwarp();
-  int c = *((volatile int*)wcount);
-  return c > HCAP ? -1 : c;
+  return total > HCAP ? -1 : total;
 }
 
 __global__ void __launch_bounds__(SG_WARPS * 32)
@@ -83,12 +136,11 @@ k_spgemm_count(int64_t n, const int32_t* __restrict__ rows, const int64_t* __res
                const int32_t* __restrict__ Aci, const int64_t* __restrict__ Brp, const int32_t* __restrict__ Bci,
                int64_t* __restrict__ cnt, int32_t* __restrict__ big, unsigned long long* __restrict__ nbig) {
   __shared__ int32_t keys_all[SG_WARPS][HB];
-  __shared__ int wcount_all[SG_WARPS];
   const int w = threadIdx.x >> 5;
   int32_t* keys = keys_all[w];
   for (int64_t t = global_warp(); t < n; t += warp_stride()) {
     const int64_t i = rows ? rows[t] : t;  // rows: the rows the thread tier could not hold
-    int c = warp_build_row(i, Arp, Aci, Brp, Bci, keys, &wcount_all[w]);
+    int c = warp_build_row(i, Arp, Aci, Brp, Bci, keys);
     if (lane_id() == 0) {
       if (c < 0) {
         unsigned long long slot = atomicAdd(nbig, 1ull);
@@ -112,19 +164,20 @@ k_spgemm_fill(int64_t n, const int32_t* __restrict__ rows, const int64_t* __rest
   // row wider than the table goes to `defer` (the big tier), the distinct
   // count of every other row to cnt[i + 1]
   __shared__ int32_t keys_all[SG_WARPS][HB];
-  __shared__ int32_t rank_all[SG_WARPS][HB];
+  __shared__ uint8_t rank_all[SG_WARPS][HB];
   __shared__ int32_t cols_all[SG_WARPS][HCAP];
+  __shared__ uint8_t slot_all[SG_WARPS][HCAP];
   __shared__ double acc_all[SG_WARPS][HCAP];
-  __shared__ int wcount_all[SG_WARPS];
   const int w = threadIdx.x >> 5, lane = lane_id();
   int32_t* keys = keys_all[w];
-  int32_t* rank_of = rank_all[w];
+  uint8_t* rank_of = rank_all[w];
   int32_t* cols = cols_all[w];
+  uint8_t* slot_of = slot_all[w];
   double* acc = acc_all[w];
   for (int64_t t = global_warp(); t < n; t += warp_stride()) {
     const int64_t i = rows ? rows[t] : t;
     if (isbig && isbig[i]) continue;  // warp-uniform
-    const int c = warp_build_row(i, Arp, Aci, Brp, Bci, keys, &wcount_all[w]);
+    const int c = warp_build_row(i, Arp, Aci, Brp, Bci, keys);
     if (!isbig && lane == 0) {
       if (c < 0) defer[atomicAdd(ndefer, 1ull)] = (int32_t)i;
       else cnt[i + 1] = c;
@@ -133,54 +186,68 @@ k_spgemm_fill(int64_t n, const int32_t* __restrict__ rows, const int64_t* __rest
     // compact the keys (slot order), remember each key's slot
     int out = 0;
     for (int t0 = 0; t0 < HB; t0 += 32) {
-      int t = t0 + lane;
-      int32_t k = keys[t];
-      bool has = k != -1;
-      unsigned m = __ballot_sync(FULL, has);
+      const int32_t k = keys[t0 + lane];
+      const bool has = k != -1;
+      const unsigned m = __ballot_sync(FULL, has);
       if (has) {
-        int pos = out + __popc(m & ((1u << lane) - 1u));
+        const int pos = out + __popc(m & ((1u << lane) - 1u));
         cols[pos] = k;
-        rank_of[t] = pos;  // temporarily: compact position
+        slot_of[pos] = (uint8_t)(t0 + lane);
       }
       out += __popc(m);
     }
     __syncwarp();
     // rank sort (keys are distinct): slot -> rank in ascending column order
     const int64_t cb = Crp[i];
-    for (int t0 = 0; t0 < HB; t0 += 32) {
-      int t = t0 + lane;
-      int32_t k = keys[t];
-      if (k != -1) {
-        int r = 0;
-        for (int u = 0; u < c; ++u) r += cols[u] < k;
-        rank_of[t] = r;
-        Cci[cb + r] = k;
-      }
+    for (int u = lane; u < c; u += 32) {
+      const int32_t k = cols[u];
+      int r = 0;
+      for (int v = 0; v < c; ++v) r += cols[v] < k;
+      rank_of[slot_of[u]] = (uint8_t)r;
+      Cci[cb + r] = k;
+      acc[u] = 0.0;
     }
-    for (int t = lane; t < c; t += 32) acc[t] = 0.0;
     __syncwarp();
-    // ordered accumulation: A columns in ascending order, lanes over the B
-    // row (distinct columns, so no two lanes touch one accumulator per step).
+    // ordered accumulation: the products in A-column order, a round of 32 at
+    // a time; lanes of one round that share an accumulator (products of
+    // successive A entries) add one after the other in lane order.
     // upper_only: entries left of the diagonal stay 0 (the caller mirrors
     // the upper triangle into them)
     const int64_t b = Arp[i], e = Arp[i + 1];
-    const int32_t jmin = upper_only ? (int32_t)i : INT32_MIN;
-    for (int64_t p = b; p < e; ++p) {
-      const int32_t k = Aci[p];
-      const double a = Av[p];
-      const int64_t qb = Brp[k], qe = Brp[k + 1];
-      for (int64_t q = qb + lane; q < qe; q += 32) {
-        const int32_t j = Bci[q];
-        if (j < jmin) continue;
-        int h = hfind(keys, j);
-        if (h >= 0) {  // always found: the keys were inserted from the same rows
-          int r = rank_of[h];
-          acc[r] = __dadd_rn(acc[r], __dmul_rn(a, Bv[q]));
+    const int32_t jmin = upper_only ? (int32_t)i : 0;
+    for (int64_t p0 = b; p0 < e; p0 += 32) {
+      const ProdChunk pc = chunk_load(p0, e, Aci, Av, Brp);
+      int32_t jn = -1;
+      double vn = 0.0, an = 0.0;
+      auto fetch = [&](int t0) {
+        const int tt = t0 + lane;
+        const int o = chunk_owner(pc, tt < pc.tot ? tt : pc.tot - 1);
+        const int64_t q = __shfl_sync(FULL, pc.qb, o) + (tt - __shfl_sync(FULL, pc.off, o));
+        an = __shfl_sync(FULL, pc.a, o);
+        const bool in = tt < pc.tot;
+        jn = in ? Bci[q] : -1;
+        vn = in ? Bv[q] : 0.0;
+      };
+      if (pc.tot > 0) fetch(0);
+      for (int t0 = 0; t0 < pc.tot; t0 += 32) {
+        const int32_t j = jn;
+        const double prod = __dmul_rn(an, vn);
+        if (t0 + 32 < pc.tot) fetch(t0 + 32);  // the next round's loads
+        int r = -1;
+        if (j >= jmin) {
+          const int h = hfind(keys, j);
+          if (h >= 0) r = rank_of[h];  // always found: the keys were inserted from the same rows
+        }
+        const unsigned same = __match_any_sync(FULL, r);
+        const int turn = r >= 0 ? __popc(same & ((1u << lane) - 1u)) : 0;
+        const int turns = __reduce_max_sync(FULL, r >= 0 ? turn + 1 : 0);
+        for (int u = 0; u < turns; ++u) {
+          if (r >= 0 && turn == u) acc[r] = __dadd_rn(acc[r], prod);
+          __syncwarp();
         }
       }
-      __syncwarp();
     }
-    for (int t = lane; t < c; t += 32) Cv[cb + t] = acc[t];
+    for (int u = lane; u < c; u += 32) Cv[cb + u] = acc[u];
     __syncwarp();
   }
 }
@@ -257,17 +324,13 @@ __global__ void __launch_bounds__(TB)
 k_spgemm_tfill(int64_t n, const int64_t* __restrict__ Arp, const int32_t* __restrict__ Aci,
                const double* __restrict__ Av, const int64_t* __restrict__ Brp, const int32_t* __restrict__ Bci,
                const double* __restrict__ Bv, const int64_t* __restrict__ Crp, int32_t* __restrict__ Cci,
-               double* __restrict__ Cv, const uint8_t* __restrict__ ismid, int upper_only,
-               int32_t* __restrict__ defer, unsigned long long* __restrict__ ndefer, int64_t* __restrict__ cnt) {
-  // one-pass mode (ismid NULL): Crp holds each row's upper-bound offset, a
-  // row with more than TCAP distinct columns goes to `defer` (the warp
-  // tier), the distinct count of every other row to cnt[i + 1]
+               double* __restrict__ Cv, const uint8_t* __restrict__ ismid, int upper_only) {
   __shared__ int32_t cols_all[TCAP * TB];
   __shared__ double vals_all[TCAP * TB];
   int32_t* cols = cols_all + threadIdx.x;
   double* vals = vals_all + threadIdx.x;
   const int64_t i = (int64_t)blockIdx.x * TB + threadIdx.x;
-  if (i >= n || (ismid && ismid[i])) return;
+  if (i >= n || ismid[i]) return;
   const int32_t jmin = upper_only ? (int32_t)i : INT32_MIN;
   int c = 0;
   const int64_t e = Arp[i + 1];
@@ -292,10 +355,7 @@ k_spgemm_tfill(int64_t n, const int64_t* __restrict__ Arp, const int32_t* __rest
         const int32_t j = Bci[q];
         const int pos = tlower(cols, c, j);
         if (!(pos < c && cols[pos * TB] == j)) {
-          if (c == TCAP) {  // two-phase: cannot happen (the count held this row)
-            if (!ismid) defer[atomicAdd(ndefer, 1ull)] = (int32_t)i;
-            return;
-          }
+          if (c == TCAP) return;  // cannot happen (the count held this row)
           for (int t = c; t > pos; --t) {
             cols[t * TB] = cols[(t - 1) * TB];
             vals[t * TB] = vals[(t - 1) * TB];
@@ -313,7 +373,96 @@ k_spgemm_tfill(int64_t n, const int64_t* __restrict__ Arp, const int32_t* __rest
     Cci[cb + t] = cols[t * TB];
     Cv[cb + t] = vals[t * TB];
   }
-  if (!ismid) cnt[i + 1] = c;
+}
+
+// the thread tier of the one-pass form: the same sums on an open-addressing
+// table of TCAP slots per thread (its own column of shared memory) instead of
+// the sorted list -- inserting into that list shifted up to TCAP columns and
+// values, and with 32 rows a warp nearly every product met a lane that did.
+// The row is written in table order; the packing pass sorts it.
+__global__ void __launch_bounds__(TB)
+k_spgemm_thash(int64_t n, const int64_t* __restrict__ Arp, const int32_t* __restrict__ Aci,
+               const double* __restrict__ Av, const int64_t* __restrict__ Brp, const int32_t* __restrict__ Bci,
+               const double* __restrict__ Bv, const int64_t* __restrict__ ub, int32_t* __restrict__ Cci,
+               double* __restrict__ Cv, int upper_only, int32_t* __restrict__ defer,
+               unsigned long long* __restrict__ ndefer, int64_t* __restrict__ cnt) {
+  __shared__ int32_t cols_all[TCAP * TB];
+  __shared__ double vals_all[TCAP * TB];
+  int32_t* cols = cols_all + threadIdx.x;
+  double* vals = vals_all + threadIdx.x;
+  const int64_t i = (int64_t)blockIdx.x * TB + threadIdx.x;
+  if (i >= n) return;
+#pragma unroll
+  for (int t = 0; t < TCAP; ++t) cols[t * TB] = -1;
+  const int32_t jmin = upper_only ? (int32_t)i : 0;
+  int c = 0;
+  const int64_t e = Arp[i + 1];
+  for (int64_t p0 = Arp[i]; p0 < e; p0 += TG) {
+    int64_t qb[TG], qe[TG];
+    double av[TG];
+#pragma unroll
+    for (int u = 0; u < TG; ++u) {
+      qb[u] = 0;
+      qe[u] = 0;
+      av[u] = 0.0;
+      if (p0 + u < e) {
+        const int32_t k = Aci[p0 + u];
+        av[u] = Av[p0 + u];
+        qb[u] = Brp[k];
+        qe[u] = Brp[k + 1];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < TG; ++u) {
+      const double a = av[u];
+      for (int64_t q0 = qb[u]; q0 < qe[u]; q0 += TG) {
+        // B entries of one row in groups, loaded together
+        int32_t jj[TG];
+        double bv[TG];
+#pragma unroll
+        for (int v = 0; v < TG; ++v) {
+          const bool in = q0 + v < qe[u];
+          jj[v] = in ? Bci[q0 + v] : -1;
+          bv[v] = in ? Bv[q0 + v] : 0.0;
+        }
+#pragma unroll
+        for (int v = 0; v < TG; ++v) {
+          const int32_t j = jj[v];
+          if (j >= 0) {
+            int h = (int)__umulhi((uint32_t)j * 0x9E3779B1u, (uint32_t)TCAP);
+            int32_t k = cols[h * TB];
+            while (k != j && k != -1) {
+              h = h + 1 < TCAP ? h + 1 : 0;
+              k = cols[h * TB];
+              // (a full table without j: every slot holds another column)
+              if (c == TCAP && h == (int)__umulhi((uint32_t)j * 0x9E3779B1u, (uint32_t)TCAP)) break;
+            }
+            if (k != j) {
+              if (c == TCAP) {
+                defer[atomicAdd(ndefer, 1ull)] = (int32_t)i;
+                return;
+              }
+              cols[h * TB] = j;
+              vals[h * TB] = 0.0;
+              ++c;
+            }
+            if (j >= jmin) vals[h * TB] = __dadd_rn(vals[h * TB], __dmul_rn(a, bv[v]));
+          }
+        }
+      }
+    }
+  }
+  int64_t o = ub[i];
+#pragma unroll
+  for (int t = 0; t < TCAP; ++t) {
+    const int32_t j = cols[t * TB];
+    if (j >= 0) {
+      Cci[o] = j;
+      Cv[o] = vals[t * TB];
+      ++o;
+    }
+  }
+  cnt[i + 1] = c;
 }
 
 // ---------------------------------------------------------------------------
@@ -402,13 +551,25 @@ __global__ void k_spgemm_pcount(int64_t n, const int64_t* __restrict__ Arp, cons
   ub[i + 1] = t;
 }
 
-// rows from their upper-bound slots to the packed CSR (a warp per row)
+// rows from their upper-bound slots to the packed CSR (a warp per row); rows of
+// up to 32 columns are ranked on the way (the thread tier leaves them in table
+// order), longer ones come sorted
 __global__ void k_spgemm_compact(int64_t n, const int64_t* __restrict__ ub, const int32_t* __restrict__ uci,
                                  const double* __restrict__ uv, const int64_t* __restrict__ Crp,
                                  int32_t* __restrict__ Cci, double* __restrict__ Cv) {
   const int lane = lane_id();
   for (int64_t i = global_warp(); i < n; i += warp_stride()) {
     const int64_t src = ub[i], dst = Crp[i], c = Crp[i + 1] - dst;
+    if (c <= 32) {
+      const int32_t k = lane < c ? uci[src + lane] : INT32_MAX;
+      int r = 0;
+      for (int t = 0; t < (int)c; ++t) r += __shfl_sync(FULL, k, t) < k;
+      if (lane < c) {
+        Cci[dst + r] = k;
+        Cv[dst + r] = uv[src + lane];
+      }
+      continue;
+    }
     for (int64_t t = lane; t < c; t += 32) {
       Cci[dst + t] = uci[src + t];
       Cv[dst + t] = uv[src + t];
@@ -475,7 +636,7 @@ static int spgemm_two_phase(Alloc& al, int64_t n, int64_t m, const int64_t* Arp,
   SA_TRY(Cv.alloc(&al, *nnzC));
   if (thread_tier) {
     k_spgemm_tfill<<<blocks_for(n, TB), TB, 0, s>>>(n, Arp, Aci, Av, Brp, Bci, Bv, Crp.p, Cci.p, Cv.p, ismid.p,
-                                                    upper_only, nullptr, nullptr, nullptr);
+                                                    upper_only);
     SA_LAUNCHED();
   }
   if (nwarp > 0) {
@@ -513,8 +674,8 @@ static int spgemm_one_pass(Alloc& al, int64_t n, int64_t m, const int64_t* Arp, 
   int64_t nwarp = n;
   const int32_t* wrows = nullptr;
   if (thread_tier) {
-    k_spgemm_tfill<<<blocks_for(n, TB), TB, 0, s>>>(n, Arp, Aci, Av, Brp, Bci, Bv, ub, uci.p, uv.p, nullptr,
-                                                    upper_only, defw.p, nd.p, Crp.p);
+    k_spgemm_thash<<<blocks_for(n, TB), TB, 0, s>>>(n, Arp, Aci, Av, Brp, Bci, Bv, ub, uci.p, uv.p, upper_only,
+                                                    defw.p, nd.p, Crp.p);
     SA_LAUNCHED();
     unsigned long long h = 0;
     SA_TRY(copy_d2h(&h, nd.p, sizeof(h), s));
