@@ -162,39 +162,6 @@ __global__ void k_node_tensor_direct(int64_t n, int dim, const double* __restric
 }
 
 // ---------------------------------------------------------------------------
-// a3. classical measure + pointwise dropping (Sec. 2.1):
-//   keep_ij <=> a_ij*a_ij >= (theta*theta) * |a_ii*a_jj|, diagonal kept,
-//   Dirichlet nodes excluded.  Warp per row; also counts kept entries per
-//   row (diagonal included) into cnt[i+1].
-// ---------------------------------------------------------------------------
-__global__ void k_strength_classical(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                                     const double* __restrict__ v, const double* __restrict__ diag,
-                                     const uint8_t* __restrict__ dir, double t2, uint8_t* __restrict__ keep,
-                                     int64_t* __restrict__ cnt) {
-  const int lane = lane_id();
-  for (int64_t i = global_warp(); i < n; i += warp_stride()) {
-    const int64_t b = rp[i], e = rp[i + 1];
-    const double di = diag[i];
-    const bool diri = dir && dir[i];
-    int kept = 0;
-    for (int64_t p = b + lane; p < e; p += 32) {
-      int32_t j = ci[p];
-      uint8_t k;
-      if (j == (int32_t)i) k = 1;
-      else if (diri || (dir && dir[j])) k = 0;
-      else {
-        double a = v[p];
-        k = (a * a >= t2 * fabs(di * diag[j])) ? 1 : 0;
-      }
-      keep[p] = k;
-      kept += k;
-    }
-    for (int o = 16; o > 0; o >>= 1) kept += __shfl_xor_sync(FULL, kept, o);
-    if (lane == 0) cnt[i + 1] = kept;
-  }
-}
-
-// ---------------------------------------------------------------------------
 // a4. material-aware distance Laplacian (Sec. 2.1 distance Laplacian,
 // Sec. 3 material distance with max symmetrisation):
 //   w_ij = 1 / max(d^T sinv_i d, d^T sinv_j d), d = x_i - x_j,
@@ -382,8 +349,8 @@ __global__ void k_row_sum_ordered(int64_t n, const int64_t* __restrict__ rp, con
   D[i] = acc;
 }
 
-// keep_ij <=> w_ij*w_ij >= (theta*theta) * (D_i*D_j), the products rounded in
-// FP64.  Four FP64 instructions a pair bound this kernel (2.1M rows 538 us), so
+// keep_ij <=> w_ij*w_ij >= (theta*theta) * (D_i*D_j) (classical measure:
+// a_ij*a_ij >= (theta*theta) * |a_ii*a_jj|), the products rounded in FP64.  Four FP64 instructions a pair bound this kernel (2.1M rows 538 us), so
 // the comparison is first made on the exponents and on the leading 20 bits of
 // the significands in FP32: 1 when w w is larger by more than their error, 0
 // when it is smaller, -1 when neither is certain (or an operand's exponent is
@@ -410,6 +377,10 @@ __device__ __forceinline__ int keep_sure(double w, double t2, double Di, double 
   return -1;
 }
 
+template <bool ABS>
+__device__ __forceinline__ double keep_arg(double v) {
+  return ABS ? fabs(v) : v;
+}
 // keep flag of entry p = (i, j), j != i
 __device__ __forceinline__ int keep_entry(double wv, double t2, double Di, double Dj, bool dirichlet) {
   if (dirichlet) return 0;
@@ -417,11 +388,16 @@ __device__ __forceinline__ int keep_entry(double wv, double t2, double Di, doubl
   return sure >= 0 ? sure : ((wv * wv >= t2 * (Di * Dj)) ? 1 : 0);
 }
 
-// a warp takes KEEP_ROWS consecutive rows at a time, their loads together (one
+// a3 / a4: the pointwise criterion, diagonal kept, Dirichlet nodes excluded;
+// kept entries per row (diagonal included) into cnt[i+1].
+// A warp takes KEEP_ROWS consecutive rows at a time, their loads together (one
 // row after another was a chain of dependent loads: 458 us), the entries past
-// the 32nd of a row after them
+// the 32nd of a row after them.  ABS: the classical measure, |a_ij| and
+// |a_ii a_jj| in place of w and D (192^3 inclusions, FP64 comparisons of one row
+// at a time: 677 us a level on average)
 constexpr int KEEP_ROWS = 4;
-__global__ void __launch_bounds__(256) k_material_keep(int64_t n, const int64_t* __restrict__ rp,
+template <bool ABS>
+__global__ void __launch_bounds__(256) k_keep(int64_t n, const int64_t* __restrict__ rp,
                                                        const int32_t* __restrict__ ci, const double* __restrict__ w,
                                                        const double* __restrict__ D, const uint8_t* __restrict__ dir,
                                                        double t2, uint8_t* __restrict__ keep,
@@ -441,14 +417,14 @@ __global__ void __launch_bounds__(256) k_material_keep(int64_t n, const int64_t*
       e[u] = __shfl_sync(FULL, rpl, u + 1);
       const bool in = b[u] + lane < e[u];
       j[u] = in ? ci[b[u] + lane] : -1;
-      wv[u] = in ? w[b[u] + lane] : 0.0;
+      wv[u] = in ? keep_arg<ABS>(w[b[u] + lane]) : 0.0;
       const int64_t i = i0 + u < n ? i0 + u : n - 1;
-      Di[u] = D[i];
+      Di[u] = keep_arg<ABS>(D[i]);
       dd[u] = dir && dir[i];
     }
 #pragma unroll
     for (int u = 0; u < KEEP_ROWS; ++u) {
-      Dj[u] = j[u] >= 0 ? D[j[u]] : 0.0;
+      Dj[u] = j[u] >= 0 ? keep_arg<ABS>(D[j[u]]) : 0.0;
       if (dir && j[u] >= 0) dd[u] |= dir[j[u]] != 0;
     }
 #pragma unroll
@@ -468,7 +444,8 @@ __global__ void __launch_bounds__(256) k_material_keep(int64_t n, const int64_t*
         int c = 0;
         for (int64_t p = b[u] + 32 + lane; p < e[u]; p += 32) {
           const int32_t jj = ci[p];
-          const int k = jj == (int32_t)i ? 1 : keep_entry(w[p], t2, Di[u], D[jj], diri || (dir && dir[jj]));
+          const int k = jj == (int32_t)i ? 1 : keep_entry(keep_arg<ABS>(w[p]), t2, Di[u], keep_arg<ABS>(D[jj]),
+                                                           diri || (dir && dir[jj]));
           keep[p] = (uint8_t)k;
           c += k;
         }
@@ -639,29 +616,55 @@ __global__ void k_cut_symmetrize(int64_t n, const int64_t* __restrict__ rp, cons
 // of its row of A (every off-diagonal dropped, lumped row sum ~ 0) gets
 // Dt = +inf: it is not smoothed.
 // ---------------------------------------------------------------------------
-__global__ void k_filter(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                         const double* __restrict__ v, const uint8_t* __restrict__ keep,
-                         const int64_t* __restrict__ rpF, int32_t* __restrict__ ciF, double* __restrict__ vF,
-                         double* __restrict__ Dt) {
-  // thread per row: the three ordered sums are sequential FP64 chains, so
-  // one warp instruction advances 32 rows
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Thread per row: the three ordered sums are sequential FP64 chains, so one
+// warp instruction advances 32 rows.  The block's rows are one segment of the
+// CSR arrays, copied to shared memory first: three passes over rows 216 bytes
+// apart cost each warp load 32 lines of a cache that 64 warps shared (1.06M
+// rows of 26 entries 341 us).  A segment above FILT_CAP entries is read in
+// place.
+constexpr int FILT_ROWS = 64;
+constexpr int FILT_CAP = 2048;
+__global__ void __launch_bounds__(FILT_ROWS) k_filter(int64_t n, const int64_t* __restrict__ rp,
+                                                      const int32_t* __restrict__ ci, const double* __restrict__ v,
+                                                      const uint8_t* __restrict__ keep,
+                                                      const int64_t* __restrict__ rpF, int32_t* __restrict__ ciF,
+                                                      double* __restrict__ vF, double* __restrict__ Dt) {
+  __shared__ double s_v[FILT_CAP];
+  __shared__ int32_t s_c[FILT_CAP];
+  __shared__ uint8_t s_k[FILT_CAP];
+  const int64_t i0 = (int64_t)blockIdx.x * FILT_ROWS, i1 = i0 + FILT_ROWS < n ? i0 + FILT_ROWS : n;
+  const int64_t i = i0 + threadIdx.x;
+  const int64_t b0 = rp[i0], tot = rp[i1] - b0;
+  const double* V = v + b0;
+  const int32_t* C = ci + b0;
+  const uint8_t* K = keep + b0;
+  if (tot <= FILT_CAP) {
+    for (int p = (int)threadIdx.x; p < (int)tot; p += FILT_ROWS) {
+      s_v[p] = V[p];
+      s_c[p] = C[p];
+      s_k[p] = K[p];
+    }
+    __syncthreads();
+    V = s_v;
+    C = s_c;
+    K = s_k;
+  }
   if (i >= n) return;
-  const int64_t b = rp[i], e = rp[i + 1];
+  const int64_t b = rp[i] - b0, e = rp[i + 1] - b0;
   // lumped diagonal: a_ii, then the dropped entries in ascending order
   double dg = 0.0;
   for (int64_t p = b; p < e; ++p)
-    if (ci[p] == (int32_t)i) dg = v[p];
+    if (C[p] == (int32_t)i) dg = V[p];
   for (int64_t p = b; p < e; ++p)
-    if (ci[p] != (int32_t)i && !keep[p]) dg += v[p];
+    if (C[p] != (int32_t)i && !K[p]) dg += V[p];
   // the filtered row and both 1-norms in ascending order
   int64_t out = rpF[i];
   double s = 0.0, a1 = 0.0;
   for (int64_t p = b; p < e; ++p) {
-    const int32_t j = ci[p];
-    const double a = v[p];
+    const int32_t j = C[p];
+    const double a = V[p];
     a1 += fabs(a);
-    if (j == (int32_t)i || keep[p]) {
+    if (j == (int32_t)i || K[p]) {
       const double fv = (j == (int32_t)i) ? dg : a;
       ciF[out] = j;
       vF[out] = fv;
@@ -773,7 +776,7 @@ int launch_strength_classical(cudaStream_t s, int64_t n, const int64_t* rp, cons
                               int64_t* cnt) {
   if (n <= 0) return SA_OK;
   const double t2 = theta * theta;
-  k_strength_classical<<<warp_rows_grid(n), 256, 0, s>>>(n, rp, ci, v, diag, dir, t2, keep, cnt);
+  k_keep<true><<<warp_rows_grid((n + KEEP_ROWS - 1) / KEEP_ROWS), 256, 0, s>>>(n, rp, ci, v, diag, dir, t2, keep, cnt);
   SA_LAUNCHED();
   return SA_OK;
 }
@@ -792,7 +795,7 @@ int launch_strength_material(cudaStream_t s, int dim, int64_t n, const int64_t* 
   SA_LAUNCHED();
   k_row_sum_ordered<<<blocks_for(n, 128), 128, 0, s>>>(n, rp, w, D);
   SA_LAUNCHED();
-  k_material_keep<<<warp_rows_grid((n + KEEP_ROWS - 1) / KEEP_ROWS), 256, 0, s>>>(n, rp, ci, w, D, dir, t2, keep, cnt);
+  k_keep<false><<<warp_rows_grid((n + KEEP_ROWS - 1) / KEEP_ROWS), 256, 0, s>>>(n, rp, ci, w, D, dir, t2, keep, cnt);
   SA_LAUNCHED();
   return SA_OK;
 }
@@ -820,7 +823,7 @@ int launch_cut_drop(Alloc& al, int measure_classical, int64_t n, int64_t nnz, co
 int launch_filter(cudaStream_t s, int64_t n, const int64_t* rp, const int32_t* ci, const double* v,
                   const uint8_t* keep, const int64_t* rpF, int32_t* ciF, double* vF, double* Dt) {
   if (n <= 0) return SA_OK;
-  k_filter<<<blocks_for(n, 128), 128, 0, s>>>(n, rp, ci, v, keep, rpF, ciF, vF, Dt);
+  k_filter<<<blocks_for(n, FILT_ROWS), FILT_ROWS, 0, s>>>(n, rp, ci, v, keep, rpF, ciF, vF, Dt);
   SA_LAUNCHED();
   return SA_OK;
 }
