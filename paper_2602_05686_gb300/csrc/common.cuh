@@ -191,6 +191,13 @@ int scan_inplace(Alloc& al, int64_t* a, int64_t n);
 // sums the partials in index order; deterministic for a given n.
 constexpr int RED_BLOCKS = 304;   // 2 x 152 SMs
 constexpr int RED_THREADS = 512;
+// device values to the host, waited for; several with one wait
+struct ReadBack {
+  void* dst;
+  const void* src;
+  size_t bytes;
+};
+int read_back(const ReadBack* r, int count, cudaStream_t s);
 int copy_d2h(void* dst, const void* src, size_t bytes, cudaStream_t s);
 int copy_h2d(void* dst, const void* src, size_t bytes, cudaStream_t s);
 int memset_d(void* dst, int v, size_t bytes, cudaStream_t s);

@@ -244,8 +244,8 @@ int run_mis2(Alloc& al, int64_t n, const int64_t* gcrp, const int32_t* gcci, con
       k_mis_listfill<<<blocks_for(nn, 256), 256, 0, s>>>(nn, N, tag, flag.p, cu.p, cn.p, ul.p, nnew);
       SA_LAUNCHED();
       int64_t tot[2] = {0, 0};
-      SA_TRY(copy_d2h(&tot[0], cu.p + nn, sizeof(int64_t), s));
-      SA_TRY(copy_d2h(&tot[1], cn.p + nn, sizeof(int64_t), s));
+      const ReadBack rb[2] = {{&tot[0], cu.p + nn, sizeof(int64_t)}, {&tot[1], cn.p + nn, sizeof(int64_t)}};
+      SA_TRY(read_back(rb, 2, s));
       U = ul.p;
       N = nnew;
       nu = tot[0];
@@ -419,11 +419,9 @@ __global__ void k_rank_sort_rows(int64_t m, const int64_t* __restrict__ rp, cons
   }
 }
 
-int run_transpose(Alloc& al, int64_t n, int64_t m, const int64_t* rp, const int32_t* ci, const double* v,
-                  Buf<int64_t>& Rrp, Buf<int32_t>& Rci, Buf<double>* Rv) {
+int run_transpose(Alloc& al, int64_t n, int64_t m, int64_t nnz, const int64_t* rp, const int32_t* ci,
+                  const double* v, Buf<int64_t>& Rrp, Buf<int32_t>& Rci, Buf<double>* Rv) {
   cudaStream_t s = al.stream;
-  int64_t nnz = 0;
-  SA_TRY(copy_d2h(&nnz, rp + n, sizeof(int64_t), s));
   SA_TRY(Rrp.alloc(&al, m + 1));
   SA_TRY(Rci.alloc(&al, nnz));
   if (Rv) SA_TRY(Rv->alloc(&al, nnz));

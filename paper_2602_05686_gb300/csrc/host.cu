@@ -41,7 +41,7 @@ struct Level {
   // optional diagnostics
   Buf<uint8_t> keep, root, dir;
   double omega = 0, lam_omega = 0, lmax = 0, lmin = 0;
-
+  Buf<double> scal;  // setup: {lambda, omega} on the device until they are read
 };
 
 }  // namespace sa
@@ -197,23 +197,21 @@ static int coarsen(sa_handle h, int l, int* err, int* stop) {
   SA_TRY(sc.alloc(&al, n));
   SA_TRY(scal.alloc(&al, 2));
   SA_TRY(launch_rsqrt_scale(s, n, Dt.p, sc.p));
-  SA_TRY(run_power(al, n, rpF.p, ciF.p, vF.p, sc.p, o.power_iters, (uint32_t)(2 * l + 1), o.seed, scal.p));
+  SA_TRY(run_power(al, n, nnzF, rpF.p, ciF.p, vF.p, sc.p, o.power_iters, (uint32_t)(2 * l + 1), o.seed, scal.p));
   SA_TRY(launch_omega(s, scal.p, o.omega_sym, scal.p + 1));
   PHASE_END(PK_S_OMEGA);
 
   // a12: P = P^ - omega D~^-1 A_F P^
   PHASE_BEGIN(PK_S_SMOOTHP, l);
-  SA_TRY(run_spgemm(al, n, nc, n, rpF.p, ciF.p, vF.p, Trp.p, Tci.p, Tv.p, L.Prp, L.Pci, L.Pv, &L.nnzP));
+  SA_TRY(run_spgemm(al, n, nc, n, nnzF, nnzT, rpF.p, ciF.p, vF.p, Trp.p, Tci.p, Tv.p, L.Prp, L.Pci, L.Pv,
+                    &L.nnzP));
   SA_TRY(launch_smooth_p_values(s, n, L.Prp.p, L.Pci.p, L.Pv.p, L.agg.p, Dt.p, scal.p + 1, L.Pv.p));
   PHASE_END(PK_S_SMOOTHP);
-  double hs[2];
-  SA_TRY(copy_d2h(hs, scal.p, sizeof(hs), s));
-  L.lam_omega = hs[0];
-  L.omega = hs[1];
+  L.scal = std::move(scal);  // lambda and omega, read with the Chebyshev bounds
 
   // a13: R = P^T, A_{l+1} = R (A P), exactly symmetric
   PHASE_BEGIN(PK_S_TRANSPOSE, l);
-  SA_TRY(run_transpose(al, n, nc, L.Prp.p, L.Pci.p, L.Pv.p, L.Rrp, L.Rci, &L.Rv));
+  SA_TRY(run_transpose(al, n, nc, L.nnzP, L.Prp.p, L.Pci.p, L.Pv.p, L.Rrp, L.Rci, &L.Rv));
   PHASE_END(PK_S_TRANSPOSE);
   PHASE_BEGIN(PK_S_RAP, l);
   Buf<int64_t> APrp;
@@ -221,14 +219,15 @@ static int coarsen(sa_handle h, int l, int* err, int* stop) {
   Buf<double> APv;
   int64_t nnzAP = 0;
   PHASE_BEGIN(PK_S_RAP_AP, l);
-  SA_TRY(run_spgemm(al, n, nc, n, L.rp.p, L.ci.p, L.v.p, L.Prp.p, L.Pci.p, L.Pv.p, APrp, APci, APv, &nnzAP));
+  SA_TRY(run_spgemm(al, n, nc, n, nnz, L.nnzP, L.rp.p, L.ci.p, L.v.p, L.Prp.p, L.Pci.p, L.Pv.p, APrp, APci, APv,
+                    &nnzAP));
   PHASE_END(PK_S_RAP_AP);
   std::unique_ptr<Level> N(new Level());
   N->n = nc;
   // R (A P) is symmetric: only its upper triangle is accumulated, the lower
   // one is mirrored from it
   PHASE_BEGIN(PK_S_RAP_RAP, l);
-  SA_TRY(run_spgemm(al, nc, nc, n, L.Rrp.p, L.Rci.p, L.Rv.p, APrp.p, APci.p, APv.p, N->rp, N->ci, N->v, &N->nnz,
+  SA_TRY(run_spgemm(al, nc, nc, n, L.nnzP, nnzAP, L.Rrp.p, L.Rci.p, L.Rv.p, APrp.p, APci.p, APv.p, N->rp, N->ci, N->v, &N->nnz,
                     1));
   SA_TRY(launch_symmetrize(s, nc, N->rp.p, N->ci.p, N->v.p, err));
   PHASE_END(PK_S_RAP_RAP);
@@ -240,7 +239,7 @@ static int coarsen(sa_handle h, int l, int* err, int* stop) {
     PHASE_BEGIN(PK_S_AUX, l);
     Buf<int64_t> Mrp;
     Buf<int32_t> Mci;
-    SA_TRY(run_transpose(al, n, nc, Trp.p, Tci.p, nullptr, Mrp, Mci, nullptr));
+    SA_TRY(run_transpose(al, n, nc, nnzT, Trp.p, Tci.p, nullptr, Mrp, Mci, nullptr));
     const int kp = h->dim == 3 ? 6 : 3;
     SA_TRY(N->x.alloc(&al, nc * h->dim));
     SA_TRY(N->sigma.alloc(&al, nc * kp));
@@ -868,19 +867,31 @@ static int setup_impl(const sa_problem* P, const sa_options* o, sa_handle h) {
     SA_TRY(vh_build<double>(al, in.data(), nlev, o->cheb_degree, coarse_view(h->cf, h->nL), &h->v64));
   }
   PHASE_END(PK_S_SELL);
-  for (int l = 0; l + 1 < nlev; ++l) {
-    PHASE_BEGIN(PK_S_CHEB, l);
-    Level& L = *h->lev[l];
+  {
+    // every level's estimate, then one wait for them all (and for the
+    // prolongators' damping)
     Buf<double> lam;
-    SA_TRY(lam.alloc(&al, 1));
-    SA_TRY(vh_power(al, h->v64, l, o->power_iters, (uint32_t)(2 * l + 2), o->seed, lam.p));
-    double hl = 0;
-    SA_TRY(copy_d2h(&hl, lam.p, sizeof(double), s));
-    L.lmax = o->cheb_boost * hl;
-    L.lmin = L.lmax / o->cheb_ratio;
-    h->v64->lev[l]->lmax = L.lmax;
-    h->v64->lev[l]->lmin = L.lmin;
-    PHASE_END(PK_S_CHEB);
+    SA_TRY(lam.alloc(&al, nlev));
+    std::vector<double> hl(nlev), hs(2 * nlev);
+    std::vector<ReadBack> rb;
+    for (int l = 0; l + 1 < nlev; ++l) {
+      PHASE_BEGIN(PK_S_CHEB, l);
+      SA_TRY(vh_power(al, h->v64, l, o->power_iters, (uint32_t)(2 * l + 2), o->seed, lam.p + l));
+      PHASE_END(PK_S_CHEB);
+      rb.push_back({&hl[l], lam.p + l, sizeof(double)});
+      rb.push_back({&hs[2 * l], h->lev[l]->scal.p, 2 * sizeof(double)});
+    }
+    SA_TRY(read_back(rb.data(), (int)rb.size(), s));
+    for (int l = 0; l + 1 < nlev; ++l) {
+      Level& L = *h->lev[l];
+      L.lmax = o->cheb_boost * hl[l];
+      L.lmin = L.lmax / o->cheb_ratio;
+      h->v64->lev[l]->lmax = L.lmax;
+      h->v64->lev[l]->lmin = L.lmin;
+      L.lam_omega = hs[2 * l];
+      L.omega = hs[2 * l + 1];
+      L.scal.release();
+    }
   }
   if (o->precision == SA_PREC_FP32_VCYCLE) SA_TRY(build_mixed(h));
   SA_TRY(dense_finish(dj));

@@ -49,8 +49,8 @@ int launch_tentative(cudaStream_t s, int64_t n, const int32_t* agg, const int64_
 int launch_tentative_count(cudaStream_t s, int64_t n, const int32_t* agg, int64_t* cnt);
 // R = P^T (m x n) with each row of R sorted by source row; Rv may be NULL
 // (pattern only).  Allocates Rrp/Rci/Rv.
-int run_transpose(Alloc& al, int64_t n, int64_t m, const int64_t* rp, const int32_t* ci, const double* v,
-                  Buf<int64_t>& Rrp, Buf<int32_t>& Rci, Buf<double>* Rv);
+int run_transpose(Alloc& al, int64_t n, int64_t m, int64_t nnz, const int64_t* rp, const int32_t* ci,
+                  const double* v, Buf<int64_t>& Rrp, Buf<int32_t>& Rci, Buf<double>* Rv);
 
 // ---- spgemm.cu -------------------------------------------------------------
 // C = A * B (n x k times k x m) by count / fill with per-warp shared hash
@@ -59,7 +59,7 @@ int run_transpose(Alloc& al, int64_t n, int64_t m, const int64_t* rp, const int3
 // warp path leaves entries left of the diagonal at 0 (for a symmetric result
 // whose lower triangle is mirrored from the upper one afterwards).  A is
 // n x kdim, B is kdim x m.
-int run_spgemm(Alloc& al, int64_t n, int64_t m, int64_t kdim, const int64_t* Arp, const int32_t* Aci,
+int run_spgemm(Alloc& al, int64_t n, int64_t m, int64_t kdim, int64_t nnzA, int64_t nnzB, const int64_t* Arp, const int32_t* Aci,
                const double* Av, const int64_t* Brp, const int32_t* Bci, const double* Bv, Buf<int64_t>& Crp,
                Buf<int32_t>& Cci, Buf<double>& Cv, int64_t* nnzC, int upper_only = 0);
 // lower triangle takes the value of the mirrored upper-triangle entry
@@ -69,7 +69,7 @@ int launch_symmetrize(cudaStream_t s, int64_t n, const int64_t* rp, const int32_
 struct PowerScratch;
 // spectral-radius estimate of diag(s) A diag(s) by `steps` power steps from
 // the hash-uniform start (tag, seed); result in *lam_dev (device scalar)
-int run_power(Alloc& al, int64_t n, const int64_t* rp, const int32_t* ci, const double* v, const double* s,
+int run_power(Alloc& al, int64_t n, int64_t nnz, const int64_t* rp, const int32_t* ci, const double* v, const double* s,
               int steps, uint32_t tag, uint32_t seed, double* lam_dev);
 // the same iteration on an operator given by its product: apply(y, w)
 // writes w = M y (the V-cycle's pre-scaled copy of D^-1/2 A D^-1/2)

@@ -91,11 +91,57 @@ int num_sms() {
   return sms;
 }
 
-int copy_d2h(void* dst, const void* src, size_t bytes, cudaStream_t s) {
-  if (!bytes) return SA_OK;
-  SA_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s));
+// Readbacks of sizes and flags land in a small pinned buffer of the calling
+// thread (4 KB, released with the thread): a copy to pageable memory goes
+// through the driver's staging, and a setup makes a few hundred.
+namespace {
+constexpr size_t PIN_BYTES = 4096;
+struct ThreadPin {
+  void* p = nullptr;
+  bool tried = false;
+  ~ThreadPin() {
+    if (p) cudaFreeHost(p);
+  }
+  unsigned char* get() {
+    if (!tried) {
+      tried = true;
+      if (cudaMallocHost(&p, PIN_BYTES) != cudaSuccess) {
+        cudaGetLastError();
+        p = nullptr;
+      }
+    }
+    return static_cast<unsigned char*>(p);
+  }
+};
+thread_local ThreadPin t_pin;
+}  // namespace
+
+int read_back(const ReadBack* r, int count, cudaStream_t s) {
+  unsigned char* pin = t_pin.get();
+  size_t tot = 0;
+  for (int k = 0; k < count; ++k) tot += (r[k].bytes + 15) & ~size_t(15);
+  if (!tot) return SA_OK;
+  if (tot > PIN_BYTES) pin = nullptr;
+  size_t off = 0;
+  for (int k = 0; k < count; ++k) {
+    if (!r[k].bytes) continue;
+    SA_CUDA(cudaMemcpyAsync(pin ? pin + off : r[k].dst, r[k].src, r[k].bytes, cudaMemcpyDeviceToHost, s));
+    off += (r[k].bytes + 15) & ~size_t(15);
+  }
   SA_CUDA(cudaStreamSynchronize(s));
+  if (pin) {
+    off = 0;
+    for (int k = 0; k < count; ++k) {
+      if (r[k].bytes) memcpy(r[k].dst, pin + off, r[k].bytes);
+      off += (r[k].bytes + 15) & ~size_t(15);
+    }
+  }
   return SA_OK;
+}
+
+int copy_d2h(void* dst, const void* src, size_t bytes, cudaStream_t s) {
+  const ReadBack r = {dst, src, bytes};
+  return read_back(&r, 1, s);
 }
 
 int copy_h2d(void* dst, const void* src, size_t bytes, cudaStream_t s) {

@@ -183,7 +183,7 @@ int launch_dots(cudaStream_t st, int64_t n, const double* a0, const double* b0, 
   return SA_OK;
 }
 
-int run_power(Alloc& al, int64_t n, const int64_t* rp, const int32_t* ci, const double* v, const double* s,
+int run_power(Alloc& al, int64_t n, int64_t nnz, const int64_t* rp, const int32_t* ci, const double* v, const double* s,
               int steps, uint32_t tag, uint32_t seed, double* lam_dev) {
   cudaStream_t st = al.stream;
   if (n <= 0) return SA_OK;
@@ -200,8 +200,6 @@ int run_power(Alloc& al, int64_t n, const int64_t* rp, const int32_t* ci, const 
   fin.tick = reinterpret_cast<unsigned*>(sc.p + 5);
   fin.sc = sc.p;
   fin.lam = lam_dev;
-  int64_t nnz = 0;
-  SA_TRY(copy_d2h(&nnz, rp + n, sizeof(int64_t), st));
   const double avg = (double)nnz / (double)n;
   const int sw = avg <= 40.0 ? 4 : (avg <= 96.0 ? 8 : 16);
   k_start_vector<<<blocks_for(n, 256), 256, 0, st>>>(n, tag, seed, x.p);

@@ -132,12 +132,14 @@ __device__ int warp_build_row(int64_t i, const int64_t* __restrict__ Arp, const 
 }
 
 __global__ void __launch_bounds__(SG_WARPS * 32)
-k_spgemm_count(int64_t n, const int32_t* __restrict__ rows, const int64_t* __restrict__ Arp,
+k_spgemm_count(int64_t n, const unsigned long long* __restrict__ nrows, const int32_t* __restrict__ rows,
+               const int64_t* __restrict__ Arp,
                const int32_t* __restrict__ Aci, const int64_t* __restrict__ Brp, const int32_t* __restrict__ Bci,
                int64_t* __restrict__ cnt, int32_t* __restrict__ big, unsigned long long* __restrict__ nbig) {
   __shared__ int32_t keys_all[SG_WARPS][HB];
   const int w = threadIdx.x >> 5;
   int32_t* keys = keys_all[w];
+  if (nrows) n = (int64_t)*nrows;
   for (int64_t t = global_warp(); t < n; t += warp_stride()) {
     const int64_t i = rows ? rows[t] : t;  // rows: the rows the thread tier could not hold
     int c = warp_build_row(i, Arp, Aci, Brp, Bci, keys);
@@ -155,7 +157,8 @@ k_spgemm_count(int64_t n, const int32_t* __restrict__ rows, const int64_t* __res
 }
 
 __global__ void __launch_bounds__(SG_WARPS * 32)
-k_spgemm_fill(int64_t n, const int32_t* __restrict__ rows, const int64_t* __restrict__ Arp,
+k_spgemm_fill(int64_t n, const unsigned long long* __restrict__ nrows, const int32_t* __restrict__ rows,
+              const int64_t* __restrict__ Arp,
               const int32_t* __restrict__ Aci, const double* __restrict__ Av, const int64_t* __restrict__ Brp,
               const int32_t* __restrict__ Bci, const double* __restrict__ Bv, const int64_t* __restrict__ Crp,
               int32_t* __restrict__ Cci, double* __restrict__ Cv, const uint8_t* __restrict__ isbig, int upper_only,
@@ -174,6 +177,7 @@ k_spgemm_fill(int64_t n, const int32_t* __restrict__ rows, const int64_t* __rest
   int32_t* cols = cols_all[w];
   uint8_t* slot_of = slot_all[w];
   double* acc = acc_all[w];
+  if (nrows) n = (int64_t)*nrows;
   for (int64_t t = global_warp(); t < n; t += warp_stride()) {
     const int64_t i = rows ? rows[t] : t;
     if (isbig && isbig[i]) continue;  // warp-uniform
@@ -533,9 +537,11 @@ k_spgemm_big(int phase, int64_t nbig, const int32_t* __restrict__ big, int64_t m
   }
 }
 
-__global__ void k_mark_big(int64_t nbig, const int32_t* __restrict__ big, uint8_t* __restrict__ isbig) {
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < nbig) isbig[big[t]] = 1;
+__global__ void k_mark_big(const unsigned long long* __restrict__ nbig, const int32_t* __restrict__ big,
+                           uint8_t* __restrict__ isbig) {
+  const int64_t n = (int64_t)*nbig;
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
+    isbig[big[t]] = 1;
 }
 
 // products of each row of A B (an upper bound of its distinct columns)
@@ -577,6 +583,13 @@ __global__ void k_spgemm_compact(int64_t n, const int64_t* __restrict__ ub, cons
   }
 }
 
+// blocks of a warp-tier launch: every row, or (row count on the device) as many
+// as stay resident
+static unsigned warp_tier_grid(int64_t n, bool listed) {
+  const unsigned g = warp_rows_grid(n, SG_WARPS * 32), r = 16u * (unsigned)num_sms();
+  return listed && g > r ? r : g;
+}
+
 static int spgemm_two_phase(Alloc& al, int64_t n, int64_t m, const int64_t* Arp, const int32_t* Aci,
                             const double* Av, const int64_t* Brp, const int32_t* Bci, const double* Bv,
                             Buf<int64_t>& Crp, Buf<int32_t>& Cci, Buf<double>& Cv, int64_t* nnzC, int upper_only,
@@ -590,8 +603,11 @@ static int spgemm_two_phase(Alloc& al, int64_t n, int64_t m, const int64_t* Arp,
   SA_TRY(isbig.alloc(&al, n));
   SA_TRY(memset_d(nbig_d.p, 0, sizeof(unsigned long long), s));
   SA_TRY(memset_d(isbig.p, 0, isbig.bytes(), s));
-  int64_t nwarp = n;             // rows on the warp tier
+  // the rows the thread tier could not hold are counted on the device: the
+  // warp tier's launches read the count instead of the host
   const int32_t* wrows = nullptr;  // NULL: every row
+  const unsigned long long* nwrows = nullptr;
+  const unsigned wgrid = warp_tier_grid(n, thread_tier);
   if (thread_tier) {
     SA_TRY(midl.alloc(&al, n));
     SA_TRY(nmid_d.alloc(&al, 1));
@@ -600,22 +616,15 @@ static int spgemm_two_phase(Alloc& al, int64_t n, int64_t m, const int64_t* Arp,
     SA_TRY(memset_d(ismid.p, 0, ismid.bytes(), s));
     k_spgemm_tcount<<<blocks_for(n, TB), TB, 0, s>>>(n, Arp, Aci, Brp, Bci, Crp.p, midl.p, nmid_d.p);
     SA_LAUNCHED();
-    unsigned long long nmid = 0;
-    SA_TRY(copy_d2h(&nmid, nmid_d.p, sizeof(nmid), s));
-    nwarp = (int64_t)nmid;
     wrows = midl.p;
-    if (nmid > 0) {
-      k_mark_big<<<blocks_for(nwarp, 256), 256, 0, s>>>(nwarp, midl.p, ismid.p);
-      SA_LAUNCHED();
-    }
-  }
-  if (nwarp > 0) {
-    k_spgemm_count<<<warp_rows_grid(nwarp, SG_WARPS * 32), SG_WARPS * 32, 0, s>>>(nwarp, wrows, Arp, Aci, Brp, Bci,
-                                                                                 Crp.p, big.p, nbig_d.p);
+    nwrows = nmid_d.p;
+    k_mark_big<<<(unsigned)num_sms(), 256, 0, s>>>(nmid_d.p, midl.p, ismid.p);
     SA_LAUNCHED();
   }
+  k_spgemm_count<<<wgrid, SG_WARPS * 32, 0, s>>>(n, nwrows, wrows, Arp, Aci, Brp, Bci, Crp.p, big.p, nbig_d.p);
+  SA_LAUNCHED();
   unsigned long long nbig = 0;
-  if (nwarp > 0) SA_TRY(copy_d2h(&nbig, nbig_d.p, sizeof(nbig), s));
+  SA_TRY(copy_d2h(&nbig, nbig_d.p, sizeof(nbig), s));
   Buf<int32_t> stamp;
   Buf<double> dacc;
   unsigned gbig = 0;
@@ -624,7 +633,7 @@ static int spgemm_two_phase(Alloc& al, int64_t n, int64_t m, const int64_t* Arp,
     SA_TRY(stamp.alloc(&al, (int64_t)gbig * m));
     SA_TRY(dacc.alloc(&al, (int64_t)gbig * m));
     SA_TRY(memset_d(stamp.p, 0xff, stamp.bytes(), s));
-    k_mark_big<<<blocks_for((int64_t)nbig, 256), 256, 0, s>>>((int64_t)nbig, big.p, isbig.p);
+    k_mark_big<<<(unsigned)num_sms(), 256, 0, s>>>(nbig_d.p, big.p, isbig.p);
     SA_LAUNCHED();
     k_spgemm_big<<<gbig, BIG_THREADS, 0, s>>>(0, (int64_t)nbig, big.p, m, Arp, Aci, Av, Brp, Bci, Bv, Crp.p,
                                                 nullptr, nullptr, nullptr, stamp.p, dacc.p);
@@ -639,11 +648,9 @@ static int spgemm_two_phase(Alloc& al, int64_t n, int64_t m, const int64_t* Arp,
                                                     upper_only);
     SA_LAUNCHED();
   }
-  if (nwarp > 0) {
-    k_spgemm_fill<<<warp_rows_grid(nwarp, SG_WARPS * 32), SG_WARPS * 32, 0, s>>>(
-        nwarp, wrows, Arp, Aci, Av, Brp, Bci, Bv, Crp.p, Cci.p, Cv.p, isbig.p, upper_only, nullptr, nullptr, nullptr);
-    SA_LAUNCHED();
-  }
+  k_spgemm_fill<<<wgrid, SG_WARPS * 32, 0, s>>>(n, nwrows, wrows, Arp, Aci, Av, Brp, Bci, Bv, Crp.p, Cci.p, Cv.p,
+                                                isbig.p, upper_only, nullptr, nullptr, nullptr);
+  SA_LAUNCHED();
   if (nbig > 0) {
     k_spgemm_big<<<gbig, BIG_THREADS, 0, s>>>(1, (int64_t)nbig, big.p, m, Arp, Aci, Av, Brp, Bci, Bv, nullptr,
                                                 Crp.p, Cci.p, Cv.p, stamp.p, dacc.p);
@@ -671,24 +678,21 @@ static int spgemm_one_pass(Alloc& al, int64_t n, int64_t m, const int64_t* Arp, 
   SA_TRY(defb.alloc(&al, n));
   SA_TRY(nd.alloc(&al, 2));
   SA_TRY(memset_d(nd.p, 0, nd.bytes(), s));
-  int64_t nwarp = n;
   const int32_t* wrows = nullptr;
+  const unsigned long long* nwrows = nullptr;  // counted on the device (as above)
   if (thread_tier) {
     k_spgemm_thash<<<blocks_for(n, TB), TB, 0, s>>>(n, Arp, Aci, Av, Brp, Bci, Bv, ub, uci.p, uv.p, upper_only,
                                                     defw.p, nd.p, Crp.p);
     SA_LAUNCHED();
-    unsigned long long h = 0;
-    SA_TRY(copy_d2h(&h, nd.p, sizeof(h), s));
-    nwarp = (int64_t)h;
     wrows = defw.p;
+    nwrows = nd.p;
   }
   unsigned long long nbig = 0;
-  if (nwarp > 0) {
-    k_spgemm_fill<<<warp_rows_grid(nwarp, SG_WARPS * 32), SG_WARPS * 32, 0, s>>>(
-        nwarp, wrows, Arp, Aci, Av, Brp, Bci, Bv, ub, uci.p, uv.p, nullptr, upper_only, defb.p, nd.p + 1, Crp.p);
-    SA_LAUNCHED();
-    SA_TRY(copy_d2h(&nbig, nd.p + 1, sizeof(nbig), s));
-  }
+  k_spgemm_fill<<<warp_tier_grid(n, thread_tier), SG_WARPS * 32, 0, s>>>(n, nwrows, wrows, Arp, Aci, Av, Brp, Bci, Bv,
+                                                                        ub, uci.p, uv.p, nullptr, upper_only, defb.p,
+                                                                        nd.p + 1, Crp.p);
+  SA_LAUNCHED();
+  SA_TRY(copy_d2h(&nbig, nd.p + 1, sizeof(nbig), s));
   if (nbig > 0) {
     const unsigned gbig = (unsigned)(nbig < 64 ? nbig : 64);
     Buf<int32_t> stamp;
@@ -709,7 +713,7 @@ static int spgemm_one_pass(Alloc& al, int64_t n, int64_t m, const int64_t* Arp, 
   return SA_OK;
 }
 
-int run_spgemm(Alloc& al, int64_t n, int64_t m, int64_t kdim, const int64_t* Arp, const int32_t* Aci,
+int run_spgemm(Alloc& al, int64_t n, int64_t m, int64_t kdim, int64_t nnzA, int64_t nnzB, const int64_t* Arp, const int32_t* Aci,
                const double* Av, const int64_t* Brp, const int32_t* Bci, const double* Bv, Buf<int64_t>& Crp,
                Buf<int32_t>& Cci, Buf<double>& Cv, int64_t* nnzC, int upper_only) {
   cudaStream_t s = al.stream;
@@ -725,9 +729,6 @@ int run_spgemm(Alloc& al, int64_t n, int64_t m, int64_t kdim, const int64_t* Arp
   // an upper bound of the distinct columns (FE products repeat columns
   // about 8 times: 90 products per row give about 11 distinct columns in the
   // aggregation prolongators); wide products go straight to the warp tier
-  int64_t nnzA = 0, nnzB = 0;
-  SA_TRY(copy_d2h(&nnzA, Arp + n, sizeof(int64_t), s));
-  if (kdim > 0) SA_TRY(copy_d2h(&nnzB, Brp + kdim, sizeof(int64_t), s));
   const double per_row = kdim > 0 ? ((double)nnzA / (double)n) * ((double)nnzB / (double)kdim) : 0.0;
   const bool thread_tier = kdim > 0 && per_row <= 256.0;
   // one pass for wide products (48 or more per row expected: the Galerkin
@@ -747,12 +748,14 @@ int run_spgemm(Alloc& al, int64_t n, int64_t m, int64_t kdim, const int64_t* Arp
   SA_TRY(scan_inplace(al, ub.p + 1, n));
   int64_t ubtot = 0;
   SA_TRY(copy_d2h(&ubtot, ub.p + n, sizeof(int64_t), s));
+  // (the query takes 20 us; 16 MB are taken without it)
   size_t fr = 0, tot = 0;
-  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+  const bool little = (double)ubtot * 12.0 <= 16e6;
+  if (!little && cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
     cudaGetLastError();
     fr = 0;
   }
-  if ((double)ubtot * 12.0 <= 0.5 * (double)fr)
+  if (little || (double)ubtot * 12.0 <= 0.5 * (double)fr)
     return spgemm_one_pass(al, n, m, Arp, Aci, Av, Brp, Bci, Bv, ub.p, ubtot, Crp, Cci, Cv, nnzC, upper_only,
                            thread_tier);
   ub.release();

@@ -274,8 +274,8 @@ int build_mat(Alloc& al, int64_t n, int64_t nnz, const int64_t* rp, const int32_
     k_slice_width<<<blocks_for(M.nslices, 256), 256, 0, s>>>(n, rp, sz.p, mx.p);
     SA_LAUNCHED();
     SA_TRY(scan_inplace(al, sz.p + 1, M.nslices));
-    SA_TRY(copy_d2h(&stored, sz.p + M.nslices, sizeof(int64_t), s));
-    SA_TRY(copy_d2h(&max_width, mx.p, sizeof(unsigned int), s));
+    const ReadBack rb[2] = {{&stored, sz.p + M.nslices, sizeof(int64_t)}, {&max_width, mx.p, sizeof(unsigned int)}};
+    SA_TRY(read_back(rb, 2, s));
   }
   // short rows (prolongators): SELL also above 25 % padding when its padding
   // costs fewer bytes than the CSR row pointers it saves (value + 32-bit
