@@ -509,6 +509,7 @@ static int cg_graph(sa_handle h, const double* b, double* x, double tol, sa_solv
   SA_CUDA(cudaMemcpyAsync(h->bb.p, b, sizeof(double) * n, cudaMemcpyDefault, s));
   SA_TRY(copy_in_guess(h, h->xb.p, x, sizeof(double) * n));
   int status = SA_ERR_NO_CONVERGENCE, it = 0;
+  bool confirmed = false;  // hp[3] holds the true residual of the final x
   SA_TRY(op_residual(h, h->bb.p, h->xb.p, h->r.p));
   SA_TRY(norm2(h, h->r.p, h->dots.p));
   SA_CUDA(cudaMemcpyAsync(hp, h->dots.p, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -542,7 +543,7 @@ static int cg_graph(sa_handle h, const double* b, double* x, double tol, sa_solv
         SA_TRY(norm2(h, h->t.p, h->dots.p + 6));
         SA_CUDA(cudaMemcpyAsync(hp + 3, h->dots.p + 6, sizeof(double), cudaMemcpyDeviceToHost, s));
         SA_CUDA(cudaStreamSynchronize(s));
-        if (sqrt(hp[3]) <= tol * r0) { status = SA_OK; break; }
+        if (sqrt(hp[3]) <= tol * r0) { status = SA_OK; confirmed = true; break; }
         SA_CUDA(cudaMemcpyAsync(h->r.p, h->t.p, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
       }
       if (it >= h->opt.maxit) break;
@@ -553,9 +554,11 @@ static int cg_graph(sa_handle h, const double* b, double* x, double tol, sa_solv
   } else {
     status = SA_OK;
   }
-  SA_TRY(op_residual(h, h->bb.p, h->xb.p, h->t.p));
-  SA_TRY(norm2(h, h->t.p, h->dots.p + 6));
-  SA_CUDA(cudaMemcpyAsync(hp + 3, h->dots.p + 6, sizeof(double), cudaMemcpyDeviceToHost, s));
+  if (!confirmed) {
+    SA_TRY(op_residual(h, h->bb.p, h->xb.p, h->t.p));
+    SA_TRY(norm2(h, h->t.p, h->dots.p + 6));
+    SA_CUDA(cudaMemcpyAsync(hp + 3, h->dots.p + 6, sizeof(double), cudaMemcpyDeviceToHost, s));
+  }
   SA_CUDA(cudaMemcpyAsync(x, h->xb.p, sizeof(double) * n, cudaMemcpyDefault, s));
   SA_CUDA(cudaStreamSynchronize(s));
   auto t1 = std::chrono::steady_clock::now();
@@ -644,7 +647,8 @@ static int cg_block(sa_handle h, int k, const double* B, double* X, double tol, 
     SA_TRY(launch_interleave(s, n, k, K, h->kStage.p, Xb, 1));
   }
   // host view of the columns
-  double r0[KMAX_BLOCK], hb[2 * KMAX_BLOCK];
+  double r0[KMAX_BLOCK], hb[2 * KMAX_BLOCK], tr[KMAX_BLOCK] = {};
+  bool known[KMAX_BLOCK] = {};  // tr holds the true residual of the column's final x (its columns are frozen)
   int act[KMAX_BLOCK], its[KMAX_BLOCK], st[KMAX_BLOCK];
   struct { double rr[KMAX_BLOCK]; CgScalars S[KMAX_BLOCK]; } hr;
   SA_TRY(launch_bsell_residual64(s, h->A0s, K, Bb, Xb, R));
@@ -694,6 +698,8 @@ static int cg_block(sa_handle h, int k, const double* B, double* X, double tol, 
           if (sqrt(hb[c]) <= tol * r0[c]) {
             st[c] = SA_OK;
             act[c] = 0;
+            tr[c] = hb[c];
+            known[c] = true;
           } else {
             SA_CUDA(cudaMemcpy2DAsync(R + c, sizeof(double) * K, T + c, sizeof(double) * K, sizeof(double), n,
                                       cudaMemcpyDeviceToDevice, s));
@@ -715,9 +721,13 @@ static int cg_block(sa_handle h, int k, const double* B, double* X, double tol, 
     }
   }
   // true residuals at exit and the solutions
-  SA_TRY(launch_bsell_residual64(s, h->A0s, K, Bb, Xb, T));
-  SA_TRY(launch_bdots(s, n, K, T, T, nullptr, nullptr, part, fin_block(h, K, FIN_STORE, dots + 3 * KMAX_BLOCK)));
-  SA_CUDA(cudaMemcpyAsync(hb, dots + 3 * KMAX_BLOCK, sizeof(double) * K, cudaMemcpyDeviceToHost, s));
+  bool all_known = true;
+  for (int c = 0; c < k; ++c) all_known = all_known && (known[c] || !(r0[c] > 0.0));
+  if (!all_known) {
+    SA_TRY(launch_bsell_residual64(s, h->A0s, K, Bb, Xb, T));
+    SA_TRY(launch_bdots(s, n, K, T, T, nullptr, nullptr, part, fin_block(h, K, FIN_STORE, dots + 3 * KMAX_BLOCK)));
+    SA_CUDA(cudaMemcpyAsync(hb, dots + 3 * KMAX_BLOCK, sizeof(double) * K, cudaMemcpyDeviceToHost, s));
+  }
   SA_TRY(launch_interleave(s, n, k, K, Xb, h->kStage.p, 0));
   SA_CUDA(cudaMemcpyAsync(X, h->kStage.p, sizeof(double) * n * k, cudaMemcpyDefault, s));
   SA_CUDA(cudaStreamSynchronize(s));
@@ -727,7 +737,7 @@ static int cg_block(sa_handle h, int k, const double* B, double* X, double tol, 
     statuses[c] = st[c];
     if (infos) {
       infos[c].iters = its[c];
-      infos[c].rel_res_true = r0[c] > 0.0 ? sqrt(hb[c]) / r0[c] : 0.0;
+      infos[c].rel_res_true = r0[c] > 0.0 ? sqrt(all_known ? tr[c] : hb[c]) / r0[c] : 0.0;
       infos[c].setup_ms = h->setup_ms;
       infos[c].solve_ms = ms;
       infos[c].status = st[c];
