@@ -32,20 +32,20 @@ constexpr int CH_STRIP = 16;             // columns of one inverse task
 constexpr int CH_BT = (int)(COARSE_BS / NB);  // tiles per diagonal block
 constexpr uint32_t CH_INV = 0x80000000u;      // task word of an inverse strip
 
-// f[i]: first nonzero tile column of tile row i (columns ascend, the first
-// entry of a row is its smallest column; at most the diagonal tile)
+// f[i]: first nonzero tile column of tile row i (at most the diagonal tile):
+// a warp over the tile row's entries, whatever their order
 __global__ void k_sky_first(int64_t n, int nb, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
                             int32_t* __restrict__ f) {
   const int i = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
   if (i >= nb) return;
-  const int64_t r = (int64_t)i * NB + (threadIdx.x & 31);
+  const int64_t o = (int64_t)i * NB, r1 = o + NB < n ? o + NB : n;
   int c = i;
-  if (r < n && rp[r + 1] > rp[r]) {
-    const int t = ci[rp[r]] / NB;
-    c = t < i ? t : i;
+  for (int64_t p = rp[o] + lane_id(); p < rp[r1]; p += 32) {
+    const int t = ci[p] / NB;
+    c = t < c ? t : c;
   }
   c = __reduce_min_sync(FULL, c);
-  if ((threadIdx.x & 31) == 0) f[i] = c;
+  if (lane_id() == 0) f[i] = c;
 }
 
 // the skyline of tile row blockIdx.x as dense rows: zeros, then the entries of
