@@ -688,15 +688,28 @@ __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_cheb_out(MatView<T>
 
 // elementwise forms over the n*K elements
 // (the first step's iterate x_1 equals its direction d_1: only d is written)
-template <typename T>
-__global__ void k_bvc_fine_in(int64_t n, int K, const double* __restrict__ r, const double* __restrict__ s, T c2,
+// fine_in: half a row of eight, or a row, per thread as one vector, its row by a
+// shift.  Bound by memory (160^3 rows, eight columns, FP32 form: a scalar and a
+// 64-bit division per thread 146 us, this 127 us, two or four vectors a thread
+// 129 and 130 us).
+template <typename T, int K>
+__global__ void k_bvc_fine_in(int64_t n, const double* __restrict__ r, const double* __restrict__ s, T c2,
                               T* __restrict__ b, T* __restrict__ d) {
   pdl_sync();
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  constexpr int G = K >= 4 ? 4 : 2;
+  const int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * G;
   if (e < n * K) {
-    const T bi = (T)(s[e / K] * r[e]);
-    b[e] = bi;
-    d[e] = c2 * bi;
+    double rv[G];
+    T bv[G], dv[G];
+    ld_row<double, G>(r + e, rv);
+    const double si = s[e / K];
+#pragma unroll
+    for (int h = 0; h < G; ++h) {
+      bv[h] = (T)(si * rv[h]);
+      dv[h] = c2 * bv[h];
+    }
+    st_row<T, G>(b + e, bv);
+    st_row<T, G>(d + e, dv);
   }
 }
 
@@ -828,8 +841,12 @@ static int mv_block(VHier<T>* m, cudaStream_t st, int l, int K, const double* r6
   // the first step writes b and d_1 = x_1 into kd; the next step reads both
   // from there and writes d into kx2 and x into kx (then in place / ping-pong)
   if (l == 0) {
+    const T c2 = (T)(1.0 / th);
     BPROF(K_FST, l, 8.0 * K * n + 8.0 * n + 2.0 * S * K * n,
-          (launch_pdl(k_bvc_fine_in<T>, g256(nk), 256, 0, st, n, K, r64, m->s0.p, (T)(1.0 / th), L->kb.p, L->kd.p)));
+          (K == 2   ? launch_pdl(k_bvc_fine_in<T, 2>, g256(n), 256, 0, st, n, r64, m->s0.p, c2, L->kb.p, L->kd.p)
+           : K == 4 ? launch_pdl(k_bvc_fine_in<T, 4>, g256(n), 256, 0, st, n, r64, m->s0.p, c2, L->kb.p, L->kd.p)
+                    : launch_pdl(k_bvc_fine_in<T, 8>, g256(2 * n), 256, 0, st, n, r64, m->s0.p, c2, L->kb.p,
+                                 L->kd.p)));
   } else {
     BPROF(K_FST, l, 2.0 * S * K * n, (launch_pdl(k_bvc_first<T>, g256(nk), 256, 0, st, nk, L->kb.p, (T)(1.0 / th), L->kd.p)));
   }

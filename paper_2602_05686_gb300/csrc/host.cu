@@ -652,7 +652,7 @@ static int cg_block(sa_handle h, int k, const double* B, double* X, double tol, 
   int act[KMAX_BLOCK], its[KMAX_BLOCK], st[KMAX_BLOCK];
   struct { double rr[KMAX_BLOCK]; CgScalars S[KMAX_BLOCK]; } hr;
   SA_TRY(launch_bsell_residual64(s, h->A0s, K, Bb, Xb, R));
-  PROF(PK_B_CG_VEC, 0, 2 * vb, launch_bdots(s, n, K, R, R, nullptr, nullptr, part, fin_block(h, K, FIN_STORE, dots)));
+  PROF(PK_B_CG_VEC, 0, 2 * vb, launch_bdots(s, n, K, R, R, nullptr, part, fin_block(h, K, FIN_STORE, dots)));
   SA_CUDA(cudaMemcpyAsync(hb, dots, sizeof(double) * K, cudaMemcpyDeviceToHost, s));
   SA_CUDA(cudaStreamSynchronize(s));
   int nact = 0;
@@ -670,7 +670,7 @@ static int cg_block(sa_handle h, int k, const double* B, double* X, double tol, 
     SA_TRY(precondition_block(h, K, R, &Z));
     PROF(PK_B_CG_VEC, 0, 2 * vb, launch_bcg_pupdate(s, n, K, h->kS.p, h->kact.p, Z, P, 1));
     PROF(PK_B_CG_VEC, 0, 2 * vb,
-         launch_bdots(s, n, K, R, Z, nullptr, nullptr, part, fin_block(h, K, FIN_BETA, dots, -1)));
+         launch_bdots(s, n, K, R, Z, nullptr, part, fin_block(h, K, FIN_BETA, dots, -1)));
     for (int it = 1;; ++it) {
       SA_TRY(launch_bsell_spmv_dot(s, h->A0s, K, P, Q, part, fin_block(h, K, FIN_ALPHA, dots)));
       PROF(PK_B_CG_VEC, 0, (flexible ? 7 : 6) * vb,
@@ -690,7 +690,7 @@ static int cg_block(sa_handle h, int k, const double* B, double* X, double tol, 
       }
       if (cand) {
         SA_TRY(launch_bsell_residual64(s, h->A0s, K, Bb, Xb, T));
-        SA_TRY(launch_bdots(s, n, K, T, T, nullptr, nullptr, part, fin_block(h, K, FIN_STORE, dots + 3 * KMAX_BLOCK)));
+        SA_TRY(launch_bdots(s, n, K, T, T, nullptr, part, fin_block(h, K, FIN_STORE, dots + 3 * KMAX_BLOCK)));
         SA_CUDA(cudaMemcpyAsync(hb, dots + 3 * KMAX_BLOCK, sizeof(double) * K, cudaMemcpyDeviceToHost, s));
         SA_CUDA(cudaStreamSynchronize(s));
         for (int c = 0; c < K; ++c) {
@@ -715,7 +715,7 @@ static int cg_block(sa_handle h, int k, const double* B, double* X, double tol, 
       if (nact == 0) break;
       SA_TRY(precondition_block(h, K, R, &Z));
       PROF(PK_B_CG_VEC, 0, (flexible ? 3 : 2) * vb,
-           launch_bdots(s, n, K, R, Z, flexible ? Z : nullptr, flexible ? Rp : nullptr, part,
+           launch_bdots(s, n, K, R, Z, flexible ? Rp : nullptr, part,
                         fin_block(h, K, FIN_BETA, dots, flexible)));
       PROF(PK_B_CG_VEC, 0, 3 * vb, launch_bcg_pupdate(s, n, K, h->kS.p, h->kact.p, Z, P, 0));
     }
@@ -725,7 +725,7 @@ static int cg_block(sa_handle h, int k, const double* B, double* X, double tol, 
   for (int c = 0; c < k; ++c) all_known = all_known && (known[c] || !(r0[c] > 0.0));
   if (!all_known) {
     SA_TRY(launch_bsell_residual64(s, h->A0s, K, Bb, Xb, T));
-    SA_TRY(launch_bdots(s, n, K, T, T, nullptr, nullptr, part, fin_block(h, K, FIN_STORE, dots + 3 * KMAX_BLOCK)));
+    SA_TRY(launch_bdots(s, n, K, T, T, nullptr, part, fin_block(h, K, FIN_STORE, dots + 3 * KMAX_BLOCK)));
     SA_CUDA(cudaMemcpyAsync(hb, dots + 3 * KMAX_BLOCK, sizeof(double) * K, cudaMemcpyDeviceToHost, s));
   }
   SA_TRY(launch_interleave(s, n, k, K, Xb, h->kStage.p, 0));

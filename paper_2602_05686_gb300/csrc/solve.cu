@@ -363,13 +363,55 @@ int launch_cg_pupdate(cudaStream_t st, int64_t n, const CgScalars* s, const doub
 // ---------------------------------------------------------------------------
 constexpr int KB = KMAX_BLOCK;
 
-// Rows of an interleaved n x KK block move as whole vectors, in groups of
-// G = 4 columns (one 256-bit access; rows on 32-byte boundaries) or G = 2
-// (KK = 2: one 128-bit access).  Element-wise pieces at the row stride leave
-// every warp store writing partial sectors.  The kernels keep the one-vector
-// kernels' grid, per-thread stride and reduction trees (each column's
-// arithmetic is theirs) and fit two 512-thread blocks per SM (64 registers):
-// the per-column scalars are read from shared memory, not held.
+// Rows of an interleaved n x KK block move as vectors of G = 4 columns (one
+// 256-bit access; rows on 32-byte boundaries) or G = 2 (KK = 2).  A row of
+// eight columns takes two lanes: a warp's access is then 1 KB of whole lines
+// (a lane that took both halves of its row left every access a line of half
+// used sectors, and its second half's loads behind the first half's store).
+// The kernels keep the one-vector kernels' grid, per-thread stride and
+// reduction trees: a warp holds the 32 rows of the one-vector kernel's 32
+// threads, slot u of lane l row l / LPR + u * (32 / LPR), so that the first
+// stage of the butterfly (rows 16 apart) is an addition in the lane and the
+// others are shuffles.  Bound by memory; the three kernels of an iteration
+// average 194 us (before: 236 us) on 160^3 rows, eight columns, FP32 form, 89 us
+// (97 us) on 128^3 rows, FP64 form.  Two 512-thread blocks per SM (64 registers).
+template <int KK>
+struct BRow {
+  static constexpr int G = KK >= 4 ? 4 : 2;
+  static constexpr int LPR = KK / G;      // lanes per row
+  static constexpr int RPL = 32 / LPR;    // rows of one access
+};
+
+// sums of D values per column (val[d][u][h]: slot u, column h of the lane's
+// group) into out[(d * KB + c) * stride + block]; columns KK .. KB - 1 get 0
+template <int KK, int D>
+__device__ __forceinline__ void bblock_sum_to(double (&val)[D][BRow<KK>::LPR][BRow<KK>::G], double* __restrict__ out,
+                                              int stride) {
+  using B = BRow<KK>;
+  __shared__ double sh[D * KMAX_BLOCK][RED_THREADS / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int d = 0; d < D; ++d)
+#pragma unroll
+    for (int h = 0; h < B::G; ++h) {
+      double t = val[d][0][h];
+      if constexpr (B::LPR == 2) t += val[d][1][h];
+#pragma unroll
+      for (int o = 16; o >= B::LPR; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
+      if (lane < B::LPR) sh[d * KMAX_BLOCK + lane * B::G + h][w] = t;
+    }
+  if constexpr (KK < KMAX_BLOCK) {
+#pragma unroll
+    for (int d = 0; d < D; ++d)
+      if (lane >= KK && lane < KMAX_BLOCK) sh[d * KMAX_BLOCK + lane][w] = 0.0;
+  }
+  __syncthreads();
+  for (int k = w; k < D * KMAX_BLOCK; k += RED_THREADS / 32) {
+    const double t = warp_sum(lane < RED_THREADS / 32 ? sh[k][lane] : 0.0);
+    if (lane == 0) out[(int64_t)k * stride + blockIdx.x] = t;
+  }
+}
+
 template <int G>
 __device__ __forceinline__ void ldgrp(const double* p, double (&v)[G]) {
   if constexpr (G == 4) {
@@ -389,36 +431,55 @@ __device__ __forceinline__ void stgrp(double* p, const double (&v)[G]) {
   }
 }
 
-// NV = KB: one dot per column (a1 unused); NV = 2 KB: two (a0.b0, a1.b1)
-template <int KK, int NV>
-__global__ void __launch_bounds__(RED_THREADS, 2) k_bdots(int64_t n, const double* __restrict__ a0,
-                                                          const double* __restrict__ b0, const double* __restrict__ a1,
-                                                          const double* __restrict__ b1, double* __restrict__ part,
-                                                          Fin fin) {
+// D = 1: a . b per column; D = 2: and b . c
+template <int KK, int D>
+__global__ void __launch_bounds__(RED_THREADS, 2) k_bdots(int64_t n, const double* __restrict__ a,
+                                                          const double* __restrict__ b, const double* __restrict__ c,
+                                                          double* __restrict__ part, Fin fin) {
   pdl_sync();
-  constexpr int G = KK >= 4 ? 4 : 2;
-  double acc[NV];
+  using B = BRow<KK>;
+  constexpr int G = B::G, L = B::LPR;
+  const int lane = threadIdx.x & 31;
+  double acc[D][L][G];
 #pragma unroll
-  for (int c = 0; c < NV; ++c) acc[c] = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t o = i * KK;
+  for (int d = 0; d < D; ++d)
 #pragma unroll
-    for (int g = 0; g < KK; g += G) {
-      double a[G], b[G];
-      ldgrp<G>(a0 + o + g, a);
-      ldgrp<G>(b0 + o + g, b);
+    for (int u = 0; u < L; ++u)
 #pragma unroll
-      for (int h = 0; h < G; ++h) acc[g + h] = fma(a[h], b[h], acc[g + h]);
-      if constexpr (NV == 2 * KB) {
-        ldgrp<G>(a1 + o + g, a);
-        ldgrp<G>(b1 + o + g, b);
+      for (int h = 0; h < G; ++h) acc[d][u][h] = 0.0;
+  for (int64_t i0 = (int64_t)blockIdx.x * RED_THREADS + (threadIdx.x & ~31u); i0 < n;
+       i0 += (int64_t)gridDim.x * RED_THREADS) {
+    const int64_t i = i0 + lane / L;
+    const int64_t o = i * KK + lane % L * G;
+    if (D == 1 && i + (L - 1) * B::RPL < n) {  // all slots' loads together
+      double av[L][G], bv[L][G];
 #pragma unroll
-        for (int h = 0; h < G; ++h) acc[KB + g + h] = fma(a[h], b[h], acc[KB + g + h]);
+      for (int u = 0; u < L; ++u) {
+        ldgrp<G>(a + o + u * B::RPL * KK, av[u]);
+        ldgrp<G>(b + o + u * B::RPL * KK, bv[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < L; ++u)
+#pragma unroll
+        for (int h = 0; h < G; ++h) acc[0][u][h] = fma(av[u][h], bv[u][h], acc[0][u][h]);
+    } else {
+#pragma unroll
+      for (int u = 0; u < L; ++u) {
+        if (i + u * B::RPL >= n) continue;
+        double av[G], bv[G], cv[G];
+        ldgrp<G>(a + o + u * B::RPL * KK, av);
+        ldgrp<G>(b + o + u * B::RPL * KK, bv);
+        if constexpr (D == 2) ldgrp<G>(c + o + u * B::RPL * KK, cv);
+#pragma unroll
+        for (int h = 0; h < G; ++h) {
+          acc[0][u][h] = fma(av[h], bv[h], acc[0][u][h]);
+          if constexpr (D == 2) acc[1][u][h] = fma(bv[h], cv[h], acc[1][u][h]);
+        }
       }
     }
   }
-  block_sum_to<NV>(acc, part, RED_BLOCKS);
-  fin_inline<NV, RED_THREADS>(fin, part, (int)gridDim.x, RED_BLOCKS, KB);
+  bblock_sum_to<KK, D>(acc, part, RED_BLOCKS);
+  fin_inline<D * KB, RED_THREADS>(fin, part, (int)gridDim.x, RED_BLOCKS, KB);
 }
 
 template <int KK>
@@ -427,7 +488,8 @@ __global__ void __launch_bounds__(RED_THREADS, 2)
                  const double* __restrict__ p, const double* __restrict__ q, double* __restrict__ x,
                  double* __restrict__ r, double* __restrict__ rprev, double* __restrict__ part, Fin fin) {
   pdl_sync();
-  constexpr int G = KK >= 4 ? 4 : 2;
+  using B = BRow<KK>;
+  constexpr int G = B::G, L = B::LPR;
   __shared__ double alpha[KB];
   __shared__ int on[KB];
   if (threadIdx.x < KB) {
@@ -439,38 +501,43 @@ __global__ void __launch_bounds__(RED_THREADS, 2)
   bool any = false;
 #pragma unroll
   for (int c = 0; c < KK; ++c) any |= on[c] != 0;
-  double acc[KB];
+  const int lane = threadIdx.x & 31, g = lane % L * G;
+  double acc[1][L][G];
 #pragma unroll
-  for (int c = 0; c < KB; ++c) acc[c] = 0.0;
+  for (int u = 0; u < L; ++u)
+#pragma unroll
+    for (int h = 0; h < G; ++h) acc[0][u][h] = 0.0;
   // each column updated and summed exactly as in the one-vector kernel; a
   // frozen column's values are written back unchanged
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t o = i * KK;
+  for (int64_t i0 = (int64_t)blockIdx.x * RED_THREADS + (threadIdx.x & ~31u); i0 < n;
+       i0 += (int64_t)gridDim.x * RED_THREADS) {
 #pragma unroll
-    for (int g = 0; g < KK; g += G) {
-      // r with q, then x with p: two groups live at a time
+    for (int u = 0; u < L; ++u) {
+      const int64_t i = i0 + lane / L + u * B::RPL;
+      if (i >= n) continue;
+      const int64_t o = i * KK + g;
       double rv[G];
-      ldgrp<G>(r + o + g, rv);
+      ldgrp<G>(r + o, rv);
       if (any) {
-        double u[G], v[G];
-        if (rprev) stgrp<G>(rprev + o + g, rv);
-        ldgrp<G>(q + o + g, u);
+        double qv[G], xv[G], pv[G];
+        ldgrp<G>(q + o, qv);
+        ldgrp<G>(x + o, xv);
+        ldgrp<G>(p + o, pv);
+        if (rprev) stgrp<G>(rprev + o, rv);
 #pragma unroll
         for (int h = 0; h < G; ++h)
-          if (on[g + h]) rv[h] = fma(-alpha[g + h], u[h], rv[h]);
-        stgrp<G>(r + o + g, rv);
-        ldgrp<G>(x + o + g, u);
-        ldgrp<G>(p + o + g, v);
+          if (on[g + h]) rv[h] = fma(-alpha[g + h], qv[h], rv[h]);
+        stgrp<G>(r + o, rv);
 #pragma unroll
         for (int h = 0; h < G; ++h)
-          if (on[g + h]) u[h] = fma(alpha[g + h], v[h], u[h]);
-        stgrp<G>(x + o + g, u);
+          if (on[g + h]) xv[h] = fma(alpha[g + h], pv[h], xv[h]);
+        stgrp<G>(x + o, xv);
       }
 #pragma unroll
-      for (int h = 0; h < G; ++h) acc[g + h] = fma(rv[h], rv[h], acc[g + h]);
+      for (int h = 0; h < G; ++h) acc[0][u][h] = fma(rv[h], rv[h], acc[0][u][h]);
     }
   }
-  block_sum_to<KB>(acc, part, RED_BLOCKS);
+  bblock_sum_to<KK, 1>(acc, part, RED_BLOCKS);
   fin_inline<KB, RED_THREADS>(fin, part, (int)gridDim.x, RED_BLOCKS, 0);
 }
 
@@ -479,7 +546,8 @@ __global__ void __launch_bounds__(RED_THREADS, 2)
     k_bcg_pupdate(int64_t n, const CgScalars* __restrict__ s, const int* __restrict__ active,
                   const double* __restrict__ z, double* __restrict__ p, int first) {
   pdl_sync();
-  constexpr int G = KK >= 4 ? 4 : 2;
+  using B = BRow<KK>;
+  constexpr int G = B::G, L = B::LPR;
   __shared__ double beta[KB];
   __shared__ int on[KB];
   if (threadIdx.x < KB) {
@@ -492,17 +560,27 @@ __global__ void __launch_bounds__(RED_THREADS, 2)
 #pragma unroll
   for (int c = 0; c < KK; ++c) any |= on[c] != 0;
   if (!any) return;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t o = i * KK;
+  const int lane = threadIdx.x & 31, g = lane % L * G;
+  for (int64_t i0 = (int64_t)blockIdx.x * RED_THREADS + (threadIdx.x & ~31u); i0 < n;
+       i0 += (int64_t)gridDim.x * RED_THREADS) {
+    const int64_t i = i0 + lane / L;
+    const int64_t o = i * KK + g;
+    double zv[L][G], pv[L][G];
 #pragma unroll
-    for (int g = 0; g < KK; g += G) {
-      double zv[G], pv[G];
-      ldgrp<G>(z + o + g, zv);
-      ldgrp<G>(p + o + g, pv);
+    for (int u = 0; u < L; ++u) {
+      if (i + u * B::RPL < n) {
+        ldgrp<G>(z + o + u * B::RPL * KK, zv[u]);
+        ldgrp<G>(p + o + u * B::RPL * KK, pv[u]);
+      }
+    }
 #pragma unroll
-      for (int h = 0; h < G; ++h)
-        if (on[g + h]) pv[h] = first ? zv[h] : fma(beta[g + h], pv[h], zv[h]);
-      stgrp<G>(p + o + g, pv);
+    for (int u = 0; u < L; ++u) {
+      if (i + u * B::RPL < n) {
+#pragma unroll
+        for (int h = 0; h < G; ++h)
+          if (on[g + h]) pv[u][h] = first ? zv[u][h] : fma(beta[g + h], pv[u][h], zv[u][h]);
+        stgrp<G>(p + o + u * B::RPL * KK, pv[u]);
+      }
     }
   }
 }
@@ -518,19 +596,19 @@ __global__ void k_interleave(int64_t n, int k, int K, const double* __restrict__
   else if (c < k) dst[(int64_t)c * n + i] = src[e];
 }
 
-int launch_bdots(cudaStream_t st, int64_t n, int k, const double* a0, const double* b0, const double* a1,
-                 const double* b1, double* part, const Fin& fin) {
+int launch_bdots(cudaStream_t st, int64_t n, int k, const double* a, const double* b, const double* c, double* part,
+                 const Fin& fin) {
   if (k != 2 && k != 4 && k != 8) return SA_ERR_INVALID_ARG;  // whole-row vectors
   const unsigned g = red_blocks(n);
-  // one dot per column, or two (a1 . b1 into out[KB + c])
-  if (a1) {
-    if (k == 2) launch_pdl(k_bdots<2, 2 * KB>, g, RED_THREADS, 0, st, n, a0, b0, a1, b1, part, fin);
-    else if (k == 4) launch_pdl(k_bdots<4, 2 * KB>, g, RED_THREADS, 0, st, n, a0, b0, a1, b1, part, fin);
-    else launch_pdl(k_bdots<8, 2 * KB>, g, RED_THREADS, 0, st, n, a0, b0, a1, b1, part, fin);
+  // one dot per column (a . b), or two (b . c into out[KB + column])
+  if (c) {
+    if (k == 2) launch_pdl(k_bdots<2, 2>, g, RED_THREADS, 0, st, n, a, b, c, part, fin);
+    else if (k == 4) launch_pdl(k_bdots<4, 2>, g, RED_THREADS, 0, st, n, a, b, c, part, fin);
+    else launch_pdl(k_bdots<8, 2>, g, RED_THREADS, 0, st, n, a, b, c, part, fin);
   } else {
-    if (k == 2) launch_pdl(k_bdots<2, KB>, g, RED_THREADS, 0, st, n, a0, b0, a1, b1, part, fin);
-    else if (k == 4) launch_pdl(k_bdots<4, KB>, g, RED_THREADS, 0, st, n, a0, b0, a1, b1, part, fin);
-    else launch_pdl(k_bdots<8, KB>, g, RED_THREADS, 0, st, n, a0, b0, a1, b1, part, fin);
+    if (k == 2) launch_pdl(k_bdots<2, 1>, g, RED_THREADS, 0, st, n, a, b, c, part, fin);
+    else if (k == 4) launch_pdl(k_bdots<4, 1>, g, RED_THREADS, 0, st, n, a, b, c, part, fin);
+    else launch_pdl(k_bdots<8, 1>, g, RED_THREADS, 0, st, n, a, b, c, part, fin);
   }
   SA_LAUNCHED();
   return SA_OK;

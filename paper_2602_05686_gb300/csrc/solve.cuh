@@ -36,8 +36,9 @@ int launch_cg_pupdate(cudaStream_t st, int64_t n, const CgScalars* s, const doub
 
 // k-column versions (k <= KMAX_BLOCK), each column summed in the one-vector
 // order so that a column of a block solve equals the one-vector solve bitwise
-int launch_bdots(cudaStream_t st, int64_t n, int k, const double* a0, const double* b0, const double* a1,
-                 const double* b1, double* part, const Fin& fin);
+// (bdots: a . b per column, and b . c where c is given)
+int launch_bdots(cudaStream_t st, int64_t n, int k, const double* a, const double* b, const double* c, double* part,
+                 const Fin& fin);
 int launch_bcg_update(cudaStream_t st, int64_t n, int k, const CgScalars* s, const int* active, const double* p,
                       const double* q, double* x, double* r, double* rprev, double* part, const Fin& fin);
 int launch_bcg_pupdate(cudaStream_t st, int64_t n, int k, const CgScalars* s, const int* active, const double* z,
