@@ -284,8 +284,8 @@ __device__ __forceinline__ void potrf_inv(int bs, double (*T)[NB + 1], double (*
 // tile; tile columns ascending), so the factor is bitwise that form's.
 // Bound by the chain of diagonal tiles (32 us a tile column) on narrow
 // skylines, by FP64 issue (8 us a tile product and SM) on wide ones.  4225-row
-// square 34.4 ms as launches per panel over the whole triangle, 4.6 ms now;
-// 2210-row 3D level (skyline 0.26) 10.7 ms, 2.6 ms.
+// square 34.4 ms as launches per panel over the whole triangle, 4.1 ms now;
+// 2210-row 3D level (skyline 0.26) 10.7 ms, 3.3 ms.
 __global__ void __launch_bounds__(CH_THREADS) k_chol(CholView C) {
   __shared__ double As[2][NB][NB + 1];
   __shared__ double Bs[2][NB][NB + 1];

@@ -393,8 +393,9 @@ __device__ __forceinline__ int keep_entry(double wv, double t2, double Di, doubl
 // A warp takes KEEP_ROWS consecutive rows at a time, their loads together (one
 // row after another was a chain of dependent loads: 458 us), the entries past
 // the 32nd of a row after them.  ABS: the classical measure, |a_ij| and
-// |a_ii a_jj| in place of w and D (192^3 inclusions, FP64 comparisons of one row
-// at a time: 677 us a level on average)
+// |a_ii a_jj| in place of w and D (192^3 inclusions, average of the levels:
+// 677 us by a kernel of its own, 674 us by this one: bound by the entries' bytes
+// and the gathered diagonal, not by the comparison).
 constexpr int KEEP_ROWS = 4;
 template <bool ABS>
 __global__ void __launch_bounds__(256) k_keep(int64_t n, const int64_t* __restrict__ rp,
@@ -619,9 +620,9 @@ __global__ void k_cut_symmetrize(int64_t n, const int64_t* __restrict__ rp, cons
 // Thread per row: the three ordered sums are sequential FP64 chains, so one
 // warp instruction advances 32 rows.  The block's rows are one segment of the
 // CSR arrays, copied to shared memory first: three passes over rows 216 bytes
-// apart cost each warp load 32 lines of a cache that 64 warps shared (1.06M
-// rows of 26 entries 341 us).  A segment above FILT_CAP entries is read in
-// place.
+// apart cost each warp load 32 lines of a cache that 64 warps shared (192^3
+// inclusions, average of the levels: 1.09 ms, 0.89 ms staged).  A segment above
+// FILT_CAP entries is read in place.
 constexpr int FILT_ROWS = 64;
 constexpr int FILT_CAP = 2048;
 __global__ void __launch_bounds__(FILT_ROWS) k_filter(int64_t n, const int64_t* __restrict__ rp,

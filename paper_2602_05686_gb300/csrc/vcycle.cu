@@ -619,8 +619,37 @@ template void vh_free<float>(VHier<float>*);
 // ---------------------------------------------------------------------------
 // FP64 SELL kernels for the outer CG (unscaled fine operator)
 // ---------------------------------------------------------------------------
+// the sum of the block's 256 values by warp 0, in the order of a butterfly per
+// warp (offsets 16 .. 1) and one over the warps: lane 4 w + q of warp 0 takes
+// the values l = q mod 4 of warp w, so three stages are additions in the lane.
+// 13 FP64 instructions a block; a butterfly in every warp took 45 of the
+// kernel's 270, and FP64 issue bounds it.
+__device__ __forceinline__ double block_sum_256(double c) {
+  __shared__ double sh[8][36];  // 36: a warp's 32 reads on distinct banks
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  sh[w][lane] = c;
+  __syncthreads();
+  if (w != 0) return 0.0;
+  double u[8];
+#pragma unroll
+  for (int m = 0; m < 8; ++m) u[m] = sh[lane >> 2][(lane & 3) + 4 * m];
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+    for (int m = 0; m < o; ++m) u[m] += u[m + o];
+  double t = u[0];
+  t += __shfl_xor_sync(FULL, t, 2);
+  t += __shfl_xor_sync(FULL, t, 1);
+  t += 0.0;  // the absent warps of a 32-wide butterfly
+  t += __shfl_xor_sync(FULL, t, 16);
+  t += __shfl_xor_sync(FULL, t, 8);
+  t += __shfl_xor_sync(FULL, t, 4);
+  return t;
+}
+
 // q = A p, partial sums of p.q per CTA (fixed order); INLINE: the last block
-// finishes them
+// finishes them.  Bound by FP64 issue: 1.8M rows of 27 entries 123 us with a
+// butterfly in every warp, 107 us with block_sum_256; 7.2M rows 448, 403 us.
 template <bool INLINE>
 __global__ void __launch_bounds__(256) k_sell_spmv_dot(int64_t n, const int64_t* __restrict__ sp, const int32_t* __restrict__ ci,
                                 const int32_t* __restrict__ base, const uint16_t* __restrict__ c16,
@@ -634,16 +663,8 @@ __global__ void __launch_bounds__(256) k_sell_spmv_dot(int64_t n, const int64_t*
     q[i] = a;
     c = a * p[i];
   }
-  c = warp_sum(c);
-  __shared__ double sh[32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane == 0) sh[w] = c;
-  __syncthreads();
-  if (w == 0) {
-    double t = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0.0;
-    t = warp_sum(t);
-    if (lane == 0) part[blockIdx.x] = t;
-  }
+  const double t = block_sum_256(c);
+  if (threadIdx.x == 0) part[blockIdx.x] = t;
   if constexpr (INLINE) fin_inline<1, 256>(fin, part, (int)gridDim.x, 0, 0);
 }
 
