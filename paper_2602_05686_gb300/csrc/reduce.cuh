@@ -35,7 +35,7 @@ struct Fin {
   int op = FIN_STORE;
   double* out = nullptr;
   unsigned* tick = nullptr;   // zero before and after every launch
-  double* wsum = nullptr;     // 16 x 32 doubles (the wide form's group sums)
+  double* wsum = nullptr;     // KMAX_BLOCK x 32 doubles (the wide form's group sums)
   CgScalars* cg = nullptr;    // one problem, or k columns
   int k = 0;                  // columns (0: one vector)
   const int* active = nullptr;
@@ -54,14 +54,14 @@ inline unsigned red_blocks(int64_t n) {
   return (unsigned)(b < 1 ? 1 : (b < RED_BLOCKS ? b : RED_BLOCKS));
 }
 
-__device__ __forceinline__ void cg_alpha_step(CgScalars* s, double pq) {
+__host__ __device__ __forceinline__ void cg_alpha_step(CgScalars* s, double pq) {
   s->pq = pq;
   if (!(pq > 0.0)) { s->breakdown = 1; s->alpha = 0.0; return; }
   s->alpha = s->rz / pq;
 }
 
 // beta from the new r.z (and z.r_prev for flexible CG)
-__device__ __forceinline__ void cg_beta_step(CgScalars* s, double rz_new, double zr, int flexible) {
+__host__ __device__ __forceinline__ void cg_beta_step(CgScalars* s, double rz_new, double zr, int flexible) {
   if (flexible < 0) {
     s->rz = rz_new;
     s->beta = 0.0;
@@ -116,11 +116,13 @@ __device__ __forceinline__ void fin_sums(const double* __restrict__ part, int np
   __syncthreads();
 }
 
-// the step that follows the sums res[0 .. NV); second values (flexible beta)
-// at res[off2 ...]
-template <int NV>
-__device__ __forceinline__ void fin_step(const Fin& f, const double* res, int off2) {
-  const int c = (int)threadIdx.x;
+// the step that follows the sums res[0 .. NV), by thread c; the second values
+// (flexible beta) are res[OFF2 ...], OFF2 = 0 where the reduction has none: the
+// k-column forms hold OFF2 columns of first values before as many second ones.
+// (Arithmetic only, so that it runs on the host too.)
+template <int NV, int OFF2>
+__host__ __device__ __forceinline__ void fin_step(const Fin& f, const double* res, int c) {
+  static_assert(OFF2 == 0 || 2 * OFF2 == NV, "a second value for every first one");
   if (f.op != FIN_POWER && c < NV) f.out[c] = res[c];
   if (f.k > 0) {
     if (c >= f.k) return;
@@ -128,20 +130,28 @@ __device__ __forceinline__ void fin_step(const Fin& f, const double* res, int of
       if (f.active[c]) cg_alpha_step(f.cg + c, res[c]);
       else f.cg[c].alpha = 0.0;
     } else if (f.op == FIN_BETA) {
-      if (f.active[c]) cg_beta_step(f.cg + c, res[c], res[off2 + c], f.flexible);
+      if (f.active[c]) {
+        double zr = 0.0;
+        if constexpr (OFF2 > 0) zr = res[OFF2 + c];  // c < k <= OFF2
+        cg_beta_step(f.cg + c, res[c], zr, f.flexible);
+      }
     }
     return;
   }
   if (c != 0) return;
   switch (f.op) {
     case FIN_ALPHA: cg_alpha_step(f.cg, res[0]); break;
-    case FIN_BETA: cg_beta_step(f.cg, res[0], NV > 1 ? res[off2] : 0.0, f.flexible); break;
+    case FIN_BETA: cg_beta_step(f.cg, res[0], NV > 1 ? res[NV - 1] : 0.0, f.flexible); break;
     case FIN_LOOP: {
       // count the iteration and decide whether the WHILE node runs the body again
       const int k = *f.it + 1;
       *f.it = k;
       const int cont = !f.cg->breakdown && !(sqrt(res[0]) <= f.ctl[0]) && k < f.maxit;
+#ifdef __CUDA_ARCH__
       cudaGraphSetConditional((cudaGraphConditionalHandle)f.loop, cont ? 1u : 0u);
+#else
+      (void)cont;
+#endif
       break;
     }
     case FIN_POWER: {
@@ -165,12 +175,12 @@ __device__ __forceinline__ void fin_step(const Fin& f, const double* res, int of
 
 // end of a reduction kernel whose blocks have written their partials (thread
 // 0 of each wrote or waited for them): the last block sums and steps
-template <int NV, int NT>
-__device__ __forceinline__ void fin_inline(const Fin& f, const double* part, int np, int64_t stride, int off2) {
+template <int NV, int NT, int OFF2>
+__device__ __forceinline__ void fin_inline(const Fin& f, const double* part, int np, int64_t stride) {
   __shared__ double res[NV];
   if (!last_block(f.tick, gridDim.x)) return;
   fin_sums<NV, NT>(part, np, stride, res);
-  fin_step<NV>(f, res, off2);
+  fin_step<NV, OFF2>(f, res, (int)threadIdx.x);
 }
 
 // the wide form: block q takes group q, a warp per value
@@ -205,7 +215,7 @@ __global__ void __launch_bounds__(32 * NV) k_fin_wide(const double* __restrict__
     res[threadIdx.x] = s;
   }
   __syncthreads();
-  fin_step<NV>(f, res, 0);
+  fin_step<NV, 0>(f, res, (int)threadIdx.x);
 }
 
 }  // namespace sa

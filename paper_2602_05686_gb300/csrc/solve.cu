@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_dots(int64_t n, const double* _
     }
   }
   block_sum_to<NV>(acc, part, RED_BLOCKS);
-  fin_inline<NV, RED_THREADS>(fin, part, (int)gridDim.x, RED_BLOCKS, 1);
+  fin_inline<NV, RED_THREADS, NV - 1>(fin, part, (int)gridDim.x, RED_BLOCKS);
 }
 
 // ---------------------------------------------------------------------------
@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_power_dots(int64_t n, const dou
     acc[1] += vi * vi;
   }
   block_sum_to<2>(acc, part, RED_BLOCKS);
-  fin_inline<2, RED_THREADS>(fin, part, (int)gridDim.x, RED_BLOCKS, 1);
+  fin_inline<2, RED_THREADS, 1>(fin, part, (int)gridDim.x, RED_BLOCKS);
 }
 
 __global__ void k_rsqrt_scale(int64_t n, const double* __restrict__ d, double* __restrict__ out) {
@@ -176,6 +176,7 @@ int pick_sw(int64_t n, int64_t nnz) {
 
 int launch_dots(cudaStream_t st, int64_t n, const double* a0, const double* b0, const double* a1,
                 const double* b1, double* part, const Fin& fin) {
+  if (fin.op == FIN_BETA && fin.flexible > 0 && !a1) return SA_ERR_INVALID_ARG;  // needs the second dot
   const unsigned g = red_blocks(n);
   if (a1) launch_pdl(k_dots<2>, g, RED_THREADS, 0, st, n, a0, b0, a1, b1, part, fin);
   else launch_pdl(k_dots<1>, g, RED_THREADS, 0, st, n, a0, b0, nullptr, nullptr, part, fin);
@@ -313,7 +314,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_cg_update(int64_t n, const CgSc
     }
   }
   block_sum_to<1>(acc, part, 0);
-  fin_inline<1, RED_THREADS>(fin, part, (int)gridDim.x, 0, 0);
+  fin_inline<1, RED_THREADS, 0>(fin, part, (int)gridDim.x, 0);
 }
 
 __global__ void k_cg_pupdate(int64_t n, const CgScalars* __restrict__ s, const double* __restrict__ z,
@@ -479,7 +480,7 @@ __global__ void __launch_bounds__(RED_THREADS, 2) k_bdots(int64_t n, const doubl
     }
   }
   bblock_sum_to<KK, D>(acc, part, RED_BLOCKS);
-  fin_inline<D * KB, RED_THREADS>(fin, part, (int)gridDim.x, RED_BLOCKS, KB);
+  fin_inline<D * KB, RED_THREADS, (D - 1) * KB>(fin, part, (int)gridDim.x, RED_BLOCKS);
 }
 
 template <int KK>
@@ -538,7 +539,7 @@ __global__ void __launch_bounds__(RED_THREADS, 2)
     }
   }
   bblock_sum_to<KK, 1>(acc, part, RED_BLOCKS);
-  fin_inline<KB, RED_THREADS>(fin, part, (int)gridDim.x, RED_BLOCKS, 0);
+  fin_inline<KB, RED_THREADS, 0>(fin, part, (int)gridDim.x, RED_BLOCKS);
 }
 
 template <int KK>
@@ -599,6 +600,7 @@ __global__ void k_interleave(int64_t n, int k, int K, const double* __restrict__
 int launch_bdots(cudaStream_t st, int64_t n, int k, const double* a, const double* b, const double* c, double* part,
                  const Fin& fin) {
   if (k != 2 && k != 4 && k != 8) return SA_ERR_INVALID_ARG;  // whole-row vectors
+  if (fin.op == FIN_BETA && fin.flexible > 0 && !c) return SA_ERR_INVALID_ARG;  // needs the second dot
   const unsigned g = red_blocks(n);
   // one dot per column (a . b), or two (b . c into out[KB + column])
   if (c) {

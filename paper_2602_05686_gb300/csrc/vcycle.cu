@@ -665,7 +665,7 @@ __global__ void __launch_bounds__(256) k_sell_spmv_dot(int64_t n, const int64_t*
   }
   const double t = block_sum_256(c);
   if (threadIdx.x == 0) part[blockIdx.x] = t;
-  if constexpr (INLINE) fin_inline<1, 256>(fin, part, (int)gridDim.x, 0, 0);
+  if constexpr (INLINE) fin_inline<1, 256, 0>(fin, part, (int)gridDim.x, 0);
 }
 
 __global__ void k_sell_res64(int64_t n, const int64_t* __restrict__ sp, const int32_t* __restrict__ ci,
