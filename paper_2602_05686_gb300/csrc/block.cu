@@ -23,35 +23,9 @@ namespace sa {
 // stores as partial-sector writes; measured on the 8-column FP32 Chebyshev
 // step at 320^3 that cost 1.6x in time.  Buffers start on 256-byte
 // boundaries (the allocator contract).
-//   ld_row_nc: data read-only for the whole launch (gathered x, b)
-//   ld_row:    coherent load (a vector the launch also writes, as d)
-template <typename T, int K>
-__device__ __forceinline__ void ld_row_nc(const T* __restrict__ p, T (&v)[K]) {
-  if constexpr (sizeof(T) == 4 && K == 8) {
-    asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
-        : "l"(p));
-  } else if constexpr (sizeof(T) == 8 && K % 4 == 0) {
-#pragma unroll
-    for (int q = 0; q < K / 4; ++q)
-      asm("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];"
-          : "=d"(v[4 * q]), "=d"(v[4 * q + 1]), "=d"(v[4 * q + 2]), "=d"(v[4 * q + 3])
-          : "l"(p + 4 * q));
-  } else if constexpr (sizeof(T) == 4 && K == 4) {
-    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
-    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
-  } else if constexpr (sizeof(T) == 4 && K == 2) {
-    const float2 t = __ldg(reinterpret_cast<const float2*>(p));
-    v[0] = t.x; v[1] = t.y;
-  } else if constexpr (sizeof(T) == 8 && K == 2) {
-    const double2 t = __ldg(reinterpret_cast<const double2*>(p));
-    v[0] = t.x; v[1] = t.y;
-  } else {
-#pragma unroll
-    for (int c = 0; c < K; ++c) v[c] = __ldg(p + c);
-  }
-}
-
+// ld_row is a coherent load that the compiler keeps behind pdl_sync(): the
+// vectors are written by the predecessor, which may still run when this launch
+// starts, so they are not read-only data for its whole length.
 template <typename T, int K>
 __device__ __forceinline__ void ld_row(const T* p, T (&v)[K]) {
   if constexpr (sizeof(T) == 4 && K == 8) {
@@ -67,11 +41,12 @@ __device__ __forceinline__ void ld_row(const T* p, T (&v)[K]) {
                    : "l"(p + 4 * q)
                    : "memory");
   } else if constexpr (sizeof(T) == 4 && K == 4) {
-    const float4 t = *reinterpret_cast<const float4*>(p);
-    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+    asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+                 : "l"(p)
+                 : "memory");
   } else if constexpr (sizeof(T) == 4 && K == 2) {
-    const float2 t = *reinterpret_cast<const float2*>(p);
-    v[0] = t.x; v[1] = t.y;
+    asm volatile("ld.global.v2.f32 {%0,%1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "l"(p) : "memory");
   } else if constexpr (sizeof(T) == 8 && K == 2) {
     const double2 t = *reinterpret_cast<const double2*>(p);
     v[0] = t.x; v[1] = t.y;
@@ -110,15 +85,15 @@ __device__ __forceinline__ void st_row(T* p, const T (&v)[K]) {
 // a 256-bit load's four results held at once cost the CSR kernels
 // registers and occupancy)
 template <typename T, int K>
-__device__ __forceinline__ void ldvec(const T* __restrict__ p, T (&v)[K]) {
+__device__ __forceinline__ void ldvec(const T* p, T (&v)[K]) {
   if constexpr (sizeof(T) == 8 && K % 2 == 0) {
 #pragma unroll
     for (int q = 0; q < K / 2; ++q) {
-      const double2 t = __ldg(reinterpret_cast<const double2*>(p) + q);
+      const double2 t = reinterpret_cast<const double2*>(p)[q];
       v[2 * q] = t.x; v[2 * q + 1] = t.y;
     }
   } else {
-    ld_row_nc<T, K>(p, v);
+    ld_row<T, K>(p, v);
   }
 }
 
@@ -182,7 +157,7 @@ struct BUnroll {
 };
 
 template <typename T, int SW, int K>
-__device__ __forceinline__ int brow_apply(const MatView<T>& M, const T* __restrict__ X, T (&acc)[K], int64_t& row,
+__device__ __forceinline__ int brow_apply(const MatView<T>& M, const T* X, T (&acc)[K], int64_t& row,
                                           int& c0) {
   constexpr int U = BUnroll<T, SW>::U;
   const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -197,7 +172,7 @@ __device__ __forceinline__ int brow_apply(const MatView<T>& M, const T* __restri
     row = i;
     if (i < M.n) {
       const int64_t e = M.p[sl + 1];
-      const T* __restrict__ xs = M.c16 ? X + (int64_t)M.base[sl] * K : X;
+      const T* xs = M.c16 ? X + (int64_t)M.base[sl] * K : X;
       int64_t p = M.p[sl] + 32 * h + r;
       for (; p + 64 * (U - 1) < e; p += 64 * U) {
         T a[U], xv[U][K];
@@ -259,7 +234,7 @@ __device__ __forceinline__ int brow_apply(const MatView<T>& M, const T* __restri
       }
     }
     if (row >= M.n) return 0;
-    const T* __restrict__ xs = M.c16 ? X + (int64_t)M.base[sl] * K : X;
+    const T* xs = M.c16 ? X + (int64_t)M.base[sl] * K : X;
     const uint16_t* s16 = reinterpret_cast<const uint16_t*>(scol);
     const int32_t* s32 = reinterpret_cast<const int32_t*>(scol);
     int k = 0;
@@ -294,7 +269,7 @@ __device__ __forceinline__ int brow_apply(const MatView<T>& M, const T* __restri
     if (gt >= M.n) return 0;
     const int64_t sl = gt >> 5, r = gt & 31;
     const int64_t b = M.p[sl], e = M.p[sl + 1];
-    const T* __restrict__ xs = M.c16 ? X + (int64_t)M.base[sl] * K : X;
+    const T* xs = M.c16 ? X + (int64_t)M.base[sl] * K : X;
     int64_t p = b + r;
     for (; p + 32 * (U - 1) < e; p += 32 * U) {
       T a[U], xv[U][K];
@@ -446,7 +421,7 @@ __device__ __forceinline__ int brow_apply(const MatView<T>& M, const T* __restri
           cc[t] = in ? M.ci[q + t] : 0;
         }
 #pragma unroll
-        for (int t = 0; t < R; ++t) xv[t] = q + t < e ? __ldg(&X[(int64_t)cc[t] * K + c]) : (T)0;
+        for (int t = 0; t < R; ++t) xv[t] = q + t < e ? X[(int64_t)cc[t] * K + c] : (T)0;
 #pragma unroll
         for (int u = 0; u < UC; ++u)
 #pragma unroll
@@ -535,7 +510,7 @@ struct BOcc {
 template <typename T, int SW, int K>
 // d_in and d_out may be one buffer (each thread reads and writes its own row);
 // d_in may also be x_in's buffer (after the first step, where x_1 = d_1)
-__global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_cheb(MatView<T> A, const T* __restrict__ b, const T* __restrict__ xin, T* __restrict__ xout,
+__global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_cheb(MatView<T> A, const T* b, const T* xin, T* __restrict__ xout,
                            const T* din, T* dout, T c1, T c2, int first) {
   pdl_sync();
   T y[K];
@@ -547,8 +522,8 @@ __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_cheb(MatView<T> A, 
   if constexpr (NW > 1) {
     if (nw == NW) {
       T bb[NW], xx[NW], dd[NW], xo[NW];
-      ld_row_nc<T, NW>(b + o, bb);
-      ld_row_nc<T, NW>(xin + o, xx);
+      ld_row<T, NW>(b + o, bb);
+      ld_row<T, NW>(xin + o, xx);
       if (first) {
 #pragma unroll
         for (int j = 0; j < NW; ++j) dd[j] = (T)0;
@@ -576,7 +551,7 @@ __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_cheb(MatView<T> A, 
 }
 
 template <typename T, int SW, int K>
-__global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_residual(MatView<T> A, const T* __restrict__ b, const T* __restrict__ x, T* __restrict__ r) {
+__global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_residual(MatView<T> A, const T* b, const T* x, T* __restrict__ r) {
   pdl_sync();
   T y[K];
   int64_t i;
@@ -587,7 +562,7 @@ __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_residual(MatView<T>
   if constexpr (NW > 1) {
     if (nw == NW) {
       T bb[NW];
-      ld_row_nc<T, NW>(b + o, bb);
+      ld_row<T, NW>(b + o, bb);
 #pragma unroll
       for (int j = 0; j < NW; ++j) bb[j] = bb[j] - y[j];
       st_row<T, NW>(r + o, bb);
@@ -600,7 +575,7 @@ __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_residual(MatView<T>
 }
 
 template <typename T, int SW, int K>
-__global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_spmv(MatView<T> A, const T* __restrict__ x, T* __restrict__ out) {
+__global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_spmv(MatView<T> A, const T* x, T* __restrict__ out) {
   pdl_sync();
   T y[K];
   int64_t i;
@@ -623,7 +598,7 @@ __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_spmv(MatView<T> A, 
 }
 
 template <typename T, int SW, int K>
-__global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_spmv_add(MatView<T> A, const T* __restrict__ x, T* __restrict__ out) {
+__global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_spmv_add(MatView<T> A, const T* x, T* __restrict__ out) {
   pdl_sync();
   T y[K];
   int64_t i;
@@ -647,8 +622,8 @@ __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_spmv_add(MatView<T>
 }
 
 template <typename T, int SW, int K>
-__global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_cheb_out(MatView<T> A, const T* __restrict__ b, const T* __restrict__ xin,
-                               const T* __restrict__ d, T c1, T c2, int first, const double* __restrict__ s,
+__global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_cheb_out(MatView<T> A, const T* b, const T* xin,
+                               const T* d, T c1, T c2, int first, const double* __restrict__ s,
                                double* __restrict__ z) {
   pdl_sync();
   T y[K];
@@ -663,13 +638,13 @@ __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_cheb_out(MatView<T>
     if (nw == NW) {
       T bb[NW], xx[NW], dd[NW];
       double zz[NW];
-      ld_row_nc<T, NW>(b + o, bb);
-      ld_row_nc<T, NW>(xin + o, xx);
+      ld_row<T, NW>(b + o, bb);
+      ld_row<T, NW>(xin + o, xx);
       if (first) {
 #pragma unroll
         for (int j = 0; j < NW; ++j) dd[j] = (T)0;
       } else {
-        ld_row_nc<T, NW>(d + o, dd);
+        ld_row<T, NW>(d + o, dd);
       }
 #pragma unroll
       for (int j = 0; j < NW; ++j) zz[j] = si * (double)(xx[j] + cheb_dir<T>(bb[j], y[j], dd[j], c1, c2, first));
@@ -693,7 +668,7 @@ __global__ void __launch_bounds__(256, BOcc<T, SW>::B) k_bvc_cheb_out(MatView<T>
 // 64-bit division per thread 146 us, this 127 us, two or four vectors a thread
 // 129 and 130 us).
 template <typename T, int K>
-__global__ void k_bvc_fine_in(int64_t n, const double* __restrict__ r, const double* __restrict__ s, T c2,
+__global__ void k_bvc_fine_in(int64_t n, const double* r, const double* __restrict__ s, T c2,
                               T* __restrict__ b, T* __restrict__ d) {
   pdl_sync();
   constexpr int G = K >= 4 ? 4 : 2;
@@ -714,14 +689,14 @@ __global__ void k_bvc_fine_in(int64_t n, const double* __restrict__ r, const dou
 }
 
 template <typename T>
-__global__ void k_bvc_first(int64_t nk, const T* __restrict__ b, T c2, T* __restrict__ d) {
+__global__ void k_bvc_first(int64_t nk, const T* b, T c2, T* __restrict__ d) {
   pdl_sync();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e < nk) d[e] = c2 * b[e];
 }
 
 template <typename T>
-__global__ void k_bcoarse_in(int64_t n, int K, const T* __restrict__ b, const double* __restrict__ sq,
+__global__ void k_bcoarse_in(int64_t n, int K, const T* b, const double* __restrict__ sq,
                              double* __restrict__ t) {
   pdl_sync();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -931,7 +906,7 @@ template int vh_vcycle_block<float>(Alloc&, VHier<float>*, cudaStream_t, int, co
 // one-vector reduction tree per column) and R = B - A X, FP64 SELL
 // ---------------------------------------------------------------------------
 template <int K>
-__global__ void k_bsell_spmv_dot(MatView<double> A, const double* __restrict__ P, double* __restrict__ Q,
+__global__ void k_bsell_spmv_dot(MatView<double> A, const double* P, double* __restrict__ Q,
                                  double* __restrict__ part) {
   pdl_sync();
   double y[K], c[K];
@@ -942,7 +917,7 @@ __global__ void k_bsell_spmv_dot(MatView<double> A, const double* __restrict__ P
   if (brow_apply<double, 0, K>(A, P, y, i, c0)) {
     const int64_t o = i * K;
     double pp[K];
-    ld_row_nc<double, K>(P + o, pp);
+    ld_row<double, K>(P + o, pp);
     st_row<double, K>(Q + o, y);
 #pragma unroll
     for (int j = 0; j < K; ++j) c[j] = y[j] * pp[j];
@@ -972,7 +947,7 @@ __global__ void k_bsell_spmv_dot(MatView<double> A, const double* __restrict__ P
 }
 
 template <int K>
-__global__ void k_bsell_res64(MatView<double> A, const double* __restrict__ B, const double* __restrict__ X,
+__global__ void k_bsell_res64(MatView<double> A, const double* B, const double* X,
                               double* __restrict__ R) {
   pdl_sync();
   double y[K];
@@ -981,7 +956,7 @@ __global__ void k_bsell_res64(MatView<double> A, const double* __restrict__ B, c
   if (!brow_apply<double, 0, K>(A, X, y, i, c0)) return;
   const int64_t o = i * K;
   double bb[K];
-  ld_row_nc<double, K>(B + o, bb);
+  ld_row<double, K>(B + o, bb);
 #pragma unroll
   for (int j = 0; j < K; ++j) bb[j] = bb[j] - y[j];
   st_row<double, K>(R + o, bb);

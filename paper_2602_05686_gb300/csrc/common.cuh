@@ -109,7 +109,11 @@ inline unsigned warp_rows_grid(int64_t rows, int block = 256) {
 // Programmatic dependent launch: a kernel launched by launch_pdl may start while
 // its predecessor in the stream drains, and waits in pdl_sync() for that
 // predecessor's completion before it touches anything the stream writes (it
-// may read matrices built before the solve earlier).  The trigger follows the
+// may read matrices built before the solve earlier).  Its lifetime overlaps the
+// predecessor's, so what the stream writes -- vectors, CG scalars, partial sums
+// -- is not read-only data in it: such pointers carry no __restrict__ and are
+// read with plain loads after pdl_sync(); __ldg, ld.global.nc and const
+// __restrict__ are for matrices, scalings and launch descriptors.  The trigger follows the
 // wait, so no kernel starts before the one before its predecessor has ended.
 // Every kernel launched this way calls pdl_sync() first.  The launches of one
 // V-cycle on small levels are 2 to 4 us of work with 1.3 us between them.

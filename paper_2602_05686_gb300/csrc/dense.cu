@@ -694,8 +694,8 @@ __device__ __forceinline__ void coarse_rows(const CoarseEnt& E, const CoarseProb
   const double* M = E.mode == CS_W ? P.F.W : (E.mode == CS_WT ? P.F.WT : (E.mode == CS_L ? P.F.L : P.F.LT));
   const double* __restrict__ Mi = M + (int64_t)i * n;
   // columns below `split` come from va, the others from vb
-  const double* __restrict__ va = E.mode == CS_W ? P.t : (E.mode == CS_LT ? P.x : P.y);
-  const double* __restrict__ vb = E.mode == CS_W ? P.bin : P.t;
+  const double* va = E.mode == CS_W ? P.t : (E.mode == CS_LT ? P.x : P.y);
+  const double* vb = E.mode == CS_W ? P.bin : P.t;
   double sum[CS_SEG * K];
 #pragma unroll
   for (int c = 0; c < CS_SEG * K; ++c) sum[c] = 0.0;

@@ -152,7 +152,7 @@ __device__ __forceinline__ void g_block_sum_to(double (&val)[NV], double* __rest
   }
 }
 
-__device__ __forceinline__ double g_sell_row(const GCg& D, const double* __restrict__ x, int64_t i) {
+__device__ __forceinline__ double g_sell_row(const GCg& D, const double* x, int64_t i) {
   return D.c16 ? sell_row16<double>(D.sp, D.base, D.c16, D.v, x, i) : sell_row<double>(D.sp, D.ci, D.v, x, i);
 }
 

@@ -90,7 +90,7 @@ __device__ __forceinline__ bool last_block(unsigned* tick, unsigned blocks) {
 // sums of NV values over np partials (value v at part[v * stride + t]) into
 // res (shared), by a block of NT threads
 template <int NV, int NT>
-__device__ __forceinline__ void fin_sums(const double* __restrict__ part, int np, int64_t stride, double* res) {
+__device__ __forceinline__ void fin_sums(const double* part, int np, int64_t stride, double* res) {
   __shared__ double sh[NV][33];
   const int lane = (int)(threadIdx.x & 31), w = (int)(threadIdx.x >> 5);
   const int groups = np < FIN_T ? (np + 31) >> 5 : 32;
@@ -185,7 +185,7 @@ __device__ __forceinline__ void fin_inline(const Fin& f, const double* part, int
 
 // the wide form: block q takes group q, a warp per value
 template <int NV>
-__global__ void __launch_bounds__(32 * NV) k_fin_wide(const double* __restrict__ part, int np, int64_t stride,
+__global__ void __launch_bounds__(32 * NV) k_fin_wide(const double* part, int np, int64_t stride,
                                                       Fin f) {
   pdl_sync();
   __shared__ double res[NV];

@@ -25,8 +25,8 @@ namespace sa {
 // power method: y_j = s_j v_j with v_j = X_j * sc[4] (the previous product
 // times the reciprocal of its norm; 1 for the start vector), formed once per
 // step so that the product below costs one FP64 FMA per stored entry
-__global__ void k_power_prep(int64_t n, const double* __restrict__ X, const double* __restrict__ s,
-                             const double* __restrict__ sc, double* __restrict__ y) {
+__global__ void k_power_prep(int64_t n, const double* X, const double* __restrict__ s,
+                             const double* sc, double* __restrict__ y) {
   pdl_sync();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) y[i] = s ? s[i] * (X[i] * sc[4]) : X[i] * sc[4];  // s NULL: a pre-scaled operator
@@ -35,7 +35,7 @@ __global__ void k_power_prep(int64_t n, const double* __restrict__ X, const doub
 // w_i = s_i * sum_p a_p y_j
 template <int SW>
 __global__ void k_power_spmv(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                             const double* __restrict__ v, const double* __restrict__ s, const double* __restrict__ y,
+                             const double* __restrict__ v, const double* __restrict__ s, const double* y,
                              double* __restrict__ w) {
   pdl_sync();
   ROW_SETUP(SW)
@@ -74,9 +74,9 @@ __device__ __forceinline__ void block_sum_to(double (&val)[NV], double* __restri
 
 // one or two dot products over a fixed grid, finished by the last block
 template <int NV>
-__global__ void __launch_bounds__(RED_THREADS) k_dots(int64_t n, const double* __restrict__ a0,
-                                                      const double* __restrict__ b0, const double* __restrict__ a1,
-                                                      const double* __restrict__ b1, double* __restrict__ part,
+__global__ void __launch_bounds__(RED_THREADS) k_dots(int64_t n, const double* a0,
+                                                      const double* b0, const double* a1,
+                                                      const double* b1, double* __restrict__ part,
                                                       Fin fin) {
   pdl_sync();
   double acc[NV];
@@ -125,8 +125,8 @@ __global__ void k_start_vector(int64_t n, uint32_t tag, uint32_t seed, double* _
 
 // w.w and v.v with v_j = X_j * sc[4]; the last block takes the estimate and
 // the next scale from them (FIN_POWER)
-__global__ void __launch_bounds__(RED_THREADS) k_power_dots(int64_t n, const double* __restrict__ w,
-                                                            const double* __restrict__ X, const double* sc,
+__global__ void __launch_bounds__(RED_THREADS) k_power_dots(int64_t n, const double* w,
+                                                            const double* X, const double* sc,
                                                             double* __restrict__ part, Fin fin) {
   pdl_sync();
   const double inv = sc[4];
@@ -276,8 +276,8 @@ int launch_omega(cudaStream_t s, const double* lam_dev, double omega_sym, double
 // ---------------------------------------------------------------------------
 // x += alpha p; r -= alpha q; (r_prev = r before the update, if given); r.r,
 // finished by the last block
-__global__ void __launch_bounds__(RED_THREADS) k_cg_update(int64_t n, const CgScalars* s, const double* __restrict__ p,
-                                                           const double* __restrict__ q, double* __restrict__ x,
+__global__ void __launch_bounds__(RED_THREADS) k_cg_update(int64_t n, const CgScalars* s, const double* p,
+                                                           const double* q, double* __restrict__ x,
                                                            double* __restrict__ r, double* __restrict__ rprev,
                                                            double* __restrict__ part, Fin fin) {
   pdl_sync();
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_cg_update(int64_t n, const CgSc
   fin_inline<1, RED_THREADS, 0>(fin, part, (int)gridDim.x, 0);
 }
 
-__global__ void k_cg_pupdate(int64_t n, const CgScalars* __restrict__ s, const double* __restrict__ z,
+__global__ void k_cg_pupdate(int64_t n, const CgScalars* s, const double* z,
                              double* __restrict__ p, int first) {
   pdl_sync();
   const double beta = s->beta;
@@ -434,8 +434,8 @@ __device__ __forceinline__ void stgrp(double* p, const double (&v)[G]) {
 
 // D = 1: a . b per column; D = 2: and b . c
 template <int KK, int D>
-__global__ void __launch_bounds__(RED_THREADS, 2) k_bdots(int64_t n, const double* __restrict__ a,
-                                                          const double* __restrict__ b, const double* __restrict__ c,
+__global__ void __launch_bounds__(RED_THREADS, 2) k_bdots(int64_t n, const double* a,
+                                                          const double* b, const double* c,
                                                           double* __restrict__ part, Fin fin) {
   pdl_sync();
   using B = BRow<KK>;
@@ -485,8 +485,8 @@ __global__ void __launch_bounds__(RED_THREADS, 2) k_bdots(int64_t n, const doubl
 
 template <int KK>
 __global__ void __launch_bounds__(RED_THREADS, 2)
-    k_bcg_update(const int64_t n, const CgScalars* s, const int* __restrict__ active,
-                 const double* __restrict__ p, const double* __restrict__ q, double* __restrict__ x,
+    k_bcg_update(const int64_t n, const CgScalars* s, const int* active,
+                 const double* p, const double* q, double* __restrict__ x,
                  double* __restrict__ r, double* __restrict__ rprev, double* __restrict__ part, Fin fin) {
   pdl_sync();
   using B = BRow<KK>;
@@ -544,8 +544,8 @@ __global__ void __launch_bounds__(RED_THREADS, 2)
 
 template <int KK>
 __global__ void __launch_bounds__(RED_THREADS, 2)
-    k_bcg_pupdate(int64_t n, const CgScalars* __restrict__ s, const int* __restrict__ active,
-                  const double* __restrict__ z, double* __restrict__ p, int first) {
+    k_bcg_pupdate(int64_t n, const CgScalars* s, const int* active,
+                  const double* z, double* __restrict__ p, int first) {
   pdl_sync();
   using B = BRow<KK>;
   constexpr int G = B::G, L = B::LPR;

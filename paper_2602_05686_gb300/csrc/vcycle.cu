@@ -399,7 +399,7 @@ struct VOcc {
 
 // x_out = x_in + d,  d = first ? c2 r : c1 d + c2 r,  r = b - A~ x_in
 template <typename T, int SW>
-__global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_cheb(MatView<T> A, const T* __restrict__ b, const T* __restrict__ xin, T* __restrict__ xout,
+__global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_cheb(MatView<T> A, const T* b, const T* xin, T* __restrict__ xout,
                           T* __restrict__ d, T c1, T c2, int first) {
   T y;
   int64_t i;
@@ -410,21 +410,21 @@ __global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_cheb(MatView<T> A, c
 }
 
 template <typename T, int SW>
-__global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_residual(MatView<T> A, const T* __restrict__ b, const T* __restrict__ x, T* __restrict__ r) {
+__global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_residual(MatView<T> A, const T* b, const T* x, T* __restrict__ r) {
   T y;
   int64_t i;
   if (row_apply<T, SW>(A, x, y, i)) r[i] = b[i] - y;
 }
 
 template <typename T, int SW>
-__global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_spmv(MatView<T> A, const T* __restrict__ x, T* __restrict__ out) {
+__global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_spmv(MatView<T> A, const T* x, T* __restrict__ out) {
   T y;
   int64_t i;
   if (row_apply<T, SW>(A, x, y, i)) out[i] = y;
 }
 
 template <typename T, int SW>
-__global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_spmv_add(MatView<T> A, const T* __restrict__ x, T* __restrict__ out) {
+__global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_spmv_add(MatView<T> A, const T* x, T* __restrict__ out) {
   T y;
   int64_t i;
   if (row_apply<T, SW>(A, x, y, i)) out[i] += y;
@@ -432,8 +432,8 @@ __global__ void __launch_bounds__(256, VOcc<T, SW>::B) k_vc_spmv_add(MatView<T> 
 
 // fine exit: the last post-smoothing step writes z = D^-1/2 x~ in FP64
 template <typename T, int SW>
-__global__ void k_vc_cheb_out(MatView<T> A, const T* __restrict__ b, const T* __restrict__ xin,
-                              const T* __restrict__ d, T c1, T c2, int first, const double* __restrict__ s,
+__global__ void k_vc_cheb_out(MatView<T> A, const T* b, const T* xin,
+                              const T* d, T c1, T c2, int first, const double* __restrict__ s,
                               double* __restrict__ z) {
   T y;
   int64_t i;
@@ -443,7 +443,7 @@ __global__ void k_vc_cheb_out(MatView<T> A, const T* __restrict__ b, const T* __
 }
 
 template <typename T>
-__global__ void k_vc_first(int64_t n, const T* __restrict__ b, T c2, T* __restrict__ x, T* __restrict__ d) {
+__global__ void k_vc_first(int64_t n, const T* b, T c2, T* __restrict__ x, T* __restrict__ d) {
   pdl_sync();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) {
@@ -455,7 +455,7 @@ __global__ void k_vc_first(int64_t n, const T* __restrict__ b, T c2, T* __restri
 
 // fine entry b~ = D^-1/2 r (FP64 r), fused with the first Chebyshev step
 template <typename T>
-__global__ void k_vc_fine_in(int64_t n, const double* __restrict__ r, const double* __restrict__ s, T c2,
+__global__ void k_vc_fine_in(int64_t n, const double* r, const double* __restrict__ s, T c2,
                              T* __restrict__ b, T* __restrict__ x, T* __restrict__ d) {
   pdl_sync();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -494,7 +494,7 @@ int vh_power(Alloc& al, VHier<double>* m, int l, int steps, uint32_t tag, uint32
 }
 
 template <typename T>
-__global__ void k_coarse_in(int64_t n, const T* __restrict__ b, const double* __restrict__ sq,
+__global__ void k_coarse_in(int64_t n, const T* b, const double* __restrict__ sq,
                             double* __restrict__ t) {
   pdl_sync();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -653,7 +653,7 @@ __device__ __forceinline__ double block_sum_256(double c) {
 template <bool INLINE>
 __global__ void __launch_bounds__(256) k_sell_spmv_dot(int64_t n, const int64_t* __restrict__ sp, const int32_t* __restrict__ ci,
                                 const int32_t* __restrict__ base, const uint16_t* __restrict__ c16,
-                                const double* __restrict__ v, const double* __restrict__ p, double* __restrict__ q,
+                                const double* __restrict__ v, const double* p, double* __restrict__ q,
                                 double* __restrict__ part, Fin fin) {
   pdl_sync();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -670,8 +670,8 @@ __global__ void __launch_bounds__(256) k_sell_spmv_dot(int64_t n, const int64_t*
 
 __global__ void k_sell_res64(int64_t n, const int64_t* __restrict__ sp, const int32_t* __restrict__ ci,
                              const int32_t* __restrict__ base, const uint16_t* __restrict__ c16,
-                             const double* __restrict__ v, const double* __restrict__ b,
-                             const double* __restrict__ x, double* __restrict__ r) {
+                             const double* __restrict__ v, const double* b,
+                             const double* x, double* __restrict__ r) {
   pdl_sync();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n)

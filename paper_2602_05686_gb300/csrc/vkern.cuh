@@ -22,7 +22,7 @@ struct RowUnroll {
 
 template <typename T, int U = RowUnroll<T>::U>
 __device__ __forceinline__ T sell_row(const int64_t* __restrict__ sp, const int32_t* __restrict__ ci,
-                                      const T* __restrict__ v, const T* __restrict__ x, int64_t i) {
+                                      const T* __restrict__ v, const T* x, int64_t i) {
   const int64_t sl = i >> 5, r = i & 31;
   const int64_t b = sp[sl], e = sp[sl + 1];
   T acc = (T)0;
@@ -36,11 +36,11 @@ __device__ __forceinline__ T sell_row(const int64_t* __restrict__ sp, const int3
       cc[u] = __ldcs(&ci[p + 32 * u]);
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) xx[u] = __ldg(&x[cc[u]]);
+    for (int u = 0; u < U; ++u) xx[u] = x[cc[u]];
 #pragma unroll
     for (int u = 0; u < U; ++u) acc += vv[u] * xx[u];
   }
-  for (; p < e; p += 32) acc += __ldcs(&v[p]) * __ldg(&x[__ldcs(&ci[p])]);
+  for (; p < e; p += 32) acc += __ldcs(&v[p]) * x[__ldcs(&ci[p])];
   return acc;
 }
 
@@ -48,10 +48,10 @@ __device__ __forceinline__ T sell_row(const int64_t* __restrict__ sp, const int3
 template <typename T, int U = RowUnroll<T>::U>
 __device__ __forceinline__ T sell_row16(const int64_t* __restrict__ sp, const int32_t* __restrict__ base,
                                         const uint16_t* __restrict__ c16, const T* __restrict__ v,
-                                        const T* __restrict__ x, int64_t i) {
+                                        const T* x, int64_t i) {
   const int64_t sl = i >> 5, r = i & 31;
   const int64_t b = sp[sl], e = sp[sl + 1];
-  const T* __restrict__ xs = x + base[sl];
+  const T* xs = x + base[sl];
   T acc = (T)0;
   int64_t p = b + r;
   for (; p + 32 * (U - 1) < e; p += 32 * U) {
@@ -63,11 +63,11 @@ __device__ __forceinline__ T sell_row16(const int64_t* __restrict__ sp, const in
       cc[u] = __ldcs(&c16[p + 32 * u]);
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) xx[u] = __ldg(&xs[cc[u]]);
+    for (int u = 0; u < U; ++u) xx[u] = xs[cc[u]];
 #pragma unroll
     for (int u = 0; u < U; ++u) acc += vv[u] * xx[u];
   }
-  for (; p < e; p += 32) acc += __ldcs(&v[p]) * __ldg(&xs[__ldcs(&c16[p])]);
+  for (; p < e; p += 32) acc += __ldcs(&v[p]) * xs[__ldcs(&c16[p])];
   return acc;
 }
 
@@ -77,9 +77,9 @@ __device__ __forceinline__ T sell_row16(const int64_t* __restrict__ sp, const in
 template <typename T, bool C16, int U = RowUnroll<T>::U>
 __device__ __forceinline__ T sell2_lane(const int64_t* __restrict__ sp, const int32_t* __restrict__ base,
                                         const uint16_t* __restrict__ c16, const int32_t* __restrict__ ci,
-                                        const T* __restrict__ v, const T* __restrict__ x, int64_t sl, int r, int h) {
+                                        const T* __restrict__ v, const T* x, int64_t sl, int r, int h) {
   const int64_t b = sp[sl], e = sp[sl + 1];
-  const T* __restrict__ xs = C16 ? x + base[sl] : x;
+  const T* xs = C16 ? x + base[sl] : x;
   T acc = (T)0;
   int64_t p = b + 32 * h + r;
   // the first round's values and columns before the wait for the vector
@@ -97,7 +97,7 @@ __device__ __forceinline__ T sell2_lane(const int64_t* __restrict__ sp, const in
   if (full) {
     for (;;) {
 #pragma unroll
-      for (int u = 0; u < U; ++u) xx[u] = __ldg(&xs[cc[u]]);
+      for (int u = 0; u < U; ++u) xx[u] = xs[cc[u]];
 #pragma unroll
       for (int u = 0; u < U; ++u) acc += vv[u] * xx[u];
       p += 64 * U;
@@ -111,7 +111,7 @@ __device__ __forceinline__ T sell2_lane(const int64_t* __restrict__ sp, const in
   }
   for (; p < e; p += 64) {
     const unsigned c = C16 ? (unsigned)__ldcs(&c16[p]) : (unsigned)__ldcs(&ci[p]);
-    acc += __ldcs(&v[p]) * __ldg(&xs[c]);
+    acc += __ldcs(&v[p]) * xs[c];
   }
   return acc;
 }
@@ -168,7 +168,7 @@ constexpr int LONG_UNROLL = 8;
 // few entries): full rounds and single entries, the fastest there (120^3 FP32
 // prolongation 26.7 us, 31 to 35 us with predicated or prefetched rounds).
 template <typename T, int W, int U>
-__device__ __forceinline__ T csr_lane(const MatView<T>& M, const T* __restrict__ x, int64_t b, int64_t e, int sl) {
+__device__ __forceinline__ T csr_lane(const MatView<T>& M, const T* x, int64_t b, int64_t e, int sl) {
   T acc = (T)0;
   if constexpr (W == 1) {
     pdl_sync();
@@ -182,11 +182,11 @@ __device__ __forceinline__ T csr_lane(const MatView<T>& M, const T* __restrict__
         cc[u] = M.ci[q + W * u];
       }
 #pragma unroll
-      for (int u = 0; u < U; ++u) xx[u] = __ldg(&x[cc[u]]);
+      for (int u = 0; u < U; ++u) xx[u] = x[cc[u]];
 #pragma unroll
       for (int u = 0; u < U; ++u) acc += vv[u] * xx[u];
     }
-    for (; q < e; q += W) acc += M.v[q] * __ldg(&x[M.ci[q]]);
+    for (; q < e; q += W) acc += M.v[q] * x[M.ci[q]];
   } else {
     const int len = (int)(e - b);
     const T* __restrict__ v = M.v + b;
@@ -204,7 +204,7 @@ __device__ __forceinline__ T csr_lane(const MatView<T>& M, const T* __restrict__
       T xx[U], vn[U];
       int32_t cn[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) xx[u] = q + W * u < len ? __ldg(&x[cc[u]]) : (T)0;
+      for (int u = 0; u < U; ++u) xx[u] = q + W * u < len ? x[cc[u]] : (T)0;
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const bool in = q + W * (U + u) < len;
@@ -273,7 +273,7 @@ static unsigned mat_grid(const Mat<T>& M) {
 // launch that covers several matrices one after another (the group solve)
 // gives every row exactly the threads and arithmetic of its own launch.
 template <typename T, int SW>
-__device__ __forceinline__ bool row_apply_at(const MatView<T>& M, const T* __restrict__ x, T& out, int64_t& row,
+__device__ __forceinline__ bool row_apply_at(const MatView<T>& M, const T* x, T& out, int64_t& row,
                                              unsigned blk) {
   if constexpr (SW == -2) {
     const int64_t gt = (int64_t)blk * blockDim.x + threadIdx.x;
@@ -330,7 +330,7 @@ __device__ __forceinline__ bool row_apply_at(const MatView<T>& M, const T* __res
 }
 
 template <typename T, int SW>
-__device__ __forceinline__ bool row_apply(const MatView<T>& M, const T* __restrict__ x, T& out, int64_t& row) {
+__device__ __forceinline__ bool row_apply(const MatView<T>& M, const T* x, T& out, int64_t& row) {
   return row_apply_at<T, SW>(M, x, out, row, blockIdx.x);
 }
 
