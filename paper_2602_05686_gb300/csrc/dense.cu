@@ -102,6 +102,17 @@ __device__ __forceinline__ void ch_publish(int* p, int v) {
   asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// handoff between warps of a block without a barrier: the writer's warps meet at
+// a barrier, one thread then releases the count, each reader acquires it
+__device__ __forceinline__ void cta_release(int* p, int v) {
+  asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(p)), "r"(v) : "memory");
+}
+__device__ __forceinline__ int cta_acquire(const int* p) {
+  int v;
+  asm volatile("ld.acquire.cta.shared.s32 %0, [%1];" : "=r"(v) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+  return v;
+}
+
 // s = sqrt(d) and r = 1 / s, both rounded to nearest, for a positive normal d,
 // in integer arithmetic: Newton's iteration for the reciprocal square root of
 // the significand in fixed point (two steps from the FP32 approximation: 2^-60),
@@ -228,7 +239,7 @@ __device__ __forceinline__ void potrf_inv(int bs, double (*T)[NB + 1], double (*
       }
       asm volatile("bar.sync 1, 128;" ::: "memory");
       // column j is written (the barrier): tell the inverse's warps
-      if (threadIdx.x == 32) *(volatile int*)ready = j + 1;
+      if (threadIdx.x == 32) cta_release(ready, j + 1);
     }
   } else {
     // eight lanes per column split each row's dot product; two columns a lane
@@ -237,9 +248,8 @@ __device__ __forceinline__ void potrf_inv(int bs, double (*T)[NB + 1], double (*
       if (m < bs) {
         // (the column warps end without waiting for these; bounded all the same)
         int it = 0;
-        while (*(volatile int*)ready <= m && ++it < (1 << 22)) __nanosleep(20);
+        while (cta_acquire(ready) <= m && ++it < (1 << 22)) __nanosleep(20);
         if (it >= (1 << 22)) atomicOr(err, 2);
-        asm volatile("" ::: "memory");
         double p0 = 0.0, p1 = 0.0;
 #pragma unroll
         for (int t = 0; t < 4; ++t) {

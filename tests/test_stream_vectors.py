@@ -75,3 +75,17 @@ def test_overlapping_kernels_read_vectors_with_plain_loads():
                 if not re.match(r"M\.(v|ci)\b|M \+", v):
                     bad.append(f"{f}: {n}: local const {t}* __restrict__ {p}")
     assert not bad, "\n".join(bad)
+
+
+def test_waits_acquire_what_they_wait_for():
+    """a wait on a flag that announces data acquires it, and the flag is released:
+    a volatile access orders nothing after it"""
+    fs = functions()
+    for name, order in (("potrf_inv", "cta"), ("ch_poll", "gpu"), ("ch_publish", "gpu")):
+        (_, _, _, body), = fs[name]
+        text = body + "".join(b for k in ("cta_release", "cta_acquire") if re.search(rf"\b{k}\b", body)
+                              for *_, b in fs.get(k, ()))
+        assert re.search(rf"(st\.release|ld\.acquire)\.{order}\.", text), name
+        if name == "potrf_inv":
+            assert "volatile int" not in text and f"st.release.{order}.shared" in text
+            assert f"ld.acquire.{order}.shared" in text
