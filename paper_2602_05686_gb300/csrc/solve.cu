@@ -335,8 +335,14 @@ __global__ void k_cg_pupdate(int64_t n, const CgScalars* s, const double* z,
 // the sums of np partials (k columns, or one vector with k = 0) that the
 // producing launch did not finish itself
 int launch_fin_wide(cudaStream_t st, const double* part, int np, const Fin& fin) {
-  if (fin.k > 0) launch_pdl(k_fin_wide<KMAX_BLOCK>, 32, 32 * KMAX_BLOCK, 0, st, part, np, np, fin);
-  else launch_pdl(k_fin_wide<1>, 32, 32, 0, st, part, np, 0, fin);
+  // as many values as the producing launch has columns
+  switch (fin.k) {
+    case 0: launch_pdl(k_fin_wide<1>, 32, 32, 0, st, part, np, 0, fin); break;
+    case 2: launch_pdl(k_fin_wide<2>, 32, 64, 0, st, part, np, np, fin); break;
+    case 4: launch_pdl(k_fin_wide<4>, 32, 128, 0, st, part, np, np, fin); break;
+    case 8: launch_pdl(k_fin_wide<8>, 32, 256, 0, st, part, np, np, fin); break;
+    default: return SA_ERR_INVALID_ARG;
+  }
   SA_LAUNCHED();
   return SA_OK;
 }
