@@ -8,6 +8,21 @@
 
 namespace sa {
 
+// one gathered element of a vector that the stream writes: a coherent load that
+// the compiler keeps behind pdl_sync() and, with the volatile loads of the
+// matrix, in the order of the source (as a plain load that it may move: 1.4 %
+// of a solve on 1.03M FP64 rows and 1.9 % on 1.77M FP32 rows more)
+__device__ __forceinline__ double ldx(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float ldx(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+
 // Row products of one thread: the entries of row i sit 32 apart inside its
 // slice.  Several entries per iteration keep their value / column loads and
 // gathers in flight together (the kernels are latency bound otherwise); the
@@ -36,11 +51,11 @@ __device__ __forceinline__ T sell_row(const int64_t* __restrict__ sp, const int3
       cc[u] = __ldcs(&ci[p + 32 * u]);
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) xx[u] = x[cc[u]];
+    for (int u = 0; u < U; ++u) xx[u] = ldx(x + cc[u]);
 #pragma unroll
     for (int u = 0; u < U; ++u) acc += vv[u] * xx[u];
   }
-  for (; p < e; p += 32) acc += __ldcs(&v[p]) * x[__ldcs(&ci[p])];
+  for (; p < e; p += 32) acc += __ldcs(&v[p]) * ldx(x + __ldcs(&ci[p]));
   return acc;
 }
 
@@ -63,11 +78,11 @@ __device__ __forceinline__ T sell_row16(const int64_t* __restrict__ sp, const in
       cc[u] = __ldcs(&c16[p + 32 * u]);
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) xx[u] = xs[cc[u]];
+    for (int u = 0; u < U; ++u) xx[u] = ldx(xs + cc[u]);
 #pragma unroll
     for (int u = 0; u < U; ++u) acc += vv[u] * xx[u];
   }
-  for (; p < e; p += 32) acc += __ldcs(&v[p]) * xs[__ldcs(&c16[p])];
+  for (; p < e; p += 32) acc += __ldcs(&v[p]) * ldx(xs + __ldcs(&c16[p]));
   return acc;
 }
 
@@ -97,7 +112,7 @@ __device__ __forceinline__ T sell2_lane(const int64_t* __restrict__ sp, const in
   if (full) {
     for (;;) {
 #pragma unroll
-      for (int u = 0; u < U; ++u) xx[u] = xs[cc[u]];
+      for (int u = 0; u < U; ++u) xx[u] = ldx(xs + cc[u]);
 #pragma unroll
       for (int u = 0; u < U; ++u) acc += vv[u] * xx[u];
       p += 64 * U;
@@ -111,7 +126,7 @@ __device__ __forceinline__ T sell2_lane(const int64_t* __restrict__ sp, const in
   }
   for (; p < e; p += 64) {
     const unsigned c = C16 ? (unsigned)__ldcs(&c16[p]) : (unsigned)__ldcs(&ci[p]);
-    acc += __ldcs(&v[p]) * xs[c];
+    acc += __ldcs(&v[p]) * ldx(xs + c);
   }
   return acc;
 }
@@ -182,11 +197,11 @@ __device__ __forceinline__ T csr_lane(const MatView<T>& M, const T* x, int64_t b
         cc[u] = M.ci[q + W * u];
       }
 #pragma unroll
-      for (int u = 0; u < U; ++u) xx[u] = x[cc[u]];
+      for (int u = 0; u < U; ++u) xx[u] = ldx(x + cc[u]);
 #pragma unroll
       for (int u = 0; u < U; ++u) acc += vv[u] * xx[u];
     }
-    for (; q < e; q += W) acc += M.v[q] * x[M.ci[q]];
+    for (; q < e; q += W) acc += M.v[q] * ldx(x + M.ci[q]);
   } else {
     const int len = (int)(e - b);
     const T* __restrict__ v = M.v + b;
@@ -204,7 +219,7 @@ __device__ __forceinline__ T csr_lane(const MatView<T>& M, const T* x, int64_t b
       T xx[U], vn[U];
       int32_t cn[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) xx[u] = q + W * u < len ? x[cc[u]] : (T)0;
+      for (int u = 0; u < U; ++u) xx[u] = q + W * u < len ? ldx(x + cc[u]) : (T)0;
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const bool in = q + W * (U + u) < len;
