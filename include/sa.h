@@ -329,12 +329,13 @@ int sa_solve_group(int m, sa_handle* hs, const double* const* B, double* const* 
  * and for callers that build their own pipeline.  Ordered on `stream`.
  *
  * sa_strength: the per-edge strength filter of Sec. 2.1 / Sec. 3 with
- *   pointwise dropping on CSR (n, row_ptr, col, val).  keep[nnz] receives
+ *   pointwise dropping on CSR (n, row_ptr, col, val), a row's columns in any
+ *   order.  keep[nnz] receives
  *   1 for the diagonal and for kept off-diagonals.  dirichlet[n] (may be
  *   NULL) excludes nodes.  CLASSICAL reads val; MATERIAL reads coords
  *   (n*dim) and sigma_inv (n*kp, inverse nodal tensors); DISTANCE reads
  *   coords only.  Scratch: the MATERIAL/DISTANCE measures need
- *   nnz + n doubles of device scratch, allocated and freed inside the call
+ *   nnz + n doubles and n / 64 bytes of device scratch, allocated and freed inside the call
  *   with cudaMallocAsync on `stream`.
  */
 int sa_strength(sa_measure measure, int dim, int64_t n, int64_t nnz, const int64_t* row_ptr, const int32_t* col,

@@ -1509,8 +1509,10 @@ int sa_strength(sa_measure measure, int dim, int64_t n, int64_t nnz, const int64
       SA_TRY(sa::launch_nodal_tensors(al, dim, n, 0, nullptr, 0, 0, nullptr, nullptr, sg.p, si.p, err.p));
       sinv = si.p;
     }
+    sa::Buf<uint8_t> unsorted;  // the rows need not be in order here
+    SA_TRY(unsorted.alloc(&al, sa::strength_blocks(n)));
     SA_TRY(sa::launch_strength_material(s, dim, n, row_ptr, col, coords, sinv, dirichlet, theta, w.p, D.p, keep,
-                                        cnt.p));
+                                        cnt.p, unsorted.p));
   }
   return SA_OK;
 }

@@ -187,3 +187,49 @@ def test_strength_masks(sa, orc, dim, n, kind):
         assert np.array_equal(kg.cpu().numpy(), ko), theta
         kc = sa.strength("classical", dim, g[0], g[1], g[2], None, None, g[5], theta)
         assert np.array_equal(kc.cpu().numpy(), orc.strength_classical(n, rp, ci, v, dirm, theta)), theta
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("kind", ["all", "one", "descending", "duplicates"])
+@pytest.mark.parametrize("n", [3, 64, 65, 1000])
+def test_strength_of_rows_in_any_order(sa, orc, dim, n, kind):
+    """sa_strength asks for no order of a row's columns: bit for bit the oracle's
+    mask, which takes the entries as they stand; every row shuffled, one row of
+    one 64-row block, descending rows, repeated columns"""
+    import torch
+    rng = np.random.default_rng(7 * dim + n)
+    P = sp.random(n, n, min(1.0, 20.0 / n), random_state=rng, format="csr") + sp.eye(n)
+    P = sp.csr_matrix(P + P.T)
+    P[n // 2, :min(n, 50)] = 1.0  # a row of more than a warp's lanes
+    P = sp.csr_matrix(P)
+    P.sort_indices()
+    rp, ci = P.indptr.astype(np.int64), P.indices.astype(np.int32)
+    v = rng.choice([-1.0, -0.5, 0.25], ci.size)
+    rows = [n // 2] if kind == "one" else range(n)
+    for i in rows:
+        b, e = rp[i], rp[i + 1]
+        o = np.arange(e - b)[::-1] if kind == "descending" else rng.permutation(e - b)
+        ci[b:e] = ci[b:e][o]
+        if kind == "duplicates" and e - b > 2:
+            ci[b + 1] = ci[b]
+    x = rng.random((n, dim))
+    kp = 3 if dim == 2 else 6
+    s = np.zeros((n, kp))
+    s[:, :dim] = 1.0 + rng.random((n, dim))
+    s[:, dim] = 0.2
+    dirm = (rng.random(n) < 0.05).astype(np.uint8)
+    t = lambda a, dt: torch.from_numpy(np.ascontiguousarray(a)).to("cuda", dt)  # noqa: E731
+    g = [t(rp, torch.int64), t(ci, torch.int32), t(v, torch.float64), t(x.ravel(), torch.float64),
+         t(s.ravel(), torch.float64), t(dirm, torch.uint8)]
+    iso = np.zeros((n, kp))
+    iso[:, :dim] = 1.0
+    for theta in (0.05, 0.3):
+        _, _, ko = orc.strength_material(dim, n, rp, ci, dirm, x, s, theta)
+        kg = sa.strength("material", dim, g[0], g[1], None, g[3], g[4], g[5], theta)
+        assert np.array_equal(kg.cpu().numpy(), ko), theta
+        _, _, ko = orc.strength_material(dim, n, rp, ci, dirm, x, iso, theta)
+        kg = sa.strength("distance", dim, g[0], g[1], None, g[3], None, g[5], theta)
+        assert np.array_equal(kg.cpu().numpy(), ko), theta
+        if kind != "duplicates":  # (a repeated diagonal: which of them is the diagonal is not defined)
+            kc = sa.strength("classical", dim, g[0], g[1], g[2], None, None, g[5], theta)
+            assert np.array_equal(kc.cpu().numpy(), orc.strength_classical(n, rp, ci, v, dirm, theta)), theta
