@@ -735,8 +735,8 @@ int run_spgemm(Alloc& al, int64_t n, int64_t m, int64_t kdim, int64_t nnzA, int6
   // products; measured slower than count-then-fill at 27 per row, the
   // smoothed prolongator, where the count pass is cheap) when the
   // upper-bound slots (12 bytes per product) fit in half of the device's free
-  // memory; else count then fill (SA_SPGEMM_PASSES=2 in the environment
-  // forces that, for its tests)
+  // memory and can be had; else count then fill (SA_SPGEMM_PASSES=2 in the
+  // environment forces that, for its tests)
   const char* passes = getenv("SA_SPGEMM_PASSES");
   if ((passes && passes[0] == '2') || per_row < 48.0)
     return spgemm_two_phase(al, n, m, Arp, Aci, Av, Brp, Bci, Bv, Crp, Cci, Cv, nnzC, upper_only, thread_tier);
@@ -755,9 +755,14 @@ int run_spgemm(Alloc& al, int64_t n, int64_t m, int64_t kdim, int64_t nnzA, int6
     cudaGetLastError();
     fr = 0;
   }
-  if (little || (double)ubtot * 12.0 <= 0.5 * (double)fr)
-    return spgemm_one_pass(al, n, m, Arp, Aci, Av, Brp, Bci, Bv, ub.p, ubtot, Crp, Cci, Cv, nnzC, upper_only,
-                           thread_tier);
+  if (little || (double)ubtot * 12.0 <= 0.5 * (double)fr) {
+    const int st = spgemm_one_pass(al, n, m, Arp, Aci, Av, Brp, Bci, Bv, ub.p, ubtot, Crp, Cci, Cv, nnzC, upper_only,
+                                   thread_tier);
+    if (st != SA_ERR_OOM) return st;
+    // the scratch was not to be had (a nearly full device, an allocator's
+    // limit): count then fill does without it
+    SA_TRY(memset_d(Crp.p, 0, Crp.bytes(), s));
+  }
   ub.release();
   return spgemm_two_phase(al, n, m, Arp, Aci, Av, Brp, Bci, Bv, Crp, Cci, Cv, nnzC, upper_only, thread_tier);
 }

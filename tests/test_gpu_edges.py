@@ -233,3 +233,63 @@ def test_strength_of_rows_in_any_order(sa, orc, dim, n, kind):
         if kind != "duplicates":  # (a repeated diagonal: which of them is the diagonal is not defined)
             kc = sa.strength("classical", dim, g[0], g[1], g[2], None, None, g[5], theta)
             assert np.array_equal(kc.cpu().numpy(), orc.strength_classical(n, rp, ci, v, dirm, theta)), theta
+
+
+def test_spgemm_scratch_that_cannot_be_had(sa, gen_mod, monkeypatch):
+    """an allocator that has the memory of the two-phase products but not the
+    one-pass form's scratch: setup falls back and gives the same hierarchy, bit
+    for bit"""
+    import ctypes
+    import torch
+    p = gen_mod.battery_3d(12, 12, 24)
+    t = {k: torch.from_numpy(np.ascontiguousarray(p[k])).cuda() for k in ("row_ptr", "col", "val", "coords")}
+    b = np.random.default_rng(5).standard_normal(p["n"])
+    b[p["dir_mask"] == 1] = 0.0
+    bd = torch.from_numpy(b).cuda()
+    L = sa.lib()
+
+    def run(limit):
+        live, most, refused = {}, [0], [0]
+
+        @sa.api._ALLOC
+        def alloc(nbytes, ctx):
+            if nbytes > limit:
+                refused[0] += 1
+                return None
+            most[0] = max(most[0], int(nbytes))
+            buf = torch.empty(int(nbytes) + 256, dtype=torch.uint8, device="cuda")
+            ptr = (buf.data_ptr() + 255) // 256 * 256
+            live[ptr] = buf
+            return ptr
+
+        @sa.api._FREE
+        def free(ptr, ctx):
+            live.pop(ptr, None)
+
+        o = sa.default_options()
+        o.max_coarse, o.measure = 100, 0
+        o.stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        o.alloc, o.dealloc = alloc, free
+        pr = sa.Problem()
+        pr.dim, pr.n, pr.nnz = 3, p["n"], p["nnz"]
+        pr.row_ptr, pr.col, pr.val = t["row_ptr"].data_ptr(), t["col"].data_ptr(), t["val"].data_ptr()
+        pr.coords = t["coords"].data_ptr()
+        hh = ctypes.c_void_p()
+        assert L.sa_setup(ctypes.byref(pr), ctypes.byref(o), ctypes.byref(hh)) == 0
+        x = torch.zeros_like(bd)
+        info = sa.SolveInfo()
+        assert L.sa_solve(hh, bd.data_ptr(), x.data_ptr(), 1e-8, ctypes.byref(info)) == 0
+        torch.cuda.synchronize()
+        L.sa_free(hh)
+        assert not live
+        return x.cpu(), info.iters, most[0], refused[0]
+
+    one = run(1 << 40)
+    monkeypatch.setenv("SA_SPGEMM_PASSES", "2")
+    two = run(1 << 40)
+    monkeypatch.delenv("SA_SPGEMM_PASSES")
+    assert one[2] > two[2]  # the scratch is the largest request
+    none = run(two[2])
+    assert none[3] > 0
+    for r in (two, none):
+        assert torch.equal(one[0], r[0]) and one[1] == r[1]
