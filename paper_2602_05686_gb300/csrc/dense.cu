@@ -23,6 +23,7 @@
 #include "profile.cuh"
 #include "group.cuh"
 #include "solve.cuh"
+#include "sqrt_rcp.cuh"
 
 namespace sa {
 
@@ -111,75 +112,6 @@ __device__ __forceinline__ int cta_acquire(const int* p) {
   int v;
   asm volatile("ld.acquire.cta.shared.s32 %0, [%1];" : "=r"(v) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
   return v;
-}
-
-// s = sqrt(d) and r = 1 / s, both rounded to nearest, for a positive normal d,
-// in integer arithmetic: Newton's iteration for the reciprocal square root of
-// the significand in fixed point (two steps from the FP32 approximation: 2^-60),
-// then the integer square root and quotient settled by their exact remainders
-// (taken modulo 2^64, where they fit).  No FP64 instruction: a dependent one
-// takes 65 cycles here, and this pair is the chain of a Cholesky pivot (574
-// cycles, 954 as sqrt() and a divide).  Equal to sqrt() and 1.0 / s on 5e8
-// operands of every exponent on the GPU, and on 6e7 on the host with the
-// starting value off by up to four units.
-__device__ __forceinline__ void sqrt_rcp(double d, double& s, double& r) {
-  const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
-  const int ex = (int)(hi >> 20);
-  if (ex == 0 || ex >= 2047) {  // zero exponent, infinity, NaN, negative
-    s = sqrt(d);
-    r = 1.0 / s;
-    return;
-  }
-  // d = m 2^p, p even, m in [2^52, 2^54); mu = m 2^-52 in [1, 4)
-  uint64_t m = (((uint64_t)hi << 32) | lo) & 0xfffffffffffffull | 0x10000000000000ull;
-  int p = ex - 1075;
-  const int odd = p & 1;
-  m <<= odd;
-  p -= odd;
-  const float f = __int_as_float(((127 + odd) << 23) | ((hi & 0xfffff) << 3) | (lo >> 29));
-  float yf;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(f));
-  const uint32_t yb = (uint32_t)__float_as_int(yf);
-  // y in [0.5, 1] as Q0.32
-  uint32_t y0 = yb >= 0x3f800000u ? 0xffffffffu : (((yb & 0x7fffff) | 0x800000) << 8);
-  if (yb < 0x3f000000u) y0 = 0x80000000u;
-  const uint64_t mf = m << 10;  // mu, Q2.62
-  uint64_t t = (uint64_t)y0 * y0;
-  const int64_t e1 = (int64_t)((1ull << 62) - __umul64hi(mf, t));        // 1 - mu y^2, Q.62
-  const uint64_t y1 = ((uint64_t)y0 << 31) + (uint64_t)(((int64_t)(uint64_t)y0 * (int32_t)(e1 >> 12)) >> 20);  // Q1.63
-  t = __umul64hi(y1, y1);
-  const int32_t e2 = (int32_t)((1ull << 60) - __umul64hi(mf, t));        // Q.60
-  const uint64_t y2 = y1 + (uint64_t)(((int64_t)(y1 >> 32) * e2) >> 29);
-  // S = sqrt(m 2^52) rounded: at most one off before the remainder says so
-  uint64_t S = __umul64hi(mf, y2) >> 9;
-  int64_t rem = (int64_t)((m << 52) - S * S);
-  if (rem < 0) {
-    S -= 1;
-    rem += (int64_t)(2 * S + 1);
-  } else if (rem > (int64_t)(2 * S)) {
-    rem -= (int64_t)(2 * S + 1);
-    S += 1;
-  }
-  S += rem > (int64_t)S;
-  const int e = (p - 52) / 2;
-  s = __longlong_as_double((long long)(((uint64_t)(e + 1074) << 52) + S));
-  // Q = 2^105 / S rounded (no ties: 2^106 has no odd factor)
-  uint64_t Q = y2 >> 10;
-  int64_t q = (int64_t)(0 - S * Q);
-#pragma unroll
-  for (int u = 0; u < 2; ++u)
-    if (q < 0) {
-      Q -= 1;
-      q += (int64_t)S;
-    }
-#pragma unroll
-  for (int u = 0; u < 2; ++u)
-    if (q >= (int64_t)S) {
-      Q += 1;
-      q -= (int64_t)S;
-    }
-  Q += 2 * q > (int64_t)S;
-  r = __longlong_as_double((long long)(((uint64_t)(969 - e) << 52) + Q));
 }
 
 // factor the tile in T (rows and columns < bs) in place and form its inverse
