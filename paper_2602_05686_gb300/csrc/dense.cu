@@ -32,6 +32,7 @@ constexpr int CH_THREADS = 256;
 constexpr int CH_STRIP = 16;             // columns of one inverse task
 constexpr int CH_BT = (int)(COARSE_BS / NB);  // tiles per diagonal block
 constexpr uint32_t CH_INV = 0x80000000u;      // task word of an inverse strip
+constexpr int CH_POLLS = 1 << 24;             // about ten seconds; the longest wait is some tasks of 8 us a product
 
 // f[i]: first nonzero tile column of tile row i (at most the diagonal tile):
 // a warp over the tile row's entries, whatever their order
@@ -78,12 +79,13 @@ struct CholView {
   int* flag;             // 1: the tile of L is written; on the diagonal: chunks of its inverse written
   int* ticket;
   int* err;              // 1: pivot not positive; 2: a wait ran out
+  int limit;             // polls of a wait
 };
 
 // bounded wait of one thread for *p >= want: false when it ran out or another
 // wait did
-__device__ bool ch_poll(const int* p, int want, int* err) {
-  for (int it = 0; it < (1 << 24); ++it) {
+__device__ bool ch_poll(const int* p, int want, int limit, int* err) {
+  for (int it = 0; it < limit; ++it) {
     int v;
     asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     if (v >= want) return true;
@@ -258,7 +260,7 @@ __global__ void __launch_bounds__(CH_THREADS) k_chol(CholView C) {
         const int fi = C.f[i];
         double x0 = c0 + c == oi + r ? 1.0 : 0.0, x1 = c0 + c == oi + r + 16 ? 1.0 : 0.0;
         for (int m = fi > jt ? fi : jt; m < i; ++m) {
-          const bool ok = tid != 0 || ch_poll(&C.flag[C.off[i] + m - fi], 1, C.err);
+          const bool ok = tid != 0 || ch_poll(&C.flag[C.off[i] + m - fi], 1, C.limit, C.err);
           if (!__syncthreads_and(ok)) return;
           const int64_t om = (int64_t)m * NB;
           for (int t = tid; t < NB * NB; t += CH_THREADS) {
@@ -281,7 +283,7 @@ __global__ void __launch_bounds__(CH_THREADS) k_chol(CholView C) {
           x1 -= s1;
           buf ^= 1;
         }
-        const bool ok = tid != 0 || ch_poll(&C.flag[C.off[i] + i - fi], CH_CHUNKS, C.err);
+        const bool ok = tid != 0 || ch_poll(&C.flag[C.off[i] + i - fi], CH_CHUNKS, C.limit, C.err);
         if (!__syncthreads_and(ok)) return;
         const double* D = C.Dinv + (int64_t)i * NB * NB;
         for (int t = tid; t < NB * NB; t += CH_THREADS) As[buf][t / NB][t % NB] = __ldcg(&D[t]);
@@ -340,8 +342,8 @@ __global__ void __launch_bounds__(CH_THREADS) k_chol(CholView C) {
     for (int k = diag || fi > fo ? fi : fo; k < jo; ++k) {
       const bool prod = k >= fo;  // (diagonal tasks: the off-diagonal tile's skyline may start later)
       bool ok = true;
-      if (tid == 0) ok = ch_poll(&C.flag[C.off[i] + k - fi], 1, C.err);
-      if (tid == 32 && prod) ok = ch_poll(&C.flag[C.off[jo] + k - fo], 1, C.err);
+      if (tid == 0) ok = ch_poll(&C.flag[C.off[i] + k - fi], 1, C.limit, C.err);
+      if (tid == 32 && prod) ok = ch_poll(&C.flag[C.off[jo] + k - fo], 1, C.limit, C.err);
       if (!__syncthreads_and(ok)) return;
       const int64_t kc = (int64_t)k * NB;
       for (int t = tid; t < NB * NB; t += CH_THREADS) {
@@ -387,7 +389,7 @@ __global__ void __launch_bounds__(CH_THREADS) k_chol(CholView C) {
       const double* D = C.Dinv + (int64_t)jo * NB * NB;
       for (int ch = 0; ch < CH_CHUNKS; ++ch) {
         const int r0 = ch * (NB / CH_CHUNKS);
-        const bool ok = tid != 0 || ch_poll(&C.flag[C.off[jo] + jo - fo], ch + 1, C.err);
+        const bool ok = tid != 0 || ch_poll(&C.flag[C.off[jo] + jo - fo], ch + 1, C.limit, C.err);
         if (!__syncthreads_and(ok)) return;
         Y[r0 + warp][lane] = __ldcg(&D[(r0 + warp) * NB + lane]);
         __syncthreads();
@@ -549,7 +551,7 @@ int dense_start(Alloc& al, int64_t n, const int64_t* rp, const int32_t* ci, cons
   C.n = n; C.nb = nb; C.f = F.sky.p; C.off = F.sky.p + 2 * nb;
   C.task = reinterpret_cast<const uint32_t*>(F.sky.p + 3 * nb + 1); C.ntask = (int)nt;
   C.M = F.L.p; C.LT = F.LT.p; C.W = F.W.p; C.WT = F.WT.p; C.Dinv = job.Dinv.p;
-  C.flag = job.flag.p; C.ticket = job.err.p + 1; C.err = job.err.p;
+  C.flag = job.flag.p; C.ticket = job.err.p + 1; C.err = job.err.p; C.limit = CH_POLLS;
   // one block per SM where the chain of diagonal tiles is the time (a second
   // block takes FP64 issue from it: 2210 rows, 41 products a tile column, 3.3
   // against 3.8 ms), two where the products are (1039 rows, 48 a column, 3.9
