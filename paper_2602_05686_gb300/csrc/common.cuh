@@ -108,15 +108,23 @@ inline unsigned warp_rows_grid(int64_t rows, int block = 256) {
 
 // Programmatic dependent launch: a kernel launched by launch_pdl may start while
 // its predecessor in the stream drains, and waits in pdl_sync() for that
-// predecessor's completion before it touches anything the stream writes (it
-// may read matrices built before the solve earlier).  Its lifetime overlaps the
-// predecessor's, so what the stream writes -- vectors, CG scalars, partial sums
-// -- is not read-only data in it: such pointers carry no __restrict__ and are
-// read with plain loads after pdl_sync(); __ldg, ld.global.nc and const
-// __restrict__ are for matrices, scalings and launch descriptors.  The trigger follows the
-// wait, so no kernel starts before the one before its predecessor has ended.
-// Every kernel launched this way calls pdl_sync() first.  The launches of one
-// V-cycle on small levels are 2 to 4 us of work with 1.3 us between them.
+// predecessor's completion.  The trigger follows the wait, so no kernel starts
+// before the one before its predecessor has ended.  What a kernel launched this
+// way has to keep to:
+// - Before its wait a thread reads only what was complete two launches (or a
+//   copy) earlier: matrices, row pointers, factors and launch descriptors, read
+//   ahead by the row kernels.  A kernel that builds such data is therefore
+//   followed by another launch before the first that reads it early.
+// - Whatever the stream's solves write -- vectors, CG scalars, partial sums -- is
+//   touched after the wait only.  The predecessor may still write it while this
+//   kernel is alive, so it is not read-only data: such pointers carry no
+//   __restrict__ and are read with plain loads; __ldg, ld.global.nc and const
+//   __restrict__ are for matrices, scalings and descriptors.
+// - At least one thread of the grid waits (threads and blocks without a row of
+//   their own may leave at once): the grid's end then still follows its
+//   predecessor's, which the kernel after it relies on.
+// The launches of one V-cycle on small levels are 2 to 4 us of work with 1.3 us
+// between them.
 template <typename... P, typename... A>
 inline void launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
   cudaLaunchConfig_t c = {};

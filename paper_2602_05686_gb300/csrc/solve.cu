@@ -236,6 +236,8 @@ int run_power_op(Alloc& al, int64_t n, int steps, uint32_t tag, uint32_t seed, d
   fin.tick = reinterpret_cast<unsigned*>(sc.p + 5);
   fin.sc = sc.p;
   fin.lam = lam_dev;
+  // (these two launches also stand between the kernels that built the operator
+  // and its first product, which reads it before its wait)
   k_start_vector<<<blocks_for(n, 256), 256, 0, st>>>(n, tag, seed, x.p);
   SA_LAUNCHED();
   double* X = x.p;

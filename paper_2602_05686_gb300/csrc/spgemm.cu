@@ -1,13 +1,15 @@
-// Two-phase (count, then fill) sparse matrix product C = A B used for the
-// smoothed prolongator (A_F P^, Sec. 2.2) and the Galerkin product (R (A P),
-// Sec. 2).  Three tiers by the row's distinct column count: one thread per
-// row with a sorted column list in shared memory (narrow products, e.g. the
-// aggregation prolongators with one to a few entries per row), then one warp
-// per row with an open-addressing hash table of column indices in shared
-// memory.  The fill phase sorts the row's columns
-// and accumulates each entry's products in ascending order of the A column
+// Sparse matrix product C = A B used for the smoothed prolongator (A_F P^,
+// Sec. 2.2) and the Galerkin product (R (A P), Sec. 2), in two phases (count,
+// then fill) or in one pass into slots sized by the rows' product counts, packed
+// afterwards.  Three tiers by the row's distinct column count: one thread per
+// row (narrow products, e.g. the aggregation prolongators with one to a few
+// entries per row) with a sorted column list in shared memory (two phases) or a
+// hash table of its own (one pass: rows of up to TCAP columns leave in table
+// order and the packing ranks them); then one warp per row with a hash table of
+// column indices in shared memory, whose fill sorts the row's columns.  Every
+// entry's products are accumulated in ascending order of the A column
 // (the order of Gustavson's row algorithm), with separately rounded multiply
-// and add, so the values do not depend on scheduling.  Rows whose distinct
+// and add, so the values do not depend on scheduling or form.  Rows whose distinct
 // column count exceeds the table go to a block-per-row path with a dense
 // accumulator in global scratch memory.
 #include <stdlib.h>
@@ -23,6 +25,8 @@ namespace sa {
 // resident (shared memory per warp is what limits the tiers)
 constexpr int HB = 256;             // hash slots per warp
 constexpr int HCAP = 192;           // max distinct columns on the warp path
+static_assert(HB <= 256, "hslot gives 8 bits; slots and ranks are stored in bytes");
+static_assert(HCAP + 32 < HB, "a round of 32 insertions is made before the count is checked");
 constexpr int SG_WARPS = 4;         // warps per CTA
 constexpr int BIG_THREADS = 512;
 
@@ -560,6 +564,7 @@ __global__ void k_spgemm_pcount(int64_t n, const int64_t* __restrict__ Arp, cons
 // rows from their upper-bound slots to the packed CSR (a warp per row); rows of
 // up to 32 columns are ranked on the way (the thread tier leaves them in table
 // order), longer ones come sorted
+static_assert(TCAP <= 32, "the packing ranks the thread tier's rows by one warp");
 __global__ void k_spgemm_compact(int64_t n, const int64_t* __restrict__ ub, const int32_t* __restrict__ uci,
                                  const double* __restrict__ uv, const int64_t* __restrict__ Crp,
                                  int32_t* __restrict__ Cci, double* __restrict__ Cv) {
