@@ -407,8 +407,10 @@ def setup_roofline(phases_ms, sizes, peak):
         ms = phases_ms.get("dense")
         if ms:
             fl = nL ** 3 / 3.0
-            out["dense"] = {"ms": ms, "flops": fl, "TFLOPs": round(fl / (ms * 1e-3) / 1e12, 4),
-                            "note": "coarse Cholesky factor (n_L^3/3), overlapped with other setup work"}
+            out["dense"] = {"ms": ms, "flops": fl,
+                            "note": "coarse Cholesky factor, overlapped with other setup work; flops of a dense "
+                                    "factor (n_L^3/3): this one skips the tiles outside its skyline, so they give "
+                                    "no rate"}
     return out
 
 

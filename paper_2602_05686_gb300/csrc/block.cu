@@ -800,7 +800,7 @@ static int mv_block(VHier<T>* m, cudaStream_t st, int l, int K, const double* r6
   const int nl = (int)m->lev.size();
   const int64_t n = L->n, nk = n * K;
   if (l == nl - 1) {
-    int pi = prof_begin(st, PK_B_COARSE, l, 8.0 * n * n + 48.0 * n * K);
+    int pi = prof_begin(st, PK_B_COARSE, l, 8.0 * m->cf.entries + 48.0 * n * K);
     launch_pdl(k_bcoarse_in<T>, g256(nk), 256, 0, st, n, K, L->kb.p, L->sq.p, m->kct.p);
     SA_LAUNCHED();
     SA_TRY(launch_coarse_solve(st, K, coarse_prob(m->cf, m->kct.p, m->kcs.p, m->kcy.p, m->kcx.p, L->sq.p, L->kx.p,

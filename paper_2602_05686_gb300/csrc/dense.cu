@@ -517,7 +517,7 @@ int dense_start(Alloc& al, int64_t n, const int64_t* rp, const int32_t* ci, cons
   // (pageable source: the copy has left it when the call returns)
   SA_TRY(copy_h2d(F.sky.p, tab.data(), sizeof(int32_t) * tab.size(), s));
   F.steps.clear();  // the solve's steps
-  coarse_steps(n, tab.data(), tab.data() + nb, F.steps);
+  F.entries = coarse_steps(n, tab.data(), tab.data() + nb, F.steps);
   SA_TRY(memset_d(job.flag.p, 0, job.flag.bytes(), s));
   // L^T rows are read up to the last tile row that reaches them; tiles of
   // that range outside another row's skyline stay zero
@@ -730,7 +730,7 @@ __global__ void __launch_bounds__(CS_THREADS) k_g_coarse(const CoarseEnt* __rest
 }
 
 // the steps of one problem's solve, in order
-void coarse_steps(int64_t n, const int32_t* first, const int32_t* end, std::vector<CoarseEnt>& out) {
+double coarse_steps(int64_t n, const int32_t* first, const int32_t* end, std::vector<CoarseEnt>& out) {
   const int nbk = (int)((n + COARSE_BS - 1) / COARSE_BS);
   auto push = [&](int mode, int64_t rb, int64_t re, int64_t r0, int64_t r1, int64_t split) {
     if (re <= rb) return;
@@ -756,6 +756,20 @@ void coarse_steps(int64_t n, const int32_t* first, const int32_t* end, std::vect
     push(CS_LT, sk, r1, r0, r1, n);
     push(CS_WT, r0, r1, r0, r1, sk);
   }
+  double read = 0.0;
+  for (const CoarseEnt& E : out) {
+    const int64_t rows = E.re - E.rb;
+    if (E.mode == CS_W || E.mode == CS_WT) {
+      read += 0.5 * (double)rows * (double)(rows + 1);
+      continue;
+    }
+    for (int64_t i = E.rb; i < E.re; ++i) {
+      const int64_t in = E.mode == CS_L ? E.r0 - (int64_t)first[i / NB] * NB
+                                        : ((int64_t)end[i / NB] * NB < n ? (int64_t)end[i / NB] * NB : n) - E.r1;
+      read += in > 0 ? (double)in : 0.0;
+    }
+  }
+  return read;
 }
 
 int coarse_blocks(const CoarseEnt& E) { return (E.re - E.rb + CS_ROWS - 1) / CS_ROWS; }

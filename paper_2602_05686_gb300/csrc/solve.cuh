@@ -74,6 +74,7 @@ struct CoarseFactor {
   // own tables
   Buf<int32_t> sky;
   std::vector<CoarseEnt> steps;  // of the solve
+  double entries = 0;            // matrix entries that one solve reads
 };
 
 struct CoarseView {
@@ -85,6 +86,7 @@ struct CoarseView {
   const int32_t* first = nullptr;  // skyline: first tile column per tile row
   const int32_t* end = nullptr;    // ... and end of the tile rows per tile column
   const std::vector<CoarseEnt>* steps = nullptr;  // host (the factor's)
+  double entries = 0;
 };
 
 inline CoarseView coarse_view(const CoarseFactor& F, int64_t n) {
@@ -92,6 +94,7 @@ inline CoarseView coarse_view(const CoarseFactor& F, int64_t n) {
   v.n = n; v.L = F.L.p; v.LT = F.LT.p; v.W = F.W.p; v.WT = F.WT.p;
   v.first = F.sky.p; v.end = F.sky.p + (n + 31) / 32;
   v.steps = &F.steps;
+  v.entries = F.entries;
   return v;
 }
 
@@ -136,9 +139,10 @@ int dense_start(Alloc& al, int64_t n, const int64_t* rp, const int32_t* ci, cons
 int dense_finish(DenseJob& job);
 // one solve with k in {1, 2, 4, 8} interleaved columns
 int launch_coarse_solve(cudaStream_t st, int k, const CoarseProb& P);
-// the steps of one solve (first, end: the skyline on the host); one step of
-// several problems in one launch (entries in the order of their blocks)
-void coarse_steps(int64_t n, const int32_t* first, const int32_t* end, std::vector<CoarseEnt>& out);
+// the steps of one solve (first, end: the skyline on the host), and the matrix
+// entries they read; one step of several problems in one launch (entries in the
+// order of their blocks)
+double coarse_steps(int64_t n, const int32_t* first, const int32_t* end, std::vector<CoarseEnt>& out);
 int coarse_blocks(const CoarseEnt& E);
 int launch_coarse_group(cudaStream_t st, const CoarseEnt* ent, int nent, int blocks, const CoarseProb* probs);
 

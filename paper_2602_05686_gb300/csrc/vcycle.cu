@@ -524,7 +524,7 @@ static int mv(VHier<T>* m, cudaStream_t st, int l, const double* r64, T** xo) {
   const int nl = (int)m->lev.size();
   const int64_t n = L->n;
   if (l == nl - 1) {
-    int pi = prof_begin(st, PK_COARSE, l, 8.0 * n * n + 48.0 * n);
+    int pi = prof_begin(st, PK_COARSE, l, 8.0 * m->cf.entries + 48.0 * n);
     launch_pdl(k_coarse_in<T>, g256(n), 256, 0, st, n, L->b.p, L->sq.p, m->ct.p);
     SA_LAUNCHED();
     SA_TRY(launch_coarse_solve(st, 1, coarse_prob(m->cf, m->ct.p, m->cs.p, m->cy.p, m->cx.p, L->sq.p, L->x.p,
@@ -590,7 +590,7 @@ int vh_vcycle(VHier<T>* m, cudaStream_t st, const double* r, double** z) {
   if (m->lev.size() == 1) {
     // one level: the dense solve on r directly
     const int64_t n = m->lev[0]->n;
-    int pi = prof_begin(st, PK_COARSE, 0, 8.0 * n * n + 32.0 * n);
+    int pi = prof_begin(st, PK_COARSE, 0, 8.0 * m->cf.entries + 32.0 * n);
     int s = launch_coarse_solve(st, 1, coarse_prob(m->cf, r, m->cs.p, m->cy.p, m->z.p));
     prof_end(st, pi);
     SA_TRY(s);

@@ -293,3 +293,23 @@ def test_spgemm_scratch_that_cannot_be_had(sa, gen_mod, monkeypatch):
     assert none[3] > 0
     for r in (two, none):
         assert torch.equal(one[0], r[0]) and one[1] == r[1]
+
+
+@pytest.mark.parametrize("n", [100, 1100])
+def test_coarse_solve_bytes_are_the_entries_it_reads(sa, n):
+    """the profile's algorithmic bytes of a coarse solve: the diagonal blocks'
+    triangles twice, and of the rows between blocks the tiles inside the skyline
+    (bandwidth 40: two tile rows reach back 64 and 32 columns, two tile columns
+    forward 32 and 64)"""
+    import torch
+    A = coarse_matrix(n, "band", np.random.default_rng(1))
+    h = sa.Hierarchy(problem(A), measure="material", max_coarse=5000)
+    b = torch.from_numpy(np.random.default_rng(2).standard_normal(n)).cuda()
+    sa.profile_enable(True)
+    h.vcycle(b)
+    rows = [r for r in sa.profile_read() if r["kind"] == "coarse"]
+    sa.profile_enable(False)
+    tri = n * (n + 1) if n <= 1024 else 1024 * 1025 + (n - 1024) * (n - 1023)
+    between = 0 if n <= 1024 else 2 * (32 * 64 + 32 * 32)
+    assert len(rows) == 1 and rows[0]["launches"] == 1
+    assert rows[0]["bytes"] == 8.0 * (tri + between) + 32.0 * n
