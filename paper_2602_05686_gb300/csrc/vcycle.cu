@@ -391,10 +391,17 @@ template int vh_build<float>(Alloc&, const VLevelIn*, int, int, const CoarseView
 // resident blocks per SM asked of the compiler: FP32 rows of several lanes
 // gain from occupancy (6 blocks, 40 registers: 370k rows of 60 entries 55.7 ->
 // 52.3 us), FP64 ones at 5 (183k rows of 46 entries: 51.4 us at 4 blocks, 47.6
-// at 5, 47.0 at 6; 6.9k rows of 128: 21.3, 21.2, 23.7)
+// at 5, 47.0 at 6; 6.9k rows of 128: 21.3, 21.2, 23.7).  One-thread rows, SELL
+// and CSR: 8 (32 registers).  Prolongation to 1.06M FP64 rows 22.5 us, 24.6 at 6
+// blocks, 51 unbounded (84 registers); 1.77M FP32 rows 26.6, 30.7, 40.1;
+// Chebyshev step on 1.06M FP64 SELL rows 66.5 us, 92.8 unbounded.  (The one-lane
+// CSR form spills 100 to 180 bytes in its long-row path for it.)  Two-lane SELL
+// rows hold a round across the wait: 6 blocks, nothing spilled (69k FP64 rows
+// 12.45 -> 11.8 us, 54k FP32 rows 19.0 -> 15.3, against 8 blocks and 24 to 52
+// bytes of spills).
 template <typename T, int SW>
 struct VOcc {
-  static constexpr int B = SW > 1 ? (sizeof(T) == 4 ? 6 : 5) : 8;
+  static constexpr int B = SW > 1 ? (sizeof(T) == 4 ? 6 : 5) : (SW == -2 ? 6 : 8);
 };
 
 // x_out = x_in + d,  d = first ? c2 r : c1 d + c2 r,  r = b - A~ x_in

@@ -88,8 +88,10 @@ __device__ __forceinline__ T sell_row16(const int64_t* __restrict__ sp, const in
 
 // SELL-32 with two lanes per row: lanes 2r and 2r+1 of a warp take the even
 // and the odd entries of row r of the slice (16 rows per warp), each summed in
-// entry order; one shuffle adds the two
-template <typename T, bool C16, int U = RowUnroll<T>::U>
+// entry order; one shuffle adds the two.  Rounds of four in both types: a round
+// is held across the wait, and eight FP32 entries of it spilled (275k rows: 21.9
+// us a Chebyshev step at 32 registers, 19.8 at 40; four 18.3)
+template <typename T, bool C16, int U = 4>
 __device__ __forceinline__ T sell2_lane(const int64_t* __restrict__ sp, const int32_t* __restrict__ base,
                                         const uint16_t* __restrict__ c16, const int32_t* __restrict__ ci,
                                         const T* __restrict__ v, const T* x, int64_t sl, int r, int h) {
