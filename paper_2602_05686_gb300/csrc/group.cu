@@ -62,7 +62,7 @@ __device__ __forceinline__ void g_mat_row(int op, const GMat<T>& D, unsigned blk
 
 // All formats in one body take the registers of the largest: 106 in FP64
 // unbounded, two blocks per SM.  4 blocks in FP64 (64 registers, no spills), 6 in
-// FP32 (40; what spills is the several-lane rounds): sixteen problems, FP64,
+// FP32 (40, with spills): sixteen problems, FP64,
 // 11.3 -> 10.2 ms unbounded -> 4 blocks, twenty smaller ones 14.3 -> 12.6; FP32
 // 9.3 -> 9.0 and 11.4 -> 10.9 at 6 blocks, 9.2 and 11.3 at 4.  (FP64 at 6 blocks:
 // 10.15 and 12.4, but four larger problems 2.47 -> 2.50.)
