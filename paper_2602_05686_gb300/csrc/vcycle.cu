@@ -396,12 +396,13 @@ template int vh_build<float>(Alloc&, const VLevelIn*, int, int, const CoarseView
 // blocks, 51 unbounded (84 registers); 1.77M FP32 rows 26.6, 30.7, 40.1;
 // Chebyshev step on 1.06M FP64 SELL rows 66.5 us, 92.8 unbounded.  (The one-lane
 // CSR form spills 100 to 180 bytes in its long-row path for it.)  Two-lane SELL
-// rows hold a round across the wait: 6 blocks, nothing spilled (69k FP64 rows
-// 12.45 -> 11.8 us, 54k FP32 rows 19.0 -> 15.3, against 8 blocks and 24 to 52
-// bytes of spills).
+// rows, which hold a round across the wait: 8 in FP64, since the next kernel's
+// blocks come in beside this one's (66k rows of 9 entries, a solve: 2.65 ms; 2.67 at
+// 6 with rounds of four; 69k rows of 27, a Chebyshev step: 11.8 us both), 6 in FP32 (54k rows
+// 15.3 us, 17.5 at 8 blocks; 275k rows 18.3 and 17.4).
 template <typename T, int SW>
 struct VOcc {
-  static constexpr int B = SW > 1 ? (sizeof(T) == 4 ? 6 : 5) : (SW == -2 ? 6 : 8);
+  static constexpr int B = SW > 1 ? (sizeof(T) == 4 ? 6 : 5) : (SW == -2 && sizeof(T) == 4 ? 6 : 8);
 };
 
 // x_out = x_in + d,  d = first ? c2 r : c1 d + c2 r,  r = b - A~ x_in

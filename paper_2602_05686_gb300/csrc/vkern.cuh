@@ -88,10 +88,11 @@ __device__ __forceinline__ T sell_row16(const int64_t* __restrict__ sp, const in
 
 // SELL-32 with two lanes per row: lanes 2r and 2r+1 of a warp take the even
 // and the odd entries of row r of the slice (16 rows per warp), each summed in
-// entry order; one shuffle adds the two.  Rounds of four in both types: a round
-// is held across the wait, and eight FP32 entries of it spilled (275k rows: 21.9
-// us a Chebyshev step at 32 registers, 19.8 at 40; four 18.3)
-template <typename T, bool C16, int U = 4>
+// entry order; one shuffle adds the two.  Rounds of three (FP64) or four (FP32):
+// a round is held across the wait, and four FP64 or eight FP32 entries of it
+// spilled at 32 registers (275k rows, Chebyshev step: FP64 28.6 -> 27.4 us, FP32
+// 21.9 -> 18.3)
+template <typename T, bool C16, int U = sizeof(T) == 4 ? 4 : 3>
 __device__ __forceinline__ T sell2_lane(const int64_t* __restrict__ sp, const int32_t* __restrict__ base,
                                         const uint16_t* __restrict__ c16, const int32_t* __restrict__ ci,
                                         const T* __restrict__ v, const T* x, int64_t sl, int r, int h) {
