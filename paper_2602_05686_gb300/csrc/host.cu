@@ -189,7 +189,7 @@ static int coarsen(sa_handle h, int l, int* err, int* stop) {
   SA_TRY(vF.alloc(&al, nnzF));
   SA_TRY(Dt.alloc(&al, n));
   const uint8_t* keep_p = o.keep_setup_data ? L.keep.p : keep.p;
-  SA_TRY(launch_filter(s, n, L.rp.p, L.ci.p, L.v.p, keep_p, rpF.p, ciF.p, vF.p, Dt.p));
+  SA_TRY(launch_filter(s, n, nnz, L.rp.p, L.ci.p, L.v.p, keep_p, rpF.p, ciF.p, vF.p, Dt.p));
   PHASE_END(PK_S_FILTER);
 
   // a11: omega = omega_sym / rho(D~^-1 A_F)

@@ -29,7 +29,7 @@ int launch_strength_material(cudaStream_t s, int dim, int64_t n, const int64_t* 
 int launch_cut_drop(Alloc& al, int measure_classical, int64_t n, int64_t nnz, const int64_t* rp, const int32_t* ci,
                     const double* v, const double* diag, const double* w, const double* D, const uint8_t* dir,
                     double theta, uint8_t* keep, int64_t* cnt);
-int launch_filter(cudaStream_t s, int64_t n, const int64_t* rp, const int32_t* ci, const double* v,
+int launch_filter(cudaStream_t s, int64_t n, int64_t nnz, const int64_t* rp, const int32_t* ci, const double* v,
                   const uint8_t* keep, const int64_t* rpF, int32_t* ciF, double* vF, double* Dt);
 int launch_coarse_aux(cudaStream_t s, int64_t nc, int dim, const int64_t* mrp, const int32_t* mlist,
                       const double* x, const double* sigma, double* xc, double* sc, double* sic);

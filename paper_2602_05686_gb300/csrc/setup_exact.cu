@@ -659,48 +659,33 @@ __global__ void k_cut_symmetrize(int64_t n, const int64_t* __restrict__ rp, cons
 // Thread per row: the three ordered sums are sequential FP64 chains, so one
 // warp instruction advances 32 rows.  The block's rows are one segment of the
 // CSR arrays, copied to shared memory first: three passes over rows 216 bytes
-// apart cost each warp load 32 lines of a cache that 64 warps shared (192^3
-// inclusions, average of the levels: 1.09 ms, 0.89 ms staged).  A segment above
-// FILT_CAP entries is read in place.
+// apart cost each warp load 32 lines of a cache that 64 warps shared (2.1M rows of
+// 27 entries: 785 us, 480 us staged).  Levels of longer rows, and short ones of
+// coarse 3D rows, read in place (109k rows of 59 entries: 117 us; staged, with
+// most blocks above the buffer, 377).  Rows of up to 12 entries on average take a
+// third of the buffer, for residency (160k rows of 9: 22.9 us in the larger one, 18.8).  A block above
+// its buffer reads in place too, by a copy of the row loop whose pointers stay
+// global and read-only.
 constexpr int FILT_ROWS = 64;
-constexpr int FILT_CAP = 2048;
-__global__ void __launch_bounds__(FILT_ROWS) k_filter(int64_t n, const int64_t* __restrict__ rp,
-                                                      const int32_t* __restrict__ ci, const double* __restrict__ v,
-                                                      const uint8_t* __restrict__ keep,
-                                                      const int64_t* __restrict__ rpF, int32_t* __restrict__ ciF,
-                                                      double* __restrict__ vF, double* __restrict__ Dt) {
-  __shared__ double s_v[FILT_CAP];
-  __shared__ int32_t s_c[FILT_CAP];
-  __shared__ uint8_t s_k[FILT_CAP];
-  const int64_t i0 = (int64_t)blockIdx.x * FILT_ROWS, i1 = i0 + FILT_ROWS < n ? i0 + FILT_ROWS : n;
-  const int64_t i = i0 + threadIdx.x;
-  const int64_t b0 = rp[i0], tot = rp[i1] - b0;
-  const double* V = v + b0;
-  const int32_t* C = ci + b0;
-  const uint8_t* K = keep + b0;
-  if (tot <= FILT_CAP) {
-    for (int p = (int)threadIdx.x; p < (int)tot; p += FILT_ROWS) {
-      s_v[p] = V[p];
-      s_c[p] = C[p];
-      s_k[p] = K[p];
-    }
-    __syncthreads();
-    V = s_v;
-    C = s_c;
-    K = s_k;
-  }
-  if (i >= n) return;
-  const int64_t b = rp[i] - b0, e = rp[i + 1] - b0;
+constexpr int FILT_CAP = 2048, FILT_CAP_SHORT = 768;
+constexpr int64_t FILT_MEAN = 27, FILT_SMALL = 4096;
+
+// row i, entries [b, e) of V, C, K
+template <typename I>
+__device__ __forceinline__ void filter_row(int64_t i, I b, I e, const double* __restrict__ V,
+                                           const int32_t* __restrict__ C, const uint8_t* __restrict__ K,
+                                           const int64_t* __restrict__ rpF, int32_t* __restrict__ ciF,
+                                           double* __restrict__ vF, double* __restrict__ Dt) {
   // lumped diagonal: a_ii, then the dropped entries in ascending order
   double dg = 0.0;
-  for (int64_t p = b; p < e; ++p)
+  for (I p = b; p < e; ++p)
     if (C[p] == (int32_t)i) dg = V[p];
-  for (int64_t p = b; p < e; ++p)
+  for (I p = b; p < e; ++p)
     if (C[p] != (int32_t)i && !K[p]) dg += V[p];
   // the filtered row and both 1-norms in ascending order
   int64_t out = rpF[i];
   double s = 0.0, a1 = 0.0;
-  for (int64_t p = b; p < e; ++p) {
+  for (I p = b; p < e; ++p) {
     const int32_t j = C[p];
     const double a = V[p];
     a1 += fabs(a);
@@ -713,6 +698,33 @@ __global__ void __launch_bounds__(FILT_ROWS) k_filter(int64_t n, const int64_t* 
     }
   }
   Dt[i] = (s <= 1e-12 * a1) ? INFINITY : s;
+}
+
+template <int CAP>
+__global__ void __launch_bounds__(FILT_ROWS) k_filter(int64_t n, const int64_t* __restrict__ rp,
+                                                      const int32_t* __restrict__ ci, const double* __restrict__ v,
+                                                      const uint8_t* __restrict__ keep,
+                                                      const int64_t* __restrict__ rpF, int32_t* __restrict__ ciF,
+                                                      double* __restrict__ vF, double* __restrict__ Dt) {
+  const int64_t i0 = (int64_t)blockIdx.x * FILT_ROWS, i1 = i0 + FILT_ROWS < n ? i0 + FILT_ROWS : n;
+  const int64_t i = i0 + threadIdx.x;
+  if constexpr (CAP > 0) {
+    __shared__ double s_v[CAP];
+    __shared__ int32_t s_c[CAP];
+    __shared__ uint8_t s_k[CAP];
+    const int64_t b0 = rp[i0], tot = rp[i1] - b0;
+    if (tot <= CAP) {
+      for (int p = (int)threadIdx.x; p < (int)tot; p += FILT_ROWS) {
+        s_v[p] = v[b0 + p];
+        s_c[p] = ci[b0 + p];
+        s_k[p] = keep[b0 + p];
+      }
+      __syncthreads();
+      if (i < n) filter_row<int>(i, (int)(rp[i] - b0), (int)(rp[i + 1] - b0), s_v, s_c, s_k, rpF, ciF, vF, Dt);
+      return;
+    }
+  }
+  if (i < n) filter_row<int64_t>(i, rp[i], rp[i + 1], v, ci, keep, rpF, ciF, vF, Dt);
 }
 
 // ---------------------------------------------------------------------------
@@ -867,10 +879,16 @@ int launch_cut_drop(Alloc& al, int measure_classical, int64_t n, int64_t nnz, co
   return SA_OK;
 }
 
-int launch_filter(cudaStream_t s, int64_t n, const int64_t* rp, const int32_t* ci, const double* v,
+int launch_filter(cudaStream_t s, int64_t n, int64_t nnz, const int64_t* rp, const int32_t* ci, const double* v,
                   const uint8_t* keep, const int64_t* rpF, int32_t* ciF, double* vF, double* Dt) {
   if (n <= 0) return SA_OK;
-  k_filter<<<blocks_for(n, FILT_ROWS), FILT_ROWS, 0, s>>>(n, rp, ci, v, keep, rpF, ciF, vF, Dt);
+  const unsigned g = blocks_for(n, FILT_ROWS);
+  if (nnz <= n * (FILT_CAP_SHORT / FILT_ROWS))
+    k_filter<FILT_CAP_SHORT><<<g, FILT_ROWS, 0, s>>>(n, rp, ci, v, keep, rpF, ciF, vF, Dt);
+  else if (nnz <= n * FILT_MEAN && n >= FILT_SMALL)
+    k_filter<FILT_CAP><<<g, FILT_ROWS, 0, s>>>(n, rp, ci, v, keep, rpF, ciF, vF, Dt);
+  else
+    k_filter<0><<<g, FILT_ROWS, 0, s>>>(n, rp, ci, v, keep, rpF, ciF, vF, Dt);
   SA_LAUNCHED();
   return SA_OK;
 }
