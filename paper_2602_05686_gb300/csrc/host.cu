@@ -114,7 +114,7 @@ static int coarsen(sa_handle h, int l, int* err, int* stop) {
   SA_TRY(rpF.alloc(&al, n + 1));
   SA_TRY(memset_d(rpF.p, 0, sizeof(int64_t), s));
   if (!aux) {
-    SA_TRY(launch_strength_classical(s, n, L.rp.p, L.ci.p, L.v.p, L.diag.p, dir, o.theta, keep.p, rpF.p));
+    SA_TRY(launch_strength_classical(s, n, nnz, L.rp.p, L.ci.p, L.v.p, L.diag.p, dir, o.theta, keep.p, rpF.p));
     if (o.drop == SA_DROP_CUT)
       SA_TRY(launch_cut_drop(al, 1, n, nnz, L.rp.p, L.ci.p, L.v.p, L.diag.p, nullptr, nullptr, dir, o.theta, keep.p,
                              rpF.p));
@@ -122,7 +122,7 @@ static int coarsen(sa_handle h, int l, int* err, int* stop) {
     Buf<double> w, D;
     SA_TRY(w.alloc(&al, nnz));
     SA_TRY(D.alloc(&al, n));
-    SA_TRY(launch_strength_material(s, h->dim, n, L.rp.p, L.ci.p, L.x.p, L.sinv.p, dir, o.theta, w.p, D.p, keep.p,
+    SA_TRY(launch_strength_material(s, h->dim, n, nnz, L.rp.p, L.ci.p, L.x.p, L.sinv.p, dir, o.theta, w.p, D.p, keep.p,
                                     rpF.p));
     if (o.drop == SA_DROP_CUT)
       SA_TRY(launch_cut_drop(al, 0, n, nnz, L.rp.p, L.ci.p, nullptr, nullptr, w.p, D.p, dir, o.theta, keep.p, rpF.p));
@@ -1494,7 +1494,7 @@ int sa_strength(sa_measure measure, int dim, int64_t n, int64_t nnz, const int64
     SA_TRY(err.alloc(&al, 1));
     SA_TRY(sa::memset_d(err.p, 0, sizeof(int), s));
     SA_TRY(sa::launch_dirichlet_diag(s, n, row_ptr, col, val, nullptr, diag.p, err.p));
-    SA_TRY(sa::launch_strength_classical(s, n, row_ptr, col, val, diag.p, dirichlet, theta, keep, cnt.p));
+    SA_TRY(sa::launch_strength_classical(s, n, nnz, row_ptr, col, val, diag.p, dirichlet, theta, keep, cnt.p));
   } else {
     sa::Buf<double> w, D, si, sg;
     sa::Buf<int> err;
@@ -1510,8 +1510,8 @@ int sa_strength(sa_measure measure, int dim, int64_t n, int64_t nnz, const int64
       sinv = si.p;
     }
     sa::Buf<uint8_t> unsorted;  // the rows need not be in order here
-    SA_TRY(unsorted.alloc(&al, sa::strength_blocks(n)));
-    SA_TRY(sa::launch_strength_material(s, dim, n, row_ptr, col, coords, sinv, dirichlet, theta, w.p, D.p, keep,
+    SA_TRY(unsorted.alloc(&al, sa::strength_blocks(n, nnz)));
+    SA_TRY(sa::launch_strength_material(s, dim, n, nnz, row_ptr, col, coords, sinv, dirichlet, theta, w.p, D.p, keep,
                                         cnt.p, unsorted.p));
   }
   return SA_OK;

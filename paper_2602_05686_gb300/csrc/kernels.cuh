@@ -16,12 +16,12 @@ int launch_dirichlet_diag(cudaStream_t s, int64_t n, const int64_t* rp, const in
                           uint8_t* dir, double* diag, int* err);
 int launch_nodal_tensors(Alloc& al, int dim, int64_t n, int tloc, const double* tensors, int64_t ne, int npe,
                          const int32_t* en, const double* meas, double* sigma, double* sinv, int* err);
-int launch_strength_classical(cudaStream_t s, int64_t n, const int64_t* rp, const int32_t* ci, const double* v,
+int launch_strength_classical(cudaStream_t s, int64_t n, int64_t nnz, const int64_t* rp, const int32_t* ci, const double* v,
                               const double* diag, const uint8_t* dir, double theta, uint8_t* keep, int64_t* cnt);
 // unsorted: NULL where every row's columns ascend strictly, else scratch of
-// strength_blocks(n) bytes (rows in any order)
-int64_t strength_blocks(int64_t n);
-int launch_strength_material(cudaStream_t s, int dim, int64_t n, const int64_t* rp, const int32_t* ci,
+// strength_blocks(n, nnz) bytes (rows in any order)
+int64_t strength_blocks(int64_t n, int64_t nnz);
+int launch_strength_material(cudaStream_t s, int dim, int64_t n, int64_t nnz, const int64_t* rp, const int32_t* ci,
                              const double* x, const double* sinv, const uint8_t* dir, double theta, double* w,
                              double* D, uint8_t* keep, int64_t* cnt, uint8_t* unsorted = nullptr);
 // cut-drop (replaces the pointwise mask in keep and the counts in cnt[i+1]);

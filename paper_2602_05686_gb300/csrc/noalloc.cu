@@ -74,6 +74,6 @@ extern "C" int sa_strength_material_noalloc(int dim, int64_t n, int64_t nnz, con
   }
   // w in [0, nnz), D in [nnz, nnz + n); both are fully written before they
   // are read, so nothing has to be cleared between calls
-  return sa::launch_strength_material(s, dim, n, row_ptr, col, coords, sigma_inv, dirichlet, theta, scratch,
+  return sa::launch_strength_material(s, dim, n, nnz, row_ptr, col, coords, sigma_inv, dirichlet, theta, scratch,
                                       scratch + nnz, keep, nullptr);
 }

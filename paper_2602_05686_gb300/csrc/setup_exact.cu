@@ -195,20 +195,31 @@ __device__ __forceinline__ double quad_form(int dim, const double* __restrict__ 
 // material region), q_ji = q_ij and its twelve instructions are left out.
 // 2.1M nodes, 64 Voronoi regions: 1733 us with a thread per row; coarse
 // levels of the stretched battery stack: 251 us on average with a warp per row
-constexpr int PAIR_ROWS = 64;
+// Rows of a block: 64, or 8 on small levels of long rows, where blocks of 64 leave
+// the chip idle and one long row holds up 63 (both kernels; start: a warp per row):
+//   44k rows of 29 entries   137 us, 250 at 64, 99 at 8
+//   6.6k rows of 117          71 us, 131 at 64, 59 at 8
+//   73k rows of 44           285 us, 226 at 64, 176 at 8
+//   131k rows of 26          307 us, 154 at 64, 194 at 8
+//   16k rows of 10            30 us,  17 at 64,  21 at 8
 constexpr int PAIR_THREADS = 256;
 
-// pair numbering of the block's rows r0 .. r0 + PAIR_ROWS - 1: the entries
+// a level of few rows that are long (coarse 3D levels): a row's work is then spread
+// over a warp or a block of few rows
+constexpr int64_t FEW_ROWS = 65536, LONG_MEAN = 24;
+inline bool few_long_rows(int64_t n, int64_t nnz) { return n < FEW_ROWS && nnz > LONG_MEAN * n; }
+
+// pair numbering of the block's rows r0 .. r0 + ROWS - 1: the entries
 // above (UPPER) or below the diagonal of row r0 + r are start[r] + 0, 1, ...
 // and pairs off[r] .. off[r + 1] - 1
-template <bool UPPER>
+template <bool UPPER, int ROWS>
 __device__ __forceinline__ void pair_offsets(int64_t n, const int64_t* __restrict__ rp,
                                              const int32_t* __restrict__ ci, int64_t r0, int64_t* start, int* off,
                                              double* __restrict__ w) {
   __shared__ int wsum;
   const int t = (int)threadIdx.x, lane = t & 31;
   int cnt = 0;
-  if (t < PAIR_ROWS) {
+  if (t < ROWS) {
     const int64_t i = r0 + t;
     int64_t st = 0;
     if (i < n) {
@@ -235,23 +246,24 @@ __device__ __forceinline__ void pair_offsets(int64_t n, const int64_t* __restric
   }
   if (t == 31) wsum = inc;
   __syncthreads();
-  if (t < PAIR_ROWS) off[t + 1] = inc + (t >= 32 ? wsum : 0);
+  if (t < ROWS) off[t + 1] = inc + (t >= 32 ? wsum : 0);
   if (t == 0) off[0] = 0;
   __syncthreads();
 }
 
 // whether a row of the block is not strictly ascending: a descent between
 // neighbouring entries that is not the step from one row to the next
+template <int ROWS>
 __device__ __forceinline__ bool pair_unsorted(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
                                               int64_t r0) {
-  __shared__ int64_t rs[PAIR_ROWS + 1];
+  __shared__ int64_t rs[ROWS + 1];
   const int t = (int)threadIdx.x;
-  if (t <= PAIR_ROWS) rs[t] = rp[r0 + t < n ? r0 + t : n];
+  if (t <= ROWS) rs[t] = rp[r0 + t < n ? r0 + t : n];
   __syncthreads();
   bool bad = false;
-  for (int64_t p = rs[0] + t; p + 1 < rs[PAIR_ROWS]; p += PAIR_THREADS) {
+  for (int64_t p = rs[0] + t; p + 1 < rs[ROWS]; p += PAIR_THREADS) {
     if (ci[p] < ci[p + 1]) continue;
-    int lo = 0, hi = PAIR_ROWS;  // the last row start <= p + 1
+    int lo = 0, hi = ROWS;  // the last row start <= p + 1
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
       if (rs[mid] <= p + 1) lo = mid;
@@ -263,10 +275,11 @@ __device__ __forceinline__ bool pair_unsorted(int64_t n, const int64_t* __restri
 }
 
 // the row (of the block) that pair q belongs to
+template <int ROWS>
 __device__ __forceinline__ int pair_row(const int* off, int q) {
-  int lo = 0, hi = PAIR_ROWS - 1;
+  int lo = 0, hi = ROWS - 1;
 #pragma unroll
-  for (int s = 0; s < 6; ++s) {
+  for (int s = 1; s < ROWS; s *= 2) {
     const int mid = (lo + hi + 1) >> 1;
     if (off[mid] <= q) lo = mid;
     else hi = mid - 1;
@@ -301,29 +314,29 @@ __device__ __forceinline__ double pair_weight(const double* __restrict__ x, cons
 // row out of order takes every entry of its rows by the expression and says so
 // in `unsorted`, and the mirror leaves it alone.  The check reads the columns'
 // lower half besides (strength filter on 2.1M nodes 2656 -> 2666 us).
-template <int DIM, bool CHECK>
+template <int DIM, bool CHECK, int ROWS>
 __global__ void __launch_bounds__(PAIR_THREADS) k_material_w(int64_t n, const int64_t* __restrict__ rp,
                                                              const int32_t* __restrict__ ci,
                                                              const double* __restrict__ x,
                                                              const double* __restrict__ sinv, double* __restrict__ w,
                                                              uint8_t* __restrict__ unsorted) {
-  __shared__ int64_t start[PAIR_ROWS];
-  __shared__ int off[PAIR_ROWS + 1];
-  const int64_t r0 = (int64_t)blockIdx.x * PAIR_ROWS;
+  __shared__ int64_t start[ROWS];
+  __shared__ int off[ROWS + 1];
+  const int64_t r0 = (int64_t)blockIdx.x * ROWS;
   if constexpr (CHECK) {
-    const bool any = pair_unsorted(n, rp, ci, r0);
+    const bool any = pair_unsorted<ROWS>(n, rp, ci, r0);
     if (threadIdx.x == 0) unsorted[blockIdx.x] = any;
     if (any) {
-      for (int64_t i = r0 + (threadIdx.x >> 5); i < r0 + PAIR_ROWS && i < n; i += PAIR_THREADS / 32)
+      for (int64_t i = r0 + (threadIdx.x >> 5); i < r0 + ROWS && i < n; i += PAIR_THREADS / 32)
         for (int64_t p = rp[i] + lane_id(); p < rp[i + 1]; p += 32)
           w[p] = ci[p] == (int32_t)i ? 0.0 : pair_weight<DIM>(x, sinv, i, ci[p]);
       return;
     }
   }
-  pair_offsets<true>(n, rp, ci, r0, start, off, w);
-  const int tot = off[PAIR_ROWS];
+  pair_offsets<true, ROWS>(n, rp, ci, r0, start, off, w);
+  const int tot = off[ROWS];
   for (int q = (int)threadIdx.x; q < tot; q += PAIR_THREADS) {
-    const int r = pair_row(off, q);
+    const int r = pair_row<ROWS>(off, q);
     const int64_t p = start[r] + (q - off[r]);
     w[p] = pair_weight<DIM>(x, sinv, r0 + r, ci[p]);
   }
@@ -333,20 +346,20 @@ __global__ void __launch_bounds__(PAIR_THREADS) k_material_w(int64_t n, const in
 // entry len - 1 - k of row j, which is tried first, then a binary search in
 // row j; a pattern without that entry (not structurally symmetric) gets w_ij
 // computed here by the same expression.
-template <int DIM>
+template <int DIM, int ROWS>
 __global__ void __launch_bounds__(PAIR_THREADS) k_material_w_mirror(int64_t n, const int64_t* __restrict__ rp,
                                                                     const int32_t* __restrict__ ci,
                                                                     const double* __restrict__ x,
                                                                     const double* __restrict__ sinv, double* w,
                                                                     const uint8_t* __restrict__ unsorted) {
   if (unsorted && unsorted[blockIdx.x]) return;
-  __shared__ int64_t start[PAIR_ROWS];
-  __shared__ int off[PAIR_ROWS + 1];
-  const int64_t r0 = (int64_t)blockIdx.x * PAIR_ROWS;
-  pair_offsets<false>(n, rp, ci, r0, start, off, w);
-  const int tot = off[PAIR_ROWS];
+  __shared__ int64_t start[ROWS];
+  __shared__ int off[ROWS + 1];
+  const int64_t r0 = (int64_t)blockIdx.x * ROWS;
+  pair_offsets<false, ROWS>(n, rp, ci, r0, start, off, w);
+  const int tot = off[ROWS];
   for (int q = (int)threadIdx.x; q < tot; q += PAIR_THREADS) {
-    const int r = pair_row(off, q);
+    const int r = pair_row<ROWS>(off, q);
     const int k = q - off[r];
     const int64_t p = start[r] + k, i = r0 + r;
     const int32_t j = ci[p];
@@ -430,13 +443,13 @@ __device__ __forceinline__ int keep_entry(double wv, double t2, double Di, doubl
 // a3 / a4: the pointwise criterion, diagonal kept, Dirichlet nodes excluded;
 // kept entries per row (diagonal included) into cnt[i+1].
 // A warp takes KEEP_ROWS consecutive rows at a time, their loads together (one
-// row after another was a chain of dependent loads: 458 us), the entries past
-// the 32nd of a row after them.  ABS: the classical measure, |a_ij| and
-// |a_ii a_jj| in place of w and D (192^3 inclusions, average of the levels:
-// 677 us by a kernel of its own, 674 us by this one: bound by the entries' bytes
-// and the gathered diagonal, not by the comparison).
-constexpr int KEEP_ROWS = 4;
-template <bool ABS>
+// row after another was a chain of dependent loads), the entries past the 32nd of
+// a row after them: four rows (1.06M rows of 26 entries 195 us, 268 a row at a
+// time), or one on small levels of long rows, whose further entries then go four
+// a lane together (6.6k rows of 117: 18 us a row at a time, 38 by fours, 12 so; in the
+// large levels' kernel that form's registers cost 250 against 195 us).  ABS: the
+// classical measure, |a_ij| and |a_ii a_jj| in place of w and D.
+template <bool ABS, int KEEP_ROWS>
 __global__ void __launch_bounds__(256) k_keep(int64_t n, const int64_t* __restrict__ rp,
                                                        const int32_t* __restrict__ ci, const double* __restrict__ w,
                                                        const double* __restrict__ D, const uint8_t* __restrict__ dir,
@@ -482,12 +495,39 @@ __global__ void __launch_bounds__(256) k_keep(int64_t n, const int64_t* __restri
         const int64_t i = i0 + u;
         const bool diri = dir && dir[i];
         int c = 0;
-        for (int64_t p = b[u] + 32 + lane; p < e[u]; p += 32) {
-          const int32_t jj = ci[p];
-          const int k = jj == (int32_t)i ? 1 : keep_entry(keep_arg<ABS>(w[p]), t2, Di[u], keep_arg<ABS>(D[jj]),
-                                                           diri || (dir && dir[jj]));
-          keep[p] = (uint8_t)k;
-          c += k;
+        if constexpr (KEEP_ROWS == 1) {
+          // four entries a lane, their loads together
+          for (int64_t p = b[u] + 32 + lane; p < e[u]; p += 128) {
+            int32_t jj[4];
+            double wt[4], Dt[4];
+            bool dt[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+              const bool in = p + 32 * v < e[u];
+              jj[v] = in ? ci[p + 32 * v] : -1;
+              wt[v] = in ? keep_arg<ABS>(w[p + 32 * v]) : 0.0;
+            }
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+              Dt[v] = jj[v] >= 0 ? keep_arg<ABS>(D[jj[v]]) : 0.0;
+              dt[v] = diri || (dir && jj[v] >= 0 && dir[jj[v]]);
+            }
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+              if (jj[v] >= 0) {
+                const int k = jj[v] == (int32_t)i ? 1 : keep_entry(wt[v], t2, Di[u], Dt[v], dt[v]);
+                keep[p + 32 * v] = (uint8_t)k;
+                c += k;
+              }
+          }
+        } else {
+          for (int64_t p = b[u] + 32 + lane; p < e[u]; p += 32) {
+            const int32_t jj = ci[p];
+            const int k = jj == (int32_t)i ? 1 : keep_entry(keep_arg<ABS>(w[p]), t2, Di[u], keep_arg<ABS>(D[jj]),
+                                                             diri || (dir && dir[jj]));
+            keep[p] = (uint8_t)k;
+            c += k;
+          }
         }
         kept[u] += __reduce_add_sync(FULL, c);
       }
@@ -788,7 +828,7 @@ int launch_dirichlet_diag(cudaStream_t s, int64_t n, const int64_t* rp, const in
   return SA_OK;
 }
 
-int64_t strength_blocks(int64_t n) { return (int64_t)blocks_for(n, PAIR_ROWS); }
+int64_t strength_blocks(int64_t n, int64_t nnz) { return (int64_t)blocks_for(n, few_long_rows(n, nnz) ? 8 : 64); }
 
 int launch_validate_csr(cudaStream_t s, int64_t n, int64_t ncols, int64_t nnz, const int64_t* rp, const int32_t* ci,
                         int* err) {
@@ -825,38 +865,51 @@ int launch_nodal_tensors(Alloc& al, int dim, int64_t n, int tloc, const double* 
   return SA_OK;
 }
 
-int launch_strength_classical(cudaStream_t s, int64_t n, const int64_t* rp, const int32_t* ci, const double* v,
-                              const double* diag, const uint8_t* dir, double theta, uint8_t* keep,
-                              int64_t* cnt) {
-  if (n <= 0) return SA_OK;
-  const double t2 = theta * theta;
-  k_keep<true><<<warp_rows_grid((n + KEEP_ROWS - 1) / KEEP_ROWS), 256, 0, s>>>(n, rp, ci, v, diag, dir, t2, keep, cnt);
+template <bool ABS>
+static int launch_keep(cudaStream_t s, int64_t n, int64_t nnz, const int64_t* rp, const int32_t* ci, const double* w,
+                       const double* D, const uint8_t* dir, double t2, uint8_t* keep, int64_t* cnt) {
+  if (few_long_rows(n, nnz)) k_keep<ABS, 1><<<warp_rows_grid(n), 256, 0, s>>>(n, rp, ci, w, D, dir, t2, keep, cnt);
+  else k_keep<ABS, 4><<<warp_rows_grid((n + 3) / 4), 256, 0, s>>>(n, rp, ci, w, D, dir, t2, keep, cnt);
   SA_LAUNCHED();
   return SA_OK;
 }
 
-int launch_strength_material(cudaStream_t s, int dim, int64_t n, const int64_t* rp, const int32_t* ci,
+int launch_strength_classical(cudaStream_t s, int64_t n, int64_t nnz, const int64_t* rp, const int32_t* ci, const double* v,
+                              const double* diag, const uint8_t* dir, double theta, uint8_t* keep,
+                              int64_t* cnt) {
+  if (n <= 0) return SA_OK;
+  const double t2 = theta * theta;
+  return launch_keep<true>(s, n, nnz, rp, ci, v, diag, dir, t2, keep, cnt);
+}
+
+template <int DIM, int ROWS>
+static int launch_pairs_rows(cudaStream_t s, int64_t n, const int64_t* rp, const int32_t* ci, const double* x,
+                             const double* sinv, double* w, uint8_t* unsorted) {
+  const unsigned g = blocks_for(n, ROWS);
+  if (unsorted) k_material_w<DIM, true, ROWS><<<g, PAIR_THREADS, 0, s>>>(n, rp, ci, x, sinv, w, unsorted);
+  else k_material_w<DIM, false, ROWS><<<g, PAIR_THREADS, 0, s>>>(n, rp, ci, x, sinv, w, nullptr);
+  SA_LAUNCHED();
+  k_material_w_mirror<DIM, ROWS><<<g, PAIR_THREADS, 0, s>>>(n, rp, ci, x, sinv, w, unsorted);
+  SA_LAUNCHED();
+  return SA_OK;
+}
+template <int DIM>
+static int launch_pairs(cudaStream_t s, int64_t n, int64_t nnz, const int64_t* rp, const int32_t* ci, const double* x,
+                        const double* sinv, double* w, uint8_t* unsorted) {
+  return few_long_rows(n, nnz) ? launch_pairs_rows<DIM, 8>(s, n, rp, ci, x, sinv, w, unsorted)
+                               : launch_pairs_rows<DIM, 64>(s, n, rp, ci, x, sinv, w, unsorted);
+}
+
+int launch_strength_material(cudaStream_t s, int dim, int64_t n, int64_t nnz, const int64_t* rp, const int32_t* ci,
                              const double* x, const double* sinv, const uint8_t* dir, double theta,
                              double* w, double* D, uint8_t* keep, int64_t* cnt, uint8_t* unsorted) {
   if (n <= 0) return SA_OK;
   const double t2 = theta * theta;
-  const unsigned g = blocks_for(n, PAIR_ROWS);
-  if (unsorted) {
-    if (dim == 3) k_material_w<3, true><<<g, PAIR_THREADS, 0, s>>>(n, rp, ci, x, sinv, w, unsorted);
-    else k_material_w<2, true><<<g, PAIR_THREADS, 0, s>>>(n, rp, ci, x, sinv, w, unsorted);
-  } else {
-    if (dim == 3) k_material_w<3, false><<<g, PAIR_THREADS, 0, s>>>(n, rp, ci, x, sinv, w, nullptr);
-    else k_material_w<2, false><<<g, PAIR_THREADS, 0, s>>>(n, rp, ci, x, sinv, w, nullptr);
-  }
-  SA_LAUNCHED();
-  if (dim == 3) k_material_w_mirror<3><<<g, PAIR_THREADS, 0, s>>>(n, rp, ci, x, sinv, w, unsorted);
-  else k_material_w_mirror<2><<<g, PAIR_THREADS, 0, s>>>(n, rp, ci, x, sinv, w, unsorted);
-  SA_LAUNCHED();
+  if (dim == 3) SA_TRY(launch_pairs<3>(s, n, nnz, rp, ci, x, sinv, w, unsorted));
+  else SA_TRY(launch_pairs<2>(s, n, nnz, rp, ci, x, sinv, w, unsorted));
   k_row_sum_ordered<<<blocks_for(n, 128), 128, 0, s>>>(n, rp, w, D);
   SA_LAUNCHED();
-  k_keep<false><<<warp_rows_grid((n + KEEP_ROWS - 1) / KEEP_ROWS), 256, 0, s>>>(n, rp, ci, w, D, dir, t2, keep, cnt);
-  SA_LAUNCHED();
-  return SA_OK;
+  return launch_keep<false>(s, n, nnz, rp, ci, w, D, dir, t2, keep, cnt);
 }
 
 int launch_cut_drop(Alloc& al, int measure_classical, int64_t n, int64_t nnz, const int64_t* rp, const int32_t* ci,

@@ -313,3 +313,38 @@ def test_coarse_solve_bytes_are_the_entries_it_reads(sa, n):
     between = 0 if n <= 1024 else 2 * (32 * 64 + 32 * 32)
     assert len(rows) == 1 and rows[0]["launches"] == 1
     assert rows[0]["bytes"] == 8.0 * (tri + between) + 32.0 * n
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("n", [25, 32, 33, 161, 200])
+@pytest.mark.parametrize("order", ["ascending", "any"])
+def test_strength_of_few_long_rows(sa, orc, dim, n, order):
+    """small levels of long rows (a warp per row, blocks of eight rows): dense and
+    half-dense rows of 25 to 200 entries, bit for bit the oracle's masks"""
+    import torch
+    rng = np.random.default_rng(11 * dim + n)
+    for density in (1.0, 0.6 if n > 60 else 1.0):
+        P = sp.csr_matrix((rng.random((n, n)) < density) | np.eye(n, dtype=bool))
+        P = sp.csr_matrix(P + P.T)
+        P.sort_indices()
+        rp, ci = P.indptr.astype(np.int64), P.indices.astype(np.int32)
+        assert ci.size > 24 * n
+        if order == "any":
+            for i in range(n):
+                ci[rp[i]:rp[i + 1]] = rng.permutation(ci[rp[i]:rp[i + 1]])
+        v = rng.choice([-1.0, -0.5, 0.25, 0.0, -0.0], ci.size)
+        v[ci == np.repeat(np.arange(n), np.diff(rp))] = rng.choice([1.0, -1.0], n)
+        x = rng.random((n, dim))
+        kp = 3 if dim == 2 else 6
+        s = np.zeros((n, kp))
+        s[:, :dim] = 1.0 + rng.integers(0, 3, (n, dim))
+        dirm = (rng.random(n) < 0.05).astype(np.uint8)
+        t = lambda a, dt: torch.from_numpy(np.ascontiguousarray(a)).to("cuda", dt)  # noqa: E731
+        g = [t(rp, torch.int64), t(ci, torch.int32), t(v, torch.float64), t(x.ravel(), torch.float64),
+             t(s.ravel(), torch.float64), t(dirm, torch.uint8)]
+        for theta in (0.0, 0.01, 0.25):
+            _, _, ko = orc.strength_material(dim, n, rp, ci, dirm, x, s, theta)
+            kg = sa.strength("material", dim, g[0], g[1], None, g[3], g[4], g[5], theta)
+            assert np.array_equal(kg.cpu().numpy(), ko), theta
+            kc = sa.strength("classical", dim, g[0], g[1], g[2], None, None, g[5], theta)
+            assert np.array_equal(kc.cpu().numpy(), orc.strength_classical(n, rp, ci, v, dirm, theta)), theta
