@@ -658,8 +658,11 @@ __device__ __forceinline__ double block_sum_256(double c) {
 // q = A p, partial sums of p.q per CTA (fixed order); INLINE: the last block
 // finishes them.  Bound by FP64 issue: 1.8M rows of 27 entries 123 us with a
 // butterfly in every warp, 107 us with block_sum_256; 7.2M rows 448, 403 us.
+// Eight blocks per SM (32 registers): finishing inline took 38, six blocks, and
+// 275k rows a second wave of a few blocks (39 us, 31 at eight; 1.77M rows 106.6 ->
+// 105.3).
 template <bool INLINE>
-__global__ void __launch_bounds__(256) k_sell_spmv_dot(int64_t n, const int64_t* __restrict__ sp, const int32_t* __restrict__ ci,
+__global__ void __launch_bounds__(256, 8) k_sell_spmv_dot(int64_t n, const int64_t* __restrict__ sp, const int32_t* __restrict__ ci,
                                 const int32_t* __restrict__ base, const uint16_t* __restrict__ c16,
                                 const double* __restrict__ v, const double* p, double* __restrict__ q,
                                 double* __restrict__ part, Fin fin) {
