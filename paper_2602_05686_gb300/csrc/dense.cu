@@ -611,9 +611,14 @@ constexpr int CS_SEG = 4;       // column segments of a row
 constexpr int CS_ROWS = 4;      // rows of a block, a warp each
 constexpr int CS_THREADS = CS_ROWS * 32;
 
-template <int K>
+// entries per segment loaded together; four columns take two on levels of up to
+// CS_SHORT rows (175 rows 14.7 us a solve, 17.0 with four) and four above (39.9 us,
+// 31.7 with four, 35.3 as a block per row)
+constexpr int coarse_pf(int K) { return K == 1 ? 8 : (K == 2 ? 4 : 2); }
+constexpr int64_t CS_SHORT = 512;
+
+template <int K, int PF = coarse_pf(K)>
 __device__ __forceinline__ void coarse_rows(const CoarseEnt& E, const CoarseProb& P, unsigned blk) {
-  constexpr int PF = K == 1 ? 8 : (K == 2 ? 4 : 2);  // entries per segment loaded together
   const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = (int)P.n;
   const int i = E.rb + (int)blk * CS_ROWS + warp;
@@ -711,9 +716,9 @@ __device__ __forceinline__ void coarse_rows(const CoarseEnt& E, const CoarseProb
   }
 }
 
-template <int K>
+template <int K, int PF = coarse_pf(K)>
 __global__ void __launch_bounds__(CS_THREADS) k_coarse(CoarseEnt E, CoarseProb P) {
-  coarse_rows<K>(E, P, blockIdx.x);
+  coarse_rows<K, PF>(E, P, blockIdx.x);
 }
 
 // the same step of several problems (group solve): blocks blk0 ... of entry k
@@ -788,7 +793,10 @@ int launch_coarse_solve(cudaStream_t st, int k, const CoarseProb& P) {
     switch (k) {
       case 1: launch_pdl(k_coarse<1>, g, CS_THREADS, 0, st, E, P); break;
       case 2: launch_pdl(k_coarse<2>, g, CS_THREADS, 0, st, E, P); break;
-      case 4: launch_pdl(k_coarse<4>, g, CS_THREADS, 0, st, E, P); break;
+      case 4:
+        if (P.n > CS_SHORT) launch_pdl(k_coarse<4, 4>, g, CS_THREADS, 0, st, E, P);
+        else launch_pdl(k_coarse<4>, g, CS_THREADS, 0, st, E, P);
+        break;
       case 8: launch_pdl(k_coarse<8>, g, CS_THREADS, 0, st, E, P); break;
       default: return SA_ERR_INVALID_ARG;
     }
