@@ -1,4 +1,6 @@
-"""Registers of the row kernels whose only path would pay for spills."""
+"""Registers that the row kernels' residency depends on, and spills where a kernel
+has no other path."""
+import functools
 import importlib
 import os
 import re
@@ -16,6 +18,7 @@ def ptxas(tmp_path_factory):
     except RuntimeError:
         pytest.skip("no nvcc")
 
+    @functools.lru_cache
     def get(name):
         r = subprocess.run([nvcc, *build.ARCH, *build.NVCC_FLAGS, "-Xptxas", "-v", "-c",
                             os.path.join(build.CSRC, name + ".cu"), "-o",
@@ -37,3 +40,9 @@ def test_sell_rows_spill_nothing(ptxas):
 def test_group_rows_leave_room_for_four_blocks(ptxas):
     (spilled, regs), = [v for k, v in ptxas("group").items() if "k_g_matId" in k]
     assert spilled == 0 and regs <= 64
+
+
+def test_outer_product_keeps_eight_blocks(ptxas):
+    # 65536 registers / (8 x 256 threads)
+    regs = [n for k, (_, n) in ptxas("vcycle").items() if "k_sell_spmv_dot" in k]
+    assert len(regs) == 2 and max(regs) <= 32
