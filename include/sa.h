@@ -153,6 +153,9 @@ int sa_default_options(sa_options* o);
  * smoother and coarse-solve data.  *out receives the handle on SA_OK and is
  * NULL otherwise.  Blocks the calling thread until setup has finished
  * (sizes are read back between steps).
+ * The coarse factor and solve leave out tiles outside the factor's skyline: a
+ * non-finite value in one component of a disconnected coarsest level (of the
+ * matrix or of a right-hand side) need not reach the other components.
  */
 int sa_setup(const sa_problem* prob, const sa_options* opt, sa_handle* out);
 
