@@ -1,4 +1,5 @@
 // Primitives: status text, stream-ordered allocation, prefix sums.
+#include <cuda.h>
 #include <stdio.h>
 #include <string.h>
 
@@ -93,24 +94,52 @@ int num_sms() {
 
 // Readbacks of sizes and flags land in a small pinned buffer of the calling
 // thread (4 KB, released with the thread): a copy to pageable memory goes
-// through the driver's staging, and a setup makes a few hundred.
+// through the driver's staging, and a setup makes a few hundred.  Pinned memory
+// belongs to a context and goes with it (a device reset), so a thread keeps one
+// buffer per context id (an id names one context for the life of the process);
+// past PIN_CONTEXTS of them, or without the driver's call, copies are pageable.
 namespace {
 constexpr size_t PIN_BYTES = 4096;
+constexpr int PIN_CONTEXTS = 8;
+
+// id of the current context, 0 if it cannot be had
+unsigned long long context_id() {
+  using Fn = CUresult (*)(CUcontext, unsigned long long*);
+  static const Fn fn = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<Fn>(f);
+  }();
+  unsigned long long id = 0;
+  return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
 struct ThreadPin {
-  void* p = nullptr;
-  bool tried = false;
+  unsigned long long id[PIN_CONTEXTS] = {};
+  void* p[PIN_CONTEXTS] = {};
+  int n = 0;
   ~ThreadPin() {
-    if (p) cudaFreeHost(p);
+    const unsigned long long now = n > 0 ? context_id() : 0;
+    for (int k = 0; k < n; ++k)
+      if (p[k] && id[k] == now) cudaFreeHost(p[k]);  // (of another context: freed with that)
   }
   unsigned char* get() {
-    if (!tried) {
-      tried = true;
-      if (cudaMallocHost(&p, PIN_BYTES) != cudaSuccess) {
-        cudaGetLastError();
-        p = nullptr;
-      }
+    const unsigned long long now = context_id();
+    if (!now) return nullptr;
+    for (int k = 0; k < n; ++k)
+      if (id[k] == now) return static_cast<unsigned char*>(p[k]);
+    if (n == PIN_CONTEXTS) return nullptr;
+    id[n] = now;
+    if (cudaMallocHost(&p[n], PIN_BYTES) != cudaSuccess) {
+      cudaGetLastError();
+      p[n] = nullptr;
     }
-    return static_cast<unsigned char*>(p);
+    return static_cast<unsigned char*>(p[n++]);
   }
 };
 thread_local ThreadPin t_pin;
