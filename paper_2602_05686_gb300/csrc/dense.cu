@@ -553,10 +553,18 @@ int dense_start(Alloc& al, int64_t n, const int64_t* rp, const int32_t* ci, cons
   C.M = F.L.p; C.LT = F.LT.p; C.W = F.W.p; C.WT = F.WT.p; C.Dinv = job.Dinv.p;
   C.flag = job.flag.p; C.ticket = job.err.p + 1; C.err = job.err.p; C.limit = CH_POLLS;
   // one block per SM where the chain of diagonal tiles is the time (a second
-  // block takes FP64 issue from it: 2210 rows, 41 products a tile column, 3.3
-  // against 3.8 ms), two where the products are (1039 rows, 48 a column, 3.9
-  // against 4.4 ms; 3989 rows, 410 a column, 18 against 27 ms)
-  const int64_t g = (nprod < 45 * (int64_t)nb ? 1 : 2) * (int64_t)num_sms();
+  // block takes FP64 issue from it), two from 200 tile products per SM on.  Bands
+  // and dense skylines of 512 to 5000 rows and 18 coarse levels, one against two:
+  //   2744 rows,  8 products per SM     2.9, 3.5 ms
+  //   2900 rows, 32                     4.6, 5.9
+  //   3002 rows, 80                     6.6, 7.2
+  //   1883 rows, 151                    5.5, 6.1
+  //   3000 rows, 203                    8.4, 7.7
+  //   4017 rows, 292                   21.6, 14.4
+  //   5000 rows, 510                   16.7, 14.3
+  // (Against it: 3 % of 3.7 ms at 1022 rows and 6 products, 3 to 9 % at 2000 and
+  // 2500 dense rows, 249 and 500.)
+  const int64_t g = (nprod < 200 * (int64_t)num_sms() ? 1 : 2) * (int64_t)num_sms();
   k_chol<<<(unsigned)(nt < g ? nt : g), CH_THREADS, 0, m>>>(C);
   SA_LAUNCHED();
   prof_end(m, ph);
